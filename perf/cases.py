@@ -132,7 +132,8 @@ def _starts(counts):
     return cu
 
 
-def prepare(case, seed):
+def _inputs(case, seed):
+    """Everything that a turn is given, drawn from the seed alone; and the two generators, for what follows the draft."""
     D = SHAPES[case["shape"]]
     op, B, k = case["op"], case["batch"], case["k"]
     host = torch.Generator().manual_seed(seed)                       # lengths and accept counts
@@ -154,31 +155,46 @@ def prepare(case, seed):
     if case["project"]:
         W["resid_proj"] = normal(d, d, std=0.02)
     T = _lengths(case, host)
-    extra = 1 + (k - 1) * case["topk"] if op == "tree" else k
-    dr = Drafter(D, W, max_batch=B, max_len=max(T) + 2 * k + 2 + extra, max_k=max(8, k))
-    del W
-    st = {"op": op, "B": B, "k": k, "drafter": dr, "resid": normal(4, d, std=0.02)}
-    cu = _starts([t + 1 for t in T])
-    ids, hidden = tokens(cu[-1]), normal(cu[-1], d)
-    if op == "open":
-        cu = _starts(T)
-        st.update(ids=ids[:cu[-1]], hidden=hidden[:cu[-1]], cu=cu, start=[0] * B)
-        return st
-    # rows [0, T) of every slot; then the pairs of the last turn, which every turn builds again
-    dr.prefill(ids, hidden, cu, start_pos=[0] * B, resid0=st["resid"][0])
-    n = [k] * B if op == "score" else [a + 1 for a in _accepted(case, host)]
-    cu = _starts(n)
-    st.update(ids=tokens(cu[-1]), hidden=normal(cu[-1], d), cu=cu, start=T)
+    x = {"W": W, "T": T, "resid": normal(4, d, std=0.02), "normal": normal, "host": host}
+    # the prompts: the rows [0, T) of every slot where the turn does not build them itself
+    cu = _starts(T if op == "open" else [t + 1 for t in T])
+    x["prompt"] = (tokens(cu[-1]), normal(cu[-1], d), cu)
+    if op != "open":
+        # the pairs of the last turn, which every turn builds again
+        n = [k] * B if op == "score" else [a + 1 for a in _accepted(case, host)]
+        cu = _starts(n)
+        x["pairs"] = (tokens(cu[-1]), normal(cu[-1], d), cu)
     if op == "score":
-        st["recorded"] = tokens(B * k).view(B, k)
+        x["recorded"] = tokens(B * k).view(B, k)
+    if op == "sampled":
+        x["uniforms"] = torch.empty((B, k, V), device="cuda").uniform_(1e-6, 1.0 - 1e-6, generator=gen)
+        x["u_accept"] = torch.empty((B, k), device="cuda").uniform_(0.0, 1.0, generator=gen)
+        x["u_sample"] = torch.empty((B,), device="cuda").uniform_(0.0, 1.0, generator=gen)
+    return x
+
+
+def prepare(case, seed):
+    D = SHAPES[case["shape"]]
+    op, B, k, V = case["op"], case["batch"], case["k"], D.vocab
+    x = _inputs(case, seed)
+    T, host, normal = x["T"], x["host"], x["normal"]
+    extra = 1 + (k - 1) * case["topk"] if op == "tree" else k
+    dr = Drafter(D, x.pop("W"), max_batch=B, max_len=max(T) + 2 * k + 2 + extra, max_k=max(8, k))
+    st = {"op": op, "B": B, "k": k, "drafter": dr, "resid": x["resid"]}
+    ids, hidden, cu = x["prompt"]
+    if op == "open":
+        st.update(ids=ids, hidden=hidden, cu=cu, start=[0] * B)
+        return st
+    dr.prefill(ids, hidden, cu, start_pos=[0] * B, resid0=st["resid"][0])
+    ids, hidden, cu = x["pairs"]
+    st.update(ids=ids, hidden=hidden, cu=cu, start=T)
+    if op == "score":
+        st["recorded"] = x["recorded"]
         return st
     # the target's logits: they follow the draft for a while, as a target's do
-    if op == "sampled":
-        st["uniforms"] = torch.empty((B, k, V), device="cuda").uniform_(1e-6, 1.0 - 1e-6, generator=gen)
-        st["u_accept"] = torch.empty((B, k), device="cuda").uniform_(0.0, 1.0, generator=gen)
-        st["u_sample"] = torch.empty((B,), device="cuda").uniform_(0.0, 1.0, generator=gen)
     dr.prefill(st["ids"], st["hidden"], cu, start_pos=T, resid0=st["resid"][0])
     if op == "sampled":
+        st.update(uniforms=x["uniforms"], u_accept=x["u_accept"], u_sample=x["u_sample"])
         draft_logits = dr.draft_sampled(B, k, 1.0, st["uniforms"], st["resid"])[1]
         st["target"] = torch.cat([draft_logits + normal(B, k, V, dtype=torch.float32), normal(B, 1, V, dtype=torch.float32)], 1).to(D.logits)
         return st
@@ -263,3 +279,79 @@ def tolerance(case):
     if case["batch"] > 16:
         return {"rel": 2.5e-2, "differ": 0.01}
     return {"rel": 5e-3, "differ": 0.01}
+
+
+@torch.no_grad()
+def exact(case, seed):
+    """The drafter's logits in 64 bits, from the definition of the step.  A chain that feeds its own tokens has such a value
+    only as long as every token is decided by more than 32 or 16 bits may move a logit; a tree of near-ties has none."""
+    op, B, k, D = case["op"], case["batch"], case["k"], SHAPES[case["shape"]]
+    if op == "tree":
+        return None
+    x = _inputs(case, seed)
+    W = {n: w.double() for n, w in x["W"].items() if n not in ("embed", "lm_head")}
+    rho = x["resid"].double()
+    if case["project"]:
+        rho = rho @ W["resid_proj"].T
+    half = D.head_dim // 2
+    freq = D.rope_base ** (-torch.arange(half, dtype=torch.float64, device="cuda") / half)
+
+    def norm(u, gain):
+        return u * torch.rsqrt((u * u).mean(-1, keepdim=True) + D.rms_eps) * gain
+
+    def fuse(f, ids, step):
+        return torch.cat([f.double(), x["W"]["embed"][ids.long()].double()], -1) @ W["fc"].T + rho[min(step, 3)]
+
+    def rows(h, m, heads):
+        z = h @ W["w" + m].T + (W["b" + m] if case["bias"] else 0.0)
+        return z.view(len(h), heads, D.head_dim)
+
+    def rope(z, pos):
+        a = pos.double()[:, None] * freq
+        c, s = a.cos()[:, None], a.sin()[:, None]
+        lo, hi = z[..., :half], z[..., half:]
+        return torch.cat([lo * c - hi * s, hi * c + lo * s], -1)
+
+    cached, feats, last = [], [], []                                 # per sequence: K and V; the pending pair
+    for b in range(B):
+        parts = [(x["prompt"], op != "open")] + ([(x["pairs"], False)] if op != "open" else [])
+        ids = torch.cat([p[0][p[2][b]:p[2][b + 1] - cut] for p, cut in parts])
+        hidden = torch.cat([p[1][p[2][b]:p[2][b + 1] - cut] for p, cut in parts])
+        h = norm(fuse(hidden[:-1], ids[:-1], 0), W["norm1"])
+        pos = torch.arange(len(h), device="cuda")
+        cached.append([rope(rows(h, "k", D.n_kv_heads), pos), rows(h, "v", D.n_kv_heads)])
+        feats.append(hidden[-1].double())
+        last.append(ids[-1])
+    f, tok = torch.stack(feats), torch.stack(last)
+    pos = torch.tensor([len(c[0]) for c in cached], device="cuda")
+    # what may move a logit, of the logits' root mean square: the lower half of a bf16 or fp32 number, with room for the largest of many
+    sure = 6e-3 if D.dtype == "bf16" else 1e-5
+    ids, logits = [], torch.empty((B, k, D.vocab), dtype=torch.float64, device="cuda")
+    for s in range(k):
+        u = fuse(f, tok, s)
+        h = norm(u, W["norm1"])
+        q, kk, vv = rope(rows(h, "q", D.n_q_heads), pos + s), rope(rows(h, "k", D.n_kv_heads), pos + s), rows(h, "v", D.n_kv_heads)
+        out = []
+        for b, c in enumerate(cached):
+            c[0], c[1] = torch.cat([c[0], kk[b:b + 1]]), torch.cat([c[1], vv[b:b + 1]])
+            g = q[b].view(D.n_kv_heads, -1, D.head_dim)
+            p = torch.softmax(torch.einsum("hgd,nhd->hgn", g, c[0]) / math.sqrt(D.head_dim), -1)
+            out.append(torch.einsum("hgn,nhd->hgd", p, c[1]).reshape(-1))
+        y = u + torch.stack(out) @ W["wo"].T
+        h = norm(y, W["norm2"])
+        f = y + (torch.nn.functional.silu(h @ W["w_gate"].T) * (h @ W["w_up"].T)) @ W["w_down"].T
+        for lo in range(0, D.vocab, 16384):
+            logits[:, s, lo:lo + 16384] = f @ x["W"]["lm_head"][lo:lo + 16384].double().T
+        if op == "score":
+            tok = x["recorded"][:, s]
+            continue
+        z = logits[:, s] - torch.log(-torch.log(x["uniforms"][:, s].double())) if op == "sampled" else logits[:, s]
+        top = z.topk(2)
+        if s < k - 1 and bool((top.values[:, 0] - top.values[:, 1] < sure * logits[:, s].square().mean(-1).sqrt()).any()):
+            return None
+        tok = top.indices[:, 0]
+        ids.append(tok.int())
+    out = {"logits": logits}
+    if op in ("round", "sampled"):
+        out.update(accepted=None, next=None, rows=None)
+    return out if op == "score" else {"ids": None, **out}
