@@ -256,7 +256,7 @@ int hivis_debug_tap(hivis_ctx* ctx, int which, float* out, void* stream);
  * HIVIS_OPT_CHAIN_KERNEL (default 1): a draft of ONE sequence runs all k steps in a single persistent
  * cooperative kernel of fp32 FMAs (one CTA per SM, grid barriers between the phases of a step, weights
  * prefetched across them by per-warp bulk-copy rings).
- * HIVIS_OPT_TC_KERNEL (default 1): with bf16 weights and d a multiple of 64, a draft of 2..16 sequences
+ * HIVIS_OPT_TC_KERNEL (default 1): with bf16 weights and d a multiple of 64, a draft of 2..64 sequences
  * runs all k steps in one persistent cooperative kernel that streams the weights with TMA and multiplies
  * on the tcgen05 tensor cores (weights as the M operand, batch as N); 2 = use it for one sequence as well;
  * 0 = never.  What neither kernel takes runs as separate kernel launches per step.  All paths give the

@@ -14,7 +14,7 @@ struct hivis_ctx {
     int dtype;
     size_t esize;
     int qw, kvw, qkvw;
-    int rows_cap;                 // batch rows the workspaces hold: max(max_batch, 16)
+    int rows_cap;                 // batch rows the workspaces hold: 32, or 64 for more than 32 slots
     int device;
     // weights (library-owned copies)
     void *embed, *lm_head, *fc, *norm1, *wqkv, *bqkv, *wo, *norm2, *wgu, *wdown, *resid_proj;
@@ -45,7 +45,7 @@ struct hivis_ctx {
     u64 bar_count_host;           // value of *bar_counter once everything enqueued has run
     int* error_flag;              // [0]: a device-side wait ran out; [1] (= id_flag): a token id was out of range
     int* id_flag;
-    // tensor-core chain kernel (bf16, up to 16 sequences)
+    // tensor-core chain kernel (bf16)
     bool tc_ok;                   // cooperative launch available, shapes supported, tensor maps built
     long long wait_cycles;        // option HIVIS_OPT_WAIT_LIMIT_US, in cycles
     bool debug_skew;              // option HIVIS_OPT_DEBUG_MISS_BARRIER: the next draft's grid barriers cannot complete
@@ -59,7 +59,7 @@ struct hivis_ctx {
     float2* pf_rope;              // [map_cap][head_dim / 2]
     u64* phase_t;                 // [HIVIS_MAX_K][HIVIS_PHASE_EVENTS][num_sms]
     int phase_k;                  // draft steps of the last recorded launch (0: none)
-    TcMaps tc_maps;
+    TcMaps tc_maps, tc_maps_wide; // operands of 32 rows; of 64 rows (calls of more than 32 sequences)
     float* tc_partial;
     int* tile_ctr;
     int tc_tiles;
@@ -248,7 +248,7 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
     c->qw = cfg->n_q_heads * cfg->head_dim;
     c->kvw = cfg->n_kv_heads * cfg->head_dim;
     c->qkvw = c->qw + 2 * c->kvw;
-    c->rows_cap = cfg->max_batch > TC_OP_ROWS ? cfg->max_batch : TC_OP_ROWS;
+    c->rows_cap = cfg->max_batch > TC_OP_ROWS ? HIVIS_MAX_BATCH : TC_OP_ROWS;
     c->launches = 0;
     c->err[0] = 0;
     c->tap_B = 0;
@@ -296,7 +296,8 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
     }
     c->key_stride = cfg->max_k + 1;
     c->map_cap = MB * (long long)cfg->max_len;
-    const long long tiles1 = (d + HIVIS_MMA_TILE_ROWS - 1) / HIVIS_MMA_TILE_ROWS;
+    const long long tiles1 = (d + 127) / 128 * 4;       // partial sums of squares: one per 32 rows, whole 128-row tiles
+    static_assert(HIVIS_MMA_TILE_ROWS == 32, "partial sums of squares");
 
     char *embed, *lm, *fc, *n1, *wqkv, *bqkv = nullptr, *wo, *n2, *wgu, *wdown, *rp = nullptr, *Kc, *Vc;
     bool ok = dalloc(c, &embed, V * d * es) && dalloc(c, &lm, V * d * es) && dalloc(c, &fc, 2 * d * d * es) &&
@@ -323,7 +324,7 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
          dalloc(c, &c->counters, R * cfg->n_q_heads) && dalloc(c, &c->bar_counter, 1) &&
          dalloc(c, &c->error_flag, 2) && dalloc(c, &c->slot_of, c->map_cap) &&
          dalloc(c, &c->row_of, c->map_cap) && dalloc(c, &c->xe_h, R * d) &&
-         dalloc(c, &c->rope_tab, 2 * 16 * (cfg->head_dim / 2));
+         dalloc(c, &c->rope_tab, 2 * 16 * tc_groups(cfg->max_batch) * (cfg->head_dim / 2));
     {
         TreeBufs& T = c->tree;
         ok = ok && dalloc(c, &T.P, 1) && dalloc(c, &T.fr_cand, TREE_MAX_TOPK) && dalloc(c, &T.fr_tok, TREE_MAX_TOPK) &&
@@ -409,13 +410,17 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
         ChainArgs ca;
         fill_chain_args(c, &ca);
         c->tc_tiles = tc_max_tiles(ca.ph);
-        bool ok2 = dalloc(c, &c->tc_partial, (size_t)c->num_sms * 2 * 16 * 128) && dalloc(c, &c->tile_ctr, c->tc_tiles) &&
+        bool ok2 = dalloc(c, &c->tc_partial, (size_t)c->num_sms * 2 * 16 * 128 * tc_groups(cfg->max_batch)) && dalloc(c, &c->tile_ctr, c->tc_tiles) &&
                    dalloc(c, &c->phase_t, (size_t)HIVIS_MAX_K * HIVIS_PHASE_EVENTS * c->num_sms);
         if (ok2) ok2 = cudaMemsetAsync(c->tile_ctr, 0, c->tc_tiles * sizeof(int), st) == cudaSuccess;
         if (ok2)
             ok2 = tc_build_maps(&c->tc_maps, ca.ph, cfg->d, c->qw, cfg->ffn, c->feat_h, c->xq, c->attn_h, c->xm, c->act_h,
                                 c->xe_h, c->Kc, c->Vc, MB * (long long)cfg->n_kv_heads * cfg->max_len,
-                                cfg->head_dim) == cudaSuccess;
+                                cfg->head_dim, TC_OP_ROWS) == cudaSuccess;
+        if (ok2 && cfg->max_batch > TC_OP_ROWS)
+            ok2 = tc_build_maps(&c->tc_maps_wide, ca.ph, cfg->d, c->qw, cfg->ffn, c->feat_h, c->xq, c->attn_h, c->xm, c->act_h,
+                                c->xe_h, c->Kc, c->Vc, MB * (long long)cfg->n_kv_heads * cfg->max_len,
+                                cfg->head_dim, HIVIS_MAX_BATCH) == cudaSuccess;
         if (!ok2) cudaGetLastError();
         c->tc_ok = ok2;
     }
@@ -768,8 +773,11 @@ static int draft_impl(hivis_ctx* c, int B, const int* seq_slots_host, int k, con
         c->tap_mma = false;
         return HIVIS_OK;
     }
-    if (c->tc_ok && c->opt_tc != 0 && B <= 16) {
-        // bf16, up to 16 sequences: all k steps in one cooperative tensor-core kernel
+    // The kernel numbers attention units x warps in 32 bits; a batch beyond that (hundreds of heads on long caches) takes
+    // the per-phase kernels, as do draws for more than 16 sequences (refused below).
+    const bool tc_fits = B <= 16 || (!uniforms && (long long)B * g.n_q_heads * ((max_rows + 31) / 32 + 1) * 4 * c->num_sms < (1ll << 32));
+    if (c->tc_ok && c->opt_tc != 0 && tc_fits) {
+        // bf16: all k steps in one cooperative tensor-core kernel
         const int lo = tc_lo_offset(B);
         CKP(c, CLS_OTHER, st, launch_tc_setup(sl, k, d, lo, c->d_slots, c->d_pos0, c->kv_len, c->pend_feat, c->pend_id,
                                               c->feat, c->feat_h, c->cur_id, c->keys, c->key_stride, (const bf16*)c->embed,
@@ -784,7 +792,7 @@ static int draft_impl(hivis_ctx* c, int B, const int* seq_slots_host, int k, con
             c->phase_k = k;
         }
         c->debug_skew = false;
-        CKP(c, CLS_CHAIN, st, launch_tc_chain(c->tc_maps, a, c->num_sms, st));
+        CKP(c, CLS_CHAIN, st, launch_tc_chain(B <= TC_OP_ROWS ? c->tc_maps : c->tc_maps_wide, a, c->num_sms, st));
         c->bar_count_host += (u64)c->num_sms * (u64)(tc_barriers_per_step() * k);
         CKP(c, CLS_OTHER, st, launch_draft_finish(B, k, c->keys, c->key_stride, out_ids, st));
         for (int b = 0; b < B; ++b) {

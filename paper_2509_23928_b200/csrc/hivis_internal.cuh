@@ -144,14 +144,14 @@ struct CuSeqlens {
 };
 
 // ---------------------------------------------------------------------------------------------
-// Tensor-core chain kernel (bf16 weights, 1..16 sequences): all k steps in one cooperative launch,
+// Tensor-core chain kernel (bf16 weights, 1..64 sequences): all k steps in one cooperative launch,
 // weights streamed by TMA into a shared-memory ring, tcgen05.mma with the weights as the M operand
-// (128 rows) and the batch as N (16 columns), accumulators in tensor memory.
+// (128 rows) and the batch as N (32 or 64 columns), accumulators in tensor memory.
 // ---------------------------------------------------------------------------------------------
-#define TC_OP_ROWS 32          // rows of every bf16 operand buffer that the tensor maps cover
+#define TC_OP_ROWS 32          // rows of every bf16 operand buffer that the tensor maps cover (64 for more than 32 sequences)
 enum { TCM_W = 0,              // PH_COUNT weight maps, box 64 x 128
-       TCM_X_FEAT = PH_COUNT, TCM_X_XQ, TCM_X_ATTN, TCM_X_XM, TCM_X_ACT,   // operand maps, box 64 x 16
-       TCM_X_EMB,              // gathered embedding rows, box 64 x 16
+       TCM_X_FEAT = PH_COUNT, TCM_X_XQ, TCM_X_ATTN, TCM_X_XM, TCM_X_ACT,   // operand maps, box 64 x operand rows
+       TCM_X_EMB,              // gathered embedding rows, box 64 x operand rows
        TCM_K, TCM_V,           // the caches, box 64 x 32 rows
        TCM_COUNT };
 struct TcMaps {
@@ -174,15 +174,15 @@ struct TcArgs {
     bf16 *feat_h, *xq_h, *attn_h, *xm_h, *act_h;   // bf16 operands [TC_OP_ROWS][width]
     bf16* xe_h;                // [TC_OP_ROWS][d] embedding rows of the step's tokens (the set-up kernel zeroes rows >= B)
     const bf16* embed;         // [V][d]
-    float *ssq1, *ssq2;        // [tiles*4][16] partial sums of squares of u / y
+    float *ssq1, *ssq2;        // [tiles*4][16 x column groups] partial sums of squares of u / y
     float* logits_out;         // [B][k][V], nullable
     const float* gumbel_u;     // [B][k][V] uniform numbers in (0, 1), nullable: tokens are drawn, not the maximum
     float inv_t;               // 1 / temperature of the draw
-    float* partial;            // [grid*2][16][128] split-tile partial accumulators
+    float* partial;            // [grid*2][column groups][128][16] split-tile partial accumulators
     int* tile_ctr;             // arrival counters of split tiles, zero between phases
     void *Kc, *Vc;
     const double* inv_freq;
-    float2* rope_tab;          // [2][16][dh/2] (cos, sin) per sequence at the current step, halves alternate
+    float2* rope_tab;          // [2][16 x column groups][dh/2] (cos, sin) per sequence at the current step, halves alternate
     float *part_acc, *part_ml;
     int* counters;
     int attn_nslot;            // partial slots per (sequence, head): >= 32-row blocks of the longest sequence
@@ -201,7 +201,7 @@ struct TcArgs {
 // fills `maps` for the given buffers; returns cudaSuccess or an error (driver entry point missing, bad shape)
 cudaError_t tc_build_maps(TcMaps* maps, const ChainPhase* ph, int d, int qw, int F, const bf16* feat_h,
                           const bf16* xq_h, const bf16* attn_h, const bf16* xm_h, const bf16* act_h, const bf16* xe_h,
-                          const void* Kc, const void* Vc, long long cache_rows, int dh);
+                          const void* Kc, const void* Vc, long long cache_rows, int dh, int op_rows);
 bool tc_supported(int d, int dh, int Hq, int Hkv, int F);
 int tc_max_tiles(const ChainPhase* ph);
 cudaError_t launch_tc_chain(const TcMaps& maps, const TcArgs& a, int grid, cudaStream_t st);
@@ -211,6 +211,7 @@ cudaError_t launch_tc_setup(const SlotList& sl, int k, int d, int lo, int* d_slo
                             int* id_flag, cudaStream_t st);
 int tc_barriers_per_step();
 int tc_lo_offset(int B);
+int tc_groups(int B);
 
 // ---------------------------------------------------------------------------------------------
 // Prefix build on the tensor cores (kernels_prefill_tc.cu): two tcgen05 GEMMs over all packed pairs.

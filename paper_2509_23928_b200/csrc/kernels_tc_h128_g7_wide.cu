@@ -1,0 +1,4 @@
+#include "tc_chain.cuh"
+
+template cudaError_t tc_launch_t<128, 7, false, 2>(const TcMaps&, const TcArgs&, int, cudaStream_t);
+template cudaError_t tc_launch_t<128, 7, false, 4>(const TcMaps&, const TcArgs&, int, cudaStream_t);

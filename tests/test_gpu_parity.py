@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 import hivis_inputs as hi
-from tests.harness import Case, check_draft_parity, check_kv_parity, check_verify_parity, to_dev, row_rel_err
+from tests.harness import LOGIT_RTOL, Case, check_draft_parity, check_kv_parity, check_verify_parity, to_dev, row_rel_err
 
 pytestmark = pytest.mark.gpu
 
@@ -256,6 +256,32 @@ def test_more_sequences_than_the_chain_kernels_take():
         case.drafter.status()
         check_kv_parity(case, res["ref"])
         check_verify_parity(case, res["ids_o"])
+    finally:
+        case.close()
+
+
+@pytest.mark.parametrize("base,batch,hi_len", [("mini_mha_b5_ragged", 17, 70), ("mini_gqa_b16_ragged", 32, 100),
+                                               ("mini_mha_b5_ragged", 33, 100), ("mini_gqa_b16_ragged", 49, 40),
+                                               ("gqa4_b16_ragged", 64, 70), ("wide_mha_b16_ragged", 64, 40)])
+def test_column_groups_of_the_tensor_core_chain_kernel(base, batch, hi_len):
+    """17..64 sequences: two and four groups of 16 columns, full and partly filled; tiles shared by many CTAs and (the
+    narrow shapes) phases with fewer tile-k-blocks than CTAs.  Then 5 of the slots again: what a larger batch left in
+    the operand rows must not reach a smaller one."""
+    wl = hi.scaled(hi.workload(base), batch=batch, k=3, text_len_range=(1, hi_len))
+    case = Case(wl)
+    try:
+        check_draft_parity(case)
+        ref = case.oracle_run()
+        check_kv_parity(case, ref, seqs=[0, 15, 16, batch - 1])
+        case.gpu_restore()
+        ids_all, logits_all = case.gpu_draft()
+        case.gpu_restore()
+        slots = [batch - 1, 3, 15, 0, 9]
+        out, lg = case.drafter.draft(5, wl.k, case.d_resid, slots=slots, want_logits=True)
+        case.torch.cuda.synchronize()
+        lg = lg.cpu().numpy()
+        for i, s in enumerate(slots):
+            assert row_rel_err(lg[i, 0], logits_all[s, 0]) <= LOGIT_RTOL
     finally:
         case.close()
 
