@@ -647,7 +647,7 @@ int hivis_prefill(hivis_ctx* c, int B, const int* seq_slots_host, const int32_t*
         // many pairs: the two GEMMs of the prefix build on the tensor cores, all pairs in one pass
         PrefillTcArgs a;
         memset(&a, 0, sizeof(a));
-        a.n_pairs = (int)total; a.pair_cap = (int)c->map_cap;
+        a.num_sms = c->num_sms; a.n_pairs = (int)total; a.pair_cap = (int)c->map_cap;
         a.d = d; a.kvw = c->kvw; a.Hkv = c->cfg.n_kv_heads; a.dh = c->cfg.head_dim; a.max_len = c->cfg.max_len;
         a.vocab = c->cfg.vocab; a.eps = c->cfg.rms_eps;
         a.ids = ids; a.hidden = (const bf16*)hidden; a.embed = (const bf16*)c->embed; a.fc = (const bf16*)c->fc;

@@ -217,6 +217,7 @@ int tc_groups(int B);
 // Prefix build on the tensor cores (kernels_prefill_tc.cu): two tcgen05 GEMMs over all packed pairs.
 // ---------------------------------------------------------------------------------------------
 struct PrefillTcArgs {
+    int num_sms;
     int n_pairs, pair_cap;     // packed pairs of the call; capacity of the pair-major buffers
     int d, kvw, Hkv, dh, max_len, vocab;
     float eps;

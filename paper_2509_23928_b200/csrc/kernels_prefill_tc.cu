@@ -1,18 +1,30 @@
 // Prefix build on the tensor cores (Algorithm 1, the prefix build; Eq. 1): for every packed (hidden state, token) pair
 //     u = W_fc [h ; E[id]] + rho_0,   a = gamma_1 * u / rms(u),   K = RoPE(W_k a + b_k, position),   V = W_v a + b_v
 // and K, V go to the pair's cache row.  Unlike a draft step this is a dense contraction - thousands of pairs share
-// every weight tile - so it runs as two tcgen05 GEMMs with the weights as the M operand (128 rows) and 128 pairs
-// as the N operand, both staged by TMA (128-byte swizzle) through a six-stage ring, accumulators in tensor memory:
-//   GEMM 1 (fusion FC):  [d rows] x [2d] x pairs.  The k-blocks of the hidden half come from the caller's hidden
+// every weight tile - so it runs as two tcgen05 GEMMs with the pairs as the M operand and the weight rows as N:
+//   GEMM 1 (fusion FC):  pairs x [2d] x [d rows].  The k-blocks of the hidden half come from the caller's hidden
 //                        states, those of the embedding half from a buffer of gathered embedding rows.  Output
-//                        stage: + rho_0, per-pair partial sums of squares of the tile's rows, gamma_1 * u as bf16
+//                        stage: + rho_0, per-pair partial sums of squares of the tile's columns, gamma_1 * u as bf16
 //                        (pair-major, the operand of GEMM 2).  The RMSNorm scale is applied after GEMM 2.
-//   GEMM 2 (K and V):    [2 * Hkv * dh rows] x [d] x pairs.  Output stage: scale by 1/rms, bias, rotate K at the
-//                        pair's position, scatter 16-byte pieces to the cache rows; pending pairs (row -1) are skipped.
-// One CTA computes one 128 x 128 output tile.  Warp 0 (one thread) issues the copies, warp 1 (one thread) the MMAs,
-// warps 2-5 run the output stage: each thread reads its weight row of the accumulator, the tile is turned in
-// shared memory (the ring is free by then) so that a thread then owns one PAIR and writes whole 16-byte pieces,
-// and sums over rows run in a fixed order.  Every wait is bounded; a wait that runs out raises the error word.
+//   GEMM 2 (K and V):    pairs x [d] x [2 * Hkv * dh rows].  Output stage: scale by 1/rms, bias, rotate K at the
+//                        pair's position, store to the cache rows; pending pairs (row -1) are skipped.
+//
+// What bounds it is the path from L2 to shared memory: a 128 x 128 tile computed by one CTA needs 128 bytes per SM and
+// clock of tensor time, twice what an SM can fetch.  So two CTAs (a cluster of two: the SMs of one TPC) work on one
+// tile of 256 pairs x 256 weight rows with cta_group::2 MMAs: each CTA stages its own 128 pairs and HALF of the weight
+// rows, which the tensor cores of both read - 64 bytes per SM and clock.  With the pairs as M every thread of the
+// output stage owns one pair: sums of squares, the rotation and 16-byte stores need no exchange between threads.
+// The kernel is persistent (one cluster per TPC) with two accumulators in tensor memory, so that a tile's output stage
+// runs under the next tile's MMAs; consecutive tiles go through the weight rows first (the weights stay in L2, the pairs
+// are read from memory once).
+//
+// 34 800 pairs of the LLaVA shape (16 sequences of 2176): 4.7 ms for both GEMMs, 1.0 PFLOP/s; with 128 x 128 tiles, one
+// per CTA and launch slot, and the tile turned in shared memory for the output stage 7.7 ms.
+//
+// Warp 0 (one thread, both CTAs) issues the copies, warp 1 (one thread of the leader, rank 0) the MMAs for both, warps
+// 2-5 run the output stage.  A stage's full barrier lives in the leader and counts the bytes of both CTAs; tcgen05.commit
+// hands stages and accumulators back to both CTAs.  Every wait is bounded; a wait that runs out raises the error word,
+// both CTAs let their copies land and leave together.
 #include <cuda.h>
 
 #include "attn_body.cuh"
@@ -20,17 +32,13 @@
 #define PF_THREADS 192
 #define PF_STAGES 6
 #define PF_BK 64
-#define PF_TM 128
-#define PF_TN 128
-#define PF_A_BYTES (PF_TM * PF_BK * 2)
-#define PF_B_BYTES (PF_TN * PF_BK * 2)
-#define PF_LD (PF_TM + 1)              // row stride (floats) of the turned tile: [pair][weight row]
-#define PF_IDESC ((1u << 4) | (1u << 7) | (1u << 10) | ((PF_TN >> 3) << 17) | ((PF_TM >> 4) << 24))
+#define PF_TM 256                    // pairs of a tile: 128 per CTA
+#define PF_A_BYTES (128 * PF_BK * 2)
 
 namespace {
 
 struct PfCtl {
-    u64 full[PF_STAGES], empty[PF_STAGES], tfull;
+    u64 full[PF_STAGES], empty[PF_STAGES], tfull[2], tempty[2];
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -59,6 +67,7 @@ __device__ __forceinline__ bool pf_wait(uint32_t bar, uint32_t parity, PfCtl* ct
     while (!pf_try(bar, parity)) {
         if ((++it & 63u) == 0u) {
             if (*(volatile int*)&ctl->abort_flag) return false;
+            if (*(volatile int*)error_flag != 0) { *(volatile int*)&ctl->abort_flag = 1; return false; }
             if (clock64() - t0 > limit) {
                 atomicCAS(error_flag, 0, 30);
                 *(volatile int*)&ctl->abort_flag = 1;
@@ -68,22 +77,40 @@ __device__ __forceinline__ bool pf_wait(uint32_t bar, uint32_t parity, PfCtl* ct
     }
     return true;
 }
+// The address of `bar` (own shared memory) in the CTA of the cluster with rank `rank`.
+__device__ __forceinline__ uint32_t pf_mapa(uint32_t bar, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(bar), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void pf_arrive_cluster(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void pf_cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// copy into this CTA's shared memory that completes on a barrier of the leader
 __device__ __forceinline__ void pf_tma_2d(uint32_t dst, const void* map, int x, int y, uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
         "l"(map), "r"(x), "r"(y), "r"(bar)
         : "memory");
 }
 __device__ __forceinline__ void pf_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void pf_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+// arrives on the barrier at this offset in both CTAs once the MMAs issued before are complete
 __device__ __forceinline__ void pf_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+                 "h"((unsigned short)3)
+                 : "memory");
 }
+template <int BN>
 __device__ __forceinline__ void pf_mma(uint32_t d_tmem, u64 adesc, u64 bdesc, uint32_t accumulate) {
+    constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((BN >> 3) << 17) | ((PF_TM >> 4) << 24);
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"((uint32_t)PF_IDESC), "r"(accumulate)
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(IDESC), "r"(accumulate)
         : "memory");
 }
 // K-major tile with 128-byte rows, 128-byte swizzle, 8-row groups 1024 bytes apart
@@ -94,6 +121,7 @@ __device__ __forceinline__ u64 pf_smem_desc(uint32_t addr) {
 }
 __device__ __forceinline__ void pf_ld32(uint32_t taddr, float (&v)[32]) {
     uint32_t r[32];
+    __syncwarp();               // the load is one instruction of the whole warp; lanes without a pair come here early
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,"
         "%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
@@ -109,17 +137,17 @@ __device__ __forceinline__ void pf_ld32(uint32_t taddr, float (&v)[32]) {
 }
 
 struct PfParams {
-    alignas(64) unsigned char map_w[128];      // weights [rows][K], box 64 x 128
+    alignas(64) unsigned char map_w[128];      // weights [rows][K], box 64 x BN / 2
     alignas(64) unsigned char map_x0[128];     // operand of k-blocks [0, kb_split): [pairs][.], box 64 x 128
     alignas(64) unsigned char map_x1[128];     // operand of k-blocks [kb_split, nkb)
-    int rows, K, kb_split, n_pairs;
+    int rows, K, kb_split, n_pairs, m_tiles, n_tiles;
     long long wait_cycles;
     int* error_flag;
     // GEMM 1 output stage
     const float* rho;          // [rows] nullable
     const bf16* gamma;         // [rows]
     bf16* xq;                  // [pairs][rows]
-    float* ssq;                // [row tiles][pair capacity]
+    float* ssq;                // [column tiles of 128][pair capacity]
     int pair_cap;
     // GEMM 2 output stage
     const float* ssq_in;       // [ssq_tiles][pair capacity]
@@ -132,153 +160,224 @@ struct PfParams {
     bf16 *Kc, *Vc;
 };
 
-template <int EPI>   // 0: fusion FC, 1: K and V
-__global__ void __launch_bounds__(PF_THREADS, 1) prefill_tc_kernel(const __grid_constant__ PfParams P) {
+__device__ __forceinline__ unsigned pf_pack(float x0, float x1) {
+    return (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(x0)) | ((unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(x1)) << 16);
+}
+__device__ __forceinline__ void pf_store32(bf16* dst, const float (&x)[32]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        *(uint4*)(dst + 8 * q) = make_uint4(pf_pack(x[8 * q], x[8 * q + 1]), pf_pack(x[8 * q + 2], x[8 * q + 3]),
+                                            pf_pack(x[8 * q + 4], x[8 * q + 5]), pf_pack(x[8 * q + 6], x[8 * q + 7]));
+}
+// 32 bf16 values that are the same for all threads of a warp (16-byte aligned), widened
+__device__ __forceinline__ void pf_load32(const bf16* src, float (&x)[32]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const uint4 w = __ldg((const uint4*)src + q);
+        x[8 * q] = bf16_lo(w.x); x[8 * q + 1] = bf16_hi(w.x); x[8 * q + 2] = bf16_lo(w.y); x[8 * q + 3] = bf16_hi(w.y);
+        x[8 * q + 4] = bf16_lo(w.z); x[8 * q + 5] = bf16_hi(w.z); x[8 * q + 6] = bf16_lo(w.w); x[8 * q + 7] = bf16_hi(w.w);
+    }
+}
+
+// GEMM 1 output stage of one pair: columns [n0, n0 + BN) of u.  Partial sums of squares cover 128 columns each, whatever
+// the tile's width, so that the RMSNorm scale does not depend on it.
+template <int BN>
+__device__ __forceinline__ void pf_out_fc(const PfParams& P, uint32_t tacc, int n0, int pair, bool live) {
+#pragma unroll 1
+    for (int c0 = 0; c0 < BN; c0 += 128) {
+        if (n0 + c0 >= P.rows) break;                       // (uniform)
+        float ss = 0.f;
+#pragma unroll 1
+        for (int c = c0; c < c0 + 128; c += 32) {
+            const int n = n0 + c;
+            if (n >= P.rows) break;
+            float v[32], g[32];
+            pf_ld32(tacc + c, v);
+            if (!live) continue;
+            pf_load32(P.gamma + n, g);
+            if (P.rho) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const float4 r = __ldg((const float4*)(P.rho + n) + q);
+                    v[4 * q] += r.x; v[4 * q + 1] += r.y; v[4 * q + 2] += r.z; v[4 * q + 3] += r.w;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                ss = fmaf(v[i], v[i], ss);
+                g[i] *= v[i];
+            }
+            pf_store32(P.xq + (long long)pair * P.rows + n, g);
+        }
+        if (live) P.ssq[(long long)((n0 + c0) >> 7) * P.pair_cap + pair] = ss;
+    }
+}
+
+// GEMM 2 output stage of one pair: the heads whose rows lie in [n0, n0 + BN), K heads first.
+template <int BN>
+__device__ __forceinline__ void pf_out_kv(const PfParams& P, uint32_t tacc, int n0, int pair, bool live) {
+    const int crow = live ? P.row_of[pair] : -1;
+    live = crow >= 0;
+    float sc = 0.f;
+    long long slot_base = 0;
+    if (live) {
+        float tot = 0.f;
+        for (int t = 0; t < P.ssq_tiles; ++t) tot += P.ssq_in[(long long)t * P.pair_cap + pair];
+        sc = rsqrtf(tot / (float)P.d + P.eps);
+        slot_base = (long long)P.slot_of[pair] * P.Hkv;
+    }
+    const int half = P.dh >> 1;
+#pragma unroll 1
+    for (int h0 = 0; h0 < BN; h0 += P.dh) {
+        const int g = n0 + h0;                              // row of the stacked [K ; V] projection
+        if (g >= P.rows) break;
+        const bool isK = g < P.kvw;
+        const int head = (isK ? g : g - P.kvw) / P.dh;
+        bf16* dst = (isK ? P.Kc : P.Vc) + ((slot_base + head) * P.max_len + (live ? crow : 0)) * P.dh;
+#pragma unroll 1
+        for (int e0 = 0; e0 < half; e0 += 32) {
+            float lo[32], hi[32], x[32];
+            pf_ld32(tacc + h0 + e0, lo);
+            pf_ld32(tacc + h0 + half + e0, hi);
+            if (!live) continue;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) { lo[i] *= sc; hi[i] *= sc; }
+            if (P.bias) {
+                pf_load32(P.bias + g + e0, x);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) lo[i] += x[i];
+                pf_load32(P.bias + g + half + e0, x);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) hi[i] += x[i];
+            }
+            if (isK) {
+                const float4* tab = (const float4*)(P.rope + (long long)pair * half + e0);
+#pragma unroll
+                for (int q = 0; q < 16; ++q) {
+                    const float4 t = __ldg(tab + q);
+                    const float l0 = lo[2 * q], l1 = lo[2 * q + 1], u0 = hi[2 * q], u1 = hi[2 * q + 1];
+                    lo[2 * q] = l0 * t.x - u0 * t.y;
+                    hi[2 * q] = u0 * t.x + l0 * t.y;
+                    lo[2 * q + 1] = l1 * t.z - u1 * t.w;
+                    hi[2 * q + 1] = u1 * t.z + l1 * t.w;
+                }
+            }
+            pf_store32(dst + e0, lo);
+            pf_store32(dst + half + e0, hi);
+        }
+    }
+}
+
+template <int EPI, int BN>   // EPI 0: fusion FC, 1: K and V
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1) prefill_tc_kernel(const __grid_constant__ PfParams P) {
+    constexpr int B_BYTES = (BN / 2) * PF_BK * 2;
     extern __shared__ __align__(1024) unsigned char pf_smem_raw[];
+    // (the stages must lie at the same offset in both CTAs: the window's start is the same for all CTAs of a launch)
     unsigned char* smem = (unsigned char*)(((uintptr_t)pf_smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t smemA = pf_saddr(smem), smemB = smemA + PF_STAGES * PF_A_BYTES;
-    PfCtl* ctl = (PfCtl*)(smem + PF_STAGES * (PF_A_BYTES + PF_B_BYTES));
+    PfCtl* ctl = (PfCtl*)(smem + PF_STAGES * (PF_A_BYTES + B_BYTES));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int row0 = blockIdx.x * PF_TM, pair0 = blockIdx.y * PF_TN;
-    const int nkb = P.K / PF_BK;
+    uint32_t rank;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    const int cluster = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
+    const int nkb = P.K / PF_BK, tiles = P.m_tiles * P.n_tiles;
     if (tid == 0) {
         for (int i = 0; i < PF_STAGES; ++i) {
             pf_mbar_init(pf_saddr(&ctl->full[i]), 1);
             pf_mbar_init(pf_saddr(&ctl->empty[i]), 1);
         }
-        pf_mbar_init(pf_saddr(&ctl->tfull), 1);
+        for (int i = 0; i < 2; ++i) {
+            pf_mbar_init(pf_saddr(&ctl->tfull[i]), 1);
+            pf_mbar_init(pf_saddr(&ctl->tempty[i]), 8);          // the four output warps of both CTAs
+        }
         ctl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(pf_saddr(&ctl->tmem_base)),
-                     "r"((uint32_t)PF_TN)
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(pf_saddr(&ctl->tmem_base)),
+                     "r"((uint32_t)(2 * BN))
                      : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     pf_fence_before();
     __syncthreads();
+    pf_cluster_sync();
     pf_fence_after();
 
     if (warp == 0) {
         if (lane == 0) {
-            for (int kb = 0; kb < nkb; ++kb) {
-                const int slot = kb % PF_STAGES, round = kb / PF_STAGES;
-                if (round > 0 && !pf_wait(pf_saddr(&ctl->empty[slot]), (round - 1) & 1u, ctl, P.wait_cycles, P.error_flag)) break;
-                const uint32_t bar = pf_saddr(&ctl->full[slot]);
-                pf_expect_tx(bar, PF_A_BYTES + PF_B_BYTES);
-                pf_tma_2d(smemA + slot * PF_A_BYTES, P.map_w, kb * PF_BK, row0, bar);
-                if (kb < P.kb_split) pf_tma_2d(smemB + slot * PF_B_BYTES, P.map_x0, kb * PF_BK, pair0, bar);
-                else pf_tma_2d(smemB + slot * PF_B_BYTES, P.map_x1, (kb - P.kb_split) * PF_BK, pair0, bar);
+            unsigned it = 0;
+            bool ok = true;
+            for (int t = cluster; t < tiles && ok; t += n_clusters) {
+                const int pair0 = (t / P.n_tiles) * PF_TM + (int)rank * 128, row0 = (t % P.n_tiles) * BN + (int)rank * (BN / 2);
+                for (int kb = 0; kb < nkb; ++kb, ++it) {
+                    const unsigned slot = it % PF_STAGES, round = it / PF_STAGES;
+                    ok = round == 0 || pf_wait(pf_saddr(&ctl->empty[slot]), (round - 1) & 1u, ctl, P.wait_cycles, P.error_flag);
+                    if (!ok) break;
+                    if (rank == 0) pf_expect_tx(pf_saddr(&ctl->full[slot]), 2 * (PF_A_BYTES + B_BYTES));
+                    const uint32_t bar = pf_mapa(pf_saddr(&ctl->full[slot]), 0);
+                    if (kb < P.kb_split) pf_tma_2d(smemA + slot * PF_A_BYTES, P.map_x0, kb * PF_BK, pair0, bar);
+                    else pf_tma_2d(smemA + slot * PF_A_BYTES, P.map_x1, (kb - P.kb_split) * PF_BK, pair0, bar);
+                    pf_tma_2d(smemB + slot * B_BYTES, P.map_w, kb * PF_BK, row0, bar);
+                }
+            }
+            if (!ok) {          // after a give-up: copies already issued still land in this CTA's shared memory
+                const long long t1 = clock64();
+                while (clock64() - t1 < 4000000ll) {}
             }
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (lane == 0 && rank == 0) {
             const uint32_t tmem = ctl->tmem_base;
+            unsigned it = 0, seg = 0;
             bool ok = true;
-            for (int kb = 0; kb < nkb && ok; ++kb) {
-                const int slot = kb % PF_STAGES, round = kb / PF_STAGES;
-                ok = pf_wait(pf_saddr(&ctl->full[slot]), round & 1u, ctl, P.wait_cycles, P.error_flag);
-                if (!ok) break;
+            for (int t = cluster; t < tiles && ok; t += n_clusters, ++seg) {
+                const unsigned acc = seg & 1u, use = seg >> 1;
+                ok = use == 0 || pf_wait(pf_saddr(&ctl->tempty[acc]), (use - 1) & 1u, ctl, P.wait_cycles, P.error_flag);
                 pf_fence_after();
-                const u64 ad = pf_smem_desc(smemA + slot * PF_A_BYTES), bd = pf_smem_desc(smemB + slot * PF_B_BYTES);
+                for (int kb = 0; kb < nkb && ok; ++kb, ++it) {
+                    const unsigned slot = it % PF_STAGES, round = it / PF_STAGES;
+                    ok = pf_wait(pf_saddr(&ctl->full[slot]), round & 1u, ctl, P.wait_cycles, P.error_flag);
+                    if (!ok) break;
+                    pf_fence_after();
+                    const u64 ad = pf_smem_desc(smemA + slot * PF_A_BYTES), bd = pf_smem_desc(smemB + slot * B_BYTES);
 #pragma unroll
-                for (int kk = 0; kk < PF_BK / 16; ++kk) pf_mma(tmem, ad + (u64)(kk * 2), bd + (u64)(kk * 2), (kb > 0 || kk > 0) ? 1u : 0u);
-                pf_commit(pf_saddr(&ctl->empty[slot]));
+                    for (int kk = 0; kk < PF_BK / 16; ++kk)
+                        pf_mma<BN>(tmem + acc * BN, ad + (u64)(kk * 2), bd + (u64)(kk * 2), (kb > 0 || kk > 0) ? 1u : 0u);
+                    pf_commit(pf_saddr(&ctl->empty[slot]));
+                }
+                if (ok) pf_commit(pf_saddr(&ctl->tfull[acc]));
             }
-            if (ok) pf_commit(pf_saddr(&ctl->tfull));
         }
         __syncwarp();
     } else {
-        // ---- output stage: warps 2..5 read the tensor-memory lanes their number modulo 4 selects
-        const int quarter = warp & 3, etid = tid - 64;                  // etid: 0..127
-        const int r_loc = quarter * 32 + lane, row = row0 + r_loc;
-        float* tile = (float*)smem;                                      // [PF_TN pairs][PF_LD]: the ring is free by now
-        bool ok = true;
-        if (lane == 0) ok = pf_wait(pf_saddr(&ctl->tfull), 0u, ctl, P.wait_cycles, P.error_flag);
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-        pf_fence_after();
-        if (ok) {
-#pragma unroll 1
-            for (int c0 = 0; c0 < PF_TN; c0 += 32) {
-                float v[32];
-                pf_ld32(ctl->tmem_base + ((uint32_t)(quarter * 32) << 16) + c0, v);
-                if (EPI == 0) {
-                    const float add = (P.rho && row < P.rows) ? P.rho[row] : 0.f;
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) tile[(c0 + i) * PF_LD + r_loc] = v[i] + add;
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) tile[(c0 + i) * PF_LD + r_loc] = v[i];
-                }
-            }
-        }
-        pf_fence_before();
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        // ---- a thread now owns one pair of the tile
-        const int pair = pair0 + etid;
-        const float* mine = tile + etid * PF_LD;
-        const int nrows = min(PF_TM, P.rows - row0);
-        if (ok && !*(volatile int*)&ctl->abort_flag && pair < P.n_pairs) {
-            if (EPI == 0) {
-                float ss = 0.f;
-                for (int r = 0; r < nrows; ++r) ss = fmaf(mine[r], mine[r], ss);
-                P.ssq[(long long)blockIdx.x * P.pair_cap + pair] = ss;
-                bf16* dst = P.xq + (long long)pair * P.rows + row0;
-                for (int r = 0; r < nrows; r += 8) {
-                    unsigned w[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float x0 = __bfloat162float(P.gamma[row0 + r + 2 * e]) * mine[r + 2 * e];
-                        const float x1 = __bfloat162float(P.gamma[row0 + r + 2 * e + 1]) * mine[r + 2 * e + 1];
-                        w[e] = (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(x0)) |
-                               ((unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(x1)) << 16);
-                    }
-                    *(uint4*)(dst + r) = make_uint4(w[0], w[1], w[2], w[3]);
-                }
-            } else {
-                const int crow = P.row_of[pair];
-                if (crow >= 0) {
-                    float tot = 0.f;
-                    for (int t = 0; t < P.ssq_tiles; ++t) tot += P.ssq_in[(long long)t * P.pair_cap + pair];
-                    const float sc = rsqrtf(tot / (float)P.d + P.eps);
-                    const int slot = P.slot_of[pair], half = P.dh >> 1;
-                    for (int r = 0; r < nrows; r += 8) {
-                        const int g = row0 + r;                               // row of the stacked [K ; V] projection
-                        const bool isK = g < P.kvw;
-                        const int gr = isK ? g : g - P.kvw, head = gr / P.dh, e0 = gr % P.dh;
-                        unsigned w[4];
-                        float x[8];
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            float val = mine[r + e] * sc + (P.bias ? __bfloat162float(P.bias[g + e]) : 0.f);
-                            if (isK) {
-                                const int ee = e0 + e, f = ee % half;
-                                const int pr = r + e + (ee < half ? half : -half);        // the partner row, in this tile
-                                const float part = mine[pr] * sc + (P.bias ? __bfloat162float(P.bias[row0 + pr]) : 0.f);
-                                const float2 t = __ldg(P.rope + (long long)pair * half + f);
-                                val = ee < half ? val * t.x - part * t.y : val * t.x + part * t.y;
-                            }
-                            x[e] = val;
-                        }
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            w[e] = (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(x[2 * e])) |
-                                   ((unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(x[2 * e + 1])) << 16);
-                        bf16* base = isK ? P.Kc : P.Vc;
-                        *(uint4*)(base + (((long long)slot * P.Hkv + head) * P.max_len + crow) * P.dh + e0) = make_uint4(w[0], w[1], w[2], w[3]);
-                    }
-                }
-            }
+        // ---- output stage: warps 2..5 read the tensor-memory lanes their number modulo 4 selects; a lane is a pair
+        const int quarter = warp & 3;
+        unsigned seg = 0;
+        for (int t = cluster; t < tiles; t += n_clusters, ++seg) {
+            const unsigned acc = seg & 1u, use = seg >> 1;
+            const int pair = (t / P.n_tiles) * PF_TM + (int)rank * 128 + quarter * 32 + lane, n0 = (t % P.n_tiles) * BN;
+            bool ok = true;
+            if (lane == 0) ok = pf_wait(pf_saddr(&ctl->tfull[acc]), use & 1u, ctl, P.wait_cycles, P.error_flag);
+            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+            if (!ok) break;
+            pf_fence_after();
+            const uint32_t tacc = ctl->tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN;
+            if (EPI == 0) pf_out_fc<BN>(P, tacc, n0, pair, pair < P.n_pairs);
+            else pf_out_kv<BN>(P, tacc, n0, pair, pair < P.n_pairs);
+            pf_fence_before();
+            __syncwarp();
+            if (lane == 0) pf_arrive_cluster(pf_mapa(pf_saddr(&ctl->tempty[acc]), 0));
         }
     }
     pf_fence_before();
     __syncthreads();
+    pf_cluster_sync();          // nobody leaves while its shared memory or its barriers may still be used by the other CTA
     if (warp == 1) {
         pf_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(ctl->tmem_base), "r"((uint32_t)PF_TN) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(ctl->tmem_base), "r"((uint32_t)(2 * BN)) : "memory");
     }
 }
 
@@ -306,7 +405,7 @@ __global__ void prefill_rope_kernel(const int* row_of, int n_pairs, int half, co
 typedef CUresult (*PfEncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-cudaError_t pf_encode(unsigned char* out, const void* base, long long rows, long long cols) {
+cudaError_t pf_encode(unsigned char* out, const void* base, long long rows, long long cols, int box_rows) {
     static PfEncodeFn fn = nullptr;
     if (!fn) {
         void* p = nullptr;
@@ -319,7 +418,7 @@ cudaError_t pf_encode(unsigned char* out, const void* base, long long rows, long
     }
     const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
-    const cuuint32_t box[2] = {PF_BK, 128};
+    const cuuint32_t box[2] = {PF_BK, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
     const CUresult r = fn((CUtensorMap*)out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -327,28 +426,41 @@ cudaError_t pf_encode(unsigned char* out, const void* base, long long rows, long
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <int EPI>
-cudaError_t pf_launch(const PfParams& P, cudaStream_t st) {
+template <int EPI, int BN>
+cudaError_t pf_launch_t(PfParams& P, int clusters, cudaStream_t st) {
     static bool attr_set[HIVIS_MAX_DEVICES] = {false};
-    const size_t smem = 1024 + (size_t)PF_STAGES * (PF_A_BYTES + PF_B_BYTES) + 256;
+    const size_t smem = 1024 + (size_t)PF_STAGES * (PF_A_BYTES + (BN / 2) * PF_BK * 2) + 256;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= HIVIS_MAX_DEVICES || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(prefill_tc_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(prefill_tc_kernel<EPI, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < HIVIS_MAX_DEVICES) attr_set[dev] = true;
     }
-    const dim3 grid((unsigned)((P.rows + PF_TM - 1) / PF_TM), (unsigned)((P.n_pairs + PF_TN - 1) / PF_TN));
-    prefill_tc_kernel<EPI><<<grid, PF_THREADS, smem, st>>>(P);
+    P.n_tiles = (P.rows + BN - 1) / BN;
+    const int tiles = P.m_tiles * P.n_tiles;
+    prefill_tc_kernel<EPI, BN><<<2 * (tiles < clusters ? tiles : clusters), PF_THREADS, smem, st>>>(P);
     return cudaGetLastError();
+}
+
+// Tile width: 256 weight rows where that fills the GPU's clusters as well as 128 does.  The time of a GEMM goes with the
+// number of tiles the busiest cluster gets, times their width.
+template <int EPI>
+cudaError_t pf_launch(PfParams& P, const void* W, int num_sms, cudaStream_t st) {
+    const int clusters = num_sms / 2 > 0 ? num_sms / 2 : 1;
+    P.m_tiles = (P.n_pairs + PF_TM - 1) / PF_TM;
+    auto cost = [&](int bn) { return (long long)((P.m_tiles * ((P.rows + bn - 1) / bn) + clusters - 1) / clusters) * bn; };
+    const int bn = cost(256) <= cost(128) ? 256 : 128;
+    cudaError_t e = pf_encode(P.map_w, W, P.rows, P.K, bn / 2);
+    if (e != cudaSuccess) return e;
+    return bn == 256 ? pf_launch_t<EPI, 256>(P, clusters, st) : pf_launch_t<EPI, 128>(P, clusters, st);
 }
 
 }  // namespace
 
 bool prefill_tc_supported(int d, int kvw) {
     static_assert(sizeof(CUtensorMap) == 128, "tensor map size");
-    static_assert((size_t)PF_TN * PF_LD * 4 <= (size_t)PF_STAGES * (PF_A_BYTES + PF_B_BYTES), "the turned tile must fit in the ring");
     return d % PF_BK == 0 && (2 * kvw) % 8 == 0;
 }
 
@@ -362,23 +474,21 @@ cudaError_t launch_prefill_tc(const PrefillTcArgs& a, cudaStream_t st) {
     PfParams P;
     memset(&P, 0, sizeof(P));
     // ---- GEMM 1: u = W_fc [h ; E[id]] + rho_0
-    if ((e = pf_encode(P.map_w, a.fc, d, 2 * d)) != cudaSuccess) return e;
-    if ((e = pf_encode(P.map_x0, a.hidden, a.n_pairs, d)) != cudaSuccess) return e;
-    if ((e = pf_encode(P.map_x1, a.xe, a.n_pairs, d)) != cudaSuccess) return e;
+    if ((e = pf_encode(P.map_x0, a.hidden, a.n_pairs, d, 128)) != cudaSuccess) return e;
+    if ((e = pf_encode(P.map_x1, a.xe, a.n_pairs, d, 128)) != cudaSuccess) return e;
     P.rows = d; P.K = 2 * d; P.kb_split = d / PF_BK; P.n_pairs = a.n_pairs;
     P.wait_cycles = a.wait_cycles; P.error_flag = a.error_flag;
     P.rho = a.rho0; P.gamma = a.norm1; P.xq = a.xq; P.ssq = a.ssq; P.pair_cap = a.pair_cap;
-    if ((e = pf_launch<0>(P, st)) != cudaSuccess) return e;
+    if ((e = pf_launch<0>(P, a.fc, a.num_sms, st)) != cudaSuccess) return e;
     // ---- GEMM 2: K, V
     PfParams Q;
     memset(&Q, 0, sizeof(Q));
-    if ((e = pf_encode(Q.map_w, a.wkv, 2 * a.kvw, d)) != cudaSuccess) return e;
-    if ((e = pf_encode(Q.map_x0, a.xq, a.n_pairs, d)) != cudaSuccess) return e;
+    if ((e = pf_encode(Q.map_x0, a.xq, a.n_pairs, d, 128)) != cudaSuccess) return e;
     memcpy(Q.map_x1, Q.map_x0, 128);
     Q.rows = 2 * a.kvw; Q.K = d; Q.kb_split = d / PF_BK; Q.n_pairs = a.n_pairs;
     Q.wait_cycles = a.wait_cycles; Q.error_flag = a.error_flag;
-    Q.ssq_in = a.ssq; Q.ssq_tiles = (d + PF_TM - 1) / PF_TM; Q.pair_cap = a.pair_cap; Q.d = d; Q.eps = a.eps;
+    Q.ssq_in = a.ssq; Q.ssq_tiles = (d + 127) / 128; Q.pair_cap = a.pair_cap; Q.d = d; Q.eps = a.eps;
     Q.bias = a.bkv; Q.kvw = a.kvw; Q.Hkv = a.Hkv; Q.dh = a.dh; Q.max_len = a.max_len;
     Q.slot_of = a.slot_of; Q.row_of = a.row_of; Q.rope = a.rope; Q.Kc = a.Kc; Q.Vc = a.Vc;
-    return pf_launch<1>(Q, st);
+    return pf_launch<1>(Q, a.wkv, a.num_sms, st);
 }

@@ -247,6 +247,33 @@ def test_tensor_core_prefill_against_oracle_and_per_pass_prefill(name):
         case.close()
 
 
+@pytest.mark.parametrize("name", ["mini_mha_b1", "mini_gqa_b3", "gqa4_b5_ragged", "wide_mha_b16_ragged"])
+@pytest.mark.parametrize("pairs", [17, 128, 129, 256, 257, 700])
+def test_tensor_core_prefill_tile_edges(name, pairs):
+    """Pairs around the tiles' edges (128 per CTA, 256 per cluster), weight rows that fill neither tile width, heads of
+    64 and 128: the cache rows against the 16-pairs-per-pass kernels.  Both round the same operand to bf16 and the rows
+    when they are stored; a sum in another order may move either by one unit in the last place (2^-8 of the value)."""
+    import torch
+    wl = hi.scaled(hi.workload(name), batch=2, text_len=None, text_len_range=(1, 2))
+    case = Case(wl, max_len=pairs + 8)
+    try:
+        g = torch.Generator(device="cuda").manual_seed(pairs)
+        ids = torch.randint(0, wl.dims.vocab, (pairs,), dtype=torch.int32, device="cuda", generator=g)
+        hidden = torch.randn(pairs, wl.dims.d, device="cuda", generator=g).to(torch.bfloat16)
+        cu = [0, pairs // 3 + 1, pairs]
+        rows = []
+        for tc in (True, False):
+            case.drafter.set_tc_prefill(tc)
+            case.drafter.prefill(ids, hidden, cu, start_pos=[0, 0], resid0=case.d_resid[0])
+            case.drafter.status()
+            rows.append([case.drafter.read_kv(b, 0, cu[b + 1] - cu[b] - 1) for b in range(2) if cu[b + 1] - cu[b] > 1])
+        for x, y in zip(*rows):
+            for got, want in zip(x, y):
+                assert (got - want).abs().max() <= 2.0 ** -7 * want.abs().max()
+    finally:
+        case.close()
+
+
 def test_more_sequences_than_the_chain_kernels_take():
     """20 sequences: beyond the 16 of the tensor-core chain kernel, so the per-phase kernels run in two passes."""
     wl = hi.scaled(hi.workload("mini_gqa_b16_ragged"), batch=20, k=3, seed=2103)
