@@ -14,7 +14,7 @@ struct hivis_ctx {
     int dtype;
     size_t esize;
     int qw, kvw, qkvw;
-    int rows_cap;                 // batch rows the workspaces hold: 32, or 64 for more than 32 slots
+    int rows_cap;                 // batch rows the workspaces hold: the 64 columns of the widest chain kernel
     int device;
     // weights (library-owned copies)
     void *embed, *lm_head, *fc, *norm1, *wqkv, *bqkv, *wo, *norm2, *wgu, *wdown, *resid_proj;
@@ -59,7 +59,9 @@ struct hivis_ctx {
     float2* pf_rope;              // [map_cap][head_dim / 2]
     u64* phase_t;                 // [HIVIS_MAX_K][HIVIS_PHASE_EVENTS][num_sms]
     int phase_k;                  // draft steps of the last recorded launch (0: none)
-    TcMaps tc_maps, tc_maps_wide; // operands of 32 rows; of 64 rows (calls of more than 32 sequences)
+    TcMaps tc_maps, tc_maps_wide; // operands of 32 rows; of 64 rows (more than 32 columns)
+    alignas(64) unsigned char tc_map_wkv[128];   // the K and V rows of the stacked QKV matrix
+    float *pf_u, *pf_kv;          // small prefix builds in the chain kernel: [64][d], [64][2 kvw]
     float* tc_partial;
     int* tile_ctr;
     int tc_tiles;
@@ -248,7 +250,7 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
     c->qw = cfg->n_q_heads * cfg->head_dim;
     c->kvw = cfg->n_kv_heads * cfg->head_dim;
     c->qkvw = c->qw + 2 * c->kvw;
-    c->rows_cap = cfg->max_batch > TC_OP_ROWS ? HIVIS_MAX_BATCH : TC_OP_ROWS;
+    c->rows_cap = HIVIS_MAX_BATCH;
     c->launches = 0;
     c->err[0] = 0;
     c->tap_B = 0;
@@ -262,6 +264,7 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
     cudaStream_t st = (cudaStream_t)stream;
     const size_t es = c->esize;
     const long long d = cfg->d, F = cfg->ffn, V = cfg->vocab, R = c->rows_cap, MB = cfg->max_batch;
+    const long long AR = MB > TC_OP_ROWS ? MB : TC_OP_ROWS;      // sequences the attention's partial buffers hold
     c->chunk = 128;
     c->nsplit_cap = (cfg->max_len + 31) / 32 + 1;       // blocks of 32 rows, and the rows of the running call
     if (c->nsplit_cap > 513) c->nsplit_cap = 513;
@@ -319,12 +322,12 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
          dalloc(c, &c->ssq2, tiles1 * R) && dalloc(c, &c->keys, R * c->key_stride) &&
          dalloc(c, &c->vkeys, MB * (cfg->max_k + 1)) && dalloc(c, &c->varrive, MB) &&
          dalloc(c, &c->vstats, (long long)sampled_stats_entries(cfg->max_batch, cfg->max_k, cfg->vocab)) &&
-         dalloc(c, &c->part_acc, R * cfg->n_q_heads * (long long)c->nsplit_cap * cfg->head_dim) &&
-         dalloc(c, &c->part_ml, R * cfg->n_q_heads * (long long)c->nsplit_cap * 2) &&
+         dalloc(c, &c->part_acc, AR * cfg->n_q_heads * (long long)c->nsplit_cap * cfg->head_dim) &&
+         dalloc(c, &c->part_ml, AR * cfg->n_q_heads * (long long)c->nsplit_cap * 2) &&
          dalloc(c, &c->counters, R * cfg->n_q_heads) && dalloc(c, &c->bar_counter, 1) &&
          dalloc(c, &c->error_flag, 2) && dalloc(c, &c->slot_of, c->map_cap) &&
          dalloc(c, &c->row_of, c->map_cap) && dalloc(c, &c->xe_h, R * d) &&
-         dalloc(c, &c->rope_tab, 2 * 16 * tc_groups(cfg->max_batch) * (cfg->head_dim / 2));
+         dalloc(c, &c->rope_tab, 2 * R * (cfg->head_dim / 2));
     {
         TreeBufs& T = c->tree;
         ok = ok && dalloc(c, &T.P, 1) && dalloc(c, &T.fr_cand, TREE_MAX_TOPK) && dalloc(c, &T.fr_tok, TREE_MAX_TOPK) &&
@@ -410,17 +413,20 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
         ChainArgs ca;
         fill_chain_args(c, &ca);
         c->tc_tiles = tc_max_tiles(ca.ph);
-        bool ok2 = dalloc(c, &c->tc_partial, (size_t)c->num_sms * 2 * 16 * 128 * tc_groups(cfg->max_batch)) && dalloc(c, &c->tile_ctr, c->tc_tiles) &&
+        bool ok2 = dalloc(c, &c->tc_partial, (size_t)c->num_sms * 2 * R * 128) && dalloc(c, &c->tile_ctr, c->tc_tiles) &&
                    dalloc(c, &c->phase_t, (size_t)HIVIS_MAX_K * HIVIS_PHASE_EVENTS * c->num_sms);
         if (ok2) ok2 = cudaMemsetAsync(c->tile_ctr, 0, c->tc_tiles * sizeof(int), st) == cudaSuccess;
         if (ok2)
             ok2 = tc_build_maps(&c->tc_maps, ca.ph, cfg->d, c->qw, cfg->ffn, c->feat_h, c->xq, c->attn_h, c->xm, c->act_h,
                                 c->xe_h, c->Kc, c->Vc, MB * (long long)cfg->n_kv_heads * cfg->max_len,
                                 cfg->head_dim, TC_OP_ROWS) == cudaSuccess;
-        if (ok2 && cfg->max_batch > TC_OP_ROWS)
+        if (ok2)
             ok2 = tc_build_maps(&c->tc_maps_wide, ca.ph, cfg->d, c->qw, cfg->ffn, c->feat_h, c->xq, c->attn_h, c->xm, c->act_h,
                                 c->xe_h, c->Kc, c->Vc, MB * (long long)cfg->n_kv_heads * cfg->max_len,
                                 cfg->head_dim, HIVIS_MAX_BATCH) == cudaSuccess;
+        if (ok2)
+            ok2 = dalloc(c, &c->pf_u, R * d) && dalloc(c, &c->pf_kv, R * 2 * c->kvw) &&
+                  tc_encode_weight(c->tc_map_wkv, wqkv + (long long)c->qw * d * es, 2 * c->kvw, d) == cudaSuccess;
         if (!ok2) cudaGetLastError();
         c->tc_ok = ok2;
     }
@@ -596,6 +602,84 @@ static int run_after_attention(hivis_ctx* c, bool mma, int b0, int nb, u64* keys
     return HIVIS_OK;
 }
 
+// Arguments of the tensor-core chain kernel for B columns and k steps (the whole step; callers narrow seq_first /
+// seq_last and bar_base when they run a part of it).
+static void fill_tc_args(hivis_ctx* c, TcArgs* out, int B, int k, int lo, const float* rho, int n_resid,
+                         const int32_t* forced_ids, float* out_logits) {
+    const hivis_config& g = c->cfg;
+    ChainArgs ca;
+    fill_chain_args(c, &ca);
+    TcArgs& a = *out;
+    memset(&a, 0, sizeof(a));
+    for (int p = 0; p < PH_COUNT; ++p) a.ph[p] = ca.ph[p];
+    a.k = k; a.B = B; a.lo = lo;
+    a.d = g.d; a.qw = c->qw; a.kvw = c->kvw; a.F = g.ffn; a.V = g.vocab; a.Hq = g.n_q_heads; a.Hkv = g.n_kv_heads;
+    a.dh = g.head_dim; a.max_len = g.max_len; a.eps = g.rms_eps; a.scale = 1.0f / sqrtf((float)g.head_dim);
+    a.norm1 = (const bf16*)c->norm1; a.norm2 = (const bf16*)c->norm2; a.bqkv = (const bf16*)c->bqkv;
+    a.rho = rho; a.n_resid = n_resid;
+    a.slots = c->d_slots; a.pos0 = c->d_pos0; a.cur_id = c->cur_id; a.forced = forced_ids;
+    a.keys = c->keys; a.key_stride = c->key_stride;
+    a.u = c->u; a.qkv = c->qkv; a.attn = c->attn; a.y = c->y; a.feat = c->feat;
+    a.feat_h = c->feat_h; a.xq_h = c->xq; a.attn_h = c->attn_h; a.xm_h = c->xm; a.act_h = c->act_h;
+    a.xe_h = c->xe_h; a.embed = (const bf16*)c->embed; a.rope_tab = c->rope_tab;
+    a.ssq1 = c->ssq1; a.ssq2 = c->ssq2; a.logits_out = out_logits;
+    a.partial = c->tc_partial; a.tile_ctr = c->tile_ctr;
+    a.Kc = c->Kc; a.Vc = c->Vc; a.inv_freq = c->inv_freq; a.part_acc = c->part_acc; a.part_ml = c->part_ml;
+    a.counters = c->counters;
+    a.attn_nslot = c->nsplit_cap;
+    a.bar_counter = c->bar_counter; a.bar_base = c->bar_count_host + (c->debug_skew ? (1ull << 40) : 0ull);
+    a.wait_cycles = c->wait_cycles; a.error_flag = c->error_flag; a.id_flag = c->id_flag;
+    a.l2_keep = c->opt_l2_keep;
+    a.phase_t = nullptr;
+    a.seq_first = 0; a.seq_last = 7;
+}
+
+// what every prefix build leaves in the host's mirrors
+static void prefill_done(hivis_ctx* c, const SlotList& sl, const int* new_upper, bool exact) {
+    for (int b = 0; b < sl.n; ++b) {
+        const int s = sl.slot[b];
+        c->kv_exact[s] = c->kv_exact[s] || exact;
+        c->kv_upper[s] = new_upper[b];
+        c->pending[s] = true;
+        c->have_pair[s] = true;
+        c->last_k[s] = 0;
+    }
+}
+
+// A prefix build of at most 64 pairs in the tensor-core chain kernel: bookkeeping and operand rows, then the phases fusion
+// FC and QKV with the K and V rows of the stacked matrix, then the rotation and the cache rows.  The hidden states are read
+// where the caller has them; u and the K/V values go to buffers of their own.
+static int prefill_in_chain_kernel(hivis_ctx* c, const SlotList& sl, const CuSeqlens& cu, const SlotList& start, int pairs,
+                                   const int32_t* ids, const bf16* hidden, const bf16* resid0, cudaStream_t st) {
+    const hivis_config& g = c->cfg;
+    const int d = g.d, op_rows = pairs <= TC_OP_ROWS ? TC_OP_ROWS : HIVIS_MAX_BATCH;
+    const bool fold_rho = resid0 && !c->resid_proj;
+    if (resid0 && !fold_rho) {
+        const int rc = prepare_rho(c, resid0, 1, st);
+        if (rc) return rc;
+    }
+    TcMaps maps = pairs <= TC_OP_ROWS ? c->tc_maps : c->tc_maps_wide;
+    memcpy(maps.m[TCM_W + PH_QKV], c->tc_map_wkv, 128);
+    CK(c, tc_encode_operand(maps.m[TCM_X_FEAT], hidden, pairs, d, op_rows));
+    CKL(c, launch_prefill_setup_rows(sl, cu, start, d, ids, hidden, c->kv_len, c->pend_feat, c->pend_id, c->slot_of, c->row_of,
+                                     op_rows, (const bf16*)c->embed, g.vocab, c->xe_h, c->id_flag, fold_rho ? resid0 : nullptr,
+                                     c->rho, st));
+    TcArgs a;
+    fill_tc_args(c, &a, pairs, 1, tc_lo_offset(pairs), resid0 ? c->rho : nullptr, 1, nullptr, nullptr);
+    a.ph[PH_QKV] = {(const bf16*)c->wqkv + (long long)c->qw * d, 2 * c->kvw, d};
+    a.bqkv = c->bqkv ? (const bf16*)c->bqkv + c->qw : nullptr;
+    a.u = c->pf_u;
+    a.qkv = c->pf_kv;
+    a.seq_first = 1; a.seq_last = 2;                                 // fusion FC, QKV
+    const u64 G = (u64)c->num_sms;
+    a.bar_base = c->bar_count_host - G;                              // as if the gather had been arrived on
+    CKL(c, launch_tc_chain(maps, a, c->num_sms, st));
+    c->bar_count_host += 2 * G;
+    CKL(c, launch_kv_append(c->dtype, c->pf_kv, pairs, c->slot_of, c->row_of, c->inv_freq, g.n_kv_heads, g.head_dim, g.max_len,
+                            c->Kc, c->Vc, st));
+    return HIVIS_OK;
+}
+
 int hivis_prefill(hivis_ctx* c, int B, const int* seq_slots_host, const int32_t* ids, const void* hidden,
                   const int32_t* cu_seqlens_host, const int32_t* start_pos_host, const void* resid0,
                   void* stream) {
@@ -636,6 +720,21 @@ int hivis_prefill(hivis_ctx* c, int B, const int* seq_slots_host, const int32_t*
     cudaStream_t st = (cudaStream_t)stream;
     const int d = c->cfg.d;
     const float* rho0 = nullptr;
+    // Up to 64 pairs (the rows that a verified draft left to rebuild: a few per sequence) are a batch of columns like any
+    // other: the fusion FC and the K/V projection run as two phases of the tensor-core chain kernel, in one pass over
+    // their weights with every SM at work.  The barrier counter of that kernel is counted on the host, so a call that
+    // is being captured into a graph (and replayed without the host) takes the kernels below.
+    if (c->tc_ok && c->opt_tc != 0 &&
+        (total <= 16 || (total <= HIVIS_MAX_BATCH && c->opt_tc_prefill > 0 && total >= c->opt_tc_prefill))) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CK(c, cudaStreamIsCapturing(st, &cap));
+        if (cap == cudaStreamCaptureStatusNone) {
+            rc = prefill_in_chain_kernel(c, sl, cu, start, (int)total, ids, (const bf16*)hidden, (const bf16*)resid0, st);
+            if (rc) return rc;
+            prefill_done(c, sl, new_upper, start_pos_host != nullptr);
+            return HIVIS_OK;
+        }
+    }
     if (resid0) {
         rc = prepare_rho(c, resid0, 1, st);
         if (rc) return rc;
@@ -674,47 +773,8 @@ int hivis_prefill(hivis_ctx* c, int B, const int* seq_slots_host, const int32_t*
                                 c->cfg.n_kv_heads, c->cfg.head_dim, c->cfg.max_len, c->Kc, c->Vc, st));
     }
     }
-    for (int b = 0; b < B; ++b) {
-        const int s = sl.slot[b];
-        c->kv_exact[s] = c->kv_exact[s] || start_pos_host != nullptr;
-        c->kv_upper[s] = new_upper[b];
-        c->pending[s] = true;
-        c->have_pair[s] = true;
-        c->last_k[s] = 0;
-    }
+    prefill_done(c, sl, new_upper, start_pos_host != nullptr);
     return HIVIS_OK;
-}
-
-// Arguments of the tensor-core chain kernel for B columns and k steps (the whole step; callers narrow seq_first /
-// seq_last and bar_base when they run a part of it).
-static void fill_tc_args(hivis_ctx* c, TcArgs* out, int B, int k, int lo, const float* rho, int n_resid,
-                         const int32_t* forced_ids, float* out_logits) {
-    const hivis_config& g = c->cfg;
-    ChainArgs ca;
-    fill_chain_args(c, &ca);
-    TcArgs& a = *out;
-    memset(&a, 0, sizeof(a));
-    for (int p = 0; p < PH_COUNT; ++p) a.ph[p] = ca.ph[p];
-    a.k = k; a.B = B; a.lo = lo;
-    a.d = g.d; a.qw = c->qw; a.kvw = c->kvw; a.F = g.ffn; a.V = g.vocab; a.Hq = g.n_q_heads; a.Hkv = g.n_kv_heads;
-    a.dh = g.head_dim; a.max_len = g.max_len; a.eps = g.rms_eps; a.scale = 1.0f / sqrtf((float)g.head_dim);
-    a.norm1 = (const bf16*)c->norm1; a.norm2 = (const bf16*)c->norm2; a.bqkv = (const bf16*)c->bqkv;
-    a.rho = rho; a.n_resid = n_resid;
-    a.slots = c->d_slots; a.pos0 = c->d_pos0; a.cur_id = c->cur_id; a.forced = forced_ids;
-    a.keys = c->keys; a.key_stride = c->key_stride;
-    a.u = c->u; a.qkv = c->qkv; a.attn = c->attn; a.y = c->y; a.feat = c->feat;
-    a.feat_h = c->feat_h; a.xq_h = c->xq; a.attn_h = c->attn_h; a.xm_h = c->xm; a.act_h = c->act_h;
-    a.xe_h = c->xe_h; a.embed = (const bf16*)c->embed; a.rope_tab = c->rope_tab;
-    a.ssq1 = c->ssq1; a.ssq2 = c->ssq2; a.logits_out = out_logits;
-    a.partial = c->tc_partial; a.tile_ctr = c->tile_ctr;
-    a.Kc = c->Kc; a.Vc = c->Vc; a.inv_freq = c->inv_freq; a.part_acc = c->part_acc; a.part_ml = c->part_ml;
-    a.counters = c->counters;
-    a.attn_nslot = c->nsplit_cap;
-    a.bar_counter = c->bar_counter; a.bar_base = c->bar_count_host + (c->debug_skew ? (1ull << 40) : 0ull);
-    a.wait_cycles = c->wait_cycles; a.error_flag = c->error_flag; a.id_flag = c->id_flag;
-    a.l2_keep = c->opt_l2_keep;
-    a.phase_t = nullptr;
-    a.seq_first = 0; a.seq_last = 7;
 }
 
 // hivis_draft and hivis_draft_sampled (uniforms != nullptr: every step's token is drawn with the Gumbel-max rule)

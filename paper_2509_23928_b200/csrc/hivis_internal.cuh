@@ -202,6 +202,8 @@ struct TcArgs {
 cudaError_t tc_build_maps(TcMaps* maps, const ChainPhase* ph, int d, int qw, int F, const bf16* feat_h,
                           const bf16* xq_h, const bf16* attn_h, const bf16* xm_h, const bf16* act_h, const bf16* xe_h,
                           const void* Kc, const void* Vc, long long cache_rows, int dh, int op_rows);
+cudaError_t tc_encode_weight(unsigned char* map, const void* W, long long rows, long long cols);
+cudaError_t tc_encode_operand(unsigned char* map, const void* x, long long rows, long long cols, int op_rows);
 bool tc_supported(int d, int dh, int Hq, int Hkv, int F);
 int tc_max_tiles(const ChainPhase* ph);
 cudaError_t launch_tc_chain(const TcMaps& maps, const TcArgs& a, int grid, cudaStream_t st);
@@ -306,6 +308,12 @@ cudaError_t launch_prefill_setup(int dtype, const SlotList& sl, const CuSeqlens&
                                  const SlotList& start /* -1 = append */, int d, const int32_t* ids,
                                  const void* hidden, int* kv_len, float* pend_feat, int* pend_id,
                                  int* slot_of, int* row_of, cudaStream_t st);
+// the same for a call whose pairs are one batch of the tensor-core chain kernel (bf16): also gathers the embedding rows of
+// the pairs' tokens (zero rows up to op_rows) and converts the residual row (nullable) to fp32
+cudaError_t launch_prefill_setup_rows(const SlotList& sl, const CuSeqlens& cu, const SlotList& start, int d, const int32_t* ids,
+                                      const bf16* hidden, int* kv_len, float* pend_feat, int* pend_id, int* slot_of,
+                                      int* row_of, int op_rows, const bf16* embed, int vocab, bf16* xe_h, int* id_flag,
+                                      const bf16* resid, float* rho, cudaStream_t st);
 // RoPE(K) and store K,V rows of a chunk of packed entries
 cudaError_t launch_kv_append(int dtype, const float* kv /*[P][2*kvw]*/, int P, const int* slot_of,
                              const int* row_of, const double* inv_freq, int Hkv, int dh, int max_len,

@@ -395,6 +395,16 @@ __device__ __forceinline__ TcAttInfo tc_att_info(const TcArgs& a, int cta, int G
     const int HG = a.Hq / GQ;
     TcAttInfo t;
     t.total = 0;
+    if (!seq_on(a, TC_SEQ_ATTN)) {          // no attention in this launch (the row counts need not be set)
+        t.pl.U = 0; t.pl.NW = 0;
+        t.plm.T = 0; t.plm.NW = 0; t.plm.nkeys = 0;
+#pragma unroll
+        for (int w = 0; w < TC_ATT_WARPS; ++w) {
+            t.job[w] = AttmJob{0, 0, 0, 0, 0, 1, 0u};
+            t.n[w] = 0;
+        }
+        return t;
+    }
     if constexpr (AttSel<GQ>::mma) {
         t.plm = attm_plan(a.pos0, a.B, HG, G * TC_ATT_WARPS);
         t.pl.U = 0; t.pl.NW = 0;
@@ -413,15 +423,6 @@ __device__ __forceinline__ TcAttInfo tc_att_info(const TcArgs& a, int cta, int G
             t.n[w] = u1 - u0;
         }
         t.total += t.n[w];
-    }
-    if (!seq_on(a, TC_SEQ_ATTN)) {
-#pragma unroll
-        for (int w = 0; w < TC_ATT_WARPS; ++w) {
-            t.n[w] = 0;
-            if constexpr (AttSel<GQ>::mma) t.job[w].units = 0;
-        }
-        t.total = 0;
-        t.pl.U = 0;
     }
     return t;
 }

@@ -274,6 +274,47 @@ def test_tensor_core_prefill_tile_edges(name, pairs):
         case.close()
 
 
+@pytest.mark.parametrize("name,project", [("mini_mha_b1", False), ("mini_gqa_b3", False), ("gqa4_b5_ragged", True),
+                                          ("wide_mha_b16_ragged", False)])
+@pytest.mark.parametrize("pairs", [1, 2, 16, 17, 32, 33, 64])
+def test_small_prefix_builds_in_the_chain_kernel(name, project, pairs):
+    """1..64 pairs as columns of the chain kernel (one, two and four column groups, full and partly filled) against the
+    kernels of 16 pairs per pass, after a larger call has left its rows in every buffer; then the draft that consumes the
+    pending pairs.  Both paths round the same operand (the chain kernel keeps its remainder up to 16 pairs) and the stored
+    rows to bf16: one unit in the last place (2^-8 of the value) apart."""
+    import torch
+    wl = hi.scaled(hi.workload(name), batch=2, text_len=None, text_len_range=(1, 2))
+    extra = {"resid_proj": hi.make_weights(wl.dims, 77)["fc"][:, :wl.dims.d].copy()} if project else None
+    case = Case(wl, max_len=200, extra_weights=extra)
+    try:
+        dr, g = case.drafter, torch.Generator(device="cuda").manual_seed(pairs)
+
+        def some(n):
+            return (torch.randint(0, wl.dims.vocab, (n,), dtype=torch.int32, device="cuda", generator=g),
+                    torch.randn(n, wl.dims.d, device="cuda", generator=g).to(torch.bfloat16))
+        big, old, new = some(64), some(60), some(pairs)
+        cu = [0, pairs] if pairs == 1 else [0, pairs // 3 + (pairs < 3), pairs]
+        B = len(cu) - 1
+        rows, drafts = [], []
+        for tc in (True, False):
+            dr.set_tc_kernel("auto")
+            dr.prefill(*big, [0, 64], start_pos=[0], resid0=case.d_resid[0])
+            dr.set_tc_kernel("auto" if tc else 0)
+            dr.set_tc_prefill(tc)
+            dr.prefill(*old, [0, 25, 60], start_pos=[0, 0], resid0=case.d_resid[0])
+            dr.prefill(*new, cu, start_pos=[20, 30][:B], resid0=case.d_resid[0])
+            drafts.append(dr.draft(B, 1, case.d_resid, want_logits=True)[1])
+            dr.status()
+            rows.append([dr.read_kv(b, 0, [20, 30][b] + cu[b + 1] - cu[b]) for b in range(B)])
+        for x, y in zip(*rows):
+            for got, want in zip(x, y):
+                assert (got - want).abs().max() <= 2.0 ** -7 * want.abs().max()
+        err = row_rel_err(drafts[0].cpu().numpy(), drafts[1].cpu().numpy())
+        assert err.max() <= LOGIT_RTOL
+    finally:
+        case.close()
+
+
 def test_more_sequences_than_the_chain_kernels_take():
     """20 sequences: beyond the 16 of the tensor-core chain kernel, so the per-phase kernels run in two passes."""
     wl = hi.scaled(hi.workload("mini_gqa_b16_ragged"), batch=20, k=3, seed=2103)
