@@ -86,6 +86,8 @@ struct hivis_ctx {
     int64_t launches;
     char err[256];
     std::vector<void*> allocs;
+    char* arena;                  // the rest of the chunk that small buffers are carved from
+    size_t arena_left;
     // optional per-kernel-class timing of hivis_draft (events around every launch)
     bool prof_on;
     std::vector<cudaEvent_t> prof_ev;
@@ -152,16 +154,32 @@ static void fill_chain_args(hivis_ctx* c, ChainArgs* a);
 
 static bool misaligned(const void* p) { return (((uintptr_t)p) & 15u) != 0; }
 
+// A context has some seventy buffers, most of them small, and every device allocation (and its release) costs tens to
+// hundreds of microseconds: requests of up to ARENA_MAX bytes are carved out of chunks.
+#define ARENA_CHUNK ((size_t)24 << 20)
+#define ARENA_MAX ((size_t)6 << 20)
 template <typename T>
 static bool dalloc(hivis_ctx* c, T** p, size_t count) {
+    size_t bytes = (count * sizeof(T) + 511) & ~(size_t)511;
+    if (!bytes) bytes = 512;
+    if (bytes <= ARENA_MAX && bytes <= c->arena_left) {
+        *p = (T*)c->arena;
+        c->arena += bytes;
+        c->arena_left -= bytes;
+        return true;
+    }
+    const size_t want = bytes <= ARENA_MAX ? ARENA_CHUNK : bytes;
     void* q = nullptr;
-    const size_t bytes = (count * sizeof(T) + 255) & ~(size_t)255;
-    if (cudaMalloc(&q, bytes ? bytes : 256) != cudaSuccess) {
+    if (cudaMalloc(&q, want) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
     c->allocs.push_back(q);
     *p = (T*)q;
+    if (want != bytes) {
+        c->arena = (char*)q + bytes;
+        c->arena_left = want - bytes;
+    }
     return true;
 }
 
@@ -253,6 +271,8 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
     c->rows_cap = HIVIS_MAX_BATCH;
     c->launches = 0;
     c->err[0] = 0;
+    c->arena = nullptr;
+    c->arena_left = 0;
     c->tap_B = 0;
     c->tap_mma = false;
     c->prof_on = false;
@@ -451,6 +471,16 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
 // residual rows in the context dtype -> fp32 rho rows (projected by resid_proj when present)
 static int prepare_rho(hivis_ctx* c, const void* resid, int R, cudaStream_t st) {
     const int d = c->cfg.d;
+    if (c->resid_proj && c->dtype == HIVIS_BF16) {
+        // the rows are bf16 as they are: one pass over the projection for all of them on the tensor cores (fp32 sums of
+        // exact products, as on the FMA path, which reads the matrix once per row: 24 us for 4 rows of 4096)
+        LinArgs a;
+        memset(&a, 0, sizeof(a));
+        a.W = c->resid_proj; a.N = d; a.K = d; a.B = R; a.ldb = c->rows_cap;
+        a.xin_h = (const bf16*)resid; a.out = c->rho;
+        CKL(c, launch_gemm_mma(PRO_PLAIN, EPI_QKV, a, st));
+        return HIVIS_OK;
+    }
     float* dst = c->resid_proj ? c->rho_raw : c->rho;
     CKL(c, launch_convert_rows(c->dtype, resid, dst, (long long)R * d, st));
     if (c->resid_proj) {
@@ -653,8 +683,8 @@ static int prefill_in_chain_kernel(hivis_ctx* c, const SlotList& sl, const CuSeq
                                    const int32_t* ids, const bf16* hidden, const bf16* resid0, cudaStream_t st) {
     const hivis_config& g = c->cfg;
     const int d = g.d, op_rows = pairs <= TC_OP_ROWS ? TC_OP_ROWS : HIVIS_MAX_BATCH;
-    const bool fold_rho = resid0 && !c->resid_proj;
-    if (resid0 && !fold_rho) {
+    const bool raw_rho = resid0 && !c->resid_proj;
+    if (resid0 && !raw_rho) {
         const int rc = prepare_rho(c, resid0, 1, st);
         if (rc) return rc;
     }
@@ -662,10 +692,10 @@ static int prefill_in_chain_kernel(hivis_ctx* c, const SlotList& sl, const CuSeq
     memcpy(maps.m[TCM_W + PH_QKV], c->tc_map_wkv, 128);
     CK(c, tc_encode_operand(maps.m[TCM_X_FEAT], hidden, pairs, d, op_rows));
     CKL(c, launch_prefill_setup_rows(sl, cu, start, d, ids, hidden, c->kv_len, c->pend_feat, c->pend_id, c->slot_of, c->row_of,
-                                     op_rows, (const bf16*)c->embed, g.vocab, c->xe_h, c->id_flag, fold_rho ? resid0 : nullptr,
-                                     c->rho, st));
+                                     op_rows, (const bf16*)c->embed, g.vocab, c->xe_h, c->id_flag, st));
     TcArgs a;
-    fill_tc_args(c, &a, pairs, 1, tc_lo_offset(pairs), resid0 ? c->rho : nullptr, 1, nullptr, nullptr);
+    fill_tc_args(c, &a, pairs, 1, tc_lo_offset(pairs), resid0 && !raw_rho ? c->rho : nullptr, 1, nullptr, nullptr);
+    a.rho_h = raw_rho ? resid0 : nullptr;
     a.ph[PH_QKV] = {(const bf16*)c->wqkv + (long long)c->qw * d, 2 * c->kvw, d};
     a.bqkv = c->bqkv ? (const bf16*)c->bqkv + c->qw : nullptr;
     a.u = c->pf_u;
@@ -802,16 +832,24 @@ static int draft_impl(hivis_ctx* c, int B, const int* seq_slots_host, int k, con
     cudaStream_t st = (cudaStream_t)stream;
     const hivis_config& g = c->cfg;
     const int d = g.d, F = g.ffn, V = g.vocab;
-    if (resid) {
+    // The chain kernels read rows that need no projection where the caller has them.
+    const bool one_seq = B == 1 && c->opt_chain && c->chain_ok && !(c->tc_ok && c->opt_tc == 2);
+    // The kernel numbers attention units x warps in 32 bits; a batch beyond that (hundreds of heads on long caches) takes
+    // the per-phase kernels, as do draws for more than 16 sequences (refused below).
+    const bool tc_fits = B <= 16 || (!uniforms && (long long)B * g.n_q_heads * ((max_rows + 31) / 32 + 1) * 4 * c->num_sms < (1ll << 32));
+    const bool in_tc = !one_seq && c->tc_ok && c->opt_tc != 0 && tc_fits;
+    const bool raw_rho = resid && !c->resid_proj && (one_seq || in_tc);
+    if (resid && !raw_rho) {
         rc = prepare_rho(c, resid, n_resid, st);
         if (rc) return rc;
     }
-    if (B == 1 && c->opt_chain && c->chain_ok && !(c->tc_ok && c->opt_tc == 2)) {
+    if (one_seq) {
         // one sequence: all k steps in one persistent cooperative kernel
         ChainArgs a;
         fill_chain_args(c, &a);
         a.k = k;
-        a.rho = resid ? c->rho : nullptr;
+        a.rho = resid && !raw_rho ? c->rho : nullptr;
+        a.rho_w = raw_rho ? resid : nullptr;
         a.n_resid = resid ? n_resid : 1;
         a.slot = sl.slot[0];
         a.forced = forced_ids;
@@ -833,17 +871,16 @@ static int draft_impl(hivis_ctx* c, int B, const int* seq_slots_host, int k, con
         c->tap_mma = false;
         return HIVIS_OK;
     }
-    // The kernel numbers attention units x warps in 32 bits; a batch beyond that (hundreds of heads on long caches) takes
-    // the per-phase kernels, as do draws for more than 16 sequences (refused below).
-    const bool tc_fits = B <= 16 || (!uniforms && (long long)B * g.n_q_heads * ((max_rows + 31) / 32 + 1) * 4 * c->num_sms < (1ll << 32));
-    if (c->tc_ok && c->opt_tc != 0 && tc_fits) {
+    if (in_tc) {
         // bf16: all k steps in one cooperative tensor-core kernel
         const int lo = tc_lo_offset(B);
         CKP(c, CLS_OTHER, st, launch_tc_setup(sl, k, d, lo, c->d_slots, c->d_pos0, c->kv_len, c->pend_feat, c->pend_id,
                                               c->feat, c->feat_h, c->cur_id, c->keys, c->key_stride, (const bf16*)c->embed,
                                               V, c->xe_h, c->id_flag, st));
         TcArgs a;
-        fill_tc_args(c, &a, B, k, lo, resid ? c->rho : nullptr, resid ? n_resid : 1, forced_ids, out_logits);
+        fill_tc_args(c, &a, B, k, lo, resid && !raw_rho ? c->rho : nullptr, resid ? n_resid : 1, forced_ids, out_logits);
+        a.rho_h = raw_rho ? (const bf16*)resid : nullptr;
+        a.out_ids = out_ids;
         a.gumbel_u = uniforms;
         a.inv_t = inv_t;
         if (c->opt_phase_times) {
@@ -854,7 +891,6 @@ static int draft_impl(hivis_ctx* c, int B, const int* seq_slots_host, int k, con
         c->debug_skew = false;
         CKP(c, CLS_CHAIN, st, launch_tc_chain(B <= TC_OP_ROWS ? c->tc_maps : c->tc_maps_wide, a, c->num_sms, st));
         c->bar_count_host += (u64)c->num_sms * (u64)(tc_barriers_per_step() * k);
-        CKP(c, CLS_OTHER, st, launch_draft_finish(B, k, c->keys, c->key_stride, out_ids, st));
         for (int b = 0; b < B; ++b) {
             const int s = sl.slot[b];
             c->kv_upper[s] += k;
@@ -1019,7 +1055,9 @@ int hivis_draft_tree(hivis_ctx* c, int slot, int topk, int depth, int keep, cons
     const hivis_config& g = c->cfg;
     const int d = g.d, V = g.vocab;
     int rc;
-    if (resid) {
+    const bool tc = c->tc_ok && c->opt_tc != 0;
+    const bool raw_rho = resid && !c->resid_proj && tc;              // rows that need no projection are read where they are
+    if (resid && !raw_rho) {
         rc = prepare_rho(c, resid, n_resid, st);
         if (rc) return rc;
     }
@@ -1027,12 +1065,11 @@ int hivis_draft_tree(hivis_ctx* c, int slot, int topk, int depth, int keep, cons
     CKL(c, launch_tree_begin(slot, d, c->kv_len, c->pend_feat, c->pend_id, c->feat, c->feat_h, c->cur_id, c->d_slots, T, st));
     // bf16 drafters with up to 16 nodes per level (always, by the limit on topk) run the levels' GEMMs in the
     // tensor-core chain kernel, one step long and in two parts around the tree's own attention
-    const bool tc = c->tc_ok && c->opt_tc != 0;
     for (int level = 0; level < depth; ++level) {
         const int nb = level == 0 ? 1 : topk;
         if (level > 0 && !tc) CKL(c, launch_tree_gather(nb, d, c->tree_g, T, c->feat, c->feat_h, c->cur_id, st));
         const int row = level < n_resid - 1 ? level : n_resid - 1;
-        const float* rho = resid ? c->rho + (long long)row * d : nullptr;
+        const float* rho = resid && !raw_rho ? c->rho + (long long)row * d : nullptr;
         if (tc) {
             const int lo = tc_lo_offset(nb);
             const u64 G = (u64)c->num_sms;
@@ -1040,6 +1077,7 @@ int hivis_draft_tree(hivis_ctx* c, int slot, int topk, int depth, int keep, cons
                                            (const bf16*)c->embed, V, c->feat_h, c->xe_h, c->d_pos0, c->id_flag, st));
             TcArgs a;
             fill_tc_args(c, &a, nb, 1, lo, rho, 1, nullptr, c->tree_logits);
+            a.rho_h = raw_rho ? (const bf16*)resid + (long long)row * d : nullptr;
             a.seq_first = 0; a.seq_last = 2;                         // gather, fusion FC, QKV
             c->debug_skew = false;
             CKL(c, launch_tc_chain(c->tc_maps, a, c->num_sms, st));

@@ -106,6 +106,7 @@ struct ChainArgs {
     float eps, scale;
     const void *norm1, *norm2, *bqkv, *embed;
     const float* rho;          // [n_resid][d] fp32, nullable
+    const void* rho_w;         // the caller's residual rows in the context dtype, read where rho is null (nullable)
     int n_resid;
     int slot;
     int* kv_len;
@@ -165,8 +166,10 @@ struct TcArgs {
     float eps, scale;
     const bf16 *norm1, *norm2, *bqkv;
     const float* rho;          // [n_resid][d] fp32, nullable
+    const bf16* rho_h;         // the caller's residual rows, read where rho is null (nullable)
     int n_resid;
     const int *slots, *pos0, *cur_id;     // [B]
+    int32_t* out_ids;          // [B][k], nullable: the chosen tokens, written when the last LM head is complete
     const int* forced;         // [B][k], nullable
     u64* keys;                 // [B][key_stride]
     int key_stride;
@@ -309,11 +312,11 @@ cudaError_t launch_prefill_setup(int dtype, const SlotList& sl, const CuSeqlens&
                                  const void* hidden, int* kv_len, float* pend_feat, int* pend_id,
                                  int* slot_of, int* row_of, cudaStream_t st);
 // the same for a call whose pairs are one batch of the tensor-core chain kernel (bf16): also gathers the embedding rows of
-// the pairs' tokens (zero rows up to op_rows) and converts the residual row (nullable) to fp32
+// the pairs' tokens (zero rows up to op_rows)
 cudaError_t launch_prefill_setup_rows(const SlotList& sl, const CuSeqlens& cu, const SlotList& start, int d, const int32_t* ids,
                                       const bf16* hidden, int* kv_len, float* pend_feat, int* pend_id, int* slot_of,
                                       int* row_of, int op_rows, const bf16* embed, int vocab, bf16* xe_h, int* id_flag,
-                                      const bf16* resid, float* rho, cudaStream_t st);
+                                      cudaStream_t st);
 // RoPE(K) and store K,V rows of a chunk of packed entries
 cudaError_t launch_kv_append(int dtype, const float* kv /*[P][2*kvw]*/, int P, const int* slot_of,
                              const int* row_of, const double* inv_freq, int Hkv, int dh, int max_len,

@@ -308,9 +308,9 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
             __syncthreads();
             if (misc->abort_flag) break;
             const int r0 = misc->r0[PH_FC], rows = misc->units[PH_FC] / misc->cpr[PH_FC];
-            const float* rho = a.rho ? a.rho + (long long)(s < a.n_resid - 1 ? s : a.n_resid - 1) * d : nullptr;
+            const long long rho_row = (long long)(s < a.n_resid - 1 ? s : a.n_resid - 1) * d;
             for (int rl = tid; rl < rows; rl += CHAIN_THREADS)
-                a.u[r0 + rl] = row_sum(PH_FC, rl) + (rho ? rho[r0 + rl] : 0.f);
+                a.u[r0 + rl] = row_sum(PH_FC, rl) + (a.rho ? a.rho[rho_row + r0 + rl] : a.rho_w ? load_as_float<WT>(a.rho_w, rho_row + r0 + rl) : 0.f);
             if (!barrier()) break;
         }
         // ============================================================ RMSNorm + QKV

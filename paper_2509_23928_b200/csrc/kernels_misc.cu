@@ -113,11 +113,10 @@ cudaError_t launch_prefill_setup(int dtype, const SlotList& sl, const CuSeqlens&
 }
 
 // Blocks [0, op_rows): the embedding row of pair j, 16 bytes per thread and turn (a zero row beyond the pairs); then one
-// block per sequence (rows, pending pair, row count); then the residual row.  What bounds it is a chain of two loads.
+// block per sequence (rows, pending pair, row count).  What bounds it is a chain of two loads.
 __global__ void prefill_setup_rows_kernel(SlotList sl, CuSeqlens cu, SlotList start, int d, const int32_t* ids,
                                           const bf16* hidden, int* kv_len, float* pend_feat, int* pend_id, int* slot_of,
-                                          int* row_of, int op_rows, const bf16* embed, int vocab, bf16* xe_h, int* id_flag,
-                                          const bf16* resid, float* rho) {
+                                          int* row_of, int op_rows, const bf16* embed, int vocab, bf16* xe_h, int* id_flag) {
     const int upr = d >> 3;
     if ((int)blockIdx.x < op_rows) {
         const int j = blockIdx.x;
@@ -131,29 +130,22 @@ __global__ void prefill_setup_rows_kernel(SlotList sl, CuSeqlens cu, SlotList st
         return;
     }
     const int b = blockIdx.x - op_rows;
-    const uint4* src;
-    float* dst;
-    if (b < sl.n) {
-        __shared__ int s_base;
-        const int slot = sl.slot[b];
-        const int lo = cu.v[b], hi = cu.v[b + 1];
-        if (threadIdx.x == 0) {
-            const int base = start.slot[b] >= 0 ? start.slot[b] : kv_len[slot];
-            s_base = base;
-            pend_id[slot] = ids[hi - 1];
-            kv_len[slot] = base + (hi - lo) - 1;
-        }
-        __syncthreads();
-        for (int j = lo + threadIdx.x; j < hi; j += blockDim.x) {
-            slot_of[j] = slot;
-            row_of[j] = (j == hi - 1) ? -1 : s_base + (j - lo);
-        }
-        src = (const uint4*)(hidden + (long long)(hi - 1) * d);
-        dst = pend_feat + (long long)slot * d;
-    } else {
-        src = (const uint4*)resid;
-        dst = rho;
+    __shared__ int s_base;
+    const int slot = sl.slot[b];
+    const int lo = cu.v[b], hi = cu.v[b + 1];
+    if (threadIdx.x == 0) {
+        const int base = start.slot[b] >= 0 ? start.slot[b] : kv_len[slot];
+        s_base = base;
+        pend_id[slot] = ids[hi - 1];
+        kv_len[slot] = base + (hi - lo) - 1;
     }
+    __syncthreads();
+    for (int j = lo + threadIdx.x; j < hi; j += blockDim.x) {
+        slot_of[j] = slot;
+        row_of[j] = (j == hi - 1) ? -1 : s_base + (j - lo);
+    }
+    const uint4* src = (const uint4*)(hidden + (long long)(hi - 1) * d);
+    float* dst = pend_feat + (long long)slot * d;
     for (int i = threadIdx.x; i < upr; i += blockDim.x) {
         const uint4 w = src[i];
         ((float4*)dst)[2 * i] = make_float4(bf16_lo(w.x), bf16_hi(w.x), bf16_lo(w.y), bf16_hi(w.y));
@@ -163,9 +155,9 @@ __global__ void prefill_setup_rows_kernel(SlotList sl, CuSeqlens cu, SlotList st
 cudaError_t launch_prefill_setup_rows(const SlotList& sl, const CuSeqlens& cu, const SlotList& start, int d, const int32_t* ids,
                                       const bf16* hidden, int* kv_len, float* pend_feat, int* pend_id, int* slot_of,
                                       int* row_of, int op_rows, const bf16* embed, int vocab, bf16* xe_h, int* id_flag,
-                                      const bf16* resid, float* rho, cudaStream_t st) {
-    prefill_setup_rows_kernel<<<op_rows + sl.n + (resid ? 1 : 0), 512, 0, st>>>(
-        sl, cu, start, d, ids, hidden, kv_len, pend_feat, pend_id, slot_of, row_of, op_rows, embed, vocab, xe_h, id_flag, resid, rho);
+                                      cudaStream_t st) {
+    prefill_setup_rows_kernel<<<op_rows + sl.n, 512, 0, st>>>(
+        sl, cu, start, d, ids, hidden, kv_len, pend_feat, pend_id, slot_of, row_of, op_rows, embed, vocab, xe_h, id_flag);
     return cudaGetLastError();
 }
 

@@ -12,44 +12,57 @@ template <int DH, int GQ, bool SMP, int NG>
 cudaError_t tc_launch_t(const TcMaps& maps, const TcArgs& a, int grid, cudaStream_t st);
 
 // ------------------------------------------------------------------------------------------ set-up kernel
-__global__ void tc_setup_kernel(SlotList sl, int k, int d, int lo, int* d_slots, int* d_pos0, int* kv_len,
+// One CTA per operand row, eight elements per thread and turn (d is a multiple of 64): a chain of two loads, 11.5 us with
+// an element per thread and turn.
+__global__ void __launch_bounds__(512) tc_setup_kernel(SlotList sl, int k, int d, int lo, int* d_slots, int* d_pos0, int* kv_len,
                                 const float* pend_feat, const int* pend_id, float* feat, bf16* feat_h, int* cur_id,
                                 u64* keys, int key_stride, const bf16* embed, int vocab, bf16* xe_h, int* id_flag) {
-    const int b = blockIdx.x;
+    const int b = blockIdx.x, upr = d >> 3;
+    uint4* xe = (uint4*)(xe_h + (long long)b * d);
     if (b >= sl.n) {
         // Rows of the embedding operand beyond the batch: the tiled copy always brings all rows, and the accumulator
         // columns of the remainder rows are added to those of the batch rows (an embedding row is exact in bf16, so
         // its remainder is zero).  An earlier, larger batch may have left rows here.
-        for (int i = threadIdx.x; i < (d >> 3); i += blockDim.x)
-            ((uint4*)(xe_h + (long long)b * d))[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = threadIdx.x; i < upr; i += blockDim.x) xe[i] = make_uint4(0u, 0u, 0u, 0u);
         return;
     }
     const int slot = sl.slot[b];
+    const int tok = pend_id[slot];
     if (threadIdx.x == 0) {
         d_slots[b] = slot;
         const int rows = kv_len[slot];
         d_pos0[b] = rows;
         kv_len[slot] = rows + k;            // every draft step appends one K/V row
-        cur_id[b] = pend_id[slot];
+        cur_id[b] = tok;
     }
     if (threadIdx.x < k) keys[(long long)b * key_stride + threadIdx.x] = 0ull;
-    for (int i = threadIdx.x; i < d; i += blockDim.x) {
-        const float v = pend_feat[(long long)slot * d + i];
-        feat[(long long)b * d + i] = v;
-        const bf16 hi = __float2bfloat16_rn(v);
-        feat_h[(long long)b * d + i] = hi;
-        if (lo) feat_h[(long long)(b + lo) * d + i] = __float2bfloat16_rn(v - __bfloat162float(hi));
-    }
     // embedding row of the pending token: the fusion FC's embedding operand of step 0
-    const int id = checked_token(pend_id[slot], vocab, id_flag);
-    for (int i = threadIdx.x; i < (d >> 3); i += blockDim.x)
-        ((uint4*)(xe_h + (long long)b * d))[i] = ((const uint4*)(embed + (long long)id * d))[i];
+    const uint4* er = (const uint4*)(embed + (long long)checked_token(tok, vocab, id_flag) * d);
+    const float4* pf = (const float4*)(pend_feat + (long long)slot * d);
+    float4* ff = (float4*)(feat + (long long)b * d);
+    for (int i = threadIdx.x; i < upr; i += blockDim.x) {
+        const float4 x = pf[2 * i], y = pf[2 * i + 1];
+        xe[i] = er[i];
+        ff[2 * i] = x;
+        ff[2 * i + 1] = y;
+        const float v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+        unsigned hi[4], rem[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const bf16 h0 = __float2bfloat16_rn(v[2 * q]), h1 = __float2bfloat16_rn(v[2 * q + 1]);
+            hi[q] = (unsigned)__bfloat16_as_ushort(h0) | ((unsigned)__bfloat16_as_ushort(h1) << 16);
+            rem[q] = (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(v[2 * q] - __bfloat162float(h0))) |
+                     ((unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(v[2 * q + 1] - __bfloat162float(h1))) << 16);
+        }
+        ((uint4*)(feat_h + (long long)b * d))[i] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        if (lo) ((uint4*)(feat_h + (long long)(b + lo) * d))[i] = make_uint4(rem[0], rem[1], rem[2], rem[3]);
+    }
 }
 cudaError_t launch_tc_setup(const SlotList& sl, int k, int d, int lo, int* d_slots, int* d_pos0, int* kv_len,
                             const float* pend_feat, const int* pend_id, float* feat, bf16* feat_h, int* cur_id,
                             u64* keys, int key_stride, const bf16* embed, int vocab, bf16* xe_h, int* id_flag,
                             cudaStream_t st) {
-    tc_setup_kernel<<<sl.n <= TC_OP_ROWS ? TC_OP_ROWS : HIVIS_MAX_BATCH, 256, 0, st>>>(sl, k, d, lo, d_slots, d_pos0, kv_len, pend_feat, pend_id, feat, feat_h,
+    tc_setup_kernel<<<sl.n <= TC_OP_ROWS ? TC_OP_ROWS : HIVIS_MAX_BATCH, 512, 0, st>>>(sl, k, d, lo, d_slots, d_pos0, kv_len, pend_feat, pend_id, feat, feat_h,
                                                 cur_id, keys, key_stride, embed, vocab, xe_h, id_flag);
     return cudaGetLastError();
 }

@@ -820,7 +820,8 @@ __device__ __forceinline__ void epi_preload(const TcArgs& a, int p, int s, int t
     if (!rok) return;
     if (p == PH_FC) {
         pre.g = __bfloat162float(a.norm1[row]);
-        const float add0 = a.rho ? a.rho[(long long)(s < a.n_resid - 1 ? s : a.n_resid - 1) * a.d + row] : 0.f;
+        const long long ri = (long long)(s < a.n_resid - 1 ? s : a.n_resid - 1) * a.d + row;
+        const float add0 = a.rho ? a.rho[ri] : a.rho_h ? __bfloat162float(a.rho_h[ri]) : 0.f;
 #pragma unroll
         for (int b = 0; b < 16; ++b) pre.add[b] = add0;
     } else if (p == PH_O) {
@@ -1318,6 +1319,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_chain_kernel(const __grid_co
                 tc_epilogue_phase<SMP, NG>(P, ctl, s, PH_DOWN, seg_cnt, cta, G, w4, lane);
                 tc_epilogue_phase<SMP, NG>(P, ctl, s, PH_LM, seg_cnt, cta, G, w4, lane);
             }
+        }
+        if (a.out_ids && cta == 0) {
+            // the chosen tokens, once every CTA's part of the last LM head has reached the keys
+            if (atid == 0)
+                wait_grid(a.bar_counter, a.bar_base + (u64)G * (u64)(a.k * TC_BARS_PER_STEP), ctl, a.error_flag, 19);
+            named_sync(TC_BAR_EPI, TC_EPI_THREADS);
+            for (int i = atid; i < a.B * a.k; i += TC_EPI_THREADS)
+                a.out_ids[i] = key_index(__ldcg(a.keys + (long long)(i / a.k) * a.key_stride + i % a.k));
         }
     }
     tc_fence_before();
