@@ -356,7 +356,7 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
              dalloc(c, &T.top_tok, TREE_MAX_TOPK * TREE_MAX_TOPK) && dalloc(c, &T.top_lp, TREE_MAX_TOPK * TREE_MAX_TOPK) &&
              dalloc(c, &T.cand_n, 1) && dalloc(c, &T.cand_tok, TREE_MAX_CAND) && dalloc(c, &T.cand_par, TREE_MAX_CAND) &&
              dalloc(c, &T.cand_depth, TREE_MAX_CAND) && dalloc(c, &T.cand_store, TREE_MAX_CAND) &&
-             dalloc(c, &T.cand_keep, TREE_MAX_CAND) && dalloc(c, &T.cand_pos, TREE_MAX_CAND) &&
+             dalloc(c, &T.arrive, TREE_MAX_TOPK + 1) &&
              dalloc(c, &T.cand_score, TREE_MAX_CAND) && dalloc(c, &T.kept_n, 1) && dalloc(c, &T.kept_tok, HIVIS_TREE_MAX_KEEP) &&
              dalloc(c, &T.kept_par, HIVIS_TREE_MAX_KEEP) && dalloc(c, &T.kept_store, HIVIS_TREE_MAX_KEEP) &&
              dalloc(c, &T.row_keys, HIVIS_TREE_MAX_KEEP + 1) && dalloc(c, &T.piece_stats, (long long)TREE_MAX_TOPK * tree_topk_pieces((int)V)) &&
@@ -406,6 +406,7 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
         CK(c, cudaMemsetAsync(c->error_flag, 0, 2 * sizeof(int), st));
         CK(c, cudaMemsetAsync(c->vkeys, 0, MB * (cfg->max_k + 1) * sizeof(u64), st));
         CK(c, cudaMemsetAsync(c->varrive, 0, MB * sizeof(int), st));
+        CK(c, cudaMemsetAsync(c->tree.arrive, 0, (TREE_MAX_TOPK + 1) * sizeof(int), st));
         CK(c, cudaMemsetAsync(c->xe_h, 0, R * d * sizeof(bf16), st));
         CK(c, cudaMemsetAsync(c->feat_h, 0, R * d * sizeof(bf16), st));
         CK(c, cudaMemsetAsync(c->xq, 0, R * d * sizeof(bf16), st));
@@ -1062,7 +1063,7 @@ int hivis_draft_tree(hivis_ctx* c, int slot, int topk, int depth, int keep, cons
         if (rc) return rc;
     }
     const TreeBufs& T = c->tree;
-    CKL(c, launch_tree_begin(slot, d, c->kv_len, c->pend_feat, c->pend_id, c->feat, c->feat_h, c->cur_id, c->d_slots, T, st));
+    if (!tc) CKL(c, launch_tree_begin(slot, d, c->kv_len, c->pend_feat, c->pend_id, c->feat, c->feat_h, c->cur_id, c->d_slots, T, st));
     // bf16 drafters with up to 16 nodes per level (always, by the limit on topk) run the levels' GEMMs in the
     // tensor-core chain kernel, one step long and in two parts around the tree's own attention
     for (int level = 0; level < depth; ++level) {
@@ -1073,18 +1074,20 @@ int hivis_draft_tree(hivis_ctx* c, int slot, int topk, int depth, int keep, cons
         if (tc) {
             const int lo = tc_lo_offset(nb);
             const u64 G = (u64)c->num_sms;
-            CKL(c, launch_tree_operands_tc(nb, TC_OP_ROWS, d, lo, c->feat, c->cur_id, level > 0 ? c->feat : nullptr, T,
-                                           (const bf16*)c->embed, V, c->feat_h, c->xe_h, c->d_pos0, c->id_flag, st));
+            CKL(c, launch_tree_operands_tc(nb, TC_OP_ROWS, d, lo, slot, c->kv_len, c->pend_feat, c->pend_id,
+                                           level > 0 ? c->feat : nullptr, T, (const bf16*)c->embed, V, c->feat_h, c->xe_h,
+                                           c->id_flag, st));
             TcArgs a;
             fill_tc_args(c, &a, nb, 1, lo, rho, 1, nullptr, c->tree_logits);
             a.rho_h = raw_rho ? (const bf16*)resid + (long long)row * d : nullptr;
-            a.seq_first = 0; a.seq_last = 2;                         // gather, fusion FC, QKV
+            a.seq_first = 1; a.seq_last = 2;                         // fusion FC, QKV (the operands are gathered already)
+            a.bar_base = c->bar_count_host - G + (c->debug_skew ? (1ull << 40) : 0ull);
             c->debug_skew = false;
             CKL(c, launch_tc_chain(c->tc_maps, a, c->num_sms, st));
-            c->bar_count_host += G * 3;
+            c->bar_count_host += G * 2;
             CK(c, launch_tree_attention(c->dtype, nb, c->qkv, c->qkvw, g.n_q_heads, g.n_kv_heads, g.head_dim, g.max_len, slot,
                                         level, T, c->inv_freq, c->Kc, c->Vc, c->attn, c->attn_h, lo, st));
-            c->launches += 2;
+            c->launches += 1;
             a.seq_first = 4; a.seq_last = 7;                         // O, gate/up, down, LM head (logits of every node)
             a.bar_base = c->bar_count_host - G * 4;                  // as if gather .. attention had been arrived on
             CKL(c, launch_tc_chain(c->tc_maps, a, c->num_sms, st));
@@ -1097,16 +1100,14 @@ int hivis_draft_tree(hivis_ctx* c, int slot, int topk, int depth, int keep, cons
             if (rc) return rc;
             CK(c, launch_tree_attention(c->dtype, nb, c->qkv, c->qkvw, g.n_q_heads, g.n_kv_heads, g.head_dim, g.max_len, slot,
                                         level, T, c->inv_freq, c->Kc, c->Vc, c->attn, c->attn_h, 0, st));
-            c->launches += 2;
+            c->launches += 1;
             rc = run_after_attention(c, mma, 0, nb, c->keys, c->key_stride, c->tree_logits, V, st);
             if (rc) return rc;
         }
-        CKL(c, launch_tree_topk(nb, c->tree_logits, V, topk, T, st));
-        c->launches += 1;                                            // (two kernels)
+        CKL(c, launch_tree_topk_select(nb, c->tree_logits, V, topk, level, depth, T, st));
         // (the tensor-core path reads the level's outputs where the down projection left them: they are overwritten only
         // by the next level's own down projection, after its operands were prepared)
         if (!tc) CK(c, cudaMemcpyAsync(c->tree_g, c->feat, (size_t)nb * d * sizeof(float), cudaMemcpyDeviceToDevice, st));
-        CKL(c, launch_tree_select(level, depth, nb, topk, T, st));
     }
     CKL(c, launch_tree_finalize(keep, T, out_tokens, out_parents, out_scores, out_count, st));
     const int total = topk + (depth - 1) * topk * topk;

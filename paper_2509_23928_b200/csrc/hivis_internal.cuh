@@ -257,7 +257,7 @@ struct TreeBufs {
     int* top_tok;              // [TOPK][TOPK] the top-k tokens of every frontier node's distribution
     float* top_lp;             //              and their log-probabilities
     // every candidate ever proposed, in creation order
-    int *cand_n, *cand_tok, *cand_par, *cand_depth, *cand_store, *cand_keep, *cand_pos;
+    int *cand_n, *cand_tok, *cand_par, *cand_depth, *cand_store;
     float* cand_score;
     // the kept nodes (the draft tree handed to the caller), for the verification
     int *kept_n, *kept_tok, *kept_par, *kept_store;
@@ -265,6 +265,7 @@ struct TreeBufs {
     // top-k of a level's logits: per node and 4096-logit piece the (max, sum exp) and the piece's largest keys
     float2* piece_stats;       // [TOPK][pieces]
     u64* piece_keys;           // [TOPK][pieces][TOPK]
+    int* arrive;               // [TOPK + 1] pieces of a node, nodes of the level done; zero between launches
 };
 int tree_topk_pieces(int V);
 cudaError_t launch_tree_begin(int slot, int d, const int* kv_len, const float* pend_feat, const int* pend_id, float* feat,
@@ -275,12 +276,13 @@ cudaError_t launch_tree_attention(int dtype, int nb, const float* qkv, int ld, i
                                   int slot, int level, const TreeBufs& T, const double* inv_freq, void* Kc, void* Vc,
                                   float* attn, bf16* attn_h, int lo_rows, cudaStream_t st);
 // the level's rows as the tensor-core chain kernel reads them (`rows` = all operand rows, so that those beyond the
-// level are cleared; g_prev non-null: the rows are gathered from the previous level's outputs on the way)
-cudaError_t launch_tree_operands_tc(int nb, int rows, int d, int lo_rows, const float* feat, const int* cur_id,
-                                    const float* g_prev, const TreeBufs& T, const bf16* embed, int vocab, bf16* feat_h,
-                                    bf16* xe_h, int* pos0, int* id_flag, cudaStream_t st);
-cudaError_t launch_tree_topk(int nb, const float* logits, int V, int topk, const TreeBufs& T, cudaStream_t st);
-cudaError_t launch_tree_select(int level, int depth, int nb, int topk, const TreeBufs& T, cudaStream_t st);
+// level are cleared); g_prev null: level 0, which also begins the tree; else the previous level's outputs
+cudaError_t launch_tree_operands_tc(int nb, int rows, int d, int lo_rows, int slot, const int* kv_len, const float* pend_feat,
+                                    const int* pend_id, const float* g_prev, const TreeBufs& T, const bf16* embed, int vocab,
+                                    bf16* feat_h, bf16* xe_h, int* id_flag, cudaStream_t st);
+// log-softmax and top-k of the level's nodes, then the next frontier
+cudaError_t launch_tree_topk_select(int nb, const float* logits, int V, int topk, int level, int depth, const TreeBufs& T,
+                                    cudaStream_t st);
 cudaError_t launch_tree_finalize(int keep, const TreeBufs& T, int32_t* out_tokens, int32_t* out_parents, float* out_scores,
                                  int32_t* out_count, cudaStream_t st);
 cudaError_t launch_tree_verify(int dtype, int logits_dtype, int slot, int depth, int rows, int V, int Hkv, int dh, int max_len,

@@ -55,77 +55,62 @@ cudaError_t launch_tree_gather(int nb, int d, const float* g_prev, const TreeBuf
 
 // The level's rows in the form the tensor-core chain kernel reads them: the features as bf16 rows with their rounding
 // remainders `lo_rows` rows further down, the embedding rows of the nodes' tokens (zero rows beyond the level: the
-// tiled copy always brings all rows), and a row count of zero per column (the kernel's own attention is not used).
-// With g_prev the rows are gathered on the way (row j = the layer output of the forward that proposed node j, and node j's
-// token); without, they are taken from feat / cur_id as tree_begin left them.
-__global__ void tree_operands_tc_kernel(int nb, int d, int lo_rows, const float* feat, const int* cur_id, const float* g_prev,
-                                        TreeBufs T, const bf16* embed, int vocab, bf16* feat_h, bf16* xe_h, int* pos0,
-                                        int* id_flag) {
-    const int j = blockIdx.x;
+// tiled copy always brings all rows).  Level 0 (g_prev null): the slot's pending pair, and the bookkeeping of a new tree;
+// later levels: row j = the layer output of the forward that proposed node j, and node j's token.  Eight elements per
+// thread: 11 us with one (and 10 us more for a level-0 launch of its own).
+__global__ void __launch_bounds__(512) tree_operands_tc_kernel(int nb, int d, int lo_rows, int slot, const int* kv_len,
+                                        const float* pend_feat, const int* pend_id, const float* g_prev,
+                                        TreeBufs T, const bf16* embed, int vocab, bf16* feat_h, bf16* xe_h, int* id_flag) {
+    const int j = blockIdx.x, upr = d >> 3;
+    uint4* xe = (uint4*)(xe_h + (long long)j * d);
     if (j >= nb) {
-        for (int i = threadIdx.x; i < (d >> 3); i += blockDim.x)
-            ((uint4*)(xe_h + (long long)j * d))[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = threadIdx.x; i < upr; i += blockDim.x) xe[i] = make_uint4(0u, 0u, 0u, 0u);
         return;
     }
-    if (threadIdx.x == 0) pos0[j] = 0;
-    const float* src = g_prev ? g_prev + (long long)T.fr_pslot[j] * d : feat + (long long)j * d;
-    for (int i = threadIdx.x; i < d; i += blockDim.x) {
-        const float v = src[i];
-        const bf16 hi = __float2bfloat16_rn(v);
-        feat_h[(long long)j * d + i] = hi;
-        feat_h[(long long)(j + lo_rows) * d + i] = __float2bfloat16_rn(v - __bfloat162float(hi));
+    const int tok = g_prev ? T.fr_tok[j] : pend_id[slot];
+    const float4* src = (const float4*)(g_prev ? g_prev + (long long)T.fr_pslot[j] * d : pend_feat + (long long)slot * d);
+    if (!g_prev && threadIdx.x == 0) {
+        *T.P = kv_len[slot];
+        *T.cand_n = 0;
+        T.fr_cand[0] = -1;
+        T.fr_store[0] = 0;
+        T.fr_score[0] = 0.f;
     }
-    const int id = checked_token(g_prev ? T.fr_tok[j] : cur_id[j], vocab, id_flag);
-    for (int i = threadIdx.x; i < (d >> 3); i += blockDim.x)
-        ((uint4*)(xe_h + (long long)j * d))[i] = ((const uint4*)(embed + (long long)id * d))[i];
+    const uint4* er = (const uint4*)(embed + (long long)checked_token(tok, vocab, id_flag) * d);
+    for (int i = threadIdx.x; i < upr; i += blockDim.x) {
+        const float4 x = src[2 * i], y = src[2 * i + 1];
+        xe[i] = er[i];
+        const float v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+        unsigned hi[4], rem[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const bf16 h0 = __float2bfloat16_rn(v[2 * q]), h1 = __float2bfloat16_rn(v[2 * q + 1]);
+            hi[q] = (unsigned)__bfloat16_as_ushort(h0) | ((unsigned)__bfloat16_as_ushort(h1) << 16);
+            rem[q] = (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(v[2 * q] - __bfloat162float(h0))) |
+                     ((unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(v[2 * q + 1] - __bfloat162float(h1))) << 16);
+        }
+        ((uint4*)(feat_h + (long long)j * d))[i] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        ((uint4*)(feat_h + (long long)(j + lo_rows) * d))[i] = make_uint4(rem[0], rem[1], rem[2], rem[3]);
+    }
 }
-cudaError_t launch_tree_operands_tc(int nb, int rows, int d, int lo_rows, const float* feat, const int* cur_id,
-                                    const float* g_prev, const TreeBufs& T, const bf16* embed, int vocab, bf16* feat_h,
-                                    bf16* xe_h, int* pos0, int* id_flag, cudaStream_t st) {
-    tree_operands_tc_kernel<<<rows, 256, 0, st>>>(nb, d, lo_rows, feat, cur_id, g_prev, T, embed, vocab, feat_h, xe_h, pos0,
-                                                  id_flag);
+cudaError_t launch_tree_operands_tc(int nb, int rows, int d, int lo_rows, int slot, const int* kv_len, const float* pend_feat,
+                                    const int* pend_id, const float* g_prev, const TreeBufs& T, const bf16* embed, int vocab,
+                                    bf16* feat_h, bf16* xe_h, int* id_flag, cudaStream_t st) {
+    tree_operands_tc_kernel<<<rows, 512, 0, st>>>(nb, d, lo_rows, slot, kv_len, pend_feat, pend_id, g_prev, T, embed, vocab,
+                                                  feat_h, xe_h, id_flag);
     return cudaGetLastError();
 }
 
-// ------------------------------------------------------------------------------------------ K/V rows of the level
-template <typename WT>
-__global__ void tree_kv_write_kernel(const float* qkv, int ld, int qw, int Hkv, int dh, int max_len, int slot, int level,
-                                     TreeBufs T, const double* inv_freq, void* Kc, void* Vc) {
-    __shared__ float2 s_cs[128];                        // (cos, sin) of the level's position: the same for every head
-    const int j = blockIdx.x;
-    const int P = *T.P;
-    const int row = P + T.fr_store[j], pos = P + level;
-    const int half = dh / 2, kvw = Hkv * dh;
-    for (int e = threadIdx.x; e < half; e += blockDim.x) {
-        float c, s;
-        rope_cs(pos, inv_freq[e], c, s);
-        s_cs[e] = make_float2(c, s);
-    }
-    __syncthreads();
-    const float* k = qkv + (long long)j * ld + qw;
-    const float* v = k + kvw;
-    for (int i = threadIdx.x; i < Hkv * half; i += blockDim.x) {
-        const int h = i / half, e = i % half;
-        const float c = s_cs[e].x, s = s_cs[e].y;
-        const float x0 = k[h * dh + e], x1 = k[h * dh + e + half];
-        const long long o = (((long long)slot * Hkv + h) * max_len + row) * dh;
-        store_from_float<WT>(Kc, o + e, x0 * c - x1 * s);
-        store_from_float<WT>(Kc, o + e + half, x1 * c + x0 * s);
-    }
-    for (int i = threadIdx.x; i < kvw; i += blockDim.x) {
-        const int h = i / dh, e = i % dh;
-        const long long o = (((long long)slot * Hkv + h) * max_len + row) * dh;
-        store_from_float<WT>(Vc, o + e, v[i]);
-    }
-}
-
 // ------------------------------------------------------------------------------------------ tree attention
-// One CTA of four warps per (query head, node).  The node attends to the prefix rows [0, P), to the rows of its
-// ancestors (the root position first) and to its own row: `level` + 1 tree rows.  Blocks of 32 rows are dealt to the
-// warps in turn.  Scores: a lane takes one row of the block and the whole dot product with the query (in shared
-// memory), so no shuffle is needed; the block's probabilities then go through an online softmax, and for the weighted
-// sum of the V rows a lane owns DH/32 output elements and every row's probability is broadcast from its lane.  The four
-// warps' (max, sum, accumulator) are merged at the end.
+// One CTA of eight warps per (query head, node).  The node attends to the prefix rows [0, P), to the rows of its
+// ancestors (the root position first) and to itself.  Its own K (rotated) and V are made here, rounded to what the cache
+// will hold, and the first head of a KV group writes them to the cache: nobody else reads that row in this level (a
+// launch of its own for the rows took 15 us).  Blocks of 32 cached rows are dealt to the warps in turn.  Scores: a lane takes
+// one row of the block and the whole dot product with the query (in shared memory), so no shuffle is needed; the block's
+// probabilities then go through an online softmax, and for the weighted sum of the V rows a lane owns DH/32 output
+// elements and every row's probability is broadcast from its lane, eight rows' loads in flight.  The warps' (max, sum,
+// accumulator) and the node's own row are merged at the end.
+#define TREE_ATT_WARPS 8
 template <typename WT, int DH>
 __device__ __forceinline__ float tree_row_dot(const void* Kc, long long o, const float* q) {
     float sc = 0.f;
@@ -150,45 +135,71 @@ __device__ __forceinline__ float tree_row_dot(const void* Kc, long long o, const
     }
     return sc;
 }
+template <typename WT>
+__device__ __forceinline__ float tree_as_cached(float x) {
+    return sizeof(WT) == 2 ? __bfloat162float(__float2bfloat16_rn(x)) : x;
+}
 template <typename WT, int DH>
-__global__ void __launch_bounds__(128) tree_attn_kernel(const float* qkv, int ld, int Hq, int Hkv, int max_len, int slot,
+__global__ void __launch_bounds__(TREE_ATT_WARPS * 32) tree_attn_kernel(const float* qkv, int ld, int Hq, int Hkv, int max_len, int slot,
                                                         int level, TreeBufs T, const double* inv_freq, float scale,
-                                                        const void* Kc, const void* Vc, float* attn, bf16* attn_h,
-                                                        int lo_rows) {
-    constexpr int EPL = DH / 32;
-    __shared__ float s_m[4], s_l[4], s_acc[4][DH];
-    __shared__ __align__(16) float s_q[DH];
+                                                        void* Kc, void* Vc, float* attn, bf16* attn_h, int lo_rows) {
+    constexpr int EPL = DH / 32, NT = TREE_ATT_WARPS * 32;
+    __shared__ float s_m[TREE_ATT_WARPS + 1], s_l[TREE_ATT_WARPS + 1], s_acc[TREE_ATT_WARPS + 1][DH];
+    __shared__ __align__(16) float s_q[DH], s_k[DH];
     __shared__ float2 s_cs[DH / 2];
     const int h = blockIdx.x, j = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int P = *T.P, pos = P + level, kvh = h / (Hq / Hkv), half = DH / 2;
+    const int P = *T.P, pos = P + level, G = Hq / Hkv, kvh = h / G, half = DH / 2;
+    const long long base = ((long long)slot * Hkv + kvh) * max_len;
+    const float* qh = qkv + (long long)j * ld + h * DH;
+    const float* kh = qkv + (long long)j * ld + (Hq + kvh) * DH;
+    const float* vh = kh + Hkv * DH;
     if (threadIdx.x < half) {
         float c, s;
         rope_cs(pos, inv_freq[threadIdx.x], c, s);
         s_cs[threadIdx.x] = make_float2(c, s);
     }
     __syncthreads();
-    // the rotated, scaled query
-    const float* qh = qkv + (long long)j * ld + h * DH;
-    for (int i = threadIdx.x; i < DH; i += 128) {
-        const int f = i % half;
+    // the rotated, scaled query; the node's own row
+    const long long own = (base + P + T.fr_store[j]) * DH;
+    const bool writer = h % G == 0;
+    for (int t = threadIdx.x; t < 3 * DH; t += NT) {
+        const int what = t / DH, i = t % DH, f = i % half;
+        const float* src = what == 0 ? qh : what == 1 ? kh : vh;
+        const float x = src[i];
+        if (what == 2) {
+            s_acc[TREE_ATT_WARPS][i] = tree_as_cached<WT>(x);
+            if (writer) store_from_float<WT>(Vc, own + i, x);
+            continue;
+        }
         const float c = s_cs[f].x, s = s_cs[f].y;
-        const float x = qh[i], y = qh[i < half ? i + half : i - half];
-        s_q[i] = (i < half ? x * c - y * s : x * c + y * s) * scale;
+        const float y = src[i < half ? i + half : i - half];
+        const float r = i < half ? x * c - y * s : x * c + y * s;
+        if (what == 0) {
+            s_q[i] = r * scale;
+        } else {
+            s_k[i] = tree_as_cached<WT>(r);
+            if (writer) store_from_float<WT>(Kc, own + i, r);
+        }
     }
     __syncthreads();
-    const long long base = ((long long)slot * Hkv + kvh) * max_len;
-    const int nrows = P + level + 1;
+    if (warp == TREE_ATT_WARPS - 1) {
+        float sc = 0.f;
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) sc = fmaf(s_q[e * 32 + lane], s_k[e * 32 + lane], sc);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, off);
+        if (lane == 0) { s_m[TREE_ATT_WARPS] = sc; s_l[TREE_ATT_WARPS] = 1.f; }
+    }
+    const int nrows = P + level;                                     // cached rows: the prefix and the ancestors
     float m = -INFINITY, l = 0.f, acc[EPL];
 #pragma unroll
     for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
-    for (int r0 = warp * 32; r0 < nrows; r0 += 128) {
+    for (int r0 = warp * 32; r0 < nrows; r0 += NT) {
         const int r = r0 + lane;
         const bool ok = r < nrows;
-        int row = ok ? r : 0;
-        if (ok && r >= P) {
-            const int a = r - P;                                     // a-th tree row on the path: ancestors, then the node
-            row = P + (a < level ? T.fr_anc[j * TREE_MAX_DEPTH + a] : T.fr_store[j]);
-        }
+        int row = ok ? r : r0;
+        if (ok && r >= P) row = P + T.fr_anc[j * TREE_MAX_DEPTH + (r - P)];
+        row = __shfl_sync(0xffffffffu, row, ok ? lane : 0);          // lanes beyond the rows read the block's first
         const float sc = ok ? tree_row_dot<WT, DH>(Kc, (base + row) * DH, s_q) : -INFINITY;
         float bm = sc;
 #pragma unroll
@@ -203,21 +214,31 @@ __global__ void __launch_bounds__(128) tree_attn_kernel(const float* qkv, int ld
 #pragma unroll
         for (int e = 0; e < EPL; ++e) acc[e] *= corr;
         const int nr = min(32, nrows - r0);
-#pragma unroll 4
-        for (int t = 0; t < nr; ++t) {
-            const float pj = __shfl_sync(0xffffffffu, p, t);
-            const int rowj = __shfl_sync(0xffffffffu, row, t);
-            const long long o = (base + rowj) * DH + lane * EPL;
-            if constexpr (sizeof(WT) == 2 && EPL == 4) {
-                const uint2 w = __ldg((const uint2*)((const bf16*)Vc + o));
-                acc[0] = fmaf(pj, bf16_lo(w.x), acc[0]); acc[1] = fmaf(pj, bf16_hi(w.x), acc[1]);
-                acc[2] = fmaf(pj, bf16_lo(w.y), acc[2]); acc[3] = fmaf(pj, bf16_hi(w.y), acc[3]);
-            } else if constexpr (sizeof(WT) == 2 && EPL == 2) {
-                const unsigned w = __ldg((const unsigned*)((const bf16*)Vc + o));
-                acc[0] = fmaf(pj, bf16_lo(w), acc[0]); acc[1] = fmaf(pj, bf16_hi(w), acc[1]);
-            } else {
+#pragma unroll 1
+        for (int t0 = 0; t0 < nr; t0 += 8) {
+            float vf[8][EPL];
 #pragma unroll
-                for (int e = 0; e < EPL; ++e) acc[e] = fmaf(pj, load_as_float<WT>(Vc, o + e), acc[e]);
+            for (int t = 0; t < 8; ++t) {
+                const int rowj = __shfl_sync(0xffffffffu, row, t0 + t);
+                const long long o = (base + rowj) * DH + lane * EPL;
+                if constexpr (sizeof(WT) == 2 && EPL == 4) {
+                    const uint2 w = __ldg((const uint2*)((const bf16*)Vc + o));
+                    vf[t][0] = bf16_lo(w.x); vf[t][1] = bf16_hi(w.x); vf[t][2] = bf16_lo(w.y); vf[t][3] = bf16_hi(w.y);
+                } else if constexpr (sizeof(WT) == 2 && EPL == 2) {
+                    const unsigned w = __ldg((const unsigned*)((const bf16*)Vc + o));
+                    vf[t][0] = bf16_lo(w); vf[t][1] = bf16_hi(w);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < EPL; ++e) vf[t][e] = __ldg((const float*)Vc + o + e);
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const float pj = __shfl_sync(0xffffffffu, p, t0 + t);        // 0 beyond the rows
+                if (t0 + t < nr) {
+#pragma unroll
+                    for (int e = 0; e < EPL; ++e) acc[e] = fmaf(pj, vf[t][e], acc[e]);
+                }
             }
         }
     }
@@ -228,12 +249,12 @@ __global__ void __launch_bounds__(128) tree_attn_kernel(const float* qkv, int ld
     if (warp == 0) {
         float M = -INFINITY;
 #pragma unroll
-        for (int w = 0; w < 4; ++w) M = fmaxf(M, s_m[w]);
+        for (int w = 0; w <= TREE_ATT_WARPS; ++w) M = fmaxf(M, s_m[w]);
         float L = 0.f, A[EPL];
 #pragma unroll
         for (int e = 0; e < EPL; ++e) A[e] = 0.f;
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
+        for (int w = 0; w <= TREE_ATT_WARPS; ++w) {
             const float f = s_l[w] > 0.f ? expf(s_m[w] - M) : 0.f;   // a warp without rows contributes nothing
             L += s_l[w] * f;
 #pragma unroll
@@ -254,21 +275,15 @@ __global__ void __launch_bounds__(128) tree_attn_kernel(const float* qkv, int ld
 cudaError_t launch_tree_attention(int dtype, int nb, const float* qkv, int ld, int Hq, int Hkv, int dh, int max_len,
                                   int slot, int level, const TreeBufs& T, const double* inv_freq, void* Kc, void* Vc,
                                   float* attn, bf16* attn_h, int lo_rows, cudaStream_t st) {
-    const int qw = Hq * dh;
     const float scale = 1.0f / sqrtf((float)dh);
-    if (dtype == HIVIS_BF16)
-        tree_kv_write_kernel<bf16><<<nb, 256, 0, st>>>(qkv, ld, qw, Hkv, dh, max_len, slot, level, T, inv_freq, Kc, Vc);
-    else
-        tree_kv_write_kernel<float><<<nb, 256, 0, st>>>(qkv, ld, qw, Hkv, dh, max_len, slot, level, T, inv_freq, Kc, Vc);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)Hq, (unsigned)nb);
+    const int nt = TREE_ATT_WARPS * 32;
     if (dtype == HIVIS_BF16) {
-        if (dh == 128) tree_attn_kernel<bf16, 128><<<grid, 128, 0, st>>>(qkv, ld, Hq, Hkv, max_len, slot, level, T, inv_freq, scale, Kc, Vc, attn, attn_h, lo_rows);
-        else tree_attn_kernel<bf16, 64><<<grid, 128, 0, st>>>(qkv, ld, Hq, Hkv, max_len, slot, level, T, inv_freq, scale, Kc, Vc, attn, attn_h, lo_rows);
+        if (dh == 128) tree_attn_kernel<bf16, 128><<<grid, nt, 0, st>>>(qkv, ld, Hq, Hkv, max_len, slot, level, T, inv_freq, scale, Kc, Vc, attn, attn_h, lo_rows);
+        else tree_attn_kernel<bf16, 64><<<grid, nt, 0, st>>>(qkv, ld, Hq, Hkv, max_len, slot, level, T, inv_freq, scale, Kc, Vc, attn, attn_h, lo_rows);
     } else {
-        if (dh == 128) tree_attn_kernel<float, 128><<<grid, 128, 0, st>>>(qkv, ld, Hq, Hkv, max_len, slot, level, T, inv_freq, scale, Kc, Vc, attn, attn_h, lo_rows);
-        else tree_attn_kernel<float, 64><<<grid, 128, 0, st>>>(qkv, ld, Hq, Hkv, max_len, slot, level, T, inv_freq, scale, Kc, Vc, attn, attn_h, lo_rows);
+        if (dh == 128) tree_attn_kernel<float, 128><<<grid, nt, 0, st>>>(qkv, ld, Hq, Hkv, max_len, slot, level, T, inv_freq, scale, Kc, Vc, attn, attn_h, lo_rows);
+        else tree_attn_kernel<float, 64><<<grid, nt, 0, st>>>(qkv, ld, Hq, Hkv, max_len, slot, level, T, inv_freq, scale, Kc, Vc, attn, attn_h, lo_rows);
     }
     return cudaGetLastError();
 }
@@ -300,14 +315,86 @@ __device__ __forceinline__ float block_reduce_sum(float v, float* red) {
 #define TREE_PIECE 4096          // logits of a node that one CTA covers (16 per thread, kept in registers)
 int tree_topk_pieces(int V) { return (V + TREE_PIECE - 1) / TREE_PIECE; }
 
-// One CTA per (piece of the row, node): the piece's maximum and sum of exp(x - max), and its `topk` largest keys, largest
-// first.  A thread keeps its 16 logits in registers and its current best key; a round takes the block's best, and only the
-// thread that owned it looks for its next one.
-__global__ void __launch_bounds__(256) tree_topk_piece_kernel(const float* logits, int V, int topk, float2* piece_stats,
-                                                              u64* piece_keys) {
+// One launch per level: log-softmax and top-k of every node, then the next frontier.
+//   One CTA per (piece of the row, node): the piece's maximum and sum of exp(x - max), and its `topk` largest keys, largest
+//   first.  A thread keeps its 16 logits in registers and its current best key; a round takes the block's best, and only
+//   the thread that owned it looks for its next one.
+//   The CTA that completes a node's count merges the node: log-sum-exp from the pieces, and the pieces' keys ranked by
+//   counting the larger ones (keys are unique; the order is by value, then by lower token id).
+//   The CTA that completes the level's count chooses the frontier.  Nobody waits for anybody.  As three launches the level
+//   spent 27 us here, most of it in a single warp that walked the sorted lists.
+#define TREE_MERGE_CAP 1024      // keys of a node ranked from shared memory (more: from global memory)
+
+// The nb * topk children of this level become candidates (creation order: frontier order, then rank); unless this was
+// the last level, the `topk` of them with the highest cumulative log-probability (earlier candidate first among
+// equals) form the next frontier, kept in creation order.
+__device__ void tree_select(int level, int depth, int nb, int topk, const TreeBufs& T) {
+    __shared__ float s_score[256];
+    __shared__ int s_sel[256];
+    __shared__ int s_anc[TREE_MAX_TOPK][TREE_MAX_DEPTH], s_store[TREE_MAX_TOPK], s_cand[TREE_MAX_TOPK];
+    const int i = threadIdx.x, n = nb * topk;
+    const int base = *T.cand_n;
+    const int j = i / topk, r = i % topk;
+    if (i < TREE_MAX_TOPK * TREE_MAX_DEPTH) s_anc[i / TREE_MAX_DEPTH][i % TREE_MAX_DEPTH] = T.fr_anc[i];
+    if (i < TREE_MAX_TOPK) { s_store[i] = T.fr_store[i]; s_cand[i] = T.fr_cand[i]; }
+    float score = -INFINITY;
+    int tok = 0;
+    if (i < n) {
+        tok = __ldcg(T.top_tok + j * TREE_MAX_TOPK + r);
+        score = T.fr_score[j] + __ldcg(T.top_lp + j * TREE_MAX_TOPK + r);
+        T.cand_tok[base + i] = tok;
+        T.cand_par[base + i] = T.fr_cand[j];
+        T.cand_depth[base + i] = level + 1;
+        T.cand_score[base + i] = score;
+        T.cand_store[base + i] = -1;
+    }
+    s_score[i] = score;
+    __syncthreads();
+    int sel = 0;
+    if (i < n && level + 1 < depth) {
+        int rank = 0;
+        for (int o = 0; o < n; ++o) rank += (s_score[o] > score || (s_score[o] == score && o < i)) ? 1 : 0;
+        sel = rank < topk ? 1 : 0;
+    }
+    s_sel[i] = sel;
+    __syncthreads();
+    if (sel) {
+        int pos = 0;
+        for (int o = 0; o < i; ++o) pos += s_sel[o];
+        const int store = 1 + level * topk + pos;              // the node joins the frontier of level + 1
+        T.fr_cand[pos] = base + i;
+        T.fr_tok[pos] = tok;
+        T.fr_score[pos] = score;
+        T.fr_pslot[pos] = j;
+        T.fr_store[pos] = store;
+        for (int a = 0; a < level; ++a) T.fr_anc[pos * TREE_MAX_DEPTH + a] = s_anc[j][a];
+        T.fr_anc[pos * TREE_MAX_DEPTH + level] = s_store[j];   // the parent's row (the root's when level == 0)
+        T.cand_store[base + i] = store;
+    }
+    if (i == 0) *T.cand_n = base + n;
+}
+
+// the CTA arrives on *counter; true for all its threads if it completed the count (the counter is zero again then)
+__device__ __forceinline__ bool tree_arrive(int* counter, int count) {
+    __shared__ int s_last;
+    __syncthreads();                          // every thread's stores are before the arrival
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const int last = atomicAdd(counter, 1) == count - 1;
+        if (last) *counter = 0;
+        __threadfence();
+        s_last = last;
+    }
+    __syncthreads();
+    return s_last != 0;
+}
+
+__global__ void __launch_bounds__(256) tree_topk_select_kernel(const float* logits, int V, int topk, int level, int depth,
+                                                               float2* piece_stats, u64* piece_keys, TreeBufs T) {
     __shared__ float red[8];
     __shared__ u64 kred[8];
-    const int piece = blockIdx.x, j = blockIdx.y, pieces = gridDim.x;
+    __shared__ u64 s_keys[TREE_MERGE_CAP];
+    const int piece = blockIdx.x, j = blockIdx.y, pieces = gridDim.x, nb = gridDim.y;
     const float* x = logits + (long long)j * V;
     const int c0 = piece * TREE_PIECE;
     u64 key[TREE_PIECE / 256];
@@ -353,110 +440,56 @@ __global__ void __launch_bounds__(256) tree_topk_piece_kernel(const float* logit
             }
         }
     }
-}
-
-// One warp per node: log-sum-exp of the row from its pieces, then the `topk` largest of the pieces' keys.  The packed key
-// orders by value, then by lower token id, so equal logits come out in token order.
-__global__ void __launch_bounds__(32) tree_topk_merge_kernel(const float* logits, int V, int topk, int pieces,
-                                                             const float2* piece_stats, const u64* piece_keys, TreeBufs T) {
-    const int j = blockIdx.x, lane = threadIdx.x;
-    const float* x = logits + (long long)j * V;
+    if (!tree_arrive(T.arrive + j, pieces)) return;
+    // ---- merge of the node
     const float2* ps = piece_stats + (long long)j * pieces;
-    float mx = -INFINITY;
-    for (int c = lane; c < pieces; c += 32) mx = fmaxf(mx, ps[c].x);
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        float mx2 = -INFINITY;
+        for (int c = lane; c < pieces; c += 32) mx2 = fmaxf(mx2, __ldcg(ps + c).x);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    float se = 0.f;
-    for (int c = lane; c < pieces; c += 32) se += ps[c].y * expf(ps[c].x - mx);
+        for (int o = 16; o > 0; o >>= 1) mx2 = fmaxf(mx2, __shfl_xor_sync(0xffffffffu, mx2, o));
+        float se2 = 0.f;
+        for (int c = lane; c < pieces; c += 32) {
+            const float2 w = __ldcg(ps + c);
+            se2 += w.y * expf(w.x - mx2);
+        }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
-    const float lse = mx + logf(se);
-    // every piece's list is sorted: a lane walks the lists of its pieces from their heads
+        for (int o = 16; o > 0; o >>= 1) se2 += __shfl_xor_sync(0xffffffffu, se2, o);
+        if (lane == 0) red[0] = mx2 + logf(se2);
+    }
     const u64* pk = piece_keys + (long long)j * pieces * TREE_MAX_TOPK;
-    u64 prev = ~0ull;
-    for (int r = 0; r < topk; ++r) {
-        u64 best = 0;
-        for (int c = lane; c < pieces; c += 32)
+    const int nk = pieces * topk;
+    const bool in_smem = nk <= TREE_MERGE_CAP;
+    if (in_smem)
+        for (int i = threadIdx.x; i < nk; i += 256) s_keys[i] = __ldcg(pk + (i / topk) * TREE_MAX_TOPK + i % topk);
+    __syncthreads();
+    const float lse = red[0];
+    for (int i = threadIdx.x; i < nk; i += 256) {
+        const u64 mine2 = in_smem ? s_keys[i] : __ldcg(pk + (i / topk) * TREE_MAX_TOPK + i % topk);
+        if (mine2 == 0ull) continue;                 // the piece had fewer entries
+        int rank = i % topk;                         // its own list is sorted
+        for (int c = 0; c < pieces && rank < topk; ++c) {
+            if (c == i / topk) continue;
             for (int t = 0; t < topk; ++t) {
-                const u64 key = pk[c * TREE_MAX_TOPK + t];
-                if (key < prev) {                     // the first not yet taken of this piece
-                    best = key > best ? key : best;
-                    break;
-                }
+                const u64 o = in_smem ? s_keys[c * topk + t] : __ldcg(pk + c * TREE_MAX_TOPK + t);
+                if (o < mine2) break;
+                ++rank;
             }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const u64 other = __shfl_xor_sync(0xffffffffu, best, o);
-            best = other > best ? other : best;
         }
-        prev = best;
-        if (lane == 0) {
-            const int tok = best ? key_index(best) : 0;
-            T.top_tok[j * TREE_MAX_TOPK + r] = tok;
-            T.top_lp[j * TREE_MAX_TOPK + r] = x[tok] - lse;
+        if (rank < topk) {
+            const int tok = key_index(mine2);
+            __stcg(T.top_tok + j * TREE_MAX_TOPK + rank, tok);
+            __stcg(T.top_lp + j * TREE_MAX_TOPK + rank, x[tok] - lse);
         }
     }
+    if (!tree_arrive(T.arrive + TREE_MAX_TOPK, nb)) return;
+    tree_select(level, depth, nb, topk, T);
 }
-cudaError_t launch_tree_topk(int nb, const float* logits, int V, int topk, const TreeBufs& T, cudaStream_t st) {
-    const int pieces = tree_topk_pieces(V);
-    tree_topk_piece_kernel<<<dim3((unsigned)pieces, (unsigned)nb), 256, 0, st>>>(logits, V, topk, T.piece_stats, T.piece_keys);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    tree_topk_merge_kernel<<<nb, 32, 0, st>>>(logits, V, topk, pieces, T.piece_stats, T.piece_keys, T);
-    return cudaGetLastError();
-}
-
-// ------------------------------------------------------------------------------------------ next frontier
-// The nb * topk children of this level become candidates (creation order: frontier order, then rank); unless this was
-// the last level, the `topk` of them with the highest cumulative log-probability (earlier candidate first among
-// equals) form the next frontier, kept in creation order.
-__global__ void __launch_bounds__(256) tree_select_kernel(int level, int depth, int nb, int topk, TreeBufs T) {
-    __shared__ float s_score[256];
-    __shared__ int s_sel[256];
-    __shared__ int s_anc[TREE_MAX_TOPK][TREE_MAX_DEPTH], s_store[TREE_MAX_TOPK], s_cand[TREE_MAX_TOPK];
-    const int i = threadIdx.x, n = nb * topk;
-    const int base = *T.cand_n;
-    const int j = i / topk, r = i % topk;
-    if (i < TREE_MAX_TOPK * TREE_MAX_DEPTH) s_anc[i / TREE_MAX_DEPTH][i % TREE_MAX_DEPTH] = T.fr_anc[i];
-    if (i < TREE_MAX_TOPK) { s_store[i] = T.fr_store[i]; s_cand[i] = T.fr_cand[i]; }
-    float score = -INFINITY;
-    int tok = 0;
-    if (i < n) {
-        tok = T.top_tok[j * TREE_MAX_TOPK + r];
-        score = T.fr_score[j] + T.top_lp[j * TREE_MAX_TOPK + r];
-        T.cand_tok[base + i] = tok;
-        T.cand_par[base + i] = T.fr_cand[j];
-        T.cand_depth[base + i] = level + 1;
-        T.cand_score[base + i] = score;
-        T.cand_store[base + i] = -1;
-    }
-    s_score[i] = score;
-    __syncthreads();
-    int sel = 0;
-    if (i < n && level + 1 < depth) {
-        int rank = 0;
-        for (int o = 0; o < n; ++o) rank += (s_score[o] > score || (s_score[o] == score && o < i)) ? 1 : 0;
-        sel = rank < topk ? 1 : 0;
-    }
-    s_sel[i] = sel;
-    __syncthreads();
-    if (sel) {
-        int pos = 0;
-        for (int o = 0; o < i; ++o) pos += s_sel[o];
-        const int store = 1 + level * topk + pos;              // the node joins the frontier of level + 1
-        T.fr_cand[pos] = base + i;
-        T.fr_tok[pos] = tok;
-        T.fr_score[pos] = score;
-        T.fr_pslot[pos] = j;
-        T.fr_store[pos] = store;
-        for (int a = 0; a < level; ++a) T.fr_anc[pos * TREE_MAX_DEPTH + a] = s_anc[j][a];
-        T.fr_anc[pos * TREE_MAX_DEPTH + level] = s_store[j];   // the parent's row (the root's when level == 0)
-        T.cand_store[base + i] = store;
-    }
-    if (i == 0) *T.cand_n = base + n;
-}
-cudaError_t launch_tree_select(int level, int depth, int nb, int topk, const TreeBufs& T, cudaStream_t st) {
-    tree_select_kernel<<<1, 256, 0, st>>>(level, depth, nb, topk, T);
+cudaError_t launch_tree_topk_select(int nb, const float* logits, int V, int topk, int level, int depth, const TreeBufs& T,
+                                    cudaStream_t st) {
+    tree_topk_select_kernel<<<dim3((unsigned)tree_topk_pieces(V), (unsigned)nb), 256, 0, st>>>(logits, V, topk, level, depth,
+                                                                                              T.piece_stats, T.piece_keys, T);
     return cudaGetLastError();
 }
 
@@ -465,36 +498,48 @@ cudaError_t launch_tree_select(int level, int depth, int nb, int topk, const Tre
 // listed in creation order, parents re-numbered within the list.
 __global__ void __launch_bounds__(1024) tree_finalize_kernel(int keep, TreeBufs T, int32_t* out_tokens, int32_t* out_parents,
                                                              float* out_scores, int32_t* out_count) {
-    const int n = *T.cand_n;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const float sc = T.cand_score[i];
-        int rank = 0;
-        for (int o = 0; o < n; ++o) {
-            const float so = T.cand_score[o];
-            rank += (so > sc || (so == sc && o < i)) ? 1 : 0;
+    __shared__ float s_score[TREE_MAX_CAND];
+    __shared__ unsigned short s_pos[TREE_MAX_CAND];          // 1 + position among the kept, 0 = not kept
+    __shared__ int s_sum[32];
+    const int n = *T.cand_n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int i = tid; i < n; i += 1024) s_score[i] = T.cand_score[i];
+    __syncthreads();
+    int before = 0;                                          // kept candidates of the earlier turns
+    for (int i0 = 0; i0 < n; i0 += 1024) {
+        const int i = i0 + tid;
+        bool kept = false;
+        if (i < n) {
+            const float sc = s_score[i];
+            int rank = 0;
+#pragma unroll 4
+            for (int o = 0; o < n; ++o) rank += (s_score[o] > sc || (s_score[o] == sc && o < i)) ? 1 : 0;
+            kept = rank < keep;
         }
-        T.cand_keep[i] = rank < keep ? 1 : 0;
+        const unsigned mask = __ballot_sync(0xffffffffu, kept);
+        if (lane == 0) s_sum[warp] = __popc(mask);
+        __syncthreads();
+        int pos = before + __popc(mask & ((1u << lane) - 1u));
+        for (int w = 0; w < 32; ++w) {
+            if (w < warp) pos += s_sum[w];
+            before += s_sum[w];
+        }
+        if (i < n) s_pos[i] = kept ? (unsigned short)(pos + 1) : 0;
+        __syncthreads();
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        int pos = 0;
-        for (int o = 0; o < i; ++o) pos += T.cand_keep[o];
-        T.cand_pos[i] = T.cand_keep[i] ? pos : -1;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const int pos = T.cand_pos[i];
+    for (int i = tid; i < n; i += 1024) {
+        const int pos = (int)s_pos[i] - 1;
         if (pos < 0) continue;
         const int par = T.cand_par[i];
-        const int pp = par < 0 ? -1 : T.cand_pos[par];
-        T.kept_tok[pos] = T.cand_tok[i];
+        const int pp = par < 0 ? -1 : (int)s_pos[par] - 1;
+        const int tok = T.cand_tok[i];
+        T.kept_tok[pos] = tok;
         T.kept_par[pos] = pp;
         T.kept_store[pos] = T.cand_store[i];
-        out_tokens[pos] = T.cand_tok[i];
+        out_tokens[pos] = tok;
         out_parents[pos] = pp;
-        out_scores[pos] = T.cand_score[i];
+        out_scores[pos] = s_score[i];
     }
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
         const int cnt = n < keep ? n : keep;
         *T.kept_n = cnt;
         if (out_count) *out_count = cnt;
@@ -531,59 +576,65 @@ __global__ void __launch_bounds__(256) tree_row_argmax_kernel(const void* logits
     }
 }
 
-// The walk: from the root, follow the child that carries the target's argmax for as long as there is one.  Then
-// the K/V rows of the accepted nodes that have one are moved right behind the root's row, in path order (a row's
-// destination never lies beyond its source, and the moves are made one after the other), and the slot gets its new
-// row count.
+// The walk: from the root, follow the child that carries the target's argmax for as long as there is one (the kept nodes
+// in shared memory, one per lane and turn).  Then the K/V rows of the accepted nodes that have one are moved right behind
+// the root's row, in path order, and the slot gets its new row count.  Every CTA walks, and moves a slice of the rows: a
+// thread reads its 16 bytes of all rows before it writes the first, and nobody else touches them.
+#define TREE_WALK_CTAS 8
 template <typename WT>
 __global__ void __launch_bounds__(256) tree_walk_kernel(int slot, int depth, int Hkv, int dh, int max_len, TreeBufs T,
                                                         const u64* keys, void* Kc, void* Vc, int* kv_len, int32_t* out_accept,
                                                         int32_t* out_path, int32_t* out_next, int32_t* out_kv_len) {
-    __shared__ int s_path[TREE_MAX_DEPTH], s_n, s_rows;
-    const int n = *T.kept_n, P = *T.P;
-    if (threadIdx.x == 0) {
+    __shared__ int s_path[TREE_MAX_DEPTH], s_src[TREE_MAX_DEPTH], s_rows;
+    __shared__ int s_tok[HIVIS_TREE_MAX_KEEP], s_par[HIVIS_TREE_MAX_KEEP], s_store[HIVIS_TREE_MAX_KEEP], s_arg[HIVIS_TREE_MAX_KEEP + 1];
+    const int n = *T.kept_n, P = *T.P, lane = threadIdx.x & 31;
+    for (int i = threadIdx.x; i < n; i += 256) {
+        s_tok[i] = T.kept_tok[i];
+        s_par[i] = T.kept_par[i];
+        s_store[i] = T.kept_store[i];
+    }
+    for (int i = threadIdx.x; i <= n; i += 256) s_arg[i] = key_index(keys[i]);
+    __syncthreads();
+    if (threadIdx.x < 32) {
         int cur = -1, acc = 0, t = 0;
         for (;;) {
-            t = key_index(keys[cur + 1]);
-            int nxt = -1;
-            for (int i = 0; i < n; ++i)
-                if (T.kept_par[i] == cur && T.kept_tok[i] == t) { nxt = i; break; }
-            if (nxt < 0 || acc >= depth) break;
-            cur = nxt;
-            s_path[acc++] = cur;
+            t = s_arg[cur + 1];
+            unsigned nxt = 0xffffffffu;
+            for (int i = lane; i < n; i += 32)
+                if (s_par[i] == cur && s_tok[i] == t) { nxt = (unsigned)i; break; }
+            nxt = __reduce_min_sync(0xffffffffu, nxt);
+            if (nxt == 0xffffffffu || acc >= depth) break;
+            cur = (int)nxt;
+            if (lane == 0) s_path[acc] = cur;
+            ++acc;
         }
+        __syncwarp();
         int rows = 0;
-        while (rows < acc && T.kept_store[s_path[rows]] >= 0) ++rows;
-        s_n = acc;
-        s_rows = rows;
-        *out_accept = acc;
-        *out_next = t;
-        for (int i = 0; i < depth; ++i) out_path[i] = i < acc ? s_path[i] : -1;
-        kv_len[slot] = P + 1 + rows;
-        if (out_kv_len) *out_kv_len = P + 1 + rows;
+        while (rows < acc && s_store[s_path[rows]] >= 0) ++rows;
+        if (lane < rows) s_src[lane] = P + s_store[s_path[lane]];
+        if (lane == 0) s_rows = rows;
+        if (blockIdx.x == 0) {
+            if (lane < depth) out_path[lane] = lane < acc ? s_path[lane] : -1;
+            if (lane == 0) {
+                *out_accept = acc;
+                *out_next = t;
+                kv_len[slot] = P + 1 + rows;
+                if (out_kv_len) *out_kv_len = P + 1 + rows;
+            }
+        }
     }
     __syncthreads();
-    const int rows = s_rows, kvw = Hkv * dh;
-    for (int m = 0; m < rows; ++m) {
-        const int src = P + T.kept_store[s_path[m]], dst = P + 1 + m;
-        if (src == dst) continue;                               // uniform over the CTA
-        for (int i0 = 0; i0 < kvw; i0 += 256) {
-            const int i = i0 + threadIdx.x;
-            float kx = 0.f, vx = 0.f;
-            long long od = 0;
-            if (i < kvw) {
-                const int h = i / dh, e = i % dh;
-                const long long os = (((long long)slot * Hkv + h) * max_len + src) * dh + e;
-                od = (((long long)slot * Hkv + h) * max_len + dst) * dh + e;
-                kx = load_as_float<WT>(Kc, os);
-                vx = load_as_float<WT>(Vc, os);
-            }
-            if (i < kvw) {
-                store_from_float<WT>(Kc, od, kx);
-                store_from_float<WT>(Vc, od, vx);
-            }
-        }
-        __syncthreads();
+    const int rows = s_rows, vpr = dh * (int)sizeof(WT) / 16;        // 16-byte units of a head's row
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < 2 * Hkv * vpr; i += TREE_WALK_CTAS * 256) {
+        const int h = (i / vpr) % Hkv, e = i % vpr;
+        uint4* base = (uint4*)(i < Hkv * vpr ? Kc : Vc) + ((long long)slot * Hkv + h) * max_len * vpr + e;
+        uint4 w[TREE_MAX_DEPTH];
+#pragma unroll
+        for (int m = 0; m < TREE_MAX_DEPTH; ++m)
+            if (m < rows) w[m] = base[(long long)s_src[m] * vpr];
+#pragma unroll
+        for (int m = 0; m < TREE_MAX_DEPTH; ++m)
+            if (m < rows) base[(long long)(P + 1 + m) * vpr] = w[m];
     }
 }
 
@@ -598,8 +649,8 @@ cudaError_t launch_tree_verify(int dtype, int logits_dtype, int slot, int depth,
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (dtype == HIVIS_BF16)
-        tree_walk_kernel<bf16><<<1, 256, 0, st>>>(slot, depth, Hkv, dh, max_len, T, T.row_keys, Kc, Vc, kv_len, out_accept, out_path, out_next, out_kv_len);
+        tree_walk_kernel<bf16><<<TREE_WALK_CTAS, 256, 0, st>>>(slot, depth, Hkv, dh, max_len, T, T.row_keys, Kc, Vc, kv_len, out_accept, out_path, out_next, out_kv_len);
     else
-        tree_walk_kernel<float><<<1, 256, 0, st>>>(slot, depth, Hkv, dh, max_len, T, T.row_keys, Kc, Vc, kv_len, out_accept, out_path, out_next, out_kv_len);
+        tree_walk_kernel<float><<<TREE_WALK_CTAS, 256, 0, st>>>(slot, depth, Hkv, dh, max_len, T, T.row_keys, Kc, Vc, kv_len, out_accept, out_path, out_next, out_kv_len);
     return cudaGetLastError();
 }
