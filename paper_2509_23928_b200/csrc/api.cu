@@ -86,8 +86,6 @@ struct hivis_ctx {
     int64_t launches;
     char err[256];
     std::vector<void*> allocs;
-    char* arena;                  // the rest of the chunk that small buffers are carved from
-    size_t arena_left;
     // optional per-kernel-class timing of hivis_draft (events around every launch)
     bool prof_on;
     std::vector<cudaEvent_t> prof_ev;
@@ -154,31 +152,31 @@ static void fill_chain_args(hivis_ctx* c, ChainArgs* a);
 
 static bool misaligned(const void* p) { return (((uintptr_t)p) & 15u) != 0; }
 
-// A context has some seventy buffers, most of them small, and every device allocation (and its release) costs tens to
-// hundreds of microseconds: requests of up to ARENA_MAX bytes are carved out of chunks.
-#define ARENA_CHUNK ((size_t)24 << 20)
-#define ARENA_MAX ((size_t)6 << 20)
 template <typename T>
 static bool dalloc(hivis_ctx* c, T** p, size_t count) {
-    size_t bytes = (count * sizeof(T) + 511) & ~(size_t)511;
-    if (!bytes) bytes = 512;
-    if (bytes <= ARENA_MAX && bytes <= c->arena_left) {
-        *p = (T*)c->arena;
-        c->arena += bytes;
-        c->arena_left -= bytes;
-        return true;
-    }
-    const size_t want = bytes <= ARENA_MAX ? ARENA_CHUNK : bytes;
     void* q = nullptr;
-    if (cudaMalloc(&q, want) != cudaSuccess) {
+    const size_t bytes = (count * sizeof(T) + 255) & ~(size_t)255;
+    if (cudaMalloc(&q, bytes ? bytes : 256) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
     c->allocs.push_back(q);
     *p = (T*)q;
-    if (want != bytes) {
-        c->arena = (char*)q + bytes;
-        c->arena_left = want - bytes;
+    return true;
+}
+// Several buffers of a megabyte or so in one allocation: each of its own costs a few hundred microseconds at that size.
+struct Carved {
+    void** p;
+    size_t bytes;
+};
+static bool dalloc_together(hivis_ctx* c, const std::vector<Carved>& list) {
+    size_t total = 0;
+    for (const Carved& x : list) total += (x.bytes + 511) & ~(size_t)511;
+    char* base = nullptr;
+    if (!dalloc(c, &base, total)) return false;
+    for (const Carved& x : list) {
+        *x.p = base;
+        base += (x.bytes + 511) & ~(size_t)511;
     }
     return true;
 }
@@ -271,8 +269,6 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
     c->rows_cap = HIVIS_MAX_BATCH;
     c->launches = 0;
     c->err[0] = 0;
-    c->arena = nullptr;
-    c->arena_left = 0;
     c->tap_B = 0;
     c->tap_mma = false;
     c->prof_on = false;
@@ -333,11 +329,14 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
     if (ok && w->resid_proj) ok = dalloc(c, &rp, d * d * es);
     ok = ok && dalloc(c, &c->inv_freq, cfg->head_dim / 2) && dalloc(c, &c->kv_len, MB) &&
          dalloc(c, &c->pend_id, MB) && dalloc(c, &c->pend_feat, MB * d) && dalloc(c, &c->d_slots, R) &&
-         dalloc(c, &c->d_pos0, R) && dalloc(c, &c->cur_id, R) && dalloc(c, &c->feat, R * d) &&
-         dalloc(c, &c->feat_h, R * d) && dalloc(c, &c->u, R * d) && dalloc(c, &c->xq, R * d) &&
-         dalloc(c, &c->qkv, R * c->qkvw) && dalloc(c, &c->attn, R * c->qw) && dalloc(c, &c->attn_h, R * c->qw) &&
-         dalloc(c, &c->y, R * d) && dalloc(c, &c->xm, R * d) && dalloc(c, &c->act, R * F) &&
-         dalloc(c, &c->act_h, R * F) && dalloc(c, &c->rho_raw, (long long)HIVIS_MAX_K * d) &&
+         dalloc(c, &c->d_pos0, R) && dalloc(c, &c->cur_id, R) &&
+         dalloc_together(c, {{(void**)&c->feat, 4ull * R * d}, {(void**)&c->feat_h, 2ull * R * d}, {(void**)&c->u, 4ull * R * d},
+                             {(void**)&c->xq, 2ull * R * d}, {(void**)&c->qkv, 4ull * R * c->qkvw},
+                             {(void**)&c->attn, 4ull * R * c->qw}, {(void**)&c->attn_h, 2ull * R * c->qw},
+                             {(void**)&c->y, 4ull * R * d}, {(void**)&c->xm, 2ull * R * d}, {(void**)&c->act, 4ull * R * F},
+                             {(void**)&c->act_h, 2ull * R * F}, {(void**)&c->xe_h, 2ull * R * d},
+                             {(void**)&c->pf_u, 4ull * R * d}, {(void**)&c->pf_kv, 8ull * R * c->kvw}}) &&
+         dalloc(c, &c->rho_raw, (long long)HIVIS_MAX_K * d) &&
          dalloc(c, &c->rho, (long long)HIVIS_MAX_K * d) && dalloc(c, &c->ssq1, tiles1 * R) &&
          dalloc(c, &c->ssq2, tiles1 * R) && dalloc(c, &c->keys, R * c->key_stride) &&
          dalloc(c, &c->vkeys, MB * (cfg->max_k + 1)) && dalloc(c, &c->varrive, MB) &&
@@ -346,7 +345,7 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
          dalloc(c, &c->part_ml, AR * cfg->n_q_heads * (long long)c->nsplit_cap * 2) &&
          dalloc(c, &c->counters, R * cfg->n_q_heads) && dalloc(c, &c->bar_counter, 1) &&
          dalloc(c, &c->error_flag, 2) && dalloc(c, &c->slot_of, c->map_cap) &&
-         dalloc(c, &c->row_of, c->map_cap) && dalloc(c, &c->xe_h, R * d) &&
+         dalloc(c, &c->row_of, c->map_cap) &&
          dalloc(c, &c->rope_tab, 2 * R * (cfg->head_dim / 2));
     {
         TreeBufs& T = c->tree;
@@ -446,8 +445,7 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
                                 c->xe_h, c->Kc, c->Vc, MB * (long long)cfg->n_kv_heads * cfg->max_len,
                                 cfg->head_dim, HIVIS_MAX_BATCH) == cudaSuccess;
         if (ok2)
-            ok2 = dalloc(c, &c->pf_u, R * d) && dalloc(c, &c->pf_kv, R * 2 * c->kvw) &&
-                  tc_encode_weight(c->tc_map_wkv, wqkv + (long long)c->qw * d * es, 2 * c->kvw, d) == cudaSuccess;
+            ok2 = tc_encode_weight(c->tc_map_wkv, wqkv + (long long)c->qw * d * es, 2 * c->kvw, d) == cudaSuccess;
         if (!ok2) cudaGetLastError();
         c->tc_ok = ok2;
     }
