@@ -55,7 +55,9 @@ struct hivis_ctx {
     int opt_tc_prefill;           // option HIVIS_OPT_TC_PREFILL: 0 = never, else the smallest call (pairs) that takes the tensor-core path
     bool pf_ok;                   // the tensor-core prefill can run (bf16, shapes, buffers)
     bf16 *pf_xe, *pf_xq;          // [map_cap][d] pair-major operands of the tensor-core prefill
-    float* pf_ssq;                // [ceil(d / 128)][map_cap]
+    float* pf_ssq;                // [ceil(d / 64)][map_cap]
+    float* pf_partial;            // shared tiles of the tensor-core prefill: accumulators and counters
+    int* pf_ctr;
     float2* pf_rope;              // [map_cap][head_dim / 2]
     u64* phase_t;                 // [HIVIS_MAX_K][HIVIS_PHASE_EVENTS][num_sms]
     int phase_k;                  // draft steps of the last recorded launch (0: none)
@@ -450,9 +452,13 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
         c->tc_ok = ok2;
     }
     if (c->dtype == HIVIS_BF16 && prefill_tc_supported(cfg->d, c->kvw)) {
-        c->pf_ok = dalloc(c, &c->pf_xe, (size_t)c->map_cap * d) && dalloc(c, &c->pf_xq, (size_t)c->map_cap * d) &&
-                   dalloc(c, &c->pf_ssq, (size_t)((d + 127) / 128) * c->map_cap) &&
-                   dalloc(c, &c->pf_rope, (size_t)c->map_cap * (cfg->head_dim / 2));
+        const size_t cap = (size_t)c->map_cap;
+        c->pf_ok = dalloc_together(c, {{(void**)&c->pf_xe, cap * d * 2}, {(void**)&c->pf_xq, cap * d * 2},
+                                       {(void**)&c->pf_ssq, (size_t)((d + 63) / 64) * cap * 4},
+                                       {(void**)&c->pf_rope, cap * (cfg->head_dim / 2) * sizeof(float2)},
+                                       {(void**)&c->pf_partial, prefill_tc_partial_floats(c->num_sms) * 4},
+                                       {(void**)&c->pf_ctr, (size_t)(c->num_sms + 2) * sizeof(int)}}) &&
+                   cudaMemsetAsync(c->pf_ctr, 0, (size_t)(c->num_sms + 2) * sizeof(int), st) == cudaSuccess;
     }
     for (int s = 0; s < HIVIS_MAX_BATCH; ++s) {
         c->kv_upper[s] = 0;
@@ -693,7 +699,8 @@ static int prefill_in_chain_kernel(hivis_ctx* c, const SlotList& sl, const CuSeq
     CKL(c, launch_prefill_setup_rows(sl, cu, start, d, ids, hidden, c->kv_len, c->pend_feat, c->pend_id, c->slot_of, c->row_of,
                                      op_rows, (const bf16*)c->embed, g.vocab, c->xe_h, c->id_flag, st));
     TcArgs a;
-    fill_tc_args(c, &a, pairs, 1, tc_lo_offset(pairs), resid0 && !raw_rho ? c->rho : nullptr, 1, nullptr, nullptr);
+    // (no remainders: the hidden states are bf16, and the K/V projection's operand is rounded as in a large build)
+    fill_tc_args(c, &a, pairs, 1, 0, resid0 && !raw_rho ? c->rho : nullptr, 1, nullptr, nullptr);
     a.rho_h = raw_rho ? resid0 : nullptr;
     a.ph[PH_QKV] = {(const bf16*)c->wqkv + (long long)c->qw * d, 2 * c->kvw, d};
     a.bqkv = c->bqkv ? (const bf16*)c->bqkv + c->qw : nullptr;
@@ -764,31 +771,37 @@ int hivis_prefill(hivis_ctx* c, int B, const int* seq_slots_host, const int32_t*
             return HIVIS_OK;
         }
     }
-    if (resid0) {
+    const bool gemms = c->pf_ok && c->opt_tc_prefill > 0 && total >= c->opt_tc_prefill;
+    const bool raw_rho = gemms && resid0 && !c->resid_proj;          // the row is read where the caller has it
+    if (resid0 && !raw_rho) {
         rc = prepare_rho(c, resid0, 1, st);
         if (rc) return rc;
         rho0 = c->rho;
     }
-    CKL(c, launch_prefill_setup(c->dtype, sl, cu, start, d, ids, hidden, c->kv_len, c->pend_feat, c->pend_id,
-                                c->slot_of, c->row_of, st));
-    if (c->pf_ok && c->opt_tc_prefill > 0 && total >= c->opt_tc_prefill) {
+    if (gemms) {
         // many pairs: the two GEMMs of the prefix build on the tensor cores, all pairs in one pass
+        CKL(c, launch_prefill_setup_rows(sl, cu, start, d, ids, (const bf16*)hidden, c->kv_len, c->pend_feat, c->pend_id,
+                                         c->slot_of, c->row_of, (int)total, (const bf16*)c->embed, c->cfg.vocab, c->pf_xe,
+                                         c->id_flag, st));
         PrefillTcArgs a;
         memset(&a, 0, sizeof(a));
         a.num_sms = c->num_sms; a.n_pairs = (int)total; a.pair_cap = (int)c->map_cap;
         a.d = d; a.kvw = c->kvw; a.Hkv = c->cfg.n_kv_heads; a.dh = c->cfg.head_dim; a.max_len = c->cfg.max_len;
-        a.vocab = c->cfg.vocab; a.eps = c->cfg.rms_eps;
-        a.ids = ids; a.hidden = (const bf16*)hidden; a.embed = (const bf16*)c->embed; a.fc = (const bf16*)c->fc;
+        a.eps = c->cfg.rms_eps;
+        a.hidden = (const bf16*)hidden; a.fc = (const bf16*)c->fc;
         a.wkv = (const bf16*)c->wqkv + (long long)c->qw * d;
         a.bkv = c->bqkv ? (const bf16*)c->bqkv + c->qw : nullptr;
-        a.norm1 = (const bf16*)c->norm1; a.rho0 = rho0;
+        a.norm1 = (const bf16*)c->norm1; a.rho0 = rho0; a.rho0_h = raw_rho ? (const bf16*)resid0 : nullptr;
         a.xe = c->pf_xe; a.xq = c->pf_xq; a.ssq = c->pf_ssq; a.rope = c->pf_rope;
+        a.partial = c->pf_partial; a.unit_ctr = c->pf_ctr;
         a.slot_of = c->slot_of; a.row_of = c->row_of; a.inv_freq = c->inv_freq;
         a.Kc = (bf16*)c->Kc; a.Vc = (bf16*)c->Vc;
-        a.wait_cycles = c->wait_cycles; a.error_flag = c->error_flag; a.id_flag = c->id_flag;
+        a.wait_cycles = c->wait_cycles; a.error_flag = c->error_flag;
         CK(c, launch_prefill_tc(a, st));
-        c->launches += 4;
+        c->launches += 3;
     } else {
+    CKL(c, launch_prefill_setup(c->dtype, sl, cu, start, d, ids, hidden, c->kv_len, c->pend_feat, c->pend_id,
+                                c->slot_of, c->row_of, st));
     const bool mma = use_mma(c, 16, true);
     for (long long j0 = 0; j0 < total; j0 += 16) {
         const int P = (int)(total - j0 < 16 ? total - j0 : 16);

@@ -224,22 +224,25 @@ int tc_groups(int B);
 struct PrefillTcArgs {
     int num_sms;
     int n_pairs, pair_cap;     // packed pairs of the call; capacity of the pair-major buffers
-    int d, kvw, Hkv, dh, max_len, vocab;
+    int d, kvw, Hkv, dh, max_len;
     float eps;
-    const int32_t* ids;        // [n_pairs]
     const bf16* hidden;        // [n_pairs][d] the caller's hidden states
-    const bf16 *embed, *fc, *wkv, *bkv, *norm1;      // wkv: rows [K ; V] of the stacked QKV matrix, bkv nullable
+    const bf16 *fc, *wkv, *bkv, *norm1;      // wkv: rows [K ; V] of the stacked QKV matrix, bkv nullable
     const float* rho0;         // [d] nullable
-    bf16 *xe, *xq;             // [pair_cap][d] gathered embedding rows; gamma_1 * u
-    float* ssq;                // [ceil(d / 128)][pair_cap]
+    const bf16* rho0_h;        // [d] nullable: the caller's row, read where rho0 is null
+    bf16 *xe, *xq;             // [pair_cap][d] gathered embedding rows (launch_prefill_setup_rows); gamma_1 * u
+    float* ssq;                // [ceil(d / 64)][pair_cap]
+    float* partial;            // accumulators of tiles that several clusters share (prefill_tc_partial_floats)
+    int* unit_ctr;             // [2 x clusters] their counters, zero between calls
     float2* rope;              // [pair_cap][dh / 2] scratch: (cos, sin) at every pair's position
     const int *slot_of, *row_of;
     const double* inv_freq;
     bf16 *Kc, *Vc;
     long long wait_cycles;
-    int *error_flag, *id_flag;
+    int* error_flag;
 };
 bool prefill_tc_supported(int d, int kvw);
+size_t prefill_tc_partial_floats(int num_sms);
 cudaError_t launch_prefill_tc(const PrefillTcArgs& a, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------

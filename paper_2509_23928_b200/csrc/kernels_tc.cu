@@ -156,7 +156,8 @@ cudaError_t tc_encode_operand(unsigned char* map, const void* x, long long rows,
 
 template <int DH, int GQ>
 static cudaError_t tc_launch_greedy(const TcMaps& maps, const TcArgs& a, int grid, cudaStream_t st) {
-    switch (tc_groups(a.B)) {
+    // (a batch whose operands carry no remainders takes the two-group kernel, however small)
+    switch (a.lo == 0 && a.B <= 16 ? 2 : tc_groups(a.B)) {
         case 1: return tc_launch_t<DH, GQ, false, 1>(maps, a, grid, st);
         case 2: return tc_launch_t<DH, GQ, false, 2>(maps, a, grid, st);
         default: return tc_launch_t<DH, GQ, false, 4>(maps, a, grid, st);

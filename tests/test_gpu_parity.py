@@ -280,7 +280,7 @@ def test_tensor_core_prefill_tile_edges(name, pairs):
 def test_small_prefix_builds_in_the_chain_kernel(name, project, pairs):
     """1..64 pairs as columns of the chain kernel (one, two and four column groups, full and partly filled) against the
     kernels of 16 pairs per pass, after a larger call has left its rows in every buffer; then the draft that consumes the
-    pending pairs.  Both paths round the same operand (the chain kernel keeps its remainder up to 16 pairs) and the stored
+    pending pairs.  Both paths round the same operand and the stored
     rows to bf16: one unit in the last place (2^-8 of the value) apart."""
     import torch
     wl = hi.scaled(hi.workload(name), batch=2, text_len=None, text_len_range=(1, 2))
