@@ -849,7 +849,13 @@ static int draft_impl(hivis_ctx* c, int B, const int* seq_slots_host, int k, con
     // The kernel numbers attention units x warps in 32 bits; a batch beyond that (hundreds of heads on long caches) takes
     // the per-phase kernels, as do draws for more than 16 sequences (refused below).
     const bool tc_fits = B <= 16 || (!uniforms && (long long)B * g.n_q_heads * ((max_rows + 31) / 32 + 1) * 4 * c->num_sms < (1ll << 32));
-    const bool in_tc = !one_seq && c->tc_ok && c->opt_tc != 0 && tc_fits;
+    bool in_tc = !one_seq && c->tc_ok && c->opt_tc != 0 && tc_fits;
+    if (in_tc && B > 16) {
+        // (the kernel's barrier counter is counted on the host: a captured call would be replayed with a stale count)
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CK(c, cudaStreamIsCapturing(st, &cap));
+        in_tc = cap == cudaStreamCaptureStatusNone;
+    }
     const bool raw_rho = resid && !c->resid_proj && (one_seq || in_tc);
     if (resid && !raw_rho) {
         rc = prepare_rho(c, resid, n_resid, st);

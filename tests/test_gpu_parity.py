@@ -315,6 +315,46 @@ def test_small_prefix_builds_in_the_chain_kernel(name, project, pairs):
         case.close()
 
 
+def test_captured_refresh_and_wide_draft_replay():
+    """A small prefix build and a draft of 20 sequences captured into a graph take the kernels without a host-counted
+    barrier: every replay gives what the calls give."""
+    import torch
+    wl = hi.scaled(hi.workload("mini_mha_b5_ragged"), batch=20, k=3, text_len_range=(2, 40))
+    case = Case(wl)
+    try:
+        dr = case.drafter
+        case.gpu_prefill()
+        _, want = case.gpu_draft()
+        rows = [int(x) - 1 for x in case.lens]
+        ids, hidden = case.d_ids[:4].contiguous(), case.d_hidden[:4].contiguous()
+        n = min(rows[0], 1)
+
+        def turn():
+            dr.set_kv_len_batch(rows, restore_pending=True)
+            dr.prefill(ids, hidden, [0, 4], slots=[0], start_pos=[n], resid0=case.d_resid[0])
+            dr.set_kv_len_batch(rows[1:], slots=list(range(1, 20)), restore_pending=True)
+            return dr.draft(20, wl.k, case.d_resid, want_logits=True)
+        eager = turn()[1].clone()
+        kv = dr.read_kv(0, 0, n + 3)
+        g, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(g, stream=s):
+            out = turn()
+        for _ in range(2):
+            out[1].zero_()
+            g.replay()
+            torch.cuda.synchronize()
+            err = row_rel_err(out[1].cpu().numpy(), eager.cpu().numpy())
+            assert err.max() <= LOGIT_RTOL
+            for x, y in zip(dr.read_kv(0, 0, n + 3), kv):
+                assert (x - y).abs().max() <= 2.0 ** -7 * y.abs().max()
+        assert row_rel_err(eager.cpu().numpy()[1:], want[1:]).max() <= LOGIT_RTOL
+        del g
+        dr.status()
+    finally:
+        case.close()
+
+
 def test_more_sequences_than_the_chain_kernels_take():
     """20 sequences: beyond the 16 of the tensor-core chain kernel, so the per-phase kernels run in two passes."""
     wl = hi.scaled(hi.workload("mini_gqa_b16_ragged"), batch=20, k=3, seed=2103)
