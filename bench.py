@@ -55,7 +55,7 @@ def measured_peaks():
     return 6650.0, "fallback"
 
 
-CHAIN_KERNEL_SOURCES = ("kernels_tc.cu", "kernels_chain.cu", "attn_body.cuh", "attn_warp.cuh", "attn_mma.cuh")
+CHAIN_KERNEL_SOURCES = ("tc_chain.cuh", "kernels_tc.cu", "kernels_chain.cu", "attn_body.cuh", "attn_warp.cuh", "attn_mma.cuh")
 
 
 def kernel_source_hash() -> str:
