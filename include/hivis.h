@@ -274,11 +274,9 @@ int hivis_debug_tap(hivis_ctx* ctx, int which, float* out, void* stream);
  * keep-in-L2 policy instead of streaming them through: with k chained steps in one launch a subset that fits
  * in L2 beside the KV cache is then read from HBM once per launch rather than once per step.
  * HIVIS_OPT_TC_PREFILL (default 1): with bf16 weights, a hivis_prefill call of HIVIS_TC_PREFILL_MIN_PAIRS pairs or more
- * builds the prefix for all pairs at once on the tcgen05 tensor cores: up to 64 pairs as columns of the chain kernel's
- * first two GEMM phases, more as two GEMMs of their own (256 pairs x 256 weight rows per pair of CTAs); 0 = in passes of
- * 16 pairs; a value n > 1 = calls of n pairs or more.  A call of at most 16 pairs is one pass either way: in the chain
- * kernel, or with HIVIS_OPT_TC_KERNEL = 0 (or while the stream is captured into a graph) in kernels of its own.
- * Same results up to fp32 summation order.                                                                     */
+ * builds the prefix with two tcgen05 GEMMs over all pairs at once (256 pairs x 128 or 256 weight rows per pair of CTAs); 0 =
+ * always in passes of 16 pairs, which smaller calls are in any case; a value n > 1 = calls of n pairs or more.  Both ways round
+ * the K/V projection's operand and the cached rows to bf16 after fp32 sums in orders of their own.              */
 #define HIVIS_TC_PREFILL_MIN_PAIRS 17     /* more than one pass of 16 pairs */
 enum { HIVIS_OPT_CHAIN_KERNEL = 0, HIVIS_OPT_TC_KERNEL = 1, HIVIS_OPT_WAIT_LIMIT_US = 2, HIVIS_OPT_DEBUG_MISS_BARRIER = 3,
        HIVIS_OPT_PHASE_TIMES = 4, HIVIS_OPT_L2_KEEP = 5, HIVIS_OPT_TC_PREFILL = 6 };

@@ -397,7 +397,7 @@ class Drafter:
         hivis_set_option(self.ctx, HIVIS_OPT_DEBUG_MISS_BARRIER, 1)
 
     def set_tc_prefill(self, on):
-        """False: hivis_prefill always uses the 16-pairs-per-pass kernels; True: the default threshold; an int n > 1:
+        """False: hivis_prefill always works in passes of 16 pairs; True: the default threshold; an int n > 1:
         calls of n pairs or more take the tensor-core path."""
         hivis_set_option(self.ctx, HIVIS_OPT_TC_PREFILL, int(on))
 

@@ -14,7 +14,7 @@ struct hivis_ctx {
     int dtype;
     size_t esize;
     int qw, kvw, qkvw;
-    int rows_cap;                 // batch rows the workspaces hold: the 64 columns of the widest chain kernel
+    int rows_cap;                 // batch rows the workspaces hold: the operand rows of the widest chain kernel that the context launches
     int device;
     // weights (library-owned copies)
     void *embed, *lm_head, *fc, *norm1, *wqkv, *bqkv, *wo, *norm2, *wgu, *wdown, *resid_proj;
@@ -55,15 +55,11 @@ struct hivis_ctx {
     int opt_tc_prefill;           // option HIVIS_OPT_TC_PREFILL: 0 = never, else the smallest call (pairs) that takes the tensor-core path
     bool pf_ok;                   // the tensor-core prefill can run (bf16, shapes, buffers)
     bf16 *pf_xe, *pf_xq;          // [map_cap][d] pair-major operands of the tensor-core prefill
-    float* pf_ssq;                // [ceil(d / 64)][map_cap]
-    float* pf_partial;            // shared tiles of the tensor-core prefill: accumulators and counters
-    int* pf_ctr;
+    float* pf_ssq;                // [ceil(d / 128)][map_cap]
     float2* pf_rope;              // [map_cap][head_dim / 2]
     u64* phase_t;                 // [HIVIS_MAX_K][HIVIS_PHASE_EVENTS][num_sms]
     int phase_k;                  // draft steps of the last recorded launch (0: none)
-    TcMaps tc_maps, tc_maps_wide; // operands of 32 rows; of 64 rows (more than 32 columns)
-    alignas(64) unsigned char tc_map_wkv[128];   // the K and V rows of the stacked QKV matrix
-    float *pf_u, *pf_kv;          // small prefix builds in the chain kernel: [64][d], [64][2 kvw]
+    TcMaps tc_maps, tc_maps_wide; // operands of 32 rows; of 64 rows (contexts of more than 32 sequences)
     float* tc_partial;
     int* tile_ctr;
     int tc_tiles;
@@ -268,7 +264,7 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
     c->qw = cfg->n_q_heads * cfg->head_dim;
     c->kvw = cfg->n_kv_heads * cfg->head_dim;
     c->qkvw = c->qw + 2 * c->kvw;
-    c->rows_cap = HIVIS_MAX_BATCH;
+    c->rows_cap = cfg->max_batch > TC_OP_ROWS ? HIVIS_MAX_BATCH : TC_OP_ROWS;
     c->launches = 0;
     c->err[0] = 0;
     c->tap_B = 0;
@@ -336,8 +332,7 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
                              {(void**)&c->xq, 2ull * R * d}, {(void**)&c->qkv, 4ull * R * c->qkvw},
                              {(void**)&c->attn, 4ull * R * c->qw}, {(void**)&c->attn_h, 2ull * R * c->qw},
                              {(void**)&c->y, 4ull * R * d}, {(void**)&c->xm, 2ull * R * d}, {(void**)&c->act, 4ull * R * F},
-                             {(void**)&c->act_h, 2ull * R * F}, {(void**)&c->xe_h, 2ull * R * d},
-                             {(void**)&c->pf_u, 4ull * R * d}, {(void**)&c->pf_kv, 8ull * R * c->kvw}}) &&
+                             {(void**)&c->act_h, 2ull * R * F}, {(void**)&c->xe_h, 2ull * R * d}}) &&
          dalloc(c, &c->rho_raw, (long long)HIVIS_MAX_K * d) &&
          dalloc(c, &c->rho, (long long)HIVIS_MAX_K * d) && dalloc(c, &c->ssq1, tiles1 * R) &&
          dalloc(c, &c->ssq2, tiles1 * R) && dalloc(c, &c->keys, R * c->key_stride) &&
@@ -435,30 +430,26 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
         ChainArgs ca;
         fill_chain_args(c, &ca);
         c->tc_tiles = tc_max_tiles(ca.ph);
-        bool ok2 = dalloc(c, &c->tc_partial, (size_t)c->num_sms * 2 * R * 128) && dalloc(c, &c->tile_ctr, c->tc_tiles) &&
+        bool ok2 = dalloc(c, &c->tc_partial, (size_t)c->num_sms * 2 * 16 * tc_groups((int)MB) * 128) &&
+                   dalloc(c, &c->tile_ctr, c->tc_tiles) &&
                    dalloc(c, &c->phase_t, (size_t)HIVIS_MAX_K * HIVIS_PHASE_EVENTS * c->num_sms);
         if (ok2) ok2 = cudaMemsetAsync(c->tile_ctr, 0, c->tc_tiles * sizeof(int), st) == cudaSuccess;
         if (ok2)
             ok2 = tc_build_maps(&c->tc_maps, ca.ph, cfg->d, c->qw, cfg->ffn, c->feat_h, c->xq, c->attn_h, c->xm, c->act_h,
                                 c->xe_h, c->Kc, c->Vc, MB * (long long)cfg->n_kv_heads * cfg->max_len,
                                 cfg->head_dim, TC_OP_ROWS) == cudaSuccess;
-        if (ok2)
+        if (ok2 && R > TC_OP_ROWS)
             ok2 = tc_build_maps(&c->tc_maps_wide, ca.ph, cfg->d, c->qw, cfg->ffn, c->feat_h, c->xq, c->attn_h, c->xm, c->act_h,
                                 c->xe_h, c->Kc, c->Vc, MB * (long long)cfg->n_kv_heads * cfg->max_len,
                                 cfg->head_dim, HIVIS_MAX_BATCH) == cudaSuccess;
-        if (ok2)
-            ok2 = tc_encode_weight(c->tc_map_wkv, wqkv + (long long)c->qw * d * es, 2 * c->kvw, d) == cudaSuccess;
         if (!ok2) cudaGetLastError();
         c->tc_ok = ok2;
     }
     if (c->dtype == HIVIS_BF16 && prefill_tc_supported(cfg->d, c->kvw)) {
         const size_t cap = (size_t)c->map_cap;
         c->pf_ok = dalloc_together(c, {{(void**)&c->pf_xe, cap * d * 2}, {(void**)&c->pf_xq, cap * d * 2},
-                                       {(void**)&c->pf_ssq, (size_t)((d + 63) / 64) * cap * 4},
-                                       {(void**)&c->pf_rope, cap * (cfg->head_dim / 2) * sizeof(float2)},
-                                       {(void**)&c->pf_partial, prefill_tc_partial_floats(c->num_sms) * 4},
-                                       {(void**)&c->pf_ctr, (size_t)(c->num_sms + 2) * sizeof(int)}}) &&
-                   cudaMemsetAsync(c->pf_ctr, 0, (size_t)(c->num_sms + 2) * sizeof(int), st) == cudaSuccess;
+                                       {(void**)&c->pf_ssq, (size_t)((d + 127) / 128) * cap * 4},
+                                       {(void**)&c->pf_rope, cap * (cfg->head_dim / 2) * sizeof(float2)}});
     }
     for (int s = 0; s < HIVIS_MAX_BATCH; ++s) {
         c->kv_upper[s] = 0;
@@ -681,41 +672,6 @@ static void prefill_done(hivis_ctx* c, const SlotList& sl, const int* new_upper,
     }
 }
 
-// A prefix build of at most 64 pairs in the tensor-core chain kernel: bookkeeping and operand rows, then the phases fusion
-// FC and QKV with the K and V rows of the stacked matrix, then the rotation and the cache rows.  The hidden states are read
-// where the caller has them; u and the K/V values go to buffers of their own.
-static int prefill_in_chain_kernel(hivis_ctx* c, const SlotList& sl, const CuSeqlens& cu, const SlotList& start, int pairs,
-                                   const int32_t* ids, const bf16* hidden, const bf16* resid0, cudaStream_t st) {
-    const hivis_config& g = c->cfg;
-    const int d = g.d, op_rows = pairs <= TC_OP_ROWS ? TC_OP_ROWS : HIVIS_MAX_BATCH;
-    const bool raw_rho = resid0 && !c->resid_proj;
-    if (resid0 && !raw_rho) {
-        const int rc = prepare_rho(c, resid0, 1, st);
-        if (rc) return rc;
-    }
-    TcMaps maps = pairs <= TC_OP_ROWS ? c->tc_maps : c->tc_maps_wide;
-    memcpy(maps.m[TCM_W + PH_QKV], c->tc_map_wkv, 128);
-    CK(c, tc_encode_operand(maps.m[TCM_X_FEAT], hidden, pairs, d, op_rows));
-    CKL(c, launch_prefill_setup_rows(sl, cu, start, d, ids, hidden, c->kv_len, c->pend_feat, c->pend_id, c->slot_of, c->row_of,
-                                     op_rows, (const bf16*)c->embed, g.vocab, c->xe_h, c->id_flag, st));
-    TcArgs a;
-    // (no remainders: the hidden states are bf16, and the K/V projection's operand is rounded as in a large build)
-    fill_tc_args(c, &a, pairs, 1, 0, resid0 && !raw_rho ? c->rho : nullptr, 1, nullptr, nullptr);
-    a.rho_h = raw_rho ? resid0 : nullptr;
-    a.ph[PH_QKV] = {(const bf16*)c->wqkv + (long long)c->qw * d, 2 * c->kvw, d};
-    a.bqkv = c->bqkv ? (const bf16*)c->bqkv + c->qw : nullptr;
-    a.u = c->pf_u;
-    a.qkv = c->pf_kv;
-    a.seq_first = 1; a.seq_last = 2;                                 // fusion FC, QKV
-    const u64 G = (u64)c->num_sms;
-    a.bar_base = c->bar_count_host - G;                              // as if the gather had been arrived on
-    CKL(c, launch_tc_chain(maps, a, c->num_sms, st));
-    c->bar_count_host += 2 * G;
-    CKL(c, launch_kv_append(c->dtype, c->pf_kv, pairs, c->slot_of, c->row_of, c->inv_freq, g.n_kv_heads, g.head_dim, g.max_len,
-                            c->Kc, c->Vc, st));
-    return HIVIS_OK;
-}
-
 int hivis_prefill(hivis_ctx* c, int B, const int* seq_slots_host, const int32_t* ids, const void* hidden,
                   const int32_t* cu_seqlens_host, const int32_t* start_pos_host, const void* resid0,
                   void* stream) {
@@ -756,21 +712,6 @@ int hivis_prefill(hivis_ctx* c, int B, const int* seq_slots_host, const int32_t*
     cudaStream_t st = (cudaStream_t)stream;
     const int d = c->cfg.d;
     const float* rho0 = nullptr;
-    // Up to 64 pairs (the rows that a verified draft left to rebuild: a few per sequence) are a batch of columns like any
-    // other: the fusion FC and the K/V projection run as two phases of the tensor-core chain kernel, in one pass over
-    // their weights with every SM at work.  The barrier counter of that kernel is counted on the host, so a call that
-    // is being captured into a graph (and replayed without the host) takes the kernels below.
-    if (c->tc_ok && c->opt_tc != 0 &&
-        (total <= 16 || (total <= HIVIS_MAX_BATCH && c->opt_tc_prefill > 0 && total >= c->opt_tc_prefill))) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        CK(c, cudaStreamIsCapturing(st, &cap));
-        if (cap == cudaStreamCaptureStatusNone) {
-            rc = prefill_in_chain_kernel(c, sl, cu, start, (int)total, ids, (const bf16*)hidden, (const bf16*)resid0, st);
-            if (rc) return rc;
-            prefill_done(c, sl, new_upper, start_pos_host != nullptr);
-            return HIVIS_OK;
-        }
-    }
     const bool gemms = c->pf_ok && c->opt_tc_prefill > 0 && total >= c->opt_tc_prefill;
     const bool raw_rho = gemms && resid0 && !c->resid_proj;          // the row is read where the caller has it
     if (resid0 && !raw_rho) {
@@ -781,8 +722,7 @@ int hivis_prefill(hivis_ctx* c, int B, const int* seq_slots_host, const int32_t*
     if (gemms) {
         // many pairs: the two GEMMs of the prefix build on the tensor cores, all pairs in one pass
         CKL(c, launch_prefill_setup_rows(sl, cu, start, d, ids, (const bf16*)hidden, c->kv_len, c->pend_feat, c->pend_id,
-                                         c->slot_of, c->row_of, (int)total, (const bf16*)c->embed, c->cfg.vocab, c->pf_xe,
-                                         c->id_flag, st));
+                                         c->slot_of, c->row_of, (const bf16*)c->embed, c->cfg.vocab, c->pf_xe, c->id_flag, st));
         PrefillTcArgs a;
         memset(&a, 0, sizeof(a));
         a.num_sms = c->num_sms; a.n_pairs = (int)total; a.pair_cap = (int)c->map_cap;
@@ -793,27 +733,26 @@ int hivis_prefill(hivis_ctx* c, int B, const int* seq_slots_host, const int32_t*
         a.bkv = c->bqkv ? (const bf16*)c->bqkv + c->qw : nullptr;
         a.norm1 = (const bf16*)c->norm1; a.rho0 = rho0; a.rho0_h = raw_rho ? (const bf16*)resid0 : nullptr;
         a.xe = c->pf_xe; a.xq = c->pf_xq; a.ssq = c->pf_ssq; a.rope = c->pf_rope;
-        a.partial = c->pf_partial; a.unit_ctr = c->pf_ctr;
         a.slot_of = c->slot_of; a.row_of = c->row_of; a.inv_freq = c->inv_freq;
         a.Kc = (bf16*)c->Kc; a.Vc = (bf16*)c->Vc;
         a.wait_cycles = c->wait_cycles; a.error_flag = c->error_flag;
         CK(c, launch_prefill_tc(a, st));
         c->launches += 3;
     } else {
-    CKL(c, launch_prefill_setup(c->dtype, sl, cu, start, d, ids, hidden, c->kv_len, c->pend_feat, c->pend_id,
-                                c->slot_of, c->row_of, st));
-    const bool mma = use_mma(c, 16, true);
-    for (long long j0 = 0; j0 < total; j0 += 16) {
-        const int P = (int)(total - j0 < 16 ? total - j0 : 16);
-        const char* hid = (const char*)hidden + j0 * d * c->esize;
-        rc = run_fuse(c, mma, 0, P, mma ? nullptr : (const float*)hid, mma ? hid : nullptr, ids + j0, 1, nullptr,
-                      rho0, st);
-        if (rc) return rc;
-        rc = run_qkv(c, mma, 0, P, c->qw, 2 * c->kvw, c->qkv, st);   // K and V rows only
-        if (rc) return rc;
-        CKL(c, launch_kv_append(c->dtype, c->qkv, P, c->slot_of + j0, c->row_of + j0, c->inv_freq,
-                                c->cfg.n_kv_heads, c->cfg.head_dim, c->cfg.max_len, c->Kc, c->Vc, st));
-    }
+        CKL(c, launch_prefill_setup(c->dtype, sl, cu, start, d, ids, hidden, c->kv_len, c->pend_feat, c->pend_id,
+                                    c->slot_of, c->row_of, st));
+        const bool mma = use_mma(c, 16, true);
+        for (long long j0 = 0; j0 < total; j0 += 16) {
+            const int P = (int)(total - j0 < 16 ? total - j0 : 16);
+            const char* hid = (const char*)hidden + j0 * d * c->esize;
+            rc = run_fuse(c, mma, 0, P, mma ? nullptr : (const float*)hid, mma ? hid : nullptr, ids + j0, 1, nullptr,
+                          rho0, st);
+            if (rc) return rc;
+            rc = run_qkv(c, mma, 0, P, c->qw, 2 * c->kvw, c->qkv, st);   // K and V rows only
+            if (rc) return rc;
+            CKL(c, launch_kv_append(c->dtype, c->qkv, P, c->slot_of + j0, c->row_of + j0, c->inv_freq,
+                                    c->cfg.n_kv_heads, c->cfg.head_dim, c->cfg.max_len, c->Kc, c->Vc, st));
+        }
     }
     prefill_done(c, sl, new_upper, start_pos_host != nullptr);
     return HIVIS_OK;

@@ -205,8 +205,6 @@ struct TcArgs {
 cudaError_t tc_build_maps(TcMaps* maps, const ChainPhase* ph, int d, int qw, int F, const bf16* feat_h,
                           const bf16* xq_h, const bf16* attn_h, const bf16* xm_h, const bf16* act_h, const bf16* xe_h,
                           const void* Kc, const void* Vc, long long cache_rows, int dh, int op_rows);
-cudaError_t tc_encode_weight(unsigned char* map, const void* W, long long rows, long long cols);
-cudaError_t tc_encode_operand(unsigned char* map, const void* x, long long rows, long long cols, int op_rows);
 bool tc_supported(int d, int dh, int Hq, int Hkv, int F);
 int tc_max_tiles(const ChainPhase* ph);
 cudaError_t launch_tc_chain(const TcMaps& maps, const TcArgs& a, int grid, cudaStream_t st);
@@ -231,9 +229,7 @@ struct PrefillTcArgs {
     const float* rho0;         // [d] nullable
     const bf16* rho0_h;        // [d] nullable: the caller's row, read where rho0 is null
     bf16 *xe, *xq;             // [pair_cap][d] gathered embedding rows (launch_prefill_setup_rows); gamma_1 * u
-    float* ssq;                // [ceil(d / 64)][pair_cap]
-    float* partial;            // accumulators of tiles that several clusters share (prefill_tc_partial_floats)
-    int* unit_ctr;             // [2 x clusters] their counters, zero between calls
+    float* ssq;                // [ceil(d / 128)][pair_cap]
     float2* rope;              // [pair_cap][dh / 2] scratch: (cos, sin) at every pair's position
     const int *slot_of, *row_of;
     const double* inv_freq;
@@ -242,7 +238,6 @@ struct PrefillTcArgs {
     int* error_flag;
 };
 bool prefill_tc_supported(int d, int kvw);
-size_t prefill_tc_partial_floats(int num_sms);
 cudaError_t launch_prefill_tc(const PrefillTcArgs& a, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------
@@ -316,12 +311,10 @@ cudaError_t launch_prefill_setup(int dtype, const SlotList& sl, const CuSeqlens&
                                  const SlotList& start /* -1 = append */, int d, const int32_t* ids,
                                  const void* hidden, int* kv_len, float* pend_feat, int* pend_id,
                                  int* slot_of, int* row_of, cudaStream_t st);
-// the same for a call whose pairs are one batch of the tensor-core chain kernel (bf16): also gathers the embedding rows of
-// the pairs' tokens (zero rows up to op_rows)
+// the same for a call that the tensor-core prefix build takes (bf16): also gathers the embedding rows of the pairs' tokens
 cudaError_t launch_prefill_setup_rows(const SlotList& sl, const CuSeqlens& cu, const SlotList& start, int d, const int32_t* ids,
                                       const bf16* hidden, int* kv_len, float* pend_feat, int* pend_id, int* slot_of,
-                                      int* row_of, int op_rows, const bf16* embed, int vocab, bf16* xe_h, int* id_flag,
-                                      cudaStream_t st);
+                                      int* row_of, const bf16* embed, int vocab, bf16* xe, int* id_flag, cudaStream_t st);
 // RoPE(K) and store K,V rows of a chunk of packed entries
 cudaError_t launch_kv_append(int dtype, const float* kv /*[P][2*kvw]*/, int P, const int* slot_of,
                              const int* row_of, const double* inv_freq, int Hkv, int dh, int max_len,

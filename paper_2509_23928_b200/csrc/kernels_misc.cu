@@ -112,24 +112,20 @@ cudaError_t launch_prefill_setup(int dtype, const SlotList& sl, const CuSeqlens&
     return cudaGetLastError();
 }
 
-// Blocks [0, op_rows): the embedding row of pair j, 16 bytes per thread and turn (a zero row beyond the pairs); then one
-// block per sequence (rows, pending pair, row count).  What bounds it is a chain of two loads.
+// Blocks [0, pairs): the embedding row of pair j, 16 bytes per thread and turn; then one block per sequence (rows, pending
+// pair, row count).  What bounds it is a chain of two loads.
 __global__ void prefill_setup_rows_kernel(SlotList sl, CuSeqlens cu, SlotList start, int d, const int32_t* ids,
                                           const bf16* hidden, int* kv_len, float* pend_feat, int* pend_id, int* slot_of,
-                                          int* row_of, int op_rows, const bf16* embed, int vocab, bf16* xe_h, int* id_flag) {
-    const int upr = d >> 3;
-    if ((int)blockIdx.x < op_rows) {
+                                          int* row_of, const bf16* embed, int vocab, bf16* xe, int* id_flag) {
+    const int upr = d >> 3, pairs = cu.v[sl.n];
+    if ((int)blockIdx.x < pairs) {
         const int j = blockIdx.x;
-        uint4* dst = (uint4*)(xe_h + (long long)j * d);
-        if (j >= cu.v[sl.n]) {
-            for (int i = threadIdx.x; i < upr; i += blockDim.x) dst[i] = make_uint4(0u, 0u, 0u, 0u);
-            return;
-        }
+        uint4* dst = (uint4*)(xe + (long long)j * d);
         const uint4* src = (const uint4*)(embed + (long long)checked_token(ids[j], vocab, id_flag) * d);
         for (int i = threadIdx.x; i < upr; i += blockDim.x) dst[i] = ld_stream(src + i);
         return;
     }
-    const int b = blockIdx.x - op_rows;
+    const int b = blockIdx.x - pairs;
     __shared__ int s_base;
     const int slot = sl.slot[b];
     const int lo = cu.v[b], hi = cu.v[b + 1];
@@ -154,10 +150,9 @@ __global__ void prefill_setup_rows_kernel(SlotList sl, CuSeqlens cu, SlotList st
 }
 cudaError_t launch_prefill_setup_rows(const SlotList& sl, const CuSeqlens& cu, const SlotList& start, int d, const int32_t* ids,
                                       const bf16* hidden, int* kv_len, float* pend_feat, int* pend_id, int* slot_of,
-                                      int* row_of, int op_rows, const bf16* embed, int vocab, bf16* xe_h, int* id_flag,
-                                      cudaStream_t st) {
-    prefill_setup_rows_kernel<<<op_rows + sl.n, 512, 0, st>>>(
-        sl, cu, start, d, ids, hidden, kv_len, pend_feat, pend_id, slot_of, row_of, op_rows, embed, vocab, xe_h, id_flag);
+                                      int* row_of, const bf16* embed, int vocab, bf16* xe, int* id_flag, cudaStream_t st) {
+    prefill_setup_rows_kernel<<<cu.v[sl.n] + sl.n, 512, 0, st>>>(sl, cu, start, d, ids, hidden, kv_len, pend_feat, pend_id, slot_of,
+                                                                 row_of, embed, vocab, xe, id_flag);
     return cudaGetLastError();
 }
 

@@ -22,11 +22,6 @@
 // clock drops to 1.3-1.5 GHz under the power cap); with 128 x 128 tiles, one per CTA and launch slot, and the tile turned in
 // shared memory for the output stage 7.9 ms.
 //
-// A few hundred pairs give fewer tiles than there are clusters.  In GEMM 2 the k-blocks of a tile are then split over
-// several clusters (one unit of work each, a cooperative launch).  A contributor publishes its accumulators except for the
-// columns that it finishes itself, waits (bounded) for the others and adds their parts in a fixed order: 64 columns per
-// contributor at a time, so that the output stage is split as well.
-//
 // Warp 0 (one thread, both CTAs) issues the copies, warp 1 (one thread of the leader, rank 0) the MMAs for both, warps
 // 2-5 run the output stage.  A stage's full barrier lives in the leader and counts the bytes of both CTAs; tcgen05.commit
 // hands stages and accumulators back to both CTAs.  Every wait is bounded; a wait that runs out raises the error word,
@@ -147,9 +142,6 @@ struct PfParams {
     alignas(64) unsigned char map_x0[128];     // operand of k-blocks [0, kb_split): [pairs][.], box 64 x 128
     alignas(64) unsigned char map_x1[128];     // operand of k-blocks [kb_split, nkb)
     int rows, K, kb_split, n_pairs, m_tiles, n_tiles;
-    int split;                 // clusters per tile; > 1: every cluster has one (tile, part)
-    float* partial;            // [units][2 CTAs][BN / 4][128 pairs] float4
-    int* unit_ctr;             // [tiles][2 CTAs] arrivals (low half) and departures (high half), zero between launches
     long long wait_cycles;
     int* error_flag;
     // GEMM 1 output stage
@@ -157,7 +149,7 @@ struct PfParams {
     const bf16* rho_h;         // [rows] nullable, read where rho is null
     const bf16* gamma;         // [rows]
     bf16* xq;                  // [pairs][rows]
-    float* ssq;                // [column blocks of 64][pair capacity]
+    float* ssq;                // [column blocks of 128][pair capacity]
     int pair_cap;
     // GEMM 2 output stage
     const float* ssq_in;       // [ssq_tiles][pair capacity]
@@ -192,46 +184,15 @@ __device__ __forceinline__ void pf_load32(const bf16* src, float (&x)[32]) {
 // Stages of the ring: as many as shared memory holds.
 template <int BN> struct PfRing { static constexpr unsigned STAGES = BN == 256 ? 7 : 9; };
 
-// The accumulators of this thread's pair: in tensor memory, or the sum of the parts of several clusters (added in the
-// order of the parts; this cluster's own one stays in tensor memory).
-struct PfAcc {
-    uint32_t tacc;
-    const float4* part;        // part 0 of this tile and CTA, this thread's pair
-    long long part_stride;     // float4s from one part to the next
-    int split, me;
-    __device__ __forceinline__ void get(int c, float (&v)[32]) const {
-        pf_ld32(tacc + c, v);
-        if (split == 1) return;
-        float sum[32];
-#pragma unroll
-        for (int i = 0; i < 32; ++i) sum[i] = 0.f;
-#pragma unroll 4
-        for (int s = 0; s < split; ++s) {
-            if (s == me) {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) sum[i] += v[i];
-            } else {
-                const float4* p = part + s * part_stride + (c >> 2) * 128;
-                float4 t[8];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) t[q] = __ldcg(p + q * 128);
-#pragma unroll
-                for (int q = 0; q < 8; ++q) { sum[4 * q] += t[q].x; sum[4 * q + 1] += t[q].y; sum[4 * q + 2] += t[q].z; sum[4 * q + 3] += t[q].w; }
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = sum[i];
-    }
-};
-
-// GEMM 1 output stage of one pair: 64 columns of u, from column n.
-__device__ __forceinline__ void pf_out_fc(const PfParams& P, const PfAcc& acc, int c0, int n0, int pair, bool live) {
+// GEMM 1 output stage of one pair: 128 columns of u from column c0 of the tile (fewer at the end of the rows), their
+// squares added one after the other.
+__device__ __forceinline__ void pf_out_fc(const PfParams& P, uint32_t tacc, int c0, int n0, int pair, bool live) {
     float ss = 0.f;
 #pragma unroll 1
-    for (int c = c0; c < c0 + 64; c += 32) {
+    for (int c = c0; c < c0 + 128 && n0 + c < P.rows; c += 32) {
         const int n = n0 + c;
         float v[32], g[32];
-        acc.get(c, v);
+        pf_ld32(tacc + c, v);
         if (!live) continue;
         pf_load32(P.gamma + n, g);
         if (P.rho) {
@@ -253,7 +214,7 @@ __device__ __forceinline__ void pf_out_fc(const PfParams& P, const PfAcc& acc, i
         }
         pf_store32(P.xq + (long long)pair * P.rows + n, g);
     }
-    if (live) P.ssq[(long long)((n0 + c0) >> 6) * P.pair_cap + pair] = ss;
+    if (live) P.ssq[(long long)((n0 + c0) >> 7) * P.pair_cap + pair] = ss;
 }
 
 // GEMM 2 output stage of one pair: 32 elements of a head from c and their partners half a head on.
@@ -275,24 +236,26 @@ __device__ __forceinline__ PfPair pf_pair(const PfParams& P, int pair, bool live
     }
     return p;
 }
-__device__ __forceinline__ void pf_out_kv(const PfParams& P, const PfAcc& acc, const PfPair& pp, int c, int n0, int pair) {
+__device__ __forceinline__ void pf_out_kv(const PfParams& P, uint32_t tacc, const PfPair& pp, int c, int n0, int pair) {
     const int half = P.dh >> 1, g = n0 + c;                 // row of the stacked [K ; V] projection
     const bool isK = g < P.kvw;
     const int head = (isK ? g : g - P.kvw) / P.dh, e0 = g % P.dh;
     float lo[32], hi[32], x[32];
-    acc.get(c, lo);
-    acc.get(c + half, hi);
+    pf_ld32(tacc + c, lo);
+    pf_ld32(tacc + c + half, hi);
     if (pp.crow < 0) return;
     bf16* dst = (isK ? P.Kc : P.Vc) + ((pp.slot_base + head) * P.max_len + pp.crow) * P.dh + e0;
-#pragma unroll
-    for (int i = 0; i < 32; ++i) { lo[i] *= pp.sc; hi[i] *= pp.sc; }
+    // (one rounding for scale and bias, as in the builds of 16 pairs per pass)
     if (P.bias) {
         pf_load32(P.bias + g, x);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) lo[i] += x[i];
+        for (int i = 0; i < 32; ++i) lo[i] = fmaf(lo[i], pp.sc, x[i]);
         pf_load32(P.bias + g + half, x);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) hi[i] += x[i];
+        for (int i = 0; i < 32; ++i) hi[i] = fmaf(hi[i], pp.sc, x[i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) { lo[i] *= pp.sc; hi[i] *= pp.sc; }
     }
     if (isK) {
         const float4* tab = (const float4*)(P.rope + (long long)pair * half + e0);
@@ -300,29 +263,16 @@ __device__ __forceinline__ void pf_out_kv(const PfParams& P, const PfAcc& acc, c
         for (int q = 0; q < 16; ++q) {
             const float4 t = __ldg(tab + q);
             const float l0 = lo[2 * q], l1 = lo[2 * q + 1], u0 = hi[2 * q], u1 = hi[2 * q + 1];
-            lo[2 * q] = l0 * t.x - u0 * t.y;
-            hi[2 * q] = u0 * t.x + l0 * t.y;
-            lo[2 * q + 1] = l1 * t.z - u1 * t.w;
-            hi[2 * q + 1] = u1 * t.z + l1 * t.w;
+            // (written out, so that every build of the code rounds the same product)
+            lo[2 * q] = fmaf(l0, t.x, -__fmul_rn(u0, t.y));
+            hi[2 * q] = fmaf(u0, t.x, __fmul_rn(l0, t.y));
+            lo[2 * q + 1] = fmaf(l1, t.z, -__fmul_rn(u1, t.w));
+            hi[2 * q + 1] = fmaf(u1, t.z, __fmul_rn(l1, t.w));
         }
     }
     pf_store32(dst, lo);
     pf_store32(dst + half, hi);
 }
-// First column of unit q (64 columns) of a tile: GEMM 1 takes them in order, GEMM 2 as 32 columns and their partners.
-template <int EPI>
-__device__ __forceinline__ int pf_unit_col(const PfParams& P, int q) {
-    if (EPI == 0 || P.dh == 64) return 64 * q;
-    return 128 * (q >> 1) + 32 * (q & 1);
-}
-// does 32-column chunk c of a tile belong to a unit that contributor `me` of `split` finishes?
-template <int EPI>
-__device__ __forceinline__ bool pf_mine(const PfParams& P, int c, int split, int me) {
-    const int q = (EPI == 0 || P.dh == 64) ? c >> 6 : 2 * (c >> 7) + ((c >> 5) & 1);
-    return q % split == me;
-}
-#define PF_DEPART 65536
-
 template <int EPI, int BN>   // EPI 0: fusion FC, 1: K and V
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1) prefill_tc_kernel(const __grid_constant__ PfParams P) {
     constexpr int B_BYTES = (BN / 2) * PF_BK * 2;
@@ -336,7 +286,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1) prefi
     uint32_t rank;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     const int cluster = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
-    const int nkb_all = P.K / PF_BK, units = P.m_tiles * P.n_tiles * P.split;
+    const int nkb = P.K / PF_BK, units = P.m_tiles * P.n_tiles;
     if (tid == 0) {
         for (int i = 0; i < (int)PF_STAGES; ++i) {
             pf_mbar_init(pf_saddr(&ctl->full[i]), 1);
@@ -366,10 +316,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1) prefi
             unsigned it = 0;
             bool ok = true;
             for (int w = cluster; w < units && ok; w += n_clusters) {
-                const int t = w / P.split, part = w - t * P.split;
-                const int kb_first = nkb_all * part / P.split, kb_end = nkb_all * (part + 1) / P.split;
-                const int pair0 = (t / P.n_tiles) * PF_TM + (int)rank * 128, row0 = (t % P.n_tiles) * BN + (int)rank * (BN / 2);
-                for (int kb = kb_first; kb < kb_end; ++kb, ++it) {
+                const int pair0 = (w / P.n_tiles) * PF_TM + (int)rank * 128, row0 = (w % P.n_tiles) * BN + (int)rank * (BN / 2);
+                for (int kb = 0; kb < nkb; ++kb, ++it) {
                     const unsigned slot = it % PF_STAGES, round = it / PF_STAGES;
                     ok = round == 0 || pf_wait(pf_saddr(&ctl->empty[slot]), (round - 1) & 1u, ctl, P.wait_cycles, P.error_flag);
                     if (!ok) break;
@@ -392,8 +340,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1) prefi
             unsigned it = 0, seg = 0;
             bool ok = true;
             for (int w = cluster; w < units && ok; w += n_clusters, ++seg) {
-                const int part = w % P.split;
-                const int nkb = nkb_all * (part + 1) / P.split - nkb_all * part / P.split;
                 const unsigned acc = seg & 1u, use = seg >> 1;
                 ok = use == 0 || pf_wait(pf_saddr(&ctl->tempty[acc]), (use - 1) & 1u, ctl, P.wait_cycles, P.error_flag);
                 pf_fence_after();
@@ -418,69 +364,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1) prefi
         unsigned seg = 0;
         for (int w = cluster; w < units; w += n_clusters, ++seg) {
             const unsigned acc = seg & 1u, use = seg >> 1;
-            const int t = w / P.split, part = w - t * P.split;
-            const int r_loc = quarter * 32 + lane;
-            const int pair = (t / P.n_tiles) * PF_TM + (int)rank * 128 + r_loc, n0 = (t % P.n_tiles) * BN;
+            const int pair = (w / P.n_tiles) * PF_TM + (int)rank * 128 + quarter * 32 + lane, n0 = (w % P.n_tiles) * BN;
             const bool live = pair < P.n_pairs;
             PfPair pp;
             if (EPI == 1) pp = pf_pair(P, pair, live);
             bool ok = true;
             if (lane == 0) ok = pf_wait(pf_saddr(&ctl->tfull[acc]), use & 1u, ctl, P.wait_cycles, P.error_flag);
             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-            if (!ok && P.split == 1) break;
+            if (!ok) break;
             pf_fence_after();
-            PfAcc a;
-            a.tacc = ctl->tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN;
-            a.split = P.split; a.me = part;
-            a.part_stride = 2ll * (BN / 4) * 128;
-            a.part = (const float4*)P.partial + (long long)t * P.split * a.part_stride + (long long)rank * (BN / 4) * 128 + r_loc;
-            int* ctr = P.unit_ctr + 2 * t + rank;
-            if (P.split > 1) {
-                if (ok) {
-                    float4* mine = (float4*)a.part + part * a.part_stride;
+            const uint32_t tacc = ctl->tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN;
+            if (EPI == 0) {
 #pragma unroll 1
-                    for (int c = 0; c < BN; c += 32) {
-                        if (pf_mine<EPI>(P, c, P.split, part)) continue;
-                        float v[32];
-                        pf_ld32(a.tacc + c, v);
-#pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            __stcg(mine + ((c >> 2) + q) * 128, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
-                    }
-                }
-                asm volatile("bar.sync 1, 128;" ::: "memory");
-                if (tid == 64) {
-                    // (after a give-up the CTA still arrives and leaves, so that the counter is zero for the next call)
-                    atom_add_acq_rel(ctr, 1);
-                    const long long t0 = clock64();
-                    unsigned n = 0;
-                    while (((*(volatile int*)ctr) & (PF_DEPART - 1)) < P.split) {
-                        if ((++n & 63u) == 0u) {
-                            if (*(volatile int*)&ctl->abort_flag) break;
-                            if (*(volatile int*)P.error_flag != 0 || clock64() - t0 > P.wait_cycles) {
-                                atomicCAS(P.error_flag, 0, 31);
-                                *(volatile int*)&ctl->abort_flag = 1;
-                                break;
-                            }
-                        }
-                    }
-                    __threadfence();
-                }
-                asm volatile("bar.sync 1, 128;" ::: "memory");
-                if (*(volatile int*)&ctl->abort_flag) ok = false;
-            }
-            if (ok) {
+                for (int c = 0; c < BN && n0 + c < P.rows; c += 128) pf_out_fc(P, tacc, c, n0, pair, live);
+            } else {
+                // 32 elements of a head and their partners, half a head on
 #pragma unroll 1
-                for (int q = P.split > 1 ? part : 0; q < BN / 64; q += P.split) {
-                    const int c = pf_unit_col<EPI>(P, q);
+                for (int q = 0; q < BN / 64; ++q) {
+                    const int c = P.dh == 64 ? 64 * q : 128 * (q >> 1) + 32 * (q & 1);
                     if (n0 + c >= P.rows) break;                    // (uniform)
-                    if (EPI == 0) pf_out_fc(P, a, c, n0, pair, live);
-                    else pf_out_kv(P, a, pp, c, n0, pair);
+                    pf_out_kv(P, tacc, pp, c, n0, pair);
                 }
-            }
-            if (P.split > 1) {
-                asm volatile("bar.sync 1, 128;" ::: "memory");
-                if (tid == 64 && atom_add_acq_rel(ctr, PF_DEPART) / PF_DEPART == P.split - 1) *ctr = 0;
             }
             pf_fence_before();
             __syncwarp();
@@ -544,44 +448,26 @@ cudaError_t pf_launch_t(PfParams& P, int clusters, cudaStream_t st) {
         if (dev >= 0 && dev < HIVIS_MAX_DEVICES) attr_set[dev] = true;
     }
     P.n_tiles = (P.rows + BN - 1) / BN;
-    const int units = P.m_tiles * P.n_tiles * P.split;
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(2u * (unsigned)(units < clusters ? units : clusters));
-    cfg.blockDim = dim3(PF_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    // contributors of a tile wait for one another: all of them have to be on the GPU
-    cudaLaunchAttribute coop;
-    coop.id = cudaLaunchAttributeCooperative;
-    coop.val.cooperative = 1;
-    cfg.attrs = &coop;
-    cfg.numAttrs = P.split > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<EPI, BN>, (const PfParams)P);
+    const int units = P.m_tiles * P.n_tiles;
+    prefill_tc_kernel<EPI, BN><<<2u * (unsigned)(units < clusters ? units : clusters), PF_THREADS, smem, st>>>(P);
+    return cudaGetLastError();
 }
 
-// Tile width and clusters per tile.  Time of the busiest cluster in units of 10 ns: its k-blocks (0.45 us each at 256 weight
-// rows, 0.33 at 128; below that an MMA takes as long whatever its width), and what publishing and adding the parts cost
-// (3 us, and 0.4 per part).  117 / 500 pairs (d 4096 / 2560): 92 / 69 us at 256, 90 / 62 at 128; 600 and 2048 pairs
-// (d 4096 / 3584): 123 and 130 us at 256, 174 and 193 at 128; K/V split over the idle clusters: 98 -> 92 (117 pairs), 136 ->
-// 130 (2048).  GEMM 1 is never split: u is rounded to bf16 for GEMM 2, and parts of its long sums added in fp32 instead of
-// in the tensor core's accumulator move one element in forty to the other side of a rounding.
+// Tile width, by the time of the busiest cluster in units of 10 ns a k-block (0.45 us at 256 weight rows, 0.33 at 128; below
+// that an MMA takes as long whatever its width).  117 / 500 pairs (d 4096 / 2560): 92 / 69 us at 256, 90 / 62 at 128; 600 and
+// 2048 pairs (d 4096 / 3584): 123 and 130 us at 256, 174 and 193 at 128.  A tile is never split over clusters: u and the cached
+// rows are rounded to bf16, and parts of their long sums added in fp32 instead of in the tensor core's accumulator move one
+// element in forty to the other side of a rounding.
 template <int EPI>
 cudaError_t pf_launch(PfParams& P, const void* W, int num_sms, cudaStream_t st) {
     const int clusters = num_sms / 2 > 0 ? num_sms / 2 : 1;
     P.m_tiles = (P.n_pairs + PF_TM - 1) / PF_TM;
-    const int nkb = P.K / PF_BK;
     int bn = 256;
     long long best = -1;
-    P.split = 1;
     for (int b = 256; b >= 128; b -= 128) {
         const int tiles = P.m_tiles * ((P.rows + b - 1) / b);
-        for (int s = 1; s <= (EPI == 0 ? 1 : 8); ++s) {
-            if (s > 1 && (tiles * s > clusters || nkb < 4 * s)) break;
-            const long long waves = (tiles * s + clusters - 1) / clusters;
-            const long long cost = waves * ((nkb + s - 1) / s) * (b == 256 ? 45 : 33) + (s > 1 ? 300 + 40 * s : 0);
-            if (best < 0 || cost < best) { best = cost; bn = b; P.split = s; }
-        }
+        const long long cost = (long long)((tiles + clusters - 1) / clusters) * (b == 256 ? 45 : 33);
+        if (best < 0 || cost < best) { best = cost; bn = b; }
     }
     cudaError_t e = pf_encode(P.map_w, W, P.rows, P.K, bn / 2);
     if (e != cudaSuccess) return e;
@@ -607,7 +493,6 @@ cudaError_t launch_prefill_tc(const PrefillTcArgs& a, cudaStream_t st) {
     if ((e = pf_encode(P.map_x1, a.xe, a.n_pairs, d, 128)) != cudaSuccess) return e;
     P.rows = d; P.K = 2 * d; P.kb_split = d / PF_BK; P.n_pairs = a.n_pairs;
     P.wait_cycles = a.wait_cycles; P.error_flag = a.error_flag;
-    P.partial = a.partial; P.unit_ctr = a.unit_ctr;
     P.rho = a.rho0; P.rho_h = a.rho0_h; P.gamma = a.norm1; P.xq = a.xq; P.ssq = a.ssq; P.pair_cap = a.pair_cap;
     if ((e = pf_launch<0>(P, a.fc, a.num_sms, st)) != cudaSuccess) return e;
     // ---- GEMM 2: K, V
@@ -617,12 +502,8 @@ cudaError_t launch_prefill_tc(const PrefillTcArgs& a, cudaStream_t st) {
     memcpy(Q.map_x1, Q.map_x0, 128);
     Q.rows = 2 * a.kvw; Q.K = d; Q.kb_split = d / PF_BK; Q.n_pairs = a.n_pairs;
     Q.wait_cycles = a.wait_cycles; Q.error_flag = a.error_flag;
-    Q.partial = a.partial; Q.unit_ctr = a.unit_ctr;
-    Q.ssq_in = a.ssq; Q.ssq_tiles = (d + 63) / 64; Q.pair_cap = a.pair_cap; Q.d = d; Q.eps = a.eps;
+    Q.ssq_in = a.ssq; Q.ssq_tiles = (d + 127) / 128; Q.pair_cap = a.pair_cap; Q.d = d; Q.eps = a.eps;
     Q.bias = a.bkv; Q.kvw = a.kvw; Q.Hkv = a.Hkv; Q.dh = a.dh; Q.max_len = a.max_len;
     Q.slot_of = a.slot_of; Q.row_of = a.row_of; Q.rope = a.rope; Q.Kc = a.Kc; Q.Vc = a.Vc;
     return pf_launch<1>(Q, a.wkv, a.num_sms, st);
 }
-
-// [units][2 CTAs][columns][128 pairs]: as many units as there are clusters, at 256 columns
-size_t prefill_tc_partial_floats(int num_sms) { return (size_t)(num_sms / 2 > 0 ? num_sms / 2 : 1) * 2 * 256 * 128; }

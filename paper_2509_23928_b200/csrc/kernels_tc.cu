@@ -146,18 +146,9 @@ cudaError_t tc_build_maps(TcMaps* maps, const ChainPhase* ph, int d, int qw, int
     return encode_map(maps->m[TCM_V], Vc, cache_rows, dh, 32, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
 }
 
-// one map for a matrix other than the ones above: weight tiles of 128 rows, or operand rows
-cudaError_t tc_encode_weight(unsigned char* map, const void* W, long long rows, long long cols) {
-    return encode_map(map, W, rows, cols, TC_TM, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
-}
-cudaError_t tc_encode_operand(unsigned char* map, const void* x, long long rows, long long cols, int op_rows) {
-    return encode_map(map, x, rows, cols, op_rows, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
-}
-
 template <int DH, int GQ>
 static cudaError_t tc_launch_greedy(const TcMaps& maps, const TcArgs& a, int grid, cudaStream_t st) {
-    // (a batch whose operands carry no remainders takes the two-group kernel, however small)
-    switch (a.lo == 0 && a.B <= 16 ? 2 : tc_groups(a.B)) {
+    switch (tc_groups(a.B)) {
         case 1: return tc_launch_t<DH, GQ, false, 1>(maps, a, grid, st);
         case 2: return tc_launch_t<DH, GQ, false, 2>(maps, a, grid, st);
         default: return tc_launch_t<DH, GQ, false, 4>(maps, a, grid, st);

@@ -278,10 +278,10 @@ def test_tensor_core_prefill_tile_edges(name, pairs):
                                           ("wide_mha_b16_ragged", False)])
 @pytest.mark.parametrize("pairs", [1, 2, 16, 17, 32, 33, 64])
 def test_small_prefix_builds_in_the_chain_kernel(name, project, pairs):
-    """1..64 pairs as columns of the chain kernel (one, two and four column groups, full and partly filled) against the
-    kernels of 16 pairs per pass, after a larger call has left its rows in every buffer; then the draft that consumes the
-    pending pairs.  Both paths round the same operand and the stored
-    rows to bf16: one unit in the last place (2^-8 of the value) apart."""
+    """1..64 pairs, the sizes of a refresh (a single pass up to 16, the two GEMMs from 17), against the kernels of 16 pairs
+    per pass, after a larger call has left its rows in every buffer; then the draft that consumes the pending pairs, in the
+    chain kernels and in the per-phase ones.  Both paths round the same operand and the stored rows to bf16: one unit in the
+    last place (2^-8 of the value) apart."""
     import torch
     wl = hi.scaled(hi.workload(name), batch=2, text_len=None, text_len_range=(1, 2))
     extra = {"resid_proj": hi.make_weights(wl.dims, 77)["fc"][:, :wl.dims.d].copy()} if project else None
