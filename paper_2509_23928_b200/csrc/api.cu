@@ -467,16 +467,6 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
 // residual rows in the context dtype -> fp32 rho rows (projected by resid_proj when present)
 static int prepare_rho(hivis_ctx* c, const void* resid, int R, cudaStream_t st) {
     const int d = c->cfg.d;
-    if (c->resid_proj && c->dtype == HIVIS_BF16) {
-        // the rows are bf16 as they are: one pass over the projection for all of them on the tensor cores (fp32 sums of
-        // exact products, as on the FMA path, which reads the matrix once per row: 24 us for 4 rows of 4096)
-        LinArgs a;
-        memset(&a, 0, sizeof(a));
-        a.W = c->resid_proj; a.N = d; a.K = d; a.B = R; a.ldb = c->rows_cap;
-        a.xin_h = (const bf16*)resid; a.out = c->rho;
-        CKL(c, launch_gemm_mma(PRO_PLAIN, EPI_QKV, a, st));
-        return HIVIS_OK;
-    }
     float* dst = c->resid_proj ? c->rho_raw : c->rho;
     CKL(c, launch_convert_rows(c->dtype, resid, dst, (long long)R * d, st));
     if (c->resid_proj) {

@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(256) gemm_mma_kernel(const LinArgs a) {
             if (tid < a.B) {
                 float tot = 0.f;
                 for (int i = 0; i < a.ssq_tiles; ++i) tot += __ldcg(a.ssq_in + (long long)i * a.ldb + tid);
-                if (a.ssq_tiles > 0) s = rsqrtf(tot / (float)a.K + a.eps);       // (0: a plain product)
+                s = rsqrtf(tot / (float)a.K + a.eps);
             }
             s_scale[tid] = s;
         }

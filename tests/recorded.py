@@ -79,10 +79,21 @@ def prefix_rows(shape, bias, project):
     return out
 
 
+def projected_rows(shape):
+    """What a projected residual row adds to u, at every step of a chain of one sequence (and the chain's logits)."""
+    r = Run(shape, 12, project=True)
+    r.prefill([1])
+    ids, logits = r.dr.draft(1, 5, r.resid, want_logits=True)
+    u = r.dr.tap("u", 1)
+    r.dr.status()
+    return digest(u, ids, logits)
+
+
 RECORDS = {
     "prefix_wide128": lambda: prefix_rows("wide128", False, False),
     "prefix_wide128_bias": lambda: prefix_rows("wide128", True, False),
     "prefix_wide64_bias": lambda: prefix_rows("wide64", True, False),
+    "projected_rows": lambda: projected_rows("wide128"),
 }
 
 
