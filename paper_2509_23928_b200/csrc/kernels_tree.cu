@@ -102,50 +102,48 @@ cudaError_t launch_tree_operands_tc(int nb, int rows, int d, int lo_rows, int sl
 }
 
 // ------------------------------------------------------------------------------------------ tree attention
-// One CTA of eight warps per (query head, node).  The node attends to the prefix rows [0, P), to the rows of its
-// ancestors (the root position first) and to itself.  Its own K (rotated) and V are made here, rounded to what the cache
-// will hold, and the first head of a KV group writes them to the cache: nobody else reads that row in this level (a
-// launch of its own for the rows took 15 us).  Blocks of 32 cached rows are dealt to the warps in turn.  Scores: a lane takes
-// one row of the block and the whole dot product with the query (in shared memory), so no shuffle is needed; the block's
-// probabilities then go through an online softmax, and for the weighted sum of the V rows a lane owns DH/32 output
-// elements and every row's probability is broadcast from its lane, eight rows' loads in flight.  The warps' (max, sum,
-// accumulator) and the node's own row are merged at the end.
-#define TREE_ATT_WARPS 8
+// One CTA of four warps per (query head, node).  The node attends to the prefix rows [0, P), to the rows of its ancestors
+// (the root position first) and to its own row: `level` + 1 tree rows.  Its own K (rotated) and V are made here, in the form
+// the cache holds, and read from shared memory in their place at the end of the rows; the first head of a KV group writes them
+// to the cache: nobody else reads that row in this level (a launch of its own for the rows took 15 us).  Blocks of 32 rows are
+// dealt to the warps in turn.  Scores: a lane takes one row of the block and the whole dot product with the query (in shared
+// memory), so no shuffle is needed; the block's probabilities then go through an online softmax, and for the weighted sum
+// of the V rows a lane owns DH/32 output elements and every row's probability is broadcast from its lane, eight rows' loads
+// in flight.  The four warps' (max, sum, accumulator) are merged at the end.  The order of all sums belongs to the result:
+// a tree's list of nodes is decided by differences that another order would move.
+#define TREE_ATT_WARPS 4
 template <typename WT, int DH>
-__device__ __forceinline__ float tree_row_dot(const void* Kc, long long o, const float* q) {
+__device__ __forceinline__ float tree_row_dot(const WT* k, const float* q) {
     float sc = 0.f;
     if constexpr (sizeof(WT) == 2) {
-        const uint4* kp = (const uint4*)((const bf16*)Kc + o);
+        const uint4* kp = (const uint4*)k;
 #pragma unroll
         for (int c = 0; c < DH / 8; ++c) {
-            const uint4 w = __ldg(kp + c);
+            const uint4 w = kp[c];
             sc = fmaf(q[8 * c + 0], bf16_lo(w.x), sc); sc = fmaf(q[8 * c + 1], bf16_hi(w.x), sc);
             sc = fmaf(q[8 * c + 2], bf16_lo(w.y), sc); sc = fmaf(q[8 * c + 3], bf16_hi(w.y), sc);
             sc = fmaf(q[8 * c + 4], bf16_lo(w.z), sc); sc = fmaf(q[8 * c + 5], bf16_hi(w.z), sc);
             sc = fmaf(q[8 * c + 6], bf16_lo(w.w), sc); sc = fmaf(q[8 * c + 7], bf16_hi(w.w), sc);
         }
     } else {
-        const float4* kp = (const float4*)((const float*)Kc + o);
+        const float4* kp = (const float4*)k;
 #pragma unroll
         for (int c = 0; c < DH / 4; ++c) {
-            const float4 w = __ldg(kp + c);
+            const float4 w = kp[c];
             sc = fmaf(q[4 * c + 0], w.x, sc); sc = fmaf(q[4 * c + 1], w.y, sc);
             sc = fmaf(q[4 * c + 2], w.z, sc); sc = fmaf(q[4 * c + 3], w.w, sc);
         }
     }
     return sc;
 }
-template <typename WT>
-__device__ __forceinline__ float tree_as_cached(float x) {
-    return sizeof(WT) == 2 ? __bfloat162float(__float2bfloat16_rn(x)) : x;
-}
 template <typename WT, int DH>
 __global__ void __launch_bounds__(TREE_ATT_WARPS * 32) tree_attn_kernel(const float* qkv, int ld, int Hq, int Hkv, int max_len, int slot,
                                                         int level, TreeBufs T, const double* inv_freq, float scale,
                                                         void* Kc, void* Vc, float* attn, bf16* attn_h, int lo_rows) {
     constexpr int EPL = DH / 32, NT = TREE_ATT_WARPS * 32;
-    __shared__ float s_m[TREE_ATT_WARPS + 1], s_l[TREE_ATT_WARPS + 1], s_acc[TREE_ATT_WARPS + 1][DH];
-    __shared__ __align__(16) float s_q[DH], s_k[DH];
+    __shared__ float s_m[TREE_ATT_WARPS], s_l[TREE_ATT_WARPS], s_acc[TREE_ATT_WARPS][DH];
+    __shared__ __align__(16) float s_q[DH];
+    __shared__ __align__(16) WT s_k[DH], s_v[DH];
     __shared__ float2 s_cs[DH / 2];
     const int h = blockIdx.x, j = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int P = *T.P, pos = P + level, G = Hq / Hkv, kvh = h / G, half = DH / 2;
@@ -167,7 +165,7 @@ __global__ void __launch_bounds__(TREE_ATT_WARPS * 32) tree_attn_kernel(const fl
         const float* src = what == 0 ? qh : what == 1 ? kh : vh;
         const float x = src[i];
         if (what == 2) {
-            s_acc[TREE_ATT_WARPS][i] = tree_as_cached<WT>(x);
+            store_from_float<WT>(s_v, i, x);
             if (writer) store_from_float<WT>(Vc, own + i, x);
             continue;
         }
@@ -177,20 +175,12 @@ __global__ void __launch_bounds__(TREE_ATT_WARPS * 32) tree_attn_kernel(const fl
         if (what == 0) {
             s_q[i] = r * scale;
         } else {
-            s_k[i] = tree_as_cached<WT>(r);
+            store_from_float<WT>(s_k, i, r);
             if (writer) store_from_float<WT>(Kc, own + i, r);
         }
     }
     __syncthreads();
-    if (warp == TREE_ATT_WARPS - 1) {
-        float sc = 0.f;
-#pragma unroll
-        for (int e = 0; e < EPL; ++e) sc = fmaf(s_q[e * 32 + lane], s_k[e * 32 + lane], sc);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, off);
-        if (lane == 0) { s_m[TREE_ATT_WARPS] = sc; s_l[TREE_ATT_WARPS] = 1.f; }
-    }
-    const int nrows = P + level;                                     // cached rows: the prefix and the ancestors
+    const int nrows = P + level + 1;                                 // the prefix, the ancestors, the node itself
     float m = -INFINITY, l = 0.f, acc[EPL];
 #pragma unroll
     for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
@@ -198,9 +188,9 @@ __global__ void __launch_bounds__(TREE_ATT_WARPS * 32) tree_attn_kernel(const fl
         const int r = r0 + lane;
         const bool ok = r < nrows;
         int row = ok ? r : r0;
-        if (ok && r >= P) row = P + T.fr_anc[j * TREE_MAX_DEPTH + (r - P)];
+        if (ok && r >= P) row = r - P < level ? P + T.fr_anc[j * TREE_MAX_DEPTH + (r - P)] : -1;     // -1: the node's own row
         row = __shfl_sync(0xffffffffu, row, ok ? lane : 0);          // lanes beyond the rows read the block's first
-        const float sc = ok ? tree_row_dot<WT, DH>(Kc, (base + row) * DH, s_q) : -INFINITY;
+        const float sc = ok ? tree_row_dot<WT, DH>(row < 0 ? s_k : (const WT*)Kc + (base + row) * DH, s_q) : -INFINITY;
         float bm = sc;
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, off));
@@ -220,16 +210,16 @@ __global__ void __launch_bounds__(TREE_ATT_WARPS * 32) tree_attn_kernel(const fl
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
                 const int rowj = __shfl_sync(0xffffffffu, row, t0 + t);
-                const long long o = (base + rowj) * DH + lane * EPL;
+                const WT* vp = (rowj < 0 ? s_v : (const WT*)Vc + (base + rowj) * DH) + lane * EPL;
                 if constexpr (sizeof(WT) == 2 && EPL == 4) {
-                    const uint2 w = __ldg((const uint2*)((const bf16*)Vc + o));
+                    const uint2 w = *(const uint2*)vp;
                     vf[t][0] = bf16_lo(w.x); vf[t][1] = bf16_hi(w.x); vf[t][2] = bf16_lo(w.y); vf[t][3] = bf16_hi(w.y);
                 } else if constexpr (sizeof(WT) == 2 && EPL == 2) {
-                    const unsigned w = __ldg((const unsigned*)((const bf16*)Vc + o));
+                    const unsigned w = *(const unsigned*)vp;
                     vf[t][0] = bf16_lo(w); vf[t][1] = bf16_hi(w);
                 } else {
 #pragma unroll
-                    for (int e = 0; e < EPL; ++e) vf[t][e] = __ldg((const float*)Vc + o + e);
+                    for (int e = 0; e < EPL; ++e) vf[t][e] = load_as_float<WT>(vp, e);
                 }
             }
 #pragma unroll
@@ -249,12 +239,12 @@ __global__ void __launch_bounds__(TREE_ATT_WARPS * 32) tree_attn_kernel(const fl
     if (warp == 0) {
         float M = -INFINITY;
 #pragma unroll
-        for (int w = 0; w <= TREE_ATT_WARPS; ++w) M = fmaxf(M, s_m[w]);
+        for (int w = 0; w < TREE_ATT_WARPS; ++w) M = fmaxf(M, s_m[w]);
         float L = 0.f, A[EPL];
 #pragma unroll
         for (int e = 0; e < EPL; ++e) A[e] = 0.f;
 #pragma unroll
-        for (int w = 0; w <= TREE_ATT_WARPS; ++w) {
+        for (int w = 0; w < TREE_ATT_WARPS; ++w) {
             const float f = s_l[w] > 0.f ? expf(s_m[w] - M) : 0.f;   // a warp without rows contributes nothing
             L += s_l[w] * f;
 #pragma unroll

@@ -19,8 +19,9 @@ def dims(d, hq, hkv, dh, ffn, vocab):
                            dtype="bf16")
 
 
-# long sums on few rows, with heads of 128 and of 64
-SHAPES = {"wide128": dims(2560, 20, 4, 128, 1024, 2048), "wide64": dims(2048, 12, 2, 64, 1024, 2048)}
+# long sums on few rows, with heads of 128 and of 64; and one whose sums are too short to be split evenly over the chip
+SHAPES = {"wide128": dims(2560, 20, 4, 128, 1024, 2048), "wide64": dims(2048, 12, 2, 64, 1024, 2048),
+          "narrow": dims(256, 4, 2, 64, 512, 2048)}
 
 
 class Run:
@@ -89,11 +90,23 @@ def projected_rows(shape):
     return digest(u, ids, logits)
 
 
+def trees(shape, project):
+    r = Run(shape, 13, project=project)
+    out = {}
+    for n, topk, depth, keep in ((5, 4, 3, 20), (33, 10, 6, 60), (150, 12, 5, 80), (300, 2, 8, 17)):
+        r.prefill([n])
+        toks, parents, scores, count = r.dr.draft_tree(0, topk, depth, keep, r.resid)
+        out[f"{n} rows, top {topk}, depth {depth}, {keep} kept"] = digest(toks, parents, scores, count[:1])
+    r.dr.status()
+    return out
+
+
 RECORDS = {
     "prefix_wide128": lambda: prefix_rows("wide128", False, False),
     "prefix_wide128_bias": lambda: prefix_rows("wide128", True, False),
     "prefix_wide64_bias": lambda: prefix_rows("wide64", True, False),
     "projected_rows": lambda: projected_rows("wide128"),
+    "tree_narrow": lambda: trees("narrow", False),
 }
 
 
