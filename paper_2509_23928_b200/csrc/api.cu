@@ -647,6 +647,7 @@ static void fill_tc_args(hivis_ctx* c, TcArgs* out, int B, int k, int lo, const 
     a.wait_cycles = c->wait_cycles; a.error_flag = c->error_flag; a.id_flag = c->id_flag;
     a.l2_keep = c->opt_l2_keep;
     a.phase_t = nullptr;
+    a.whole_ctas = (1 << PH_COUNT) - 1;
     a.seq_first = 0; a.seq_last = 7;
 }
 
@@ -1026,6 +1027,7 @@ int hivis_draft_tree(hivis_ctx* c, int slot, int topk, int depth, int keep, cons
             TcArgs a;
             fill_tc_args(c, &a, nb, 1, lo, rho, 1, nullptr, c->tree_logits);
             a.rho_h = raw_rho ? (const bf16*)resid + (long long)row * d : nullptr;
+            a.whole_ctas = 0;                                        // the order of the sums decides which of two near nodes is kept
             a.seq_first = 1; a.seq_last = 2;                         // fusion FC, QKV (the operands are gathered already)
             a.bar_base = c->bar_count_host - G + (c->debug_skew ? (1ull << 40) : 0ull);
             c->debug_skew = false;

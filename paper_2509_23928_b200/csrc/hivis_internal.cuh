@@ -199,6 +199,7 @@ struct TcArgs {
     // The grid barriers of a step are numbered 0 gather, 1 FC, 2 QKV, 3 attention, 4 O, 5 gate/up, 6 down, 7 LM head.
     // A launch runs the part [seq_first, seq_last] of every step (0..7: the whole step); what lies outside does no work
     // and arrives nowhere, and bar_base is set as if the barriers before seq_first had been completed already.
+    int whole_ctas;            // bit p: the tiles of phase p get whole CTAs where their number allows it
     int seq_first, seq_last;
 };
 // fills `maps` for the given buffers; returns cudaSuccess or an error (driver entry point missing, bad shape)

@@ -329,7 +329,9 @@ struct PhaseShape {
 // where that keeps TC_ALIGN_PCT of the CTAs busy: no CTA has two tiles to publish, nobody finishes two in a row, and the
 // contributors of a tile are done together.  With contiguous ranges the slowest CTA of the fusion FC had its last
 // accumulator 9 us after the median one.  Batch 16 (d 4096, 704 rows) 1180 -> 1152 us per round, d 2560 batch 5 513 -> 488,
-// 64 sequences 1726 -> 1631, a tree 1351 -> 1303; the 14 % of idle SMs cost nothing, HBM is the slower side.
+// 64 sequences 1726 -> 1631; the 14 % of idle SMs cost nothing, HBM is the slower side.  Not for the levels of a draft tree
+// (TcArgs::whole_ctas): another split adds the sums in another order, and a tree's list of nodes hangs on differences
+// smaller than that.
 #define TC_ALIGN_PCT 80
 // does this launch run the part of a step that arrives on barrier `seq`?
 __device__ __forceinline__ bool seq_on(const TcArgs& a, int seq) { return seq >= a.seq_first && seq <= a.seq_last; }
@@ -339,7 +341,7 @@ __device__ __forceinline__ PhaseShape phase_shape(const TcArgs& a, int p) {
     s.ntiles = (a.ph[p].N + TC_TM - 1) / TC_TM;
     s.W = seq_on(a, phase_seq(p)) ? (long long)s.nkb * s.ntiles : 0;      // a phase outside the launch's part has no work
     const int G = gridDim.x, per = G / s.ntiles;
-    s.split = s.W > 0 && per >= 2 && s.nkb >= 2 * per && per * s.ntiles * 100 >= TC_ALIGN_PCT * G ? per : 0;
+    s.split = ((a.whole_ctas >> p) & 1) && s.W > 0 && per >= 2 && s.nkb >= 2 * per && per * s.ntiles * 100 >= TC_ALIGN_PCT * G ? per : 0;
     return s;
 }
 // first tile-k-block of CTA c (its range ends where that of c + 1 begins)

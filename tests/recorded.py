@@ -107,6 +107,8 @@ RECORDS = {
     "prefix_wide64_bias": lambda: prefix_rows("wide64", True, False),
     "projected_rows": lambda: projected_rows("wide128"),
     "tree_narrow": lambda: trees("narrow", False),
+    "tree_wide128": lambda: trees("wide128", False),
+    "tree_wide64_projected": lambda: trees("wide64", True),
 }
 
 
