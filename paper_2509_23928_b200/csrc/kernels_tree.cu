@@ -171,7 +171,8 @@ __global__ void __launch_bounds__(TREE_ATT_WARPS * 32) tree_attn_kernel(const fl
         }
         const float c = s_cs[f].x, s = s_cs[f].y;
         const float y = src[i < half ? i + half : i - half];
-        const float r = i < half ? x * c - y * s : x * c + y * s;
+        // (written out, so that every build of the code rounds the same product)
+        const float r = i < half ? fmaf(x, c, -__fmul_rn(y, s)) : what == 0 ? fmaf(x, c, __fmul_rn(y, s)) : fmaf(y, s, __fmul_rn(x, c));
         if (what == 0) {
             s_q[i] = r * scale;
         } else {

@@ -96,7 +96,8 @@ def trees(shape, project):
     for n, topk, depth, keep in ((5, 4, 3, 20), (33, 10, 6, 60), (150, 12, 5, 80), (300, 2, 8, 17)):
         r.prefill([n])
         toks, parents, scores, count = r.dr.draft_tree(0, topk, depth, keep, r.resid)
-        out[f"{n} rows, top {topk}, depth {depth}, {keep} kept"] = digest(toks, parents, scores, count[:1])
+        out[f"{n} rows, top {topk}, depth {depth}, {keep} kept"] = digest(toks, parents, scores, count[:1],
+                                                                      *r.dr.read_kv(0, n - 1, 1 + (depth - 1) * topk))
     r.dr.status()
     return out
 
