@@ -88,6 +88,7 @@ __device__ __forceinline__ void pf_arrive_cluster(uint32_t bar) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void pf_cluster_sync() {
+    __syncwarp();               // (aligned instructions)
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // copy into this CTA's shared memory that completes on a barrier of the leader

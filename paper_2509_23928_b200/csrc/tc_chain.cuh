@@ -178,6 +178,7 @@ __device__ __forceinline__ u64 tc_smem_desc(uint32_t addr) {
     return ((u64)hi << 32) | lo;
 }
 __device__ __forceinline__ void tc_ld16_issue(uint32_t taddr, uint32_t (&r)[16]) {
+    __syncwarp();               // one instruction of the whole warp: lanes may come here one by one (a wait's loop, a row beyond N)
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
@@ -228,7 +229,11 @@ __device__ __forceinline__ void phase_stamp(const TcArgs& a, int s, int e, int c
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     a.phase_t[((long long)s * HIVIS_PHASE_EVENTS + e) * G + cta] = t;
 }
-__device__ __forceinline__ void named_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+// (bar.sync is an aligned instruction: the lanes of a warp have to come to it together, whatever they did before)
+__device__ __forceinline__ void named_sync(int id, int n) {
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
 
 // ---- bounded waits -------------------------------------------------------------------------------
 __device__ __forceinline__ bool poisoned(const TcCtl* ctl) { return *(volatile const int*)&ctl->abort_flag != 0; }
@@ -494,8 +499,9 @@ struct TcAttRing {
     __device__ __forceinline__ bool acquire(unsigned r, uint32_t& addr) {
         const unsigned idx = position(r), slot = idx % STAGES, round = idx / STAGES;
         addr = smemA + slot * TC_A_BYTES;
-        if (!wait_issued(ctl, idx, error_flag, 15)) return false;
-        return wait_mbar(saddr(&ctl->full[slot]), round & 1u, ctl, error_flag, 13);
+        // one answer for the warp: a lane that gave up alone would be missing in the shuffles and matrix loads that follow
+        const bool ok = wait_issued(ctl, idx, error_flag, 15) && wait_mbar(saddr(&ctl->full[slot]), round & 1u, ctl, error_flag, 13);
+        return __all_sync(0xffffffffu, ok);
     }
     __device__ __forceinline__ void release(unsigned r) { mbar_arrive(saddr(&ctl->empty[position(r) % STAGES])); }
 };
@@ -1295,6 +1301,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_chain_kernel(const __grid_co
         fence_proxy_async_all();
     }
     if (warp == 1) {
+        __syncwarp();
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(&ctl->tmem_base)),
                      "r"((uint32_t)TcGeo<NG>::TMEM_COLS)
                      : "memory");
@@ -1385,6 +1392,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_chain_kernel(const __grid_co
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
+        __syncwarp();
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(ctl->tmem_base), "r"((uint32_t)TcGeo<NG>::TMEM_COLS)
                      : "memory");
