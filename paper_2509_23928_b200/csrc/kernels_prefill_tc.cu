@@ -78,6 +78,11 @@ __device__ __forceinline__ bool pf_wait(uint32_t bar, uint32_t parity, PfCtl* ct
     }
     return true;
 }
+// after a give-up: time for copies and MMAs in flight
+__device__ __forceinline__ void pf_drain() {
+    const long long t1 = clock64();
+    while (clock64() - t1 < 4000000ll) {}
+}
 // The address of `bar` (own shared memory) in the CTA of the cluster with rank `rank`.
 __device__ __forceinline__ uint32_t pf_mapa(uint32_t bar, uint32_t rank) {
     uint32_t r;
@@ -329,10 +334,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1) prefi
                     pf_tma_2d(smemB + slot * B_BYTES, P.map_w, kb * PF_BK, row0, bar);
                 }
             }
-            if (!ok) {          // after a give-up: copies already issued still land in this CTA's shared memory
-                const long long t1 = clock64();
-                while (clock64() - t1 < 4000000ll) {}
-            }
+            if (!ok) pf_drain();          // copies already issued still land in this CTA's shared memory
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -357,6 +359,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1) prefi
                 }
                 if (ok) pf_commit(pf_saddr(&ctl->tfull[acc]));
             }
+            if (!ok) pf_drain();          // MMAs issued are over before tensor memory is freed
         }
         __syncwarp();
     } else {

@@ -39,9 +39,9 @@
 // fed through 16 more batch columns (rows [16, 32) of every operand buffer) and added in the output stage,
 // which keeps about 16 mantissa bits of the activations for every batch size.
 //
-// Every wait is bounded.  A wait that runs out raises the error flag and poisons the CTA: all roles then
-// run through their remaining schedule without waiting, issuing no further copies or MMAs, so that named
-// barriers still pair up, tensor memory is freed and the kernel returns.
+// Every wait is bounded.  A wait that runs out raises the error flag and poisons the CTA: the producers and the MMA issuer
+// stop where they are (after giving copies in flight time to land), the output warps run through their remaining
+// schedule without waiting, so that named barriers still pair up, tensor memory is freed and the kernel returns.
 #pragma once
 #include <cuda.h>
 
@@ -728,6 +728,10 @@ __device__ void tc_gather(const TcParams& P, TcCtl* ctl, int s, int cta, int G, 
 }
 
 // ---- MMA issuer ----------------------------------------------------------------------------------
+// A wait that is given up ends the role.  Running on through the schedule is not an option here: a barrier tells only the
+// parity of its phase, so the next round's test of a stage that never filled succeeds at once; the commit that followed it
+// handed the stage back, and the weight producer, still polling for it, armed a barrier whose phase was not over - one
+// arrival more than it counts, which the GPU reports as a launch failure.
 template <int NG>
 __device__ void tc_mma_issuer(const TcParams& P, TcCtl* ctl, uint32_t smemA, uint32_t smemB, int cta, int G,
                               unsigned att_items) {
@@ -749,27 +753,24 @@ __device__ void tc_mma_issuer(const TcParams& P, TcCtl* ctl, uint32_t smemA, uin
             while (left > 0) {
                 const int n = left < sh.nkb - kb0 ? left : sh.nkb - kb0;
                 const unsigned acc = seg_cnt & 1u, use = seg_cnt >> 1;
-                if (use > 0) wait_mbar(saddr(&ctl->tempty[acc]), (use - 1) & 1u, ctl, a.error_flag, 4);
+                if (use > 0 && !wait_mbar(saddr(&ctl->tempty[acc]), (use - 1) & 1u, ctl, a.error_flag, 4)) return;
                 tc_fence_after();
                 for (int j = 0; j < n; ++j) {
-                    bool ok = true;
                     if (check) {
-                        ok = wait_issued(ctl, round * STAGES + slot, a.error_flag, 16);
+                        if (!wait_issued(ctl, round * STAGES + slot, a.error_flag, 16)) return;
                         --check;
                     }
-                    ok = ok && wait_mbar(saddr(&ctl->full[slot]), round & 1u, ctl, a.error_flag, 5);
-                    if (ok) {
-                        tc_fence_after();
-                        const u64 ad = tc_smem_desc(smemA + slot * TC_A_BYTES);
-                        const u64 bd = tc_smem_desc(smemB + slot * TcGeo<NG>::B_BYTES);
+                    if (!wait_mbar(saddr(&ctl->full[slot]), round & 1u, ctl, a.error_flag, 5)) return;
+                    tc_fence_after();
+                    const u64 ad = tc_smem_desc(smemA + slot * TC_A_BYTES);
+                    const u64 bd = tc_smem_desc(smemB + slot * TcGeo<NG>::B_BYTES);
 #pragma unroll
-                        for (int kk = 0; kk < TC_BK / 16; ++kk)
-                            tc_mma<NG>(tmem + acc * TcGeo<NG>::TN, ad + (u64)(kk * 2), bd + (u64)(kk * 2), (j > 0 || kk > 0) ? 1u : 0u);
-                        tc_commit(saddr(&ctl->empty[slot]));
-                    }
+                    for (int kk = 0; kk < TC_BK / 16; ++kk)
+                        tc_mma<NG>(tmem + acc * TcGeo<NG>::TN, ad + (u64)(kk * 2), bd + (u64)(kk * 2), (j > 0 || kk > 0) ? 1u : 0u);
+                    tc_commit(saddr(&ctl->empty[slot]));
                     if (++slot == STAGES) { slot = 0; ++round; }
                 }
-                if (!poisoned(ctl)) tc_commit(saddr(&ctl->tfull[acc]));
+                tc_commit(saddr(&ctl->tfull[acc]));
                 ++seg_cnt;
                 left -= n;
                 kb0 = 0;
@@ -1317,7 +1318,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_chain_kernel(const __grid_co
         if (lane == 0) tc_producer_w<DH, GQ, NG>(P, ctl, smemA, cta, G, ai);
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) tc_mma_issuer<NG>(P, ctl, smemA, smemB, cta, G, ai.total);
+        if (lane == 0) {
+            tc_mma_issuer<NG>(P, ctl, smemA, smemB, cta, G, ai.total);
+            if (poisoned(ctl)) drain_after_poison();        // MMAs issued are over before tensor memory is freed
+        }
         __syncwarp();
     } else if (warp == 2) {
         if (lane == 0) tc_producer_x<NG>(P, ctl, smemB, cta, G, ai.total);
@@ -1360,7 +1364,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_chain_kernel(const __grid_co
                 wait_grid(a.bar_counter, a.bar_base + (u64)G * (u64)(s * TC_BARS_PER_STEP + TC_SEQ_ATTN), ctl, a.error_flag, 7);
             if (atid == 0) phase_stamp(a, s, 20, cta, G);
             named_sync(TC_BAR_ATT, TC_ATT_WARPS * 32);
-            if (!poisoned(ctl)) {
+            if (!__any_sync(0xffffffffu, poisoned(ctl))) {
                 aw.step = s;
                 aw.rope_tab = a.rope_tab + (long long)(s & 1) * TcGeo<NG>::NB * (DH / 2);
                 ring.base = items_before + (unsigned)s * items_step;

@@ -1,5 +1,7 @@
 """Drafts of 17..64 sequences on a shape whose phases all give their tiles whole CTAs: the column groups of a tile are dealt to
 its contributors, which wait for one another."""
+import time
+
 import numpy as np
 import pytest
 
@@ -37,3 +39,25 @@ def test_dealt_column_groups_against_the_per_phase_kernels(shape, B):
     r.dr.status()
     assert row_rel_err(got, want).max() <= LOGIT_RTOL
     assert np.abs(rows - ref).max() <= 2.0 ** -6 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("B", [17, 32, 33, 64])
+def test_waits_run_out_cleanly_and_the_context_recovers(B):
+    """The grid barriers of one draft are made impossible to complete: every wait, those for a tile's other contributors among
+    them, ends at its limit, the status says so, and the same draft then gives what it gave before, bit for bit."""
+    from paper_2509_23928_b200 import HivisError
+    r = start("wide128", B, 22)
+    want, ref = window(r, B)
+    r.dr.set_wait_limit_us(2000)
+    r.dr.miss_next_barrier()
+    t0 = time.perf_counter()
+    window(r, B)
+    assert time.perf_counter() - t0 < 10.0
+    with pytest.raises(HivisError) as e:
+        r.dr.status()
+    assert e.value.code == -7
+    r.dr.status()
+    r.dr.set_wait_limit_us(1000000)
+    got, rows = window(r, B)
+    r.dr.status()
+    assert np.array_equal(got, want) and np.array_equal(rows, ref)
