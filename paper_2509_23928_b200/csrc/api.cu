@@ -42,7 +42,6 @@ struct hivis_ctx {
     bool chain_ok_coop;           // cooperative launch available
     bool opt_chain;               // option HIVIS_OPT_CHAIN_KERNEL
     u64* bar_counter;
-    u64 bar_count_host;           // value of *bar_counter once everything enqueued has run
     int* error_flag;              // [0]: a device-side wait ran out; [1] (= id_flag): a token id was out of range
     int* id_flag;
     // tensor-core chain kernel (bf16)
@@ -299,7 +298,6 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
     c->phase_k = 0;
     c->tile_ctr = nullptr;
     c->tc_tiles = 0;
-    c->bar_count_host = 0;
     {
         int coop = 0;
         c->num_sms = 0;
@@ -619,7 +617,7 @@ static int run_after_attention(hivis_ctx* c, bool mma, int b0, int nb, u64* keys
 }
 
 // Arguments of the tensor-core chain kernel for B columns and k steps (the whole step; callers narrow seq_first /
-// seq_last and bar_base when they run a part of it).
+// seq_last and bar_off when they run a part of it).
 static void fill_tc_args(hivis_ctx* c, TcArgs* out, int B, int k, int lo, const float* rho, int n_resid,
                          const int32_t* forced_ids, float* out_logits) {
     const hivis_config& g = c->cfg;
@@ -643,7 +641,7 @@ static void fill_tc_args(hivis_ctx* c, TcArgs* out, int B, int k, int lo, const 
     a.Kc = c->Kc; a.Vc = c->Vc; a.inv_freq = c->inv_freq; a.part_acc = c->part_acc; a.part_ml = c->part_ml;
     a.counters = c->counters;
     a.attn_nslot = c->nsplit_cap;
-    a.bar_counter = c->bar_counter; a.bar_base = c->bar_count_host + (c->debug_skew ? (1ull << 40) : 0ull);
+    a.bar_counter = c->bar_counter; a.bar_off = c->debug_skew ? 1ull << 40 : 0ull;
     a.wait_cycles = c->wait_cycles; a.error_flag = c->error_flag; a.id_flag = c->id_flag;
     a.l2_keep = c->opt_l2_keep;
     a.phase_t = nullptr;
@@ -779,13 +777,7 @@ static int draft_impl(hivis_ctx* c, int B, const int* seq_slots_host, int k, con
     // The kernel numbers attention units x warps in 32 bits; a batch beyond that (hundreds of heads on long caches) takes
     // the per-phase kernels, as do draws for more than 16 sequences (refused below).
     const bool tc_fits = B <= 16 || (!uniforms && (long long)B * g.n_q_heads * ((max_rows + 31) / 32 + 1) * 4 * c->num_sms < (1ll << 32));
-    bool in_tc = !one_seq && c->tc_ok && c->opt_tc != 0 && tc_fits;
-    if (in_tc && B > 16) {
-        // (the kernel's barrier counter is counted on the host: a captured call would be replayed with a stale count)
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        CK(c, cudaStreamIsCapturing(st, &cap));
-        in_tc = cap == cudaStreamCaptureStatusNone;
-    }
+    const bool in_tc = !one_seq && c->tc_ok && c->opt_tc != 0 && tc_fits;
     const bool raw_rho = resid && !c->resid_proj && (one_seq || in_tc);
     if (resid && !raw_rho) {
         rc = prepare_rho(c, resid, n_resid, st);
@@ -806,11 +798,10 @@ static int draft_impl(hivis_ctx* c, int B, const int* seq_slots_host, int k, con
         a.inv_t = inv_t;
         a.out_ids = out_ids;
         plan_attention(c, max_rows, c->num_sms / g.n_q_heads, &a.attn_chunk, &a.attn_nsplit);
-        a.bar_base = c->bar_count_host + (c->debug_skew ? (1ull << 40) : 0ull);
+        a.bar_off = c->debug_skew ? 1ull << 40 : 0ull;
         a.wait_cycles = c->wait_cycles;
         c->debug_skew = false;
         CKP(c, CLS_CHAIN, st, launch_draft_chain(a, c->dtype, c->num_sms, st));
-        c->bar_count_host += (u64)c->num_sms * (u64)(chain_barriers_per_step() * k);
         const int s0 = sl.slot[0];
         c->kv_upper[s0] += k;
         c->pending[s0] = false;
@@ -838,7 +829,6 @@ static int draft_impl(hivis_ctx* c, int B, const int* seq_slots_host, int k, con
         }
         c->debug_skew = false;
         CKP(c, CLS_CHAIN, st, launch_tc_chain(B <= TC_OP_ROWS ? c->tc_maps : c->tc_maps_wide, a, c->num_sms, st));
-        c->bar_count_host += (u64)c->num_sms * (u64)(tc_barriers_per_step() * k);
         for (int b = 0; b < B; ++b) {
             const int s = sl.slot[b];
             c->kv_upper[s] += k;
@@ -1029,17 +1019,15 @@ int hivis_draft_tree(hivis_ctx* c, int slot, int topk, int depth, int keep, cons
             a.rho_h = raw_rho ? (const bf16*)resid + (long long)row * d : nullptr;
             a.whole_ctas = 0;                                        // the order of the sums decides which of two near nodes is kept
             a.seq_first = 1; a.seq_last = 2;                         // fusion FC, QKV (the operands are gathered already)
-            a.bar_base = c->bar_count_host - G + (c->debug_skew ? (1ull << 40) : 0ull);
+            a.bar_off -= G;                                          // as if the gather had been arrived on
             c->debug_skew = false;
             CKL(c, launch_tc_chain(c->tc_maps, a, c->num_sms, st));
-            c->bar_count_host += G * 2;
             CK(c, launch_tree_attention(c->dtype, nb, c->qkv, c->qkvw, g.n_q_heads, g.n_kv_heads, g.head_dim, g.max_len, slot,
                                         level, T, c->inv_freq, c->Kc, c->Vc, c->attn, c->attn_h, lo, st));
             c->launches += 1;
             a.seq_first = 4; a.seq_last = 7;                         // O, gate/up, down, LM head (logits of every node)
-            a.bar_base = c->bar_count_host - G * 4;                  // as if gather .. attention had been arrived on
+            a.bar_off = 0 - G * 4;                                   // as if gather .. attention had been arrived on
             CKL(c, launch_tc_chain(c->tc_maps, a, c->num_sms, st));
-            c->bar_count_host += G * 4;
         } else {
             const bool mma = use_mma(c, nb, false);
             rc = run_fuse(c, mma, 0, nb, c->feat, c->feat_h, c->cur_id, 1, nullptr, rho, st);
@@ -1221,7 +1209,6 @@ int hivis_status(hivis_ctx* c, void* stream) {
     CK(c, cudaMemsetAsync(c->counters, 0, (size_t)c->rows_cap * c->cfg.n_q_heads * sizeof(int), st));
     if (c->tile_ctr) CK(c, cudaMemsetAsync(c->tile_ctr, 0, (size_t)c->tc_tiles * sizeof(int), st));
     CK(c, cudaStreamSynchronize(st));
-    c->bar_count_host = 0;
     return fail(c, HIVIS_ERR_TIMEOUT, "a device-side wait ran out (code %d); results of that call are invalid", flag);
 }
 

@@ -89,6 +89,17 @@ struct AttnArgs {
 };
 cudaError_t launch_attention(int dtype, const AttnArgs& a, cudaStream_t st);
 
+// The grid barriers of the chain kernels count arrivals in one counter of the context, which is only ever incremented, G (the
+// number of CTAs, the same for every launch) times per barrier.  A launch finds out itself where it starts: until a CTA has
+// made its first arrival the first barrier cannot be complete, so what it reads is the value at the launch's start, a multiple
+// of G, plus at most G - 1 arrivals of others.  (A value that the host counts and passes is wrong for a captured launch that
+// is replayed.)  One thread, before the CTA's first arrival.
+__device__ __forceinline__ u64 barrier_base(const u64* counter, unsigned G) {
+    u64 v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(counter) : "memory");
+    return v - v % G;
+}
+
 // ---------------------------------------------------------------------------------------------
 // Persistent chain kernel (one sequence, all k steps in one cooperative launch).
 // ---------------------------------------------------------------------------------------------
@@ -124,8 +135,8 @@ struct ChainArgs {
     float *part_acc, *part_ml;
     int* counters;
     int attn_chunk, attn_nsplit;
-    u64* bar_counter;          // arrival counter of the grid barrier, only ever incremented
-    u64 bar_base;              // its value when this launch starts
+    u64* bar_counter;          // arrival counter of the grid barrier (barrier_base)
+    u64 bar_off;               // 0; anything large makes the barriers impossible to complete (test aid)
     long long wait_cycles;     // limit of every device-side wait, in SM clock cycles
     int* error_flag;           // set non-zero by a kernel that gave up on a wait
     int* id_flag;              // set non-zero when a token id outside [0, V) reached the embedding lookup
@@ -134,7 +145,6 @@ struct ChainArgs {
 // shared memory the kernel needs for these dimensions on `grid` CTAs; 0 = does not fit
 size_t chain_smem_bytes(const ChainArgs& a, int dtype, int grid);
 cudaError_t launch_draft_chain(ChainArgs& a, int dtype, int grid, cudaStream_t st);
-int chain_barriers_per_step();
 
 struct SlotList {
     int n;
@@ -189,8 +199,8 @@ struct TcArgs {
     float *part_acc, *part_ml;
     int* counters;
     int attn_nslot;            // partial slots per (sequence, head): >= 32-row blocks of the longest sequence
-    u64* bar_counter;
-    u64 bar_base;
+    u64* bar_counter;          // (barrier_base)
+    u64 bar_off;               // added to the counter's value at the start: the barriers of the parts that a launch leaves out
     long long wait_cycles;     // limit of every device-side wait, in SM clock cycles
     int* error_flag;
     int* id_flag;              // set non-zero when a token id outside [0, V) reached the embedding lookup
@@ -198,7 +208,7 @@ struct TcArgs {
     int l2_keep;               // bit p set: the weights of phase p are loaded with the keep-in-L2 policy
     // The grid barriers of a step are numbered 0 gather, 1 FC, 2 QKV, 3 attention, 4 O, 5 gate/up, 6 down, 7 LM head.
     // A launch runs the part [seq_first, seq_last] of every step (0..7: the whole step); what lies outside does no work
-    // and arrives nowhere, and bar_base is set as if the barriers before seq_first had been completed already.
+    // and arrives nowhere, and bar_off makes it as if the barriers before seq_first had been completed already.
     int whole_ctas;            // bit p: the tiles of phase p get whole CTAs where their number allows it
     int seq_first, seq_last;
 };
@@ -213,7 +223,6 @@ cudaError_t launch_tc_setup(const SlotList& sl, int k, int d, int lo, int* d_slo
                             const float* pend_feat, const int* pend_id, float* feat, bf16* feat_h,
                             int* cur_id, u64* keys, int key_stride, const bf16* embed, int vocab, bf16* xe_h,
                             int* id_flag, cudaStream_t st);
-int tc_barriers_per_step();
 int tc_lo_offset(int B);
 int tc_groups(int B);
 

@@ -77,6 +77,7 @@ __device__ __forceinline__ int ld_relaxed_int(const int* p) {
     return v;
 }
 
+#define CHAIN_BARRIERS 7         // grid barriers of a step
 struct ChainMisc {
     float red[CHAIN_WARPS];
     u64 kred[CHAIN_WARPS];
@@ -84,6 +85,7 @@ struct ChainMisc {
     int r0[PH_COUNT];          // first row of this CTA in each phase
     int units[PH_COUNT];       // number of units of this CTA in each phase
     int cpr[PH_COUNT];         // chunks per row
+    u64 bar_base;              // value of the barrier counter when the launch began
 };
 
 // Grid-wide barrier on a monotonically increasing counter.  false = gave up (error flag raised).
@@ -191,6 +193,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
             misc->cpr[p] = cpr;
             misc->units[p] = (int)(r1 - r0) * cpr;
         }
+        misc->bar_base = barrier_base(a.bar_counter, (unsigned)G) + a.bar_off;
         for (int i = 0; i < CHAIN_WARPS * CHAIN_STAGES; ++i) mbar_init(smem_addr(bars + i), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
@@ -276,7 +279,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
         return v;
     };
 
-    u64 bar_target = a.bar_base;
+    u64 bar_target = misc->bar_base;
     bool alive = true;
     auto barrier = [&]() {
         bar_target += (u64)G;
@@ -434,7 +437,9 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
         }
         return;                                             // every fetched unit has been consumed
     }
-    // gave up: wait (bounded) for this warp's copies that are still in flight, then leave
+    // gave up: make the arrivals that are left (the next launch counts on whole barriers), wait (bounded) for this warp's
+    // copies that are still in flight, then leave
+    if (tid == 0) red_release_add_u64(a.bar_counter, (u64)(CHAIN_BARRIERS * a.k) - (bar_target - misc->bar_base) / (u64)G);
     for (; ci < fi; ++ci) {
         const uint32_t bar = bar0 + (ci % CHAIN_STAGES) * 8;
         const uint32_t parity = (ci / CHAIN_STAGES) & 1u;
@@ -476,8 +481,6 @@ static ChainPlan chain_plan(const ChainArgs& a, int es, int dh, int grid) {
     p.smem_bytes = off;
     return p;
 }
-
-int chain_barriers_per_step() { return 7; }
 
 template <typename WT, int DH>
 static cudaError_t chain_launch_t(ChainArgs& a, int grid, size_t smem, cudaStream_t st) {

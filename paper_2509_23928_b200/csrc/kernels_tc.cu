@@ -115,8 +115,6 @@ int tc_max_tiles(const ChainPhase* ph) {
     return m;
 }
 
-int tc_barriers_per_step() { return 8; }      // the grid barriers of TcArgs::seq_first .. seq_last
-
 // column groups of 16 sequences of a launch: the kernel is built for 1, 2 and 4
 int tc_groups(int B) { return B <= 16 ? 1 : B <= 32 ? 2 : 4; }
 // Row offset of the rounding remainders in the operand buffers for a batch of B (0: none are kept).

@@ -91,6 +91,7 @@ struct TcCtl {
     unsigned issued;            // ring items the weight producer has armed so far
     int abort_flag;
     long long wait_cycles;      // limit of every wait
+    u64 bar_base;               // value of the barrier counter when the launch began
     int last_flag, early_flag;
     int cinfo[2][3];            // contributors of the CTA's first and last tile of the phase: first CTA, its slot bit, count
     float scale[HIVIS_MAX_BATCH];
@@ -658,7 +659,7 @@ __device__ void tc_producer_x(const TcParams& P, TcCtl* ctl, uint32_t smemB, int
             // the descriptor of the phase's operand is asked for while the barrier is still awaited
             prefetch_tensormap(&P.maps.m[map_idx]);
             if (need >= 0) {
-                if (!wait_grid(a.bar_counter, a.bar_base + (u64)G * (u64)(need + 1), ctl, a.error_flag, 9)) break;
+                if (!wait_grid(a.bar_counter, ctl->bar_base + (u64)G * (u64)(need + 1), ctl, a.error_flag, 9)) break;
                 // other CTAs wrote the operand through the generic proxy; TMA reads through the async proxy
                 fence_proxy_async_global();
             }
@@ -666,7 +667,7 @@ __device__ void tc_producer_x(const TcParams& P, TcCtl* ctl, uint32_t smemB, int
         }
         const bool emb = c.p == PH_FC && c.kb >= dkb;
         if (emb && gathered_step != c.step) {
-            if (!wait_grid(a.bar_counter, a.bar_base + (u64)G * (u64)(c.step * TC_BARS_PER_STEP + TC_SEQ_GATHER + 1), ctl,
+            if (!wait_grid(a.bar_counter, ctl->bar_base + (u64)G * (u64)(c.step * TC_BARS_PER_STEP + TC_SEQ_GATHER + 1), ctl,
                            a.error_flag, 11))
                 break;
             fence_proxy_async_global();
@@ -705,7 +706,7 @@ __device__ void tc_gather(const TcParams& P, TcCtl* ctl, int s, int cta, int G, 
     }
     if (s > 0) {
         if (etid == 0)
-            wait_grid(a.bar_counter, a.bar_base + (u64)G * (u64)((s - 1) * TC_BARS_PER_STEP + 8), ctl, a.error_flag, 12);
+            wait_grid(a.bar_counter, ctl->bar_base + (u64)G * (u64)((s - 1) * TC_BARS_PER_STEP + 8), ctl, a.error_flag, 12);
         named_sync(TC_BAR_EPI, TC_EPI_THREADS);
         if (!poisoned(ctl)) {
             const int upr = a.d >> 3;                    // 16-byte units per row
@@ -1064,7 +1065,7 @@ __device__ __forceinline__ void tc_epilogue_phase(const TcParams& P, TcCtl* ctl,
     if (need_scale && lo < hi) {
         // The RMSNorm scale of this phase's operand: wait here for the phase that produced it (rather than for
         // the first accumulator, which for a short range is also the last: the sums would be fetched in the tail)
-        if (etid == 0) wait_grid(a.bar_counter, a.bar_base + (u64)G * (u64)(need_seq(s, p) + 1), ctl, a.error_flag, 18);
+        if (etid == 0) wait_grid(a.bar_counter, ctl->bar_base + (u64)G * (u64)(need_seq(s, p) + 1), ctl, a.error_flag, 18);
         named_sync(TC_BAR_EPI, TC_EPI_THREADS);
         epi_compute_scales<NG>(a, ctl, p == PH_QKV ? a.ssq1 : a.ssq2, etid);
         need_scale = false;
@@ -1262,7 +1263,7 @@ __device__ __forceinline__ void tc_epilogue_phase(const TcParams& P, TcCtl* ctl,
         // (the FC phase follows the gather barrier of its step, which its hidden-half operand does not imply)
         const int need = p == PH_FC ? s * TC_BARS_PER_STEP + TC_SEQ_GATHER : need_seq(s, p);
         if ((lo == hi || p == PH_FC) && need >= 0)
-            wait_grid(a.bar_counter, a.bar_base + (u64)G * (u64)(need + 1), ctl, a.error_flag, 8);
+            wait_grid(a.bar_counter, ctl->bar_base + (u64)G * (u64)(need + 1), ctl, a.error_flag, 8);
         phase_stamp(a, s, phase_seq(p), cta, G);
         red_release_add_u64(a.bar_counter, 1ull);
     }
@@ -1301,6 +1302,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_chain_kernel(const __grid_co
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async_all();
     }
+    if (tid == 96) ctl->bar_base = barrier_base(a.bar_counter, (unsigned)G) + a.bar_off;      // (warp 3 has no role)
     if (warp == 1) {
         __syncwarp();
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(&ctl->tmem_base)),
@@ -1361,7 +1363,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_chain_kernel(const __grid_co
             // ---- attention: needs every CTA's QKV rows
             if (seq_on(a, TC_SEQ_ATTN)) {
             if (atid == 0)
-                wait_grid(a.bar_counter, a.bar_base + (u64)G * (u64)(s * TC_BARS_PER_STEP + TC_SEQ_ATTN), ctl, a.error_flag, 7);
+                wait_grid(a.bar_counter, ctl->bar_base + (u64)G * (u64)(s * TC_BARS_PER_STEP + TC_SEQ_ATTN), ctl, a.error_flag, 7);
             if (atid == 0) phase_stamp(a, s, 20, cta, G);
             named_sync(TC_BAR_ATT, TC_ATT_WARPS * 32);
             if (!__any_sync(0xffffffffu, poisoned(ctl))) {
@@ -1387,7 +1389,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_chain_kernel(const __grid_co
         if (a.out_ids && cta == 0) {
             // the chosen tokens, once every CTA's part of the last LM head has reached the keys
             if (atid == 0)
-                wait_grid(a.bar_counter, a.bar_base + (u64)G * (u64)(a.k * TC_BARS_PER_STEP), ctl, a.error_flag, 19);
+                wait_grid(a.bar_counter, ctl->bar_base + (u64)G * (u64)(a.k * TC_BARS_PER_STEP), ctl, a.error_flag, 19);
             named_sync(TC_BAR_EPI, TC_EPI_THREADS);
             for (int i = atid; i < a.B * a.k; i += TC_EPI_THREADS)
                 a.out_ids[i] = key_index(__ldcg(a.keys + (long long)(i / a.k) * a.key_stride + i % a.k));

@@ -316,8 +316,7 @@ def test_small_prefix_builds_in_the_chain_kernel(name, project, pairs):
 
 
 def test_captured_refresh_and_wide_draft_replay():
-    """A small prefix build and a draft of 20 sequences captured into a graph take the kernels without a host-counted
-    barrier: every replay gives what the calls give."""
+    """A small prefix build and a draft of 20 sequences captured into a graph: every replay gives what the calls give."""
     import torch
     wl = hi.scaled(hi.workload("mini_mha_b5_ragged"), batch=20, k=3, text_len_range=(2, 40))
     case = Case(wl)
