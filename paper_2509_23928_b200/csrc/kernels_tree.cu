@@ -316,6 +316,10 @@ int tree_topk_pieces(int V) { return (V + TREE_PIECE - 1) / TREE_PIECE; }
 //   spent 27 us here, most of it in a single warp that walked the sorted lists.
 #define TREE_MERGE_CAP 1024      // keys of a node ranked from shared memory (more: from global memory)
 
+// What a score ranks as.  A score that is not a number (weights or states that are not) ranks last: compared as it is it
+// would be beaten by nobody, and more nodes would be chosen than the lists hold.
+__device__ __forceinline__ float tree_rank_of(float score) { return score == score ? score : -INFINITY; }
+
 // The nb * topk children of this level become candidates (creation order: frontier order, then rank); unless this was
 // the last level, the `topk` of them with the highest cumulative log-probability (earlier candidate first among
 // equals) form the next frontier, kept in creation order.
@@ -339,12 +343,13 @@ __device__ void tree_select(int level, int depth, int nb, int topk, const TreeBu
         T.cand_score[base + i] = score;
         T.cand_store[base + i] = -1;
     }
-    s_score[i] = score;
+    const float mine = tree_rank_of(score);
+    s_score[i] = mine;
     __syncthreads();
     int sel = 0;
     if (i < n && level + 1 < depth) {
         int rank = 0;
-        for (int o = 0; o < n; ++o) rank += (s_score[o] > score || (s_score[o] == score && o < i)) ? 1 : 0;
+        for (int o = 0; o < n; ++o) rank += (s_score[o] > mine || (s_score[o] == mine && o < i)) ? 1 : 0;
         sel = rank < topk ? 1 : 0;
     }
     s_sel[i] = sel;
@@ -493,7 +498,7 @@ __global__ void __launch_bounds__(1024) tree_finalize_kernel(int keep, TreeBufs 
     __shared__ unsigned short s_pos[TREE_MAX_CAND];          // 1 + position among the kept, 0 = not kept
     __shared__ int s_sum[32];
     const int n = *T.cand_n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int i = tid; i < n; i += 1024) s_score[i] = T.cand_score[i];
+    for (int i = tid; i < n; i += 1024) s_score[i] = tree_rank_of(T.cand_score[i]);
     __syncthreads();
     int before = 0;                                          // kept candidates of the earlier turns
     for (int i0 = 0; i0 < n; i0 += 1024) {
@@ -528,7 +533,7 @@ __global__ void __launch_bounds__(1024) tree_finalize_kernel(int keep, TreeBufs 
         T.kept_store[pos] = T.cand_store[i];
         out_tokens[pos] = tok;
         out_parents[pos] = pp;
-        out_scores[pos] = s_score[i];
+        out_scores[pos] = T.cand_score[i];
     }
     if (tid == 0) {
         const int cnt = n < keep ? n : keep;

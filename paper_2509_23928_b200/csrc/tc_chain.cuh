@@ -85,6 +85,19 @@ struct TcParams {
     TcArgs a;
 };
 
+// A CTA's part of a phase, worked out once per launch (it is the same at every step): its run of tile-k-blocks, and who shares
+// the first and the last tile of the run.  Worked out at every phase entry, inlined for each of the six phases and the three
+// producing roles, the divisions were two fifths of the kernel's code (544 KB; 329 KB now), which an SM's instruction
+// caches do not hold: it is fetched again at every phase, and from HBM when the K/V rows of long caches push it out of L2.
+// Batch 16, d 4096, five steps: 829 -> 803 us with 128 cached rows, 1073 -> 1043 with 704, 963 -> 930 with 64..512.
+struct TcPlan {
+    int tile, kb, n;            // first tile, its first k-block, number of tile-k-blocks
+    int nkb;                    // k-blocks of a tile
+    int split;                  // > 0: that many CTAs per tile (PhaseShape)
+    int big;                    // every CTA has work: the contributors of a tile are consecutive CTAs
+    int cf[2], fs[2], nc[2];    // first / last tile: its first contributor, that one's partial slot, number of contributors
+};
+
 struct TcCtl {
     u64 full[TC_MAX_STAGES], empty[TC_MAX_STAGES], tfull[2], tempty[2];
     uint32_t tmem_base;
@@ -93,7 +106,7 @@ struct TcCtl {
     long long wait_cycles;      // limit of every wait
     u64 bar_base;               // value of the barrier counter when the launch began
     int last_flag, early_flag;
-    int cinfo[2][3];            // contributors of the CTA's first and last tile of the phase: first CTA, its slot bit, count
+    TcPlan plan[PH_COUNT];      // this CTA's part of every phase
     float scale[HIVIS_MAX_BATCH];
     alignas(16) float red[8 * HIVIS_MAX_BATCH];
     u64 kred[2][4][16];         // LM head: best key of each epilogue warp per sequence (two buffers, used in turn)
@@ -329,7 +342,7 @@ __device__ __forceinline__ int need_seq(int step, int p) {                      
 struct PhaseShape {
     int nkb, ntiles;
     int split;          // > 0: that many CTAs per tile, equal runs of its k-blocks; 0: one contiguous run over all tiles
-    long long W;
+    unsigned W;         // tile-k-blocks; times the number of CTAs it fits 32 bits for any matrix that fits the GPU's memory
 };
 // Phases with few row tiles (fusion FC, O, down) give every tile the same number of CTAs, each one run of its k-blocks,
 // where that keeps TC_ALIGN_PCT of the CTAs busy: no CTA has two tiles to publish, nobody finishes two in a row, and the
@@ -345,62 +358,90 @@ __device__ __forceinline__ PhaseShape phase_shape(const TcArgs& a, int p) {
     PhaseShape s;
     s.nkb = (a.ph[p].K + TC_BK - 1) / TC_BK;
     s.ntiles = (a.ph[p].N + TC_TM - 1) / TC_TM;
-    s.W = seq_on(a, phase_seq(p)) ? (long long)s.nkb * s.ntiles : 0;      // a phase outside the launch's part has no work
+    s.W = seq_on(a, phase_seq(p)) ? (unsigned)(s.nkb * s.ntiles) : 0u;      // a phase outside the launch's part has no work
     const int G = gridDim.x, per = G / s.ntiles;
     s.split = ((a.whole_ctas >> p) & 1) && s.W > 0 && per >= 2 && s.nkb >= 2 * per && per * s.ntiles * 100 >= TC_ALIGN_PCT * G ? per : 0;
     return s;
 }
 // first tile-k-block of CTA c (its range ends where that of c + 1 begins)
-__device__ __forceinline__ long long range_lo(const PhaseShape& s, int c, int G) {
+__device__ __forceinline__ int range_lo(const PhaseShape& s, int c, int G) {
     if (s.split) {
         const int t = c / s.split;
-        return t >= s.ntiles ? s.W : (long long)t * s.nkb + s.nkb * (c - t * s.split) / s.split;
+        return t >= s.ntiles ? (int)s.W : t * s.nkb + s.nkb * (c - t * s.split) / s.split;
     }
-    return s.W * c / G;
+    return (int)(s.W * (unsigned)c / (unsigned)G);
 }
 // CTA whose range contains tile-k-block `idx`
-__device__ __forceinline__ int owner_of(const PhaseShape& s, int G, long long idx) {
+__device__ __forceinline__ int owner_of(const PhaseShape& s, int G, int idx) {
     if (s.split) {
-        const int t = (int)(idx / s.nkb), kb = (int)(idx - (long long)t * s.nkb);
+        const int t = idx / s.nkb, kb = idx - t * s.nkb;
         int part = kb * s.split / s.nkb;
         while (part + 1 < s.split && s.nkb * (part + 1) / s.split <= kb) ++part;
         while (part > 0 && s.nkb * part / s.split > kb) --part;
         return t * s.split + part;
     }
-    int c = (int)(idx * G / s.W);
+    int c = (int)((unsigned)idx * (unsigned)G / s.W);
     if (c >= G) c = G - 1;
     while (c + 1 < G && range_lo(s, c + 1, G) <= idx) ++c;
     while (c > 0 && range_lo(s, c, G) > idx) --c;
     return c;
 }
+// The next contributor's first tile-k-block (phases with fewer tile-k-blocks than CTAs, where they are not consecutive).
+__device__ __noinline__ int owner_end(const PhaseShape s, int G, int idx, int& owner) {
+    owner = owner_of(s, G, idx);
+    return range_lo(s, owner + 1, G);
+}
+__device__ __noinline__ void tc_plan_phase(const TcArgs& a, int p, int cta, int G, TcPlan& out) {
+    const PhaseShape s = phase_shape(a, p);
+    const int lo = range_lo(s, cta, G), hi = range_lo(s, cta + 1, G);
+    out.tile = lo / s.nkb;
+    out.kb = lo % s.nkb;
+    out.n = hi - lo;
+    out.nkb = s.nkb;
+    out.split = s.split;
+    out.big = s.W >= (unsigned)G;
+    if (lo >= hi) return;
+    for (int q = 0; q < 2; ++q) {
+        const int t0 = (q == 0 ? lo : hi - 1) / s.nkb * s.nkb;
+        const int cf = owner_of(s, G, t0);
+        out.cf[q] = cf;
+        out.fs[q] = t0 == range_lo(s, cf, G) ? 0 : 1;
+        if (out.big) {
+            out.nc[q] = owner_of(s, G, t0 + s.nkb - 1) - cf + 1;
+        } else {
+            int nc = 0, owner;
+            for (int i = t0; i < t0 + s.nkb; ++nc) i = owner_end(s, G, i, owner);
+            out.nc[q] = nc;
+        }
+    }
+}
 
-// Cursor over one CTA's tile-k-blocks through all phases and steps.  Divisions happen only when a phase is
-// entered; stepping to the next k-block is a few integer instructions (the producers are single threads).
+// Cursor over one CTA's tile-k-blocks through all phases and steps (the producers are single threads: a phase entry is a few
+// loads from shared memory, a step to the next k-block a few integer instructions).
 struct Cursor {
     int step, p;
     int tile, kb, left, nkb;
     bool live, entered;         // entered: this k-block is the first of its phase for this CTA
 };
-__device__ __forceinline__ void cursor_enter(Cursor& c, const TcArgs& a, int cta, int G) {
+__device__ __forceinline__ void cursor_enter(Cursor& c, const TcPlan* plan, int steps) {
     // position on the first non-empty phase range at or after (step, p)
     while (c.live) {
-        const PhaseShape s = phase_shape(a, c.p);
-        const long long lo = range_lo(s, cta, G), hi = range_lo(s, cta + 1, G);
-        c.nkb = s.nkb;
-        c.left = (int)(hi - lo);
+        const TcPlan& s = plan[c.p];
+        c.left = s.n;
         if (c.left > 0) {
-            c.tile = (int)(lo / s.nkb);
-            c.kb = (int)(lo % s.nkb);
+            c.nkb = s.nkb;
+            c.tile = s.tile;
+            c.kb = s.kb;
             c.entered = true;
             return;
         }
         if (++c.p == PH_COUNT) {
             c.p = 0;
-            if (++c.step == a.k) c.live = false;
+            if (++c.step == steps) c.live = false;
         }
     }
 }
-__device__ __forceinline__ void cursor_next(Cursor& c, const TcArgs& a, int cta, int G) {
+__device__ __forceinline__ void cursor_next(Cursor& c, const TcPlan* plan, int steps) {
     c.entered = false;
     if (--c.left > 0) {
         if (++c.kb == c.nkb) {
@@ -411,9 +452,9 @@ __device__ __forceinline__ void cursor_next(Cursor& c, const TcArgs& a, int cta,
     }
     if (++c.p == PH_COUNT) {
         c.p = 0;
-        if (++c.step == a.k) { c.live = false; return; }
+        if (++c.step == steps) { c.live = false; return; }
     }
-    cursor_enter(c, a, cta, G);
+    cursor_enter(c, plan, steps);
 }
 
 // after a give-up: copies already issued still land in this CTA's shared memory; give them time
@@ -598,7 +639,7 @@ __device__ void tc_producer_w(const TcParams& P, TcCtl* ctl, uint32_t smemA, int
         }
     }
     Cursor c{0, 0, 0, 0, 0, 0, true, false};
-    cursor_enter(c, a, cta, G);
+    cursor_enter(c, ctl->plan, a.k);
     unsigned slot = 0, round = 0;
     int att_done = 0;               // steps whose attention items have been issued
     unsigned publish = 0;           // weight items still to be announced (those that reuse attention stages)
@@ -620,7 +661,7 @@ __device__ void tc_producer_w(const TcParams& P, TcCtl* ctl, uint32_t smemA, int
             pol_w = ((a.l2_keep >> c.p) & 1) ? pol_kv : pol_stream;
         }
         tma_load_2d(smemA + slot * TC_A_BYTES, &P.maps.m[TCM_W + c.p], c.kb * TC_BK, c.tile * TC_TM, bar, pol_w);
-        cursor_next(c, a, cta, G);
+        cursor_next(c, ctl->plan, a.k);
         if (++slot == STAGES) { slot = 0; ++round; }
         if (publish) {
             st_release_cta_u32(&ctl->issued, round * STAGES + slot);
@@ -643,7 +684,7 @@ __device__ void tc_producer_x(const TcParams& P, TcCtl* ctl, uint32_t smemB, int
     const TcArgs& a = P.a;
     const u64 pol_x = policy_evict_last();
     Cursor c{0, 0, 0, 0, 0, 0, true, false};
-    cursor_enter(c, a, cta, G);
+    cursor_enter(c, ctl->plan, a.k);
     unsigned slot = 0, round = 0;
     const int dkb = a.d / TC_BK;
     int map_idx = TCM_X_FEAT;
@@ -678,7 +719,7 @@ __device__ void tc_producer_x(const TcParams& P, TcCtl* ctl, uint32_t smemB, int
         const uint32_t dst = smemB + slot * TcGeo<NG>::B_BYTES;
         if (emb) tma_load_2d(dst, &P.maps.m[TCM_X_EMB], (c.kb - dkb) * TC_BK, 0, bar, pol_x);
         else tma_load_2d(dst, &P.maps.m[map_idx], c.kb * TC_BK, 0, bar, pol_x);
-        cursor_next(c, a, cta, G);
+        cursor_next(c, ctl->plan, a.k);
         if (++slot == STAGES) { slot = 0; ++round; }
     }
     if (poisoned(ctl)) drain_after_poison();
@@ -743,16 +784,14 @@ __device__ void tc_mma_issuer(const TcParams& P, TcCtl* ctl, uint32_t smemA, uin
     unsigned check = 0;         // items whose stage last held an attention item: see wait_issued
     for (int s = 0; s < a.k; ++s)
         for (int p = 0; p < PH_COUNT; ++p) {
-            const PhaseShape sh = phase_shape(a, p);
-            const long long lo = range_lo(sh, cta, G), hi = range_lo(sh, cta + 1, G);
-            int left = (int)(hi - lo);
-            int kb0 = left > 0 ? (int)(lo % sh.nkb) : 0;
+            const int nkb = ctl->plan[p].nkb;
+            int left = ctl->plan[p].n, kb0 = ctl->plan[p].kb;
             if (p == PH_O && att_items > 0) {                       // the attention items of this step
                 ring_skip<NG>(slot, round, att_items);
                 check = STAGES;
             }
             while (left > 0) {
-                const int n = left < sh.nkb - kb0 ? left : sh.nkb - kb0;
+                const int n = left < nkb - kb0 ? left : nkb - kb0;
                 const unsigned acc = seg_cnt & 1u, use = seg_cnt >> 1;
                 if (use > 0 && !wait_mbar(saddr(&ctl->tempty[acc]), (use - 1) & 1u, ctl, a.error_flag, 4)) return;
                 tc_fence_after();
@@ -1042,27 +1081,14 @@ __device__ __forceinline__ void tc_epilogue_phase(const TcParams& P, TcCtl* ctl,
     const TcArgs& a = P.a;
     if (!seq_on(a, phase_seq(p))) return;
     const int etid = w4 * 32 + lane;
-    const PhaseShape sh = phase_shape(a, p);
-    const long long lo = range_lo(sh, cta, G), hi = range_lo(sh, cta + 1, G);
-    long long idx = lo;
+    const TcPlan& sh = ctl->plan[p];
+    const int total = sh.n;
+    int done = 0, tile = sh.tile, kb0 = sh.kb;
     unsigned lm_calls = 0;
     bool need_scale = (p == PH_QKV || p == PH_GU);
-    const bool big = sh.W >= G;        // every CTA has work: the contributors of a tile are consecutive CTAs
-    // Contributors of the (at most two) tiles this CTA shares with others, worked out while the first
-    // accumulator is still being computed: first contributor, its slot bit, number of contributors.
-    if (etid == 0 && lo < hi && big) {
-        const long long tl[2] = {lo / sh.nkb, (hi - 1) / sh.nkb};
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const long long t0 = tl[q] * sh.nkb;
-            const int cf = owner_of(sh, G, t0);
-            ctl->cinfo[q][0] = cf;
-            ctl->cinfo[q][1] = t0 == range_lo(sh, cf, G) ? 0 : 1;
-            ctl->cinfo[q][2] = owner_of(sh, G, t0 + sh.nkb - 1) - cf + 1;
-        }
-    }
-    if (lo < hi && big) named_sync(TC_BAR_EPI, TC_EPI_THREADS);
-    if (need_scale && lo < hi) {
+    const bool big = sh.big != 0;
+    if (total > 0 && big) named_sync(TC_BAR_EPI, TC_EPI_THREADS);
+    if (need_scale && total > 0) {
         // The RMSNorm scale of this phase's operand: wait here for the phase that produced it (rather than for
         // the first accumulator, which for a short range is also the last: the sums would be fetched in the tail)
         if (etid == 0) wait_grid(a.bar_counter, ctl->bar_base + (u64)G * (u64)(need_seq(s, p) + 1), ctl, a.error_flag, 18);
@@ -1070,16 +1096,11 @@ __device__ __forceinline__ void tc_epilogue_phase(const TcParams& P, TcCtl* ctl,
         epi_compute_scales<NG>(a, ctl, p == PH_QKV ? a.ssq1 : a.ssq2, etid);
         need_scale = false;
     }
-    const int tile_first = (int)(lo / sh.nkb);
-    while (idx < hi) {
-        const int tile = (int)(idx / sh.nkb), kb0 = (int)(idx % sh.nkb);
-        const int n = (int)((hi - idx) < (long long)(sh.nkb - kb0) ? (hi - idx) : (long long)(sh.nkb - kb0));
+    while (done < total) {
+        const int n = total - done < sh.nkb - kb0 ? total - done : sh.nkb - kb0;
         const bool shared = !(kb0 == 0 && n == sh.nkb);
-        int cf = 0, fs = 0, nc = 0;
-        if (shared && big) {
-            const int q = tile == tile_first ? 0 : 1;
-            cf = ctl->cinfo[q][0]; fs = ctl->cinfo[q][1]; nc = ctl->cinfo[q][2];
-        }
+        const int q0 = done == 0 ? 0 : 1;
+        const int cf = sh.cf[q0], fs = sh.fs[q0], nc = sh.nc[q0];
         const int me = cta - cf;            // this CTA's place among the contributors (big phases)
         if constexpr (NG == 1) {
         EpiPre pre;
@@ -1089,7 +1110,7 @@ __device__ __forceinline__ void tc_epilogue_phase(const TcParams& P, TcCtl* ctl,
         float others[16];
 #pragma unroll
         for (int c = 0; c < 16; ++c) others[c] = 0.f;
-        if (shared && big && idx != lo && hi - lo >= sh.nkb) {
+        if (shared && big && done != 0 && total >= sh.nkb) {
             if (etid == 0) {
                 const int seen = ld_acquire_int(a.tile_ctr + tile);
                 ctl->early_flag = seen == nc - 1;
@@ -1100,7 +1121,7 @@ __device__ __forceinline__ void tc_epilogue_phase(const TcParams& P, TcCtl* ctl,
         }
         const unsigned acc = seg_cnt & 1u;
         wait_mbar(saddr(&ctl->tfull[acc]), (seg_cnt >> 1) & 1u, ctl, a.error_flag, 6);
-        if (etid == 0 && idx + n == hi) phase_stamp(a, s, 14 + p, cta, G);
+        if (etid == 0 && done + n == total) phase_stamp(a, s, 14 + p, cta, G);
         tc_fence_after();
         float v[16];
         tc_ld_acc<NG>(ctl->tmem_base + ((uint32_t)(w4 * 32) << 16) + acc * TcGeo<NG>::TN, v);
@@ -1120,16 +1141,11 @@ __device__ __forceinline__ void tc_epilogue_phase(const TcParams& P, TcCtl* ctl,
         } else if (shared) {
             // publish the partial accumulator ([row][16 columns], 64 bytes per thread); the last arriver
             // finishes the tile
-            float4* mine = partial_of<NG>(a, cta * 2 + (idx == lo ? 0 : 1), 0, etid);
+            float4* mine = partial_of<NG>(a, cta * 2 + q0, 0, etid);
 #pragma unroll
             for (int q = 0; q < 4; ++q) __stcg(mine + q, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
             named_sync(TC_BAR_EPI, TC_EPI_THREADS);
             if (etid == 0) {
-                if (!big) {
-                    // contributors = the CTAs whose (non-empty) ranges meet this tile, in range order
-                    const long long t0 = (long long)tile * sh.nkb;
-                    for (long long i = t0; i < t0 + sh.nkb; ++nc) i = range_lo(sh, owner_of(sh, G, i) + 1, G);
-                }
                 // release: the CTA's partial (ordered before by the barrier) is visible first; acquire: so are
                 // the partials of those that arrived before
                 const int old = atom_add_acq_rel(a.tile_ctr + tile, 1);
@@ -1149,16 +1165,18 @@ __device__ __forceinline__ void tc_epilogue_phase(const TcParams& P, TcCtl* ctl,
                     // few tile-k-blocks (tiny shapes): contributors in range order, all read back
 #pragma unroll
                     for (int c = 0; c < 16; ++c) v[c] = 0.f;
-                    const long long t0 = (long long)tile * sh.nkb;
-                    for (long long i = t0; i < t0 + sh.nkb;) {
-                        const int cc = owner_of(sh, G, i);
-                        const float4* src = partial_of<NG>(a, cc * 2 + (i == range_lo(sh, cc, G) ? 0 : 1), 0, etid);
+                    const PhaseShape ps = phase_shape(a, p);
+                    const int t0 = tile * ps.nkb;
+                    for (int i = t0; i < t0 + ps.nkb;) {
+                        int cc;
+                        const int end = owner_end(ps, G, i, cc);
+                        const float4* src = partial_of<NG>(a, cc * 2 + (i == range_lo(ps, cc, G) ? 0 : 1), 0, etid);
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             const float4 t = __ldcg(src + q);
                             v[4 * q] += t.x; v[4 * q + 1] += t.y; v[4 * q + 2] += t.z; v[4 * q + 3] += t.w;
                         }
-                        i = range_lo(sh, cc + 1, G);
+                        i = end;
                     }
                 }
             }
@@ -1167,7 +1185,7 @@ __device__ __forceinline__ void tc_epilogue_phase(const TcParams& P, TcCtl* ctl,
         if (finish) epi_output<SMP, NG>(a, ctl, p, s, tile, 0, v, pre, lm_calls, w4, lane);
         } else {
         bool early = false;
-        if (shared && big && idx != lo && hi - lo >= sh.nkb) {
+        if (shared && big && done != 0 && total >= sh.nkb) {
             if (etid == 0) ctl->early_flag = ld_acquire_int(a.tile_ctr + tile) == nc - 1;
             named_sync(TC_BAR_EPI, TC_EPI_THREADS);
             early = ctl->early_flag != 0;
@@ -1181,7 +1199,7 @@ __device__ __forceinline__ void tc_epilogue_phase(const TcParams& P, TcCtl* ctl,
         if (deal && me < groups) epi_preload<SMP>(a, p, s, tile, 16 * me, w4, lane, pre);
         const unsigned acc = seg_cnt & 1u;
         wait_mbar(saddr(&ctl->tfull[acc]), (seg_cnt >> 1) & 1u, ctl, a.error_flag, 6);
-        if (etid == 0 && idx + n == hi) phase_stamp(a, s, 14 + p, cta, G);
+        if (etid == 0 && done + n == total) phase_stamp(a, s, 14 + p, cta, G);
         tc_fence_after();
         const uint32_t tacc = ctl->tmem_base + ((uint32_t)(w4 * 32) << 16) + acc * TcGeo<NG>::TN;
         bool finish = true;
@@ -1193,16 +1211,12 @@ __device__ __forceinline__ void tc_epilogue_phase(const TcParams& P, TcCtl* ctl,
                 if (deal && cg % nc == me) continue;
                 float v[16];
                 tc_ld_acc<NG>(tacc + 16 * cg, v);
-                float4* mine = partial_of<NG>(a, cta * 2 + (idx == lo ? 0 : 1), cg, etid);
+                float4* mine = partial_of<NG>(a, cta * 2 + q0, cg, etid);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) __stcg(mine + q, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
             }
             named_sync(TC_BAR_EPI, TC_EPI_THREADS);
             if (etid == 0) {
-                if (!big) {
-                    const long long t0 = (long long)tile * sh.nkb;
-                    for (long long i = t0; i < t0 + sh.nkb; ++nc) i = range_lo(sh, owner_of(sh, G, i) + 1, G);
-                }
                 const int old = atom_add_acq_rel(a.tile_ctr + tile, 1);
                 const int last = old == nc - 1;
                 if (deal) {
@@ -1232,16 +1246,18 @@ __device__ __forceinline__ void tc_epilogue_phase(const TcParams& P, TcCtl* ctl,
                     // few tile-k-blocks (tiny shapes): contributors in range order, all read back
 #pragma unroll
                     for (int c = 0; c < 16; ++c) v[c] = 0.f;
-                    const long long t0 = (long long)tile * sh.nkb;
-                    for (long long i = t0; i < t0 + sh.nkb;) {
-                        const int cc = owner_of(sh, G, i);
-                        const float4* src = partial_of<NG>(a, cc * 2 + (i == range_lo(sh, cc, G) ? 0 : 1), cg, etid);
+                    const PhaseShape ps = phase_shape(a, p);
+                    const int t0 = tile * ps.nkb;
+                    for (int i = t0; i < t0 + ps.nkb;) {
+                        int cc;
+                        const int end = owner_end(ps, G, i, cc);
+                        const float4* src = partial_of<NG>(a, cc * 2 + (i == range_lo(ps, cc, G) ? 0 : 1), cg, etid);
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             const float4 t = __ldcg(src + q);
                             v[4 * q] += t.x; v[4 * q + 1] += t.y; v[4 * q + 2] += t.z; v[4 * q + 3] += t.w;
                         }
-                        i = range_lo(sh, cc + 1, G);
+                        i = end;
                     }
                 }
                 epi_output<SMP, NG>(a, ctl, p, s, tile, 16 * cg, v, pre, lm_calls, w4, lane);
@@ -1253,7 +1269,9 @@ __device__ __forceinline__ void tc_epilogue_phase(const TcParams& P, TcCtl* ctl,
         ++seg_cnt;
         if (shared && !early) named_sync(TC_BAR_EPI, TC_EPI_THREADS);      // last_flag may be rewritten by the next segment
         }
-        idx += n;
+        done += n;
+        kb0 = 0;
+        ++tile;
     }
     // This CTA's part of the phase is done: arrive on the grid barrier.  All arrivals are counted in one
     // counter, so a CTA may arrive for this phase only once the barrier before it is complete.  With work in
@@ -1262,14 +1280,14 @@ __device__ __forceinline__ void tc_epilogue_phase(const TcParams& P, TcCtl* ctl,
     if (etid == 0) {
         // (the FC phase follows the gather barrier of its step, which its hidden-half operand does not imply)
         const int need = p == PH_FC ? s * TC_BARS_PER_STEP + TC_SEQ_GATHER : need_seq(s, p);
-        if ((lo == hi || p == PH_FC) && need >= 0)
+        if ((total == 0 || p == PH_FC) && need >= 0)
             wait_grid(a.bar_counter, ctl->bar_base + (u64)G * (u64)(need + 1), ctl, a.error_flag, 8);
         phase_stamp(a, s, phase_seq(p), cta, G);
         red_release_add_u64(a.bar_counter, 1ull);
     }
     // Without work in the phase nothing but the wait above tells this CTA that the earlier phases are complete:
     // hold the other epilogue threads until it is over (they read those phases' results early in the next one).
-    if (lo == hi) named_sync(TC_BAR_EPI, TC_EPI_THREADS);
+    if (total == 0) named_sync(TC_BAR_EPI, TC_EPI_THREADS);
 }
 
 }  // namespace
@@ -1302,6 +1320,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_chain_kernel(const __grid_co
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async_all();
     }
+    if (tid >= 64 && tid < 64 + PH_COUNT) tc_plan_phase(a, tid - 64, cta, G, ctl->plan[tid - 64]);
     if (tid == 96) ctl->bar_base = barrier_base(a.bar_counter, (unsigned)G) + a.bar_off;      // (warp 3 has no role)
     if (warp == 1) {
         __syncwarp();
@@ -1345,8 +1364,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_chain_kernel(const __grid_co
         // ring items of this CTA per step, and those before the attention items of step 0
         unsigned items_step = ai.total, items_before = 0;
         for (int p = 0; p < PH_COUNT; ++p) {
-            const PhaseShape sh = phase_shape(a, p);
-            const unsigned cnt = (unsigned)(range_lo(sh, cta + 1, G) - range_lo(sh, cta, G));
+            const unsigned cnt = (unsigned)ctl->plan[p].n;
             items_step += cnt;
             if (p < PH_O) items_before += cnt;
         }

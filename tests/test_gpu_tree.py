@@ -194,3 +194,28 @@ def test_tree_verify_rejects_everything_and_state_errors():
         assert e.value.code == -4
     finally:
         case.close()
+
+
+@pytest.mark.parametrize("name", ["mini_mha_b1", "c1_tiny_f32_b1"])
+def test_a_tree_whose_scores_are_not_numbers_stays_within_its_lists(name):
+    """Rows of the LM head that are not numbers make every node's log-sum-exp, and with it every score, not a number.  The tree
+    still has as many nodes as were asked for, each behind its parent, and the verification walks it."""
+    import torch
+    wl = hi.scaled(hi.workload(name), batch=1)
+    W = hi.make_weights(wl.dims, wl.seed)
+    W["lm_head"][5:40] = np.nan
+    case = Case(wl, W=W, max_len=200)
+    try:
+        dr = case.drafter
+        case.gpu_prefill()
+        toks, parents, scores, count = (t.cpu().numpy() for t in dr.draft_tree(0, 10, 6, 60, case.d_resid))
+        dr.status()
+        assert count[0] == 60 and np.isnan(scores).all()
+        assert ((parents >= -1) & (parents < np.arange(60))).all()
+        assert ((toks >= 0) & (toks < wl.dims.vocab)).all()
+        n, path, _, rows = dr.verify_tree(0, 6, torch.zeros((61, wl.dims.vocab), device="cuda"))
+        torch.cuda.synchronize()
+        dr.status()
+        assert 0 <= int(n[0]) <= 6 and int(rows[0]) >= int(case.lens[0])
+    finally:
+        case.close()
