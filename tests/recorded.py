@@ -66,8 +66,8 @@ def digest(*tensors):
     return h.hexdigest()[:16]
 
 
-# pairs of one prefix build: one pass, several, and the edges of the GEMMs' tiles
-BUILDS = [[2], [9], [16], [17], [33], [64], [65], [118], [257], [1, 3, 7, 2, 4, 5, 20], [100, 1, 200, 64]]
+# pairs of one prefix build: one pass, several, the edges of the GEMMs' tiles; enough for tiles of 256 weight rows
+BUILDS = [[2], [9], [16], [17], [33], [64], [65], [118], [257], [1, 3, 7, 2, 4, 5, 20], [100, 1, 200, 64], [390] * 7]
 
 
 def prefix_rows(shape, bias, project):
