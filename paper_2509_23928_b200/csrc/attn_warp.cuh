@@ -50,8 +50,8 @@ struct AttnWArgs {
     int lo_rows;
 };
 
-// Unit ranges of the warps.  32-bit arithmetic: units * warps stays far below 2^31 for every size the
-// library accepts (<= 16 sequences x 128 head groups x 513 units, a few thousand warps would still fit).
+// Unit ranges of the warps.  32-bit arithmetic: units * warps fits 32 bits (16 sequences x 128 heads x 513 blocks on 592
+// warps do five times over; for more than 16 sequences the host checks the product before it takes this path).
 __device__ __forceinline__ unsigned attw_lo(unsigned U, int g, int NW) { return U * (unsigned)g / (unsigned)NW; }
 __device__ __forceinline__ int attw_owner(unsigned U, int NW, unsigned u) {
     int g = (int)(u * (unsigned)NW / U);

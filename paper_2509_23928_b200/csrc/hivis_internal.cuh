@@ -184,8 +184,8 @@ struct TcArgs {
     u64* keys;                 // [B][key_stride]
     int key_stride;
     float *u, *qkv, *attn, *y, *feat;     // fp32 activations [B][width]
-    bf16 *feat_h, *xq_h, *attn_h, *xm_h, *act_h;   // bf16 operands [TC_OP_ROWS][width]
-    bf16* xe_h;                // [TC_OP_ROWS][d] embedding rows of the step's tokens (the set-up kernel zeroes rows >= B)
+    bf16 *feat_h, *xq_h, *attn_h, *xm_h, *act_h;   // bf16 operands [32, or 64 for more than 32 sequences][width]
+    bf16* xe_h;                // [the same][d] embedding rows of the step's tokens (the set-up kernel zeroes rows >= B)
     const bf16* embed;         // [V][d]
     float *ssq1, *ssq2;        // [tiles*4][16 x column groups] partial sums of squares of u / y
     float* logits_out;         // [B][k][V], nullable

@@ -18,9 +18,9 @@
 // runs under the next tile's MMAs; consecutive tiles go through the weight rows first (the weights stay in L2, the pairs
 // are read from memory once).
 //
-// 34 800 pairs of the LLaVA shape (16 sequences of 2176): 3.8 ms, 1.2 PFLOP/s (of 1.4 to 1.6 for a library GEMM; the SM
+// 34 800 pairs of the LLaVA shape (16 sequences of 2176): 3.5 ms, 1.35 PFLOP/s (of 1.4 to 1.7 for a library GEMM; the SM
 // clock drops to 1.3-1.5 GHz under the power cap); with 128 x 128 tiles, one per CTA and launch slot, and the tile turned in
-// shared memory for the output stage 7.9 ms.
+// shared memory for the output stage 7.9 ms.  17 to 256 pairs: 87 to 91 us, a serial chain of 128 k-blocks in GEMM 1.
 //
 // Warp 0 (one thread, both CTAs) issues the copies, warp 1 (one thread of the leader, rank 0) the MMAs for both, warps
 // 2-5 run the output stage.  A stage's full barrier lives in the leader and counts the bytes of both CTAs; tcgen05.commit
@@ -459,9 +459,11 @@ cudaError_t pf_launch_t(PfParams& P, int clusters, cudaStream_t st) {
 
 // Tile width, by the time of the busiest cluster in units of 10 ns a k-block (0.45 us at 256 weight rows, 0.33 at 128; below
 // that an MMA takes as long whatever its width).  117 / 500 pairs (d 4096 / 2560): 92 / 69 us at 256, 90 / 62 at 128; 600 and
-// 2048 pairs (d 4096 / 3584): 123 and 130 us at 256, 174 and 193 at 128.  A tile is never split over clusters: u and the cached
-// rows are rounded to bf16, and parts of their long sums added in fp32 instead of in the tensor core's accumulator move one
-// element in forty to the other side of a rounding.
+// 2048 pairs (d 4096 / 3584): 123 and 130 us at 256, 174 and 193 at 128.
+// A tile is never split over clusters, and no call goes through the chain kernel, whose phases are split over CTAs (64 pairs:
+// 45 us there, 89 here): u and the cached rows are rounded to bf16, and parts of their long sums added in fp32 instead of
+// in the tensor core's accumulator move one element in forty to the other side of a rounding.  Two to eleven of a hundred
+// cached elements then differ, enough to exchange nodes of a draft tree and to move a token drawn by inverse CDF.
 template <int EPI>
 cudaError_t pf_launch(PfParams& P, const void* W, int num_sms, cudaStream_t st) {
     const int clusters = num_sms / 2 > 0 ? num_sms / 2 : 1;

@@ -6,16 +6,17 @@
 //                        ring with TMA (cp.async.bulk.tensor, 128-byte swizzle, mbarrier complete_tx).
 //                        Weight tiles do not depend on activations, so their loads run ahead through phase
 //                        and step boundaries, limited only by the ring.
-//   warp 2 (one thread)  operand producer: the matching batch-operand tiles (32 rows x 64 k, 4 KB) in the
-//                        same order; the first tile of a phase waits for the grid barrier before it.
-//   warp 3               no role.
-//   warp 1 (one thread)  issues tcgen05.mma (M = 128 weight rows, N = 32 batch columns, K = 16, four per
-//                        stage), accumulating in tensor memory (two 32-column accumulators, so the next
+//   warp 2 (one thread)  operand producer: the matching batch-operand tiles (32 rows x 64 k, 4 KB; 64 rows, 8 KB for
+//                        more than 32 sequences) in the same order; the first tile of a phase waits for the grid
+//                        barrier before it.
+//   warp 3               no role after the set-up.
+//   warp 1 (one thread)  issues tcgen05.mma (M = 128 weight rows, N = 32 or 64 batch columns, K = 16, four per
+//                        stage), accumulating in tensor memory (two accumulators of N columns, so the next
 //                        tile's MMAs overlap the previous tile's epilogue); tcgen05.commit frees stages.
 //   The three single threads are the pace of the whole kernel: a stage's round trip (handed back -> copy
 //   issued -> landed -> MMAs issued -> handed back) bounds the bytes in flight, so their loops hold nothing
 //   that is not needed per item (one shared-memory load more per wait cost 2-4 % of a draft step).
-//   warps 4-7            epilogue: tcgen05.ld (one weight row per thread, 16 batch values), then the fused
+//   warps 4-7            epilogue: tcgen05.ld (one weight row per thread, 16 batch values at a time), then the fused
 //                        output stage of the phase (residuals, RMSNorm statistics and gains, RoPE-free
 //                        QKV bias, SiLU*up, LM-head argmax keys) and the bf16 operand of the next phase.
 //   warps 4-7            at the start of a step: embedding gather - once the step's tokens are known, their
@@ -33,11 +34,13 @@
 // writes its partial accumulator to global scratch and bumps the tile's arrival counter; the last one adds
 // the partials in a fixed order (so results do not depend on timing) and runs the output stage.  Where a
 // range is at least a tile long, the tile at its end is finished from an early look at the counter (the other
-// contributors did their part at the start of the phase).  Nobody waits for anybody inside a phase.
+// contributors did their part at the start of the phase).  Up to 16 sequences nobody waits for anybody inside a phase;
+// with more, and whole CTAs per tile, the contributors of a tile finish a part of its columns each and wait (bounded) for
+// the others' partials.
 //
-// Batch operand: activations are rounded to bf16 for the MMA; the rounding remainder of every activation is
-// fed through 16 more batch columns (rows [16, 32) of every operand buffer) and added in the output stage,
-// which keeps about 16 mantissa bits of the activations for every batch size.
+// Batch operand: activations are rounded to bf16 for the MMA.  Up to 16 sequences the rounding remainder of every
+// activation is fed through 16 more batch columns (rows [16, 32) of every operand buffer) and added in the output
+// stage, which keeps about 16 mantissa bits of the activations; with more sequences there are no remainders.
 //
 // Every wait is bounded.  A wait that runs out raises the error flag and poisons the CTA: the producers and the MMA issuer
 // stop where they are (after giving copies in flight time to land), the output warps run through their remaining
@@ -55,11 +58,11 @@
 // Geometry by the number NG of 16-sequence column groups of the launch.
 //   NG = 1 (up to 16 sequences): 32 batch columns, [0,16) the activations rounded to bf16, [16,32) their rounding
 //          remainders (an MMA of this shape costs the same for 16 and for 32 columns).
-//   NG = 2 (17..32), NG = 4 (33..64): 16 NG columns of rounded activations, no remainders.  The operand tile grows with
-//          the batch (8 KB beside the 16 KB of weights for 64 columns), so the ring has fewer stages; its bytes of weights
+//   NG = 2 (17..32), NG = 4 (33..64): 16 NG columns of rounded activations, no remainders.  For 64 columns the operand
+//          tile is 8 KB beside the 16 KB of weights, so the ring has nine stages instead of eleven; its bytes of weights
 //          in flight (9 x 16 KB x 148 SMs) are still three times what the memory's latency asks for.  One pass over the
 //          weights for all 64 sequences: a window of 64 ragged sequences (LLaVA shape, k = 5, 64..512 rows, prefix pairs
-//          included) takes 1.71 ms, where passes of 16 sequences through the per-phase kernels took 8.14 ms.
+//          included) takes 1.48 ms, where passes of 16 sequences through the per-phase kernels took 8.04 ms.
 #define TC_MAX_STAGES 11
 #define TC_A_BYTES (TC_TM * TC_BK * 2)
 template <int NG>
@@ -347,10 +350,11 @@ struct PhaseShape {
 // Phases with few row tiles (fusion FC, O, down) give every tile the same number of CTAs, each one run of its k-blocks,
 // where that keeps TC_ALIGN_PCT of the CTAs busy: no CTA has two tiles to publish, nobody finishes two in a row, and the
 // contributors of a tile are done together.  With contiguous ranges the slowest CTA of the fusion FC had its last
-// accumulator 9 us after the median one.  Batch 16 (d 4096, 704 rows) 1180 -> 1152 us per round, d 2560 batch 5 513 -> 488,
-// 64 sequences 1726 -> 1631; the 14 % of idle SMs cost nothing, HBM is the slower side.  Not for the levels of a draft tree
-// (TcArgs::whole_ctas): another split adds the sums in another order, and a tree's list of nodes hangs on differences
-// smaller than that.
+// accumulator 9 us after the median one.  Five draft steps, contiguous -> whole CTAs: d 4096, 2 / 16 sequences of 128 rows
+// 801 -> 788 / 818 -> 808 us, 16 of 704 or 64..512 rows level (1039 / 1040, 928 / 930); d 2560, 5 sequences 627 -> 593, 16 of 900
+// rows 1037 -> 993; 24 sequences 1105 -> 1040, 64 ragged ones 1475 -> 1347.  The idle SMs cost nothing, HBM is the slower
+// side.  Not for the levels of a draft tree (TcArgs::whole_ctas): another split adds the sums in another order, and a
+// tree's list of nodes hangs on differences smaller than that.
 #define TC_ALIGN_PCT 80
 // does this launch run the part of a step that arrives on barrier `seq`?
 __device__ __forceinline__ bool seq_on(const TcArgs& a, int seq) { return seq >= a.seq_first && seq <= a.seq_last; }
