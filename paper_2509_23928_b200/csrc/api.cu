@@ -778,6 +778,9 @@ static int draft_impl(hivis_ctx* c, int B, const int* seq_slots_host, int k, con
     // the per-phase kernels, as do draws for more than 16 sequences (refused below).
     const bool tc_fits = B <= 16 || (!uniforms && (long long)B * g.n_q_heads * ((max_rows + 31) / 32 + 1) * 4 * c->num_sms < (1ll << 32));
     const bool in_tc = !one_seq && c->tc_ok && c->opt_tc != 0 && tc_fits;
+    if (uniforms && !one_seq && !in_tc)
+        return fail(c, HIVIS_ERR_SHAPE, "drawing the drafted tokens runs in the chain kernels only: one sequence, or up to 16 "
+                    "sequences of a bf16 context with the kernels switched on");
     const bool raw_rho = resid && !c->resid_proj && (one_seq || in_tc);
     if (resid && !raw_rho) {
         rc = prepare_rho(c, resid, n_resid, st);
@@ -839,9 +842,6 @@ static int draft_impl(hivis_ctx* c, int B, const int* seq_slots_host, int k, con
         c->tap_mma = true;
         return HIVIS_OK;
     }
-    if (uniforms)
-        return fail(c, HIVIS_ERR_SHAPE, "drawing the drafted tokens runs in the chain kernels only: one sequence, or up to 16 "
-                    "sequences of a bf16 context with the kernels switched on");
     CKP(c, CLS_OTHER, st, launch_draft_setup(sl, k, d, c->d_slots, c->d_pos0, c->kv_len, c->pend_feat, c->pend_id, c->feat,
                               c->feat_h, c->cur_id, c->keys, c->key_stride, st));
     const bool mma = use_mma(c, B, false);

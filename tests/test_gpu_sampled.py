@@ -165,9 +165,11 @@ def test_sampled_drafting_refusals():
         B, k, V = wl.batch, wl.k, wl.dims.vocab
         case.gpu_prefill()
         u = torch.full((B, k, V), 0.5, device="cuda")
+        before = case.drafter.launch_count()
         with pytest.raises(HivisError) as e:
             case.drafter.draft_sampled(B, k, 1.0, u, case.d_resid)
         assert e.value.code == -2
+        assert case.drafter.launch_count() == before           # a refused call launches nothing
         with pytest.raises(HivisError) as e:
             case.drafter.draft_sampled(1, k, 0.0, u, case.d_resid)
         assert e.value.code == -1
