@@ -17,6 +17,12 @@
  *     default stream) and return without waiting; outputs are valid once the
  *     stream has been synchronised.  A context must always be used with work
  *     ordered on one stream at a time, and is not thread-safe.
+ *   - All calls but those that synchronise (hivis_init, hivis_get_kv_len,
+ *     hivis_status, hivis_read_phase_times and the profiling calls) may be
+ *     captured into a CUDA graph and replayed.  What the library keeps on the
+ *     host for its argument checks (bounds of the row counts, pending pairs,
+ *     k of the last draft) advances when a call is captured, not when it is
+ *     replayed: let a captured turn set its row counts first.
  *   - Every function returns HIVIS_OK (0) or a negative error code and never
  *     throws.  After an error nothing was launched unless the code is
  *     HIVIS_ERR_CUDA.  hivis_last_error gives a text for the last failure.

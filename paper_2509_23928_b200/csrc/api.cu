@@ -4,6 +4,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 #include <vector>
 
@@ -166,7 +167,7 @@ struct Carved {
     void** p;
     size_t bytes;
 };
-static bool dalloc_together(hivis_ctx* c, const std::vector<Carved>& list) {
+static bool dalloc_together(hivis_ctx* c, std::initializer_list<Carved> list) {
     size_t total = 0;
     for (const Carved& x : list) total += (x.bytes + 511) & ~(size_t)511;
     char* base = nullptr;
