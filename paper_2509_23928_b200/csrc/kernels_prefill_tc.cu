@@ -96,6 +96,14 @@ __device__ __forceinline__ void pf_cluster_sync() {
     __syncwarp();               // (aligned instructions)
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// One thread of a converged warp, known to the compiler to be one: MMAs are issued at the tensor core's pace (under a test of
+// the lane number one every 53 to 64 clocks, however small).  117 pairs at d 4096 and a draft of five: 826 -> 808 us.
+__device__ __forceinline__ bool pf_elect() {
+    uint32_t p;
+    __syncwarp();
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
 // copy into this CTA's shared memory that completes on a barrier of the leader
 __device__ __forceinline__ void pf_tma_2d(uint32_t dst, const void* map, int x, int y, uint32_t bar) {
     asm volatile(
@@ -318,7 +326,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1) prefi
     pf_fence_after();
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (pf_elect()) {
             unsigned it = 0;
             bool ok = true;
             for (int w = cluster; w < units && ok; w += n_clusters) {
@@ -338,7 +346,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1) prefi
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0 && pf_elect()) {
             const uint32_t tmem = ctl->tmem_base;
             unsigned it = 0, seg = 0;
             bool ok = true;

@@ -246,6 +246,17 @@ __device__ __forceinline__ void phase_stamp(const TcArgs& a, int s, int e, int c
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     a.phase_t[((long long)s * HIVIS_PHASE_EVENTS + e) * G + cta] = t;
 }
+// One thread of a converged warp, by elect.sync: the compiler then knows that a single thread runs what follows and issues
+// tcgen05 and bulk-copy instructions back to back.  Under a test of the lane number an MMA costs 53 clocks to issue (64 with a
+// commit for every four), whatever its shape; under this one the tensor core sets the pace (128 x 32 x 16: 44 clocks with the
+// commits).  Batch 16 at d 4096, five steps and refresh: 1028 -> 977 us with 64..512 rows, 1141 -> 1087 with 704; 64 sequences
+// 1514 -> 1431.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    __syncwarp();
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
 // (bar.sync is an aligned instruction: the lanes of a warp have to come to it together, whatever they did before)
 __device__ __forceinline__ void named_sync(int id, int n) {
     __syncwarp();
@@ -1340,16 +1351,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_chain_kernel(const __grid_co
     // the split of the attention units (the same for every step) and this CTA's ring items per step
     const TcAttInfo ai = tc_att_info<GQ>(a, cta, G);
     if (warp == 0) {
-        if (lane == 0) tc_producer_w<DH, GQ, NG>(P, ctl, smemA, cta, G, ai);
+        if (elect_one()) tc_producer_w<DH, GQ, NG>(P, ctl, smemA, cta, G, ai);
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             tc_mma_issuer<NG>(P, ctl, smemA, smemB, cta, G, ai.total);
             if (poisoned(ctl)) drain_after_poison();        // MMAs issued are over before tensor memory is freed
         }
         __syncwarp();
     } else if (warp == 2) {
-        if (lane == 0) tc_producer_x<NG>(P, ctl, smemB, cta, G, ai.total);
+        if (elect_one()) tc_producer_x<NG>(P, ctl, smemB, cta, G, ai.total);
         __syncwarp();
     } else if (warp >= 4) {
         // warps 4..7: the embedding gather at the start of a step, the epilogue of every GEMM phase and the attention
