@@ -516,7 +516,7 @@ static bool use_mma(const hivis_ctx* c, int B, bool prefill) {
 
 // fusion FC for rows [b0, b0+nb): u, gamma1*u (bf16), partial sums of squares
 static int run_fuse(hivis_ctx* c, bool mma, int b0, int nb, const float* feat, const void* feat_h,
-                    const int* ids, int id_stride, const u64* keys, const float* rho, cudaStream_t st) {
+                    const int* ids, int id_stride, const u64* keys, const float* rho, cudaStream_t st, const void* rho_w = nullptr) {
     const int d = c->cfg.d;
     LinArgs a;
     memset(&a, 0, sizeof(a));
@@ -524,6 +524,7 @@ static int run_fuse(hivis_ctx* c, bool mma, int b0, int nb, const float* feat, c
     a.feat = feat; a.feat_h = feat_h; a.embed = c->embed; a.vocab = c->cfg.vocab; a.id_flag = c->id_flag;
     a.ids = ids; a.id_stride = id_stride; a.keys = keys; a.key_stride = c->key_stride;
     a.rho = rho;
+    a.rho_w = rho_w;
     a.out = c->u + (long long)b0 * d;
     if (mma) {
         a.out_h = c->xq + (long long)b0 * d;
@@ -703,7 +704,7 @@ int hivis_prefill(hivis_ctx* c, int B, const int* seq_slots_host, const int32_t*
     const int d = c->cfg.d;
     const float* rho0 = nullptr;
     const bool gemms = c->pf_ok && c->opt_tc_prefill > 0 && total >= c->opt_tc_prefill;
-    const bool raw_rho = gemms && resid0 && !c->resid_proj;          // the row is read where the caller has it
+    const bool raw_rho = resid0 && !c->resid_proj;                   // the row is read where the caller has it
     if (resid0 && !raw_rho) {
         rc = prepare_rho(c, resid0, 1, st);
         if (rc) return rc;
@@ -736,7 +737,7 @@ int hivis_prefill(hivis_ctx* c, int B, const int* seq_slots_host, const int32_t*
             const int P = (int)(total - j0 < 16 ? total - j0 : 16);
             const char* hid = (const char*)hidden + j0 * d * c->esize;
             rc = run_fuse(c, mma, 0, P, mma ? nullptr : (const float*)hid, mma ? hid : nullptr, ids + j0, 1, nullptr,
-                          rho0, st);
+                          rho0, st, raw_rho ? resid0 : nullptr);
             if (rc) return rc;
             rc = run_qkv(c, mma, 0, P, c->qw, 2 * c->kvw, c->qkv, st);   // K and V rows only
             if (rc) return rc;

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "../../include/hivis.h"
 
 typedef __nv_bfloat16 bf16;
@@ -47,6 +49,7 @@ struct LinArgs {
     // ---- output stage
     const void* bias;     // EPI_QKV: [N] context dtype, nullable
     const float* rho;     // EPI_FUSE: [N] fp32 residual row, nullable
+    const void* rho_w;    // EPI_FUSE: the caller's row in the context dtype, read where rho is null (nullable)
     const float* addend;  // EPI_OPROJ (u), EPI_DOWN (y): [B][N] fp32
     float* out;           // fp32 result [B][N] (EPI_GATEUP: [B][N/2]); nullable
     bf16* out_h;          // bf16 copy [B][N] (EPI_GATEUP: [B][N/2]); nullable
@@ -403,6 +406,26 @@ __device__ __forceinline__ void store_from_float<float>(void* p, long long i, fl
 template <>
 __device__ __forceinline__ void store_from_float<bf16>(void* p, long long i, float v) {
     ((bf16*)p)[i] = __float2bfloat16_rn(v);
+}
+
+// Programmatic dependent launch.  pdl_wait: the launches before this one are complete and their writes visible.  pdl_trigger:
+// the launch after this one may begin (it waits itself).  A kernel launched with launch_pdl calls pdl_wait before it reads or
+// writes what other launches of the stream may touch, and before it ends.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
 // 16-byte streaming load of weights: read-only path, do not keep in L1.

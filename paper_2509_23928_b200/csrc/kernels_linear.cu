@@ -22,8 +22,8 @@ __device__ __forceinline__ void epilogue_pair(const LinArgs& a, int b, int row, 
     if (EPI == EPI_FUSE || EPI == EPI_OPROJ) {
         float r0, r1 = 0.f;
         if (EPI == EPI_FUSE) {
-            r0 = v0 + (a.rho ? a.rho[row] : 0.f);
-            if (has2) r1 = v1 + (a.rho ? a.rho[row + 1] : 0.f);
+            r0 = v0 + (a.rho ? a.rho[row] : a.rho_w ? load_as_float<WT>(a.rho_w, row) : 0.f);
+            if (has2) r1 = v1 + (a.rho ? a.rho[row + 1] : a.rho_w ? load_as_float<WT>(a.rho_w, row + 1) : 0.f);
         } else {
             r0 = a.addend[o] + v0;
             if (has2) r1 = a.addend[o + 1] + v1;
@@ -279,7 +279,9 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], unsigned a0, unsigned a1
 template <int NI, int PRO, int EPI>
 __global__ void __launch_bounds__(256) gemm_mma_kernel(const LinArgs a) {
     constexpr int MI = HIVIS_MMA_TILE_ROWS / 16;
-    constexpr int U = 2;
+    // k-blocks per batch of loads, two batches in flight: 64 KB per CTA.  With two k-blocks, all used before the next were asked for,
+    // and launches that began when the one before was over, the prefix rows of 1..16 pairs (d 4096) took 81..99 us; now 66..75.
+    constexpr int U = 4;
     __shared__ float red[8][NI * 8][MI * 16 + 1];
     __shared__ float s_scale[NI * 8];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -288,6 +290,30 @@ __global__ void __launch_bounds__(256) gemm_mma_kernel(const LinArgs a) {
     const int nblk = (nch + 3) >> 2;
     const uint4 zero = make_uint4(0, 0, 0, 0);
 
+    const uint4* wrow[MI][2];
+    bool wok[MI][2];
+#pragma unroll
+    for (int mi = 0; mi < MI; ++mi)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const long long r = row_base + mi * 16 + g + 8 * h;
+            wok[mi][h] = r < a.N;
+            wrow[mi][h] = (const uint4*)((const bf16*)a.W + (wok[mi][h] ? r : 0) * a.K);
+        }
+    auto fetch = [&](int blk, uint4 (&A)[U][MI][2]) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int c = (blk + 8 * u) * 4 + t;
+#pragma unroll
+            for (int mi = 0; mi < MI; ++mi)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) A[u][mi][h] = (c < nch && wok[mi][h]) ? ld_stream(wrow[mi][h] + c) : zero;
+        }
+    };
+    uint4 A[U][MI][2];
+    fetch(warp, A);                 // the first weights are in flight while the launch before this one ends
+    pdl_wait();
+    pdl_trigger();
     if (EPI == EPI_QKV || EPI == EPI_GATEUP) {
         if (tid < NI * 8) {
             float s = 1.f;
@@ -300,16 +326,6 @@ __global__ void __launch_bounds__(256) gemm_mma_kernel(const LinArgs a) {
         }
     }
 
-    const uint4* wrow[MI][2];
-    bool wok[MI][2];
-#pragma unroll
-    for (int mi = 0; mi < MI; ++mi)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const long long r = row_base + mi * 16 + g + 8 * h;
-            wok[mi][h] = r < a.N;
-            wrow[mi][h] = (const uint4*)((const bf16*)a.W + (wok[mi][h] ? r : 0) * a.K);
-        }
     // batch operand: row n = g + 8*ni; for PRO_FUSE the row is [feature ; embedding of its token]
     const uint4* xa[NI];
     const uint4* xb[NI];
@@ -337,17 +353,13 @@ __global__ void __launch_bounds__(256) gemm_mma_kernel(const LinArgs a) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[mi][ni][i] = 0.f;
 
+    // (the next batch of weights is on its way while one is used; a warp's k-blocks are added in ascending order whatever U)
     for (int blk = warp; blk < nblk; blk += 8 * U) {
-        uint4 A[U][MI][2], X[U][NI];
+        uint4 X[U][NI], N[U][MI][2];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int c = (blk + 8 * u) * 4 + t;
             const bool okc = c < nch;
-#pragma unroll
-            for (int mi = 0; mi < MI; ++mi)
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-                    A[u][mi][h] = (okc && wok[mi][h]) ? ld_stream(wrow[mi][h] + c) : zero;
 #pragma unroll
             for (int ni = 0; ni < NI; ++ni) {
                 const uint4* p;
@@ -356,6 +368,7 @@ __global__ void __launch_bounds__(256) gemm_mma_kernel(const LinArgs a) {
                 X[u][ni] = (okc && xok[ni]) ? ld_act(p) : zero;
             }
         }
+        fetch(blk + 8 * U, N);
 #pragma unroll
         for (int u = 0; u < U; ++u)
 #pragma unroll
@@ -367,6 +380,12 @@ __global__ void __launch_bounds__(256) gemm_mma_kernel(const LinArgs a) {
                     mma_bf16(acc[mi][ni], A[u][mi][0].z, A[u][mi][1].z, A[u][mi][0].w, A[u][mi][1].w,
                              X[u][ni].z, X[u][ni].w);
                 }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int mi = 0; mi < MI; ++mi)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) A[u][mi][h] = N[u][mi][h];
     }
     // every warp holds a partial sum over its share of k: reduce across the 8 warps in fixed order
 #pragma unroll
@@ -415,12 +434,9 @@ __global__ void __launch_bounds__(256) gemm_mma_kernel(const LinArgs a) {
 
 template <int NI>
 static cudaError_t launch_mma_n(int pro, int epi, const LinArgs& a, cudaStream_t st) {
-    const unsigned grid = (unsigned)((a.N + HIVIS_MMA_TILE_ROWS - 1) / HIVIS_MMA_TILE_ROWS);
+    const dim3 grid((unsigned)((a.N + HIVIS_MMA_TILE_ROWS - 1) / HIVIS_MMA_TILE_ROWS));
 #define HIVIS_MMA_CASE(P, E)                                    \
-    if (pro == P && epi == E) {                                 \
-        gemm_mma_kernel<NI, P, E><<<grid, 256, 0, st>>>(a);     \
-        return cudaGetLastError();                              \
-    }
+    if (pro == P && epi == E) return launch_pdl(gemm_mma_kernel<NI, P, E>, grid, dim3(256), 0, st, a);
     HIVIS_MMA_CASE(PRO_FUSE, EPI_FUSE)
     HIVIS_MMA_CASE(PRO_PLAIN, EPI_QKV)
     HIVIS_MMA_CASE(PRO_PLAIN, EPI_OPROJ)

@@ -83,6 +83,8 @@ __global__ void prefill_setup_kernel(SlotList sl, CuSeqlens cu, SlotList start, 
                                      const void* hidden, int* kv_len, float* pend_feat, int* pend_id,
                                      int* slot_of, int* row_of) {
     __shared__ int s_base;
+    pdl_wait();
+    pdl_trigger();
     const int b = blockIdx.x, slot = sl.slot[b];
     const int lo = cu.v[b], hi = cu.v[b + 1];
     if (threadIdx.x == 0) s_base = start.slot[b] >= 0 ? start.slot[b] : kv_len[slot];
@@ -103,13 +105,8 @@ cudaError_t launch_prefill_setup(int dtype, const SlotList& sl, const CuSeqlens&
                                  int d, const int32_t* ids, const void* hidden, int* kv_len,
                                  float* pend_feat, int* pend_id, int* slot_of, int* row_of,
                                  cudaStream_t st) {
-    if (dtype == HIVIS_BF16)
-        prefill_setup_kernel<bf16><<<sl.n, 256, 0, st>>>(sl, cu, start, d, ids, hidden, kv_len, pend_feat,
-                                                         pend_id, slot_of, row_of);
-    else
-        prefill_setup_kernel<float><<<sl.n, 256, 0, st>>>(sl, cu, start, d, ids, hidden, kv_len, pend_feat,
-                                                          pend_id, slot_of, row_of);
-    return cudaGetLastError();
+    return launch_pdl(dtype == HIVIS_BF16 ? prefill_setup_kernel<bf16> : prefill_setup_kernel<float>, dim3(sl.n), dim3(256), 0, st, sl, cu,
+                      start, d, ids, hidden, kv_len, pend_feat, pend_id, slot_of, row_of);
 }
 
 // Blocks [0, pairs): the embedding row of pair j, 16 bytes per thread and turn; then one block per sequence (rows, pending
@@ -173,6 +170,8 @@ template <typename WT>
 __global__ void __launch_bounds__(256) kv_append_kernel(const float* kv, const int* slot_of, const int* row_of,
                                                         const double* inv_freq, int Hkv, int dh, int max_len, void* Kc, void* Vc) {
     __shared__ float2 s_cs[64];
+    pdl_wait();
+    pdl_trigger();
     const int j = blockIdx.x;
     const int row = row_of[j];
     if (row < 0) return;
@@ -211,11 +210,8 @@ cudaError_t launch_kv_append(int dtype, const float* kv, int P, const int* slot_
                              cudaStream_t st) {
     if (P <= 0) return cudaSuccess;
     const dim3 grid((unsigned)P, KV_APPEND_CTAS);
-    if (dtype == HIVIS_BF16)
-        kv_append_kernel<bf16><<<grid, 256, 0, st>>>(kv, slot_of, row_of, inv_freq, Hkv, dh, max_len, Kc, Vc);
-    else
-        kv_append_kernel<float><<<grid, 256, 0, st>>>(kv, slot_of, row_of, inv_freq, Hkv, dh, max_len, Kc, Vc);
-    return cudaGetLastError();
+    return launch_pdl(dtype == HIVIS_BF16 ? kv_append_kernel<bf16> : kv_append_kernel<float>, grid, dim3(256), 0, st, kv, slot_of, row_of,
+                      inv_freq, Hkv, dh, max_len, Kc, Vc);
 }
 
 // ------------------------------------------------------------------------------------------
