@@ -27,7 +27,7 @@ struct hivis_ctx {
     float* pend_feat;
     // per-call work
     int *d_slots, *d_pos0, *cur_id;
-    float *feat, *u, *qkv, *attn, *y, *act, *rho_raw, *rho, *ssq1, *ssq2;
+    float *feat, *u, *qkv, *attn, *y, *act, *rho, *ssq1, *ssq2;
     bf16 *feat_h, *xq, *attn_h, *xm, *act_h;
     u64* keys;
     int key_stride;
@@ -332,7 +332,6 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
                              {(void**)&c->attn, 4ull * R * c->qw}, {(void**)&c->attn_h, 2ull * R * c->qw},
                              {(void**)&c->y, 4ull * R * d}, {(void**)&c->xm, 2ull * R * d}, {(void**)&c->act, 4ull * R * F},
                              {(void**)&c->act_h, 2ull * R * F}, {(void**)&c->xe_h, 2ull * R * d}}) &&
-         dalloc(c, &c->rho_raw, (long long)HIVIS_MAX_K * d) &&
          dalloc(c, &c->rho, (long long)HIVIS_MAX_K * d) && dalloc(c, &c->ssq1, tiles1 * R) &&
          dalloc(c, &c->ssq2, tiles1 * R) && dalloc(c, &c->keys, R * c->key_stride) &&
          dalloc(c, &c->vkeys, MB * (cfg->max_k + 1)) && dalloc(c, &c->varrive, MB) &&
@@ -466,15 +465,8 @@ int hivis_init(hivis_ctx** out, const hivis_config* cfg, const hivis_weights* w,
 // residual rows in the context dtype -> fp32 rho rows (projected by resid_proj when present)
 static int prepare_rho(hivis_ctx* c, const void* resid, int R, cudaStream_t st) {
     const int d = c->cfg.d;
-    float* dst = c->resid_proj ? c->rho_raw : c->rho;
-    CKL(c, launch_convert_rows(c->dtype, resid, dst, (long long)R * d, st));
-    if (c->resid_proj) {
-        LinArgs a;
-        memset(&a, 0, sizeof(a));
-        a.W = c->resid_proj; a.N = d; a.K = d; a.B = R; a.ldb = c->rows_cap;
-        a.xin = c->rho_raw; a.out = c->rho;
-        CKL(c, launch_gemv_alu(c->dtype, PRO_PLAIN, EPI_QKV, a, st));
-    }
+    if (c->resid_proj) CKL(c, launch_project_rows(c->dtype, c->resid_proj, resid, R, d, c->rho, st));
+    else CKL(c, launch_convert_rows(c->dtype, resid, c->rho, (long long)R * d, st));
     return HIVIS_OK;
 }
 

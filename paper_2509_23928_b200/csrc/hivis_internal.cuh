@@ -313,7 +313,9 @@ cudaError_t launch_draft_setup(const SlotList& sl, int k, int d, int* d_slots, i
 cudaError_t launch_draft_finish(int B, int k, const u64* keys, int key_stride, int32_t* out_ids,
                                 cudaStream_t st);
 
-// residual rows (context dtype) -> fp32 rho [R][d] (no projection)
+// residual rows (context dtype) -> fp32 rho [R][d], projected by W [d][d]
+cudaError_t launch_project_rows(int dtype, const void* W, const void* rows, int R, int d, float* out, cudaStream_t st);
+// the same without a projection
 cudaError_t launch_convert_rows(int dtype, const void* src, float* dst, long long n, cudaStream_t st);
 cudaError_t launch_f32_to_bf16(const float* src, bf16* dst, long long n, cudaStream_t st);
 cudaError_t launch_bf16_to_f32(const bf16* src, float* dst, long long n, cudaStream_t st);

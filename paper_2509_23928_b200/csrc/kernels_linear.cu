@@ -251,7 +251,6 @@ template <typename WT>
 static cudaError_t launch_alu_d(int pro, int epi, const LinArgs& a, cudaStream_t st) {
     if (pro == PRO_FUSE && epi == EPI_FUSE) return launch_alu_t<WT, PRO_FUSE, EPI_FUSE>(a, st);
     if (pro == PRO_NORM && epi == EPI_QKV) return launch_alu_t<WT, PRO_NORM, EPI_QKV>(a, st);
-    if (pro == PRO_PLAIN && epi == EPI_QKV) return launch_alu_t<WT, PRO_PLAIN, EPI_QKV>(a, st);
     if (pro == PRO_PLAIN && epi == EPI_OPROJ) return launch_alu_t<WT, PRO_PLAIN, EPI_OPROJ>(a, st);
     if (pro == PRO_NORM && epi == EPI_GATEUP) return launch_alu_t<WT, PRO_NORM, EPI_GATEUP>(a, st);
     if (pro == PRO_PLAIN && epi == EPI_DOWN) return launch_alu_t<WT, PRO_PLAIN, EPI_DOWN>(a, st);
@@ -262,6 +261,110 @@ static cudaError_t launch_alu_d(int pro, int epi, const LinArgs& a, cudaStream_t
 cudaError_t launch_gemv_alu(int dtype, int pro, int epi, const LinArgs& a, cudaStream_t st) {
     if (a.B <= 0 || a.N <= 0) return cudaSuccess;
     return dtype == HIVIS_BF16 ? launch_alu_d<bf16>(pro, epi, a, st) : launch_alu_d<float>(pro, epi, a, st);
+}
+
+// ==========================================================================================
+// projected residual rows
+// ==========================================================================================
+// out[r][n] = sum_k W[n][k] rows[r][k] for up to NB rows at a time, every sum in the order of gemv_alu_kernel (with which the
+// recorded rows were made).  It is one pass over W (33 MB at d 4096): with a CTA per residual row and sixteen weight rows W came
+// from L2 once per residual row, behind a launch that widened the rows.
+template <typename WT, int NB>
+__global__ void __launch_bounds__(256) project_rows_kernel(const void* W, const void* rows, int R, int d, float* out) {
+    extern __shared__ __align__(16) float xs[];
+    constexpr int U = 4;
+    constexpr int VEC = 16 / (int)sizeof(WT);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nch = d / VEC, r0 = blockIdx.y * NB;
+    const uint4 zero = make_uint4(0, 0, 0, 0);
+    const long long row0 = ((long long)blockIdx.x * 8 + warp) * 2;
+    const bool has1 = row0 < d, has2 = row0 + 1 < d;
+    const uint4* w0 = (const uint4*)((const WT*)W + (has1 ? row0 : 0) * d);
+    const uint4* w1 = w0 + nch;
+    uint4 c0[U], c1[U];
+    auto fetch = [&](int cb, uint4* v0, uint4* v1) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int cc = cb + lane + 32 * u;
+            v0[u] = cc < nch && has1 ? ld_stream(w0 + cc) : zero;
+            v1[u] = cc < nch && has2 ? ld_stream(w1 + cc) : zero;
+        }
+    };
+    fetch(0, c0, c1);                   // the first weights are in flight while the launch before this one ends
+    pdl_wait();
+    pdl_trigger();
+    for (int b = 0; b < NB; ++b)
+        for (int k = threadIdx.x; k < d; k += 256)
+            xs[b * d + xs_index<WT>(k, d)] = r0 + b < R ? load_as_float<WT>(rows, (long long)(r0 + b) * d + k) : 0.f;
+    __syncthreads();
+    float acc0[NB], acc1[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) acc0[b] = acc1[b] = 0.f;
+    for (int cb = 0; cb < nch; cb += 32 * U) {
+        uint4 n0[U], n1[U];
+        fetch(cb + 32 * U, n0, n1);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int cc = cb + lane + 32 * u;
+            if (cc >= nch) break;
+            const uint4 p = c0[u], q = c1[u];
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                const float4 xa = ((const float4*)(xs + b * d))[cc];
+                if (sizeof(WT) == 2) {
+                    const float4 xb = ((const float4*)(xs + b * d + (d >> 1)))[cc];
+                    acc0[b] = fmaf(bf16_lo(p.x), xa.x, acc0[b]); acc0[b] = fmaf(bf16_hi(p.x), xa.y, acc0[b]);
+                    acc0[b] = fmaf(bf16_lo(p.y), xa.z, acc0[b]); acc0[b] = fmaf(bf16_hi(p.y), xa.w, acc0[b]);
+                    acc0[b] = fmaf(bf16_lo(p.z), xb.x, acc0[b]); acc0[b] = fmaf(bf16_hi(p.z), xb.y, acc0[b]);
+                    acc0[b] = fmaf(bf16_lo(p.w), xb.z, acc0[b]); acc0[b] = fmaf(bf16_hi(p.w), xb.w, acc0[b]);
+                    acc1[b] = fmaf(bf16_lo(q.x), xa.x, acc1[b]); acc1[b] = fmaf(bf16_hi(q.x), xa.y, acc1[b]);
+                    acc1[b] = fmaf(bf16_lo(q.y), xa.z, acc1[b]); acc1[b] = fmaf(bf16_hi(q.y), xa.w, acc1[b]);
+                    acc1[b] = fmaf(bf16_lo(q.z), xb.x, acc1[b]); acc1[b] = fmaf(bf16_hi(q.z), xb.y, acc1[b]);
+                    acc1[b] = fmaf(bf16_lo(q.w), xb.z, acc1[b]); acc1[b] = fmaf(bf16_hi(q.w), xb.w, acc1[b]);
+                } else {
+                    acc0[b] = fmaf(__uint_as_float(p.x), xa.x, acc0[b]); acc0[b] = fmaf(__uint_as_float(p.y), xa.y, acc0[b]);
+                    acc0[b] = fmaf(__uint_as_float(p.z), xa.z, acc0[b]); acc0[b] = fmaf(__uint_as_float(p.w), xa.w, acc0[b]);
+                    acc1[b] = fmaf(__uint_as_float(q.x), xa.x, acc1[b]); acc1[b] = fmaf(__uint_as_float(q.y), xa.y, acc1[b]);
+                    acc1[b] = fmaf(__uint_as_float(q.z), xa.z, acc1[b]); acc1[b] = fmaf(__uint_as_float(q.w), xa.w, acc1[b]);
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) { c0[u] = n0[u]; c1[u] = n1[u]; }
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            acc0[b] += __shfl_xor_sync(0xffffffffu, acc0[b], o);
+            acc1[b] += __shfl_xor_sync(0xffffffffu, acc1[b], o);
+        }
+        if (lane == 0 && r0 + b < R) {
+            if (has1) out[(long long)(r0 + b) * d + row0] = acc0[b];
+            if (has2) out[(long long)(r0 + b) * d + row0 + 1] = acc1[b];
+        }
+    }
+}
+template <typename WT, int NB>
+static cudaError_t launch_project_t(const void* W, const void* rows, int R, int d, float* out, cudaStream_t st) {
+    static bool attr_set[HIVIS_MAX_DEVICES] = {false};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= HIVIS_MAX_DEVICES || !attr_set[dev]) {
+        e = cudaFuncSetAttribute(project_rows_kernel<WT, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < HIVIS_MAX_DEVICES) attr_set[dev] = true;
+    }
+    return launch_pdl(project_rows_kernel<WT, NB>, dim3((unsigned)((d + 15) / 16), (unsigned)((R + NB - 1) / NB)), dim3(256),
+                      (size_t)NB * d * sizeof(float), st, W, rows, R, d, out);
+}
+// out = rows W^T; rows in the context dtype.  Four rows at a time where their fp32 values fit shared memory.
+cudaError_t launch_project_rows(int dtype, const void* W, const void* rows, int R, int d, float* out, cudaStream_t st) {
+    if ((size_t)d * sizeof(float) > 200 * 1024) return cudaErrorInvalidValue;
+    const bool four = R > 1 && (size_t)4 * d * sizeof(float) <= 200 * 1024;
+    if (dtype == HIVIS_BF16)
+        return four ? launch_project_t<bf16, 4>(W, rows, R, d, out, st) : launch_project_t<bf16, 1>(W, rows, R, d, out, st);
+    return four ? launch_project_t<float, 4>(W, rows, R, d, out, st) : launch_project_t<float, 1>(W, rows, R, d, out, st);
 }
 
 // ==========================================================================================
