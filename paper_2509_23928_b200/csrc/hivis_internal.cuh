@@ -143,6 +143,7 @@ struct ChainArgs {
     long long wait_cycles;     // limit of every device-side wait, in SM clock cycles
     int* error_flag;           // set non-zero by a kernel that gave up on a wait
     int* id_flag;              // set non-zero when a token id outside [0, V) reached the embedding lookup
+    int attn_rows;             // cache rows of a unit that shared memory holds, filled by the launcher
     int off_x, off_part, off_bar, off_misc;   // shared-memory layout, filled by the launcher
 };
 // shared memory the kernel needs for these dimensions on `grid` CTAs; 0 = does not fit

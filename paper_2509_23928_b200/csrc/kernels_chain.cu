@@ -88,11 +88,14 @@ struct ChainMisc {
     u64 bar_base;              // value of the barrier counter when the launch began
 };
 
-// Grid-wide barrier on a monotonically increasing counter.  false = gave up (error flag raised).
-__device__ __forceinline__ bool grid_barrier(const ChainArgs& a, ChainMisc* misc, u64 target) {
+// Grid-wide barrier on a monotonically increasing counter, in two halves: what does not need the others' results goes between.
+__device__ __forceinline__ void grid_arrive(const ChainArgs& a) {
     __syncthreads();
+    if (threadIdx.x == 0) red_release_add_u64(a.bar_counter, 1ull);
+}
+// false = gave up (error flag raised)
+__device__ __forceinline__ bool grid_wait(const ChainArgs& a, ChainMisc* misc, u64 target) {
     if (threadIdx.x == 0) {
-        red_release_add_u64(a.bar_counter, 1ull);
         const long long t0 = clock64();
         unsigned it = 0;
         bool ok = true;
@@ -161,6 +164,220 @@ __device__ __forceinline__ float dot_chunk(const uint4* wsm, const float* xs, in
     return acc;
 }
 
+// ---- attention -----------------------------------------------------------------------------------
+// A unit = (split of the cache rows, query head), a CTA each; the arithmetic and its order are attn_unit's (attn_body.cuh, one
+// head per unit), so the results are the same bits.  What bounds it is a chain of latencies: with attn_unit, one or two warps of a
+// CTA working from global memory, the phase took 29 000 clocks of a step's 286 000 (d 4096, 128 rows), 15 000 of 52 000 at d 256.
+// So the unit's rows of K and V, which earlier steps have written, are copied to shared memory by all warps before the grid
+// barrier is awaited, and the angles worked out there; q, k and v are rotated side by side, the new row being one more row of
+// the copies; warps without rows are left out of the merge; the splits' partial results come in one round trip.  Units whose
+// rows shared memory does not hold take attn_unit.
+// (No more registers than the projections need: the acquire of a grid barrier empties L1, so a spilled register comes back from
+// L2.  A variant with rows in registers spilled 100 words and made a step 24 us slower.)
+template <typename WT, int DH>
+struct ChainAttnSmem {
+    static constexpr int KROW = DH * (int)sizeof(WT) + 16;       // bytes from K row to K row: lanes read rows side by side
+    static constexpr int VROW = DH * (int)sizeof(WT);
+    alignas(16) float q[DH];
+    float2 cs[DH / 2];
+    float m[CHAIN_WARPS], l[CHAIN_WARPS];
+    alignas(16) float acc[CHAIN_WARPS][DH];
+    int last;
+    alignas(16) unsigned char rows[16];                          // K rows [attn_rows][KROW], V rows [attn_rows][VROW]
+};
+template <typename WT, int DH>
+__device__ __forceinline__ void chain_attn_prepare(const ChainArgs& a, ChainAttnSmem<WT, DH>& sm, int unit, int p, int slot) {
+    typedef ChainAttnSmem<WT, DH> S;
+    constexpr int NCH = S::VROW / 16;
+    const int split = unit % a.attn_nsplit, kvh = unit / a.attn_nsplit / (a.Hq / a.Hkv);
+    const int r0 = split * a.attn_chunk, n = min(p, r0 + a.attn_chunk) - r0;     // rows without the new one
+    const int tid = threadIdx.x;
+    const long long row0 = (((long long)slot * a.Hkv + kvh) * a.max_len + r0) * (long long)DH;
+    const char* K = (const char*)((const WT*)a.Kc + row0);
+    const char* V = (const char*)((const WT*)a.Vc + row0);
+    const uint32_t ks = smem_addr(sm.rows), vs = ks + a.attn_rows * S::KROW;
+#pragma unroll 2
+    for (int i = tid; i < n * NCH; i += CHAIN_THREADS) {
+        const int r = i / NCH, c = i - r * NCH;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(ks + r * S::KROW + c * 16), "l"(K + (long long)i * 16) : "memory");
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(vs + i * 16), "l"(V + (long long)i * 16) : "memory");
+    }
+    if (tid < DH / 2) {
+        float c, s;
+        rope_cs(p, a.inv_freq[tid], c, s);
+        sm.cs[tid] = make_float2(c, s);
+    }
+}
+template <typename WT, int DH>
+__device__ __forceinline__ void chain_attn_run(const ChainArgs& a, ChainAttnSmem<WT, DH>& sm, int unit, int p, int slot) {
+    typedef ChainAttnSmem<WT, DH> S;
+    constexpr int EPL = DH / 32;                 // head-dim elements per lane in the PV phase
+    constexpr int NCH = S::VROW / 16;            // 16-byte vectors of a row
+    constexpr int half = DH / 2;
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    const int nsplits = (p + a.attn_chunk) / a.attn_chunk, split = unit % a.attn_nsplit, h = unit / a.attn_nsplit;
+    if (split >= nsplits) return;
+    const int r0 = split * a.attn_chunk, n = min(p + 1, r0 + a.attn_chunk) - r0, kvh = h / (a.Hq / a.Hkv);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    unsigned char* const ks = sm.rows;
+    unsigned char* const vs = sm.rows + a.attn_rows * S::KROW;
+    __syncthreads();                             // the angles and the copies
+    {
+        // q of the head, and the new row of the unit that has it; one unit per KV head appends the row to the cache
+        const int pn = p - r0;
+        const bool owns_new = pn < n, writer = owns_new && h % (a.Hq / a.Hkv) == 0;
+        const long long row = (((long long)slot * a.Hkv + kvh) * a.max_len + p) * (long long)DH;
+        if (tid < DH) {
+            const bool is_q = tid < half;
+            const int j = is_q ? tid : tid - half;
+            if (is_q || owns_new) {
+                const float* x = a.qkv + (is_q ? h * DH : a.qw + kvh * DH);
+                const float x0 = __ldcg(x + j), x1 = __ldcg(x + j + half);
+                const float2 cs = sm.cs[j];
+                // (written out, so that every build of the code rounds the same product)
+                const float y0 = fmaf(x0, cs.x, -__fmul_rn(x1, cs.y)), y1 = fmaf(x1, cs.x, __fmul_rn(x0, cs.y));
+                if (is_q) {
+                    sm.q[j] = y0 * a.scale;
+                    sm.q[j + half] = y1 * a.scale;
+                } else {
+                    store_from_float<WT>(ks + pn * S::KROW, j, y0);
+                    store_from_float<WT>(ks + pn * S::KROW, j + half, y1);
+                    if (writer) {
+                        store_from_float<WT>(a.Kc, row + j, y0);
+                        store_from_float<WT>(a.Kc, row + j + half, y1);
+                    }
+                }
+            }
+        } else if (tid < 2 * DH && owns_new) {
+            const int j = tid - DH;
+            const float v = __ldcg(a.qkv + a.qw + a.kvw + kvh * DH + j);
+            store_from_float<WT>(vs + pn * S::VROW, j, v);
+            if (writer) store_from_float<WT>(a.Vc, row + j, v);
+        }
+    }
+    __syncthreads();
+
+    float m_run = -INFINITY, l_run = 0.f, acc[EPL];
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
+#pragma unroll 1
+    for (int base = warp * 32; base < n; base += CHAIN_THREADS) {
+        const int r = base + lane;
+        const bool ok = r < n;
+        float s = 0.f;
+        const uint4* k4 = (const uint4*)(ks + (ok ? r : base) * S::KROW);
+        const float4* q4 = (const float4*)sm.q;
+#pragma unroll 4
+        for (int c = 0; c < NCH; ++c) {
+            const uint4 w = k4[c];
+            if constexpr (sizeof(WT) == 2) {
+                const float4 qa = q4[2 * c], qb = q4[2 * c + 1];
+                s = fmaf(qa.x, bf16_lo(w.x), s); s = fmaf(qa.y, bf16_hi(w.x), s);
+                s = fmaf(qa.z, bf16_lo(w.y), s); s = fmaf(qa.w, bf16_hi(w.y), s);
+                s = fmaf(qb.x, bf16_lo(w.z), s); s = fmaf(qb.y, bf16_hi(w.z), s);
+                s = fmaf(qb.z, bf16_lo(w.w), s); s = fmaf(qb.w, bf16_hi(w.w), s);
+            } else {
+                const float4 qa = q4[c];
+                s = fmaf(qa.x, __uint_as_float(w.x), s); s = fmaf(qa.y, __uint_as_float(w.y), s);
+                s = fmaf(qa.z, __uint_as_float(w.z), s); s = fmaf(qa.w, __uint_as_float(w.w), s);
+            }
+        }
+        // online softmax over this block of 32 rows
+        const float sv = ok ? s : -INFINITY;
+        float mb = sv;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+        const float mn = fmaxf(m_run, mb);       // finite: the block has at least one valid row
+        const float corr = expf(m_run - mn);
+        const float pr = ok ? expf(sv - mn) : 0.f;
+        float ps = pr;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, o);
+        l_run = l_run * corr + ps;
+        m_run = mn;
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) acc[e] *= corr;
+        // PV: lane owns head-dim elements [lane * EPL, + EPL)
+        const int nrows = min(32, n - base);
+        const unsigned char* v0 = vs + base * S::VROW + lane * EPL * (int)sizeof(WT);
+#pragma unroll 8
+        for (int j = 0; j < nrows; ++j) {
+            const float pj = __shfl_sync(0xffffffffu, pr, j);
+            constexpr int VW = EPL * (int)sizeof(WT) / 4;            // words of the slice: one load
+            struct alignas(4 * VW) Slice { unsigned w[VW]; };
+            const Slice v = *(const Slice*)(v0 + j * S::VROW);
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) {
+                const float x = sizeof(WT) == 4 ? __uint_as_float(v.w[e % VW]) : (e & 1) ? bf16_hi(v.w[e / 2]) : bf16_lo(v.w[e / 2]);
+                acc[e] = fmaf(pj, x, acc[e]);
+            }
+        }
+    }
+    // merge the warps that had rows
+    if (lane == 0) {
+        sm.m[warp] = m_run;
+        sm.l[warp] = l_run;
+    }
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) sm.acc[warp][lane * EPL + e] = acc[e];
+    __syncthreads();
+    const int nw = min(CHAIN_WARPS, (n + 31) / 32);
+    float M = -INFINITY, L = 0.f, A = 0.f;
+    auto merge = [&](int count) {                // of what lies in sm.m, sm.l and sm.acc, in order
+        M = -INFINITY;
+        L = A = 0.f;
+        for (int w = 0; w < count; ++w) M = fmaxf(M, sm.m[w]);
+        for (int w = 0; w < count; ++w) {
+            const float f = expf(sm.m[w] - M);
+            L += sm.l[w] * f;
+            A += sm.acc[w][tid] * f;
+        }
+    };
+    if (tid < DH) merge(nw);
+    if (nsplits == 1) {
+        if (tid < DH) a.attn[h * DH + tid] = A / L;
+        return;
+    }
+    const long long p0 = (long long)h * a.attn_nsplit;
+    if (tid < DH) {
+        a.part_acc[(p0 + split) * DH + tid] = A;
+        if (tid == 0) {
+            a.part_ml[(p0 + split) * 2] = M;
+            a.part_ml[(p0 + split) * 2 + 1] = L;
+        }
+    }
+    // arrival counter: the last unit of the head merges the splits; nobody waits
+    __syncthreads();
+    if (tid == 0) {
+        int* ctr = a.counters + h;
+        const int old = atom_add_acq_rel(ctr, 1);
+        sm.last = (old == nsplits - 1);
+        if (sm.last) *ctr = 0;
+    }
+    __syncthreads();
+    if (!sm.last) return;
+    if (nsplits <= CHAIN_WARPS) {
+        if (tid < nsplits) {
+            sm.m[tid] = __ldcg(a.part_ml + (p0 + tid) * 2);
+            sm.l[tid] = __ldcg(a.part_ml + (p0 + tid) * 2 + 1);
+        }
+#pragma unroll 4
+        for (int i = tid; i < nsplits * DH; i += CHAIN_THREADS) sm.acc[i / DH][i % DH] = __ldcg(a.part_acc + p0 * DH + i);
+        __syncthreads();
+        if (tid < DH) merge(nsplits);
+    } else if (tid < DH) {
+        M = -INFINITY;
+        L = A = 0.f;
+        for (int q = 0; q < nsplits; ++q) M = fmaxf(M, __ldcg(a.part_ml + (p0 + q) * 2));
+        for (int q = 0; q < nsplits; ++q) {
+            const float f = expf(__ldcg(a.part_ml + (p0 + q) * 2) - M);
+            L += __ldcg(a.part_ml + (p0 + q) * 2 + 1) * f;
+            A += __ldcg(a.part_acc + (p0 + q) * DH + tid) * f;
+        }
+    }
+    if (tid < DH) a.attn[h * DH + tid] = A / L;
+}
+
 template <typename WT, int DH>
 __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const ChainArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -171,6 +388,8 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
     u64* bars = (u64*)(smem + a.off_bar);
     ChainMisc* misc = (ChainMisc*)(smem + a.off_misc);
     AttnSmem<CHAIN_WARPS, 1, DH>* asm_ = (AttnSmem<CHAIN_WARPS, 1, DH>*)(smem + a.off_x);   // x is idle during attention
+
+    ChainAttnSmem<WT, DH>* cs = (ChainAttnSmem<WT, DH>*)(smem + a.off_x);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int cta = blockIdx.x, G = gridDim.x;
@@ -281,10 +500,14 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
 
     u64 bar_target = misc->bar_base;
     bool alive = true;
-    auto barrier = [&]() {
+    auto arrive = [&]() {
         bar_target += (u64)G;
-        alive = grid_barrier(a, misc, bar_target);
-        return alive;
+        grid_arrive(a);
+    };
+    auto wait = [&]() { return alive = grid_wait(a, misc, bar_target); };
+    auto barrier = [&]() {
+        arrive();
+        return wait();
     };
 
     AttnArgs aa;
@@ -337,13 +560,25 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
             const int r0 = misc->r0[PH_QKV], rows = misc->units[PH_QKV] / misc->cpr[PH_QKV];
             for (int rl = tid; rl < rows; rl += CHAIN_THREADS)
                 a.qkv[r0 + rl] = row_sum(PH_QKV, rl) + (a.bqkv ? load_as_float<WT>(a.bqkv, r0 + rl) : 0.f);
-            if (!barrier()) break;
         }
         // ============================================================ attention over the text-only cache
         {
             const int nunits = a.Hq * a.attn_nsplit;
-            for (int unit = cta; unit < nunits; unit += G)
-                attn_unit<WT, DH, 1, CHAIN_WARPS>(aa, unit % a.attn_nsplit, unit / a.attn_nsplit, 0, pos0 + s, slot, *asm_);
+            const bool staged = a.attn_chunk <= a.attn_rows;
+            arrive();
+            if (staged && cta < nunits) chain_attn_prepare<WT, DH>(a, *cs, cta, pos0 + s, slot);
+            if (!wait()) break;
+            for (int unit = cta; unit < nunits; unit += G) {
+                if (staged) {
+                    if (unit != cta) {
+                        __syncthreads();                     // the unit before has been read
+                        chain_attn_prepare<WT, DH>(a, *cs, unit, pos0 + s, slot);
+                    }
+                    chain_attn_run<WT, DH>(a, *cs, unit, pos0 + s, slot);
+                } else {
+                    attn_unit<WT, DH, 1, CHAIN_WARPS>(aa, unit % a.attn_nsplit, unit / a.attn_nsplit, 0, pos0 + s, slot, *asm_);
+                }
+            }
             if (!barrier()) break;
         }
         // ============================================================ O projection + residual
@@ -450,8 +685,10 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
 }
 
 // ------------------------------------------------------------------------------------------ host side
+#define CHAIN_ATTN_ROWS 128     // cache rows of a unit that are staged (a head's 600 rows at 32 heads, with four units each)
 struct ChainPlan {
     int off_x, off_part, off_bar, off_misc;
+    int attn_rows;             // rows of K and V that the room of x holds
     size_t smem_bytes;
 };
 
@@ -468,6 +705,15 @@ static ChainPlan chain_plan(const ChainArgs& a, int es, int dh, int grid) {
     size_t x_bytes = (size_t)kmax * 4;
     const size_t attn_bytes = dh == 128 ? sizeof(AttnSmem<CHAIN_WARPS, 1, 128>) : sizeof(AttnSmem<CHAIN_WARPS, 1, 64>);
     if (attn_bytes > x_bytes) x_bytes = attn_bytes;
+    // the attention stages up to CHAIN_ATTN_ROWS rows of K and V, as many as fit beside the rest
+    const size_t fixed = dh == 128 ? sizeof(ChainAttnSmem<float, 128>) : sizeof(ChainAttnSmem<float, 64>);
+    const size_t row = (size_t)(2 * dh * es + 16);
+    const size_t other = (size_t)CHAIN_WARPS * CHAIN_STAGES * (CHAIN_CHUNK_BYTES + 8) + (size_t)slots * 4 + sizeof(ChainMisc) + 512;
+    const size_t room = (size_t)227 * 1024 > other ? (size_t)227 * 1024 - other : 0;
+    size_t want = fixed + CHAIN_ATTN_ROWS * row;
+    if (want > room) want = room;
+    if (want > x_bytes) x_bytes = want;
+    p.attn_rows = x_bytes > fixed ? (int)((x_bytes - fixed) / row) : 0;
     size_t off = (size_t)CHAIN_WARPS * CHAIN_STAGES * CHAIN_CHUNK_BYTES;
     p.off_x = (int)off;
     off += (x_bytes + 127) & ~(size_t)127;
@@ -507,6 +753,7 @@ size_t chain_smem_bytes(const ChainArgs& a, int dtype, int grid) {
 cudaError_t launch_draft_chain(ChainArgs& a, int dtype, int grid, cudaStream_t st) {
     const ChainPlan p = chain_plan(a, dtype == HIVIS_BF16 ? 2 : 4, a.dh, grid);
     if (p.smem_bytes > 227 * 1024) return cudaErrorInvalidValue;
+    a.attn_rows = p.attn_rows;
     a.off_x = p.off_x; a.off_part = p.off_part; a.off_bar = p.off_bar; a.off_misc = p.off_misc;
     if (dtype == HIVIS_BF16)
         return a.dh == 128 ? chain_launch_t<bf16, 128>(a, grid, p.smem_bytes, st) : chain_launch_t<bf16, 64>(a, grid, p.smem_bytes, st);
