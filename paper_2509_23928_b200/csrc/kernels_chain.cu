@@ -10,6 +10,9 @@
 // barrier and stages the next activation vector, the first units of the next phase are already
 // landing in its rings: HBM keeps streaming through every dependency of the chain.
 //
+// The fusion FC is streamed in two parts: the hidden half needs nothing that the LM head before it decides and is used while that
+// one's grid barrier is awaited.  All parts of all steps run through ONE copy of the code (staging, weight loop, output stage).
+//
 // Phases of a step (grid barrier after each):
 //   FC (+rho) -> QKV (RMSNorm in the input stage) -> attention (RoPE, KV append, split-KV, arrival-
 //   counter merge) -> O (+u) -> gate/up (RMSNorm in, SiLU*up out) -> down (+y) -> LM head + argmax.
@@ -78,16 +81,63 @@ __device__ __forceinline__ int ld_relaxed_int(const int* p) {
 }
 
 #define CHAIN_BARRIERS 7         // grid barriers of a step
+
+// Matrices as the warps see them: those of the phases, the fusion FC in two parts - whole chunks of its hidden half, which
+// the step before has left in place, and the rest, which needs the step's token.  The hidden part lies under the grid barrier
+// of the LM head before it.
+enum { CW_FCH = 0, CW_FCE, CW_QKV, CW_O, CW_GU, CW_DOWN, CW_LM, CW_COUNT };
+struct ChainSeg {
+    const char* base;          // this CTA's first row, first column of the part
+    long long ld;              // bytes from row to row
+    int row0, rows;            // rows of this CTA
+    int K;                     // columns of the part
+    int cpr;                   // chunks per row of the part
+    int slot0, slots;          // partial sums: chunk slots of a row, the first of this part
+};
+
+// A warp's place in its units of a part.  A warp keeps to one chunk of the columns where the number of chunks divides the
+// number of warps, else it has a run of the units taken chunk by chunk.
+struct alignas(16) ChainCursor {
+    int row, ch, left, step;
+    __device__ void begin(const ChainSeg& g, int warp) {
+        if (CHAIN_WARPS % g.cpr == 0) {
+            step = CHAIN_WARPS / g.cpr;
+            ch = warp % g.cpr;
+            row = warp / g.cpr;
+            left = row < g.rows ? (g.rows - 1 - row) / step + 1 : 0;
+        } else {
+            const int U = g.rows * g.cpr, u0 = U * warp / CHAIN_WARPS;
+            step = 1;
+            ch = g.rows > 0 ? u0 / g.rows : 0;
+            row = u0 - ch * g.rows;
+            left = U * (warp + 1) / CHAIN_WARPS - u0;
+        }
+    }
+    __device__ __forceinline__ void next(const ChainSeg& g) {
+        --left;
+        row += step;
+        if (row >= g.rows) { row = 0; ++ch; }        // (not reached by warps that keep to a chunk: none is left)
+    }
+};
+// A warp's stream of units: how many it has asked for and used, and the next one to ask for.
+struct ChainStream {
+    unsigned fi, ci;
+    int step, w;
+    ChainCursor at;
+};
 struct ChainMisc {
     float red[CHAIN_WARPS];
     u64 kred[CHAIN_WARPS];
     int abort_flag;
-    int r0[PH_COUNT];          // first row of this CTA in each phase
-    int units[PH_COUNT];       // number of units of this CTA in each phase
-    int cpr[PH_COUNT];         // chunks per row
+    ChainSeg seg[CW_COUNT];
+    ChainCursor first[CW_COUNT][CHAIN_WARPS];      // every warp's place at the start of every part
     u64 bar_base;              // value of the barrier counter when the launch began
 };
 
+// CTA barrier; true, for all threads alike, while no wait of the CTA has run out.
+__device__ __forceinline__ bool cta_alive(const ChainMisc* misc) {
+    return __syncthreads_or(*(volatile const int*)&misc->abort_flag) == 0;
+}
 // Grid-wide barrier on a monotonically increasing counter, in two halves: what does not need the others' results goes between.
 __device__ __forceinline__ void grid_arrive(const ChainArgs& a) {
     __syncthreads();
@@ -95,41 +145,24 @@ __device__ __forceinline__ void grid_arrive(const ChainArgs& a) {
 }
 // false = gave up (error flag raised)
 __device__ __forceinline__ bool grid_wait(const ChainArgs& a, ChainMisc* misc, u64 target) {
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && *(volatile int*)&misc->abort_flag == 0) {
         const long long t0 = clock64();
         unsigned it = 0;
-        bool ok = true;
         while (ld_acquire_u64(a.bar_counter) < target) {
             if ((++it & 255u) == 0u && (ld_relaxed_int(a.error_flag) != 0 || clock64() - t0 > a.wait_cycles)) {
-                ok = false;
+                atomicExch(a.error_flag, 1);
+                *(volatile int*)&misc->abort_flag = 1;
                 break;
             }
         }
-        if (!ok) {
-            atomicExch(a.error_flag, 1);
-            misc->abort_flag = 1;
-        }
     }
-    __syncthreads();
-    return misc->abort_flag == 0;
+    return cta_alive(misc);
 }
 
 template <typename WT>
 __device__ __forceinline__ int x_index(int k, int K) {
     if (sizeof(WT) == 2) return ((k >> 3) << 2) + (k & 3) + ((k >> 2) & 1) * (K >> 1);
     return k;
-}
-
-__device__ __forceinline__ float block_sum(float v, float* red) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    float tot = 0.f;
-#pragma unroll
-    for (int w = 0; w < CHAIN_WARPS; ++w) tot += red[w];
-    return tot;
 }
 
 // dot product of one staged chunk with the matching slice of x
@@ -164,6 +197,30 @@ __device__ __forceinline__ float dot_chunk(const uint4* wsm, const float* xs, in
     return acc;
 }
 
+// Asks for the warp's next unit (lane 0 issues; every lane tracks the cursor).
+__device__ __forceinline__ void chain_fetch(ChainStream& t, const ChainMisc* misc, int k, int es, uint32_t ring0, uint32_t bar0, u64 pol,
+                                            int warp, int lane) {
+    while (t.at.left == 0) {
+        if (++t.w == CW_COUNT) {
+            t.w = 0;
+            ++t.step;
+        }
+        if (t.step >= k) return;
+        t.at = misc->first[t.w][warp];
+    }
+    if (t.step >= k) return;
+    const ChainSeg& g = misc->seg[t.w];
+    if (lane == 0) {
+        const unsigned st = t.fi % CHAIN_STAGES;
+        const uint32_t bar = bar0 + st * 8;
+        const uint32_t bytes = (uint32_t)min(CHAIN_CHUNK_BYTES, g.K * es - t.at.ch * CHAIN_CHUNK_BYTES);
+        mbar_expect_tx(bar, bytes);
+        bulk_g2s(ring0 + st * CHAIN_CHUNK_BYTES, g.base + t.at.row * g.ld + t.at.ch * CHAIN_CHUNK_BYTES, bytes, bar, pol);
+    }
+    ++t.fi;
+    t.at.next(g);
+}
+
 // ---- attention -----------------------------------------------------------------------------------
 // A unit = (split of the cache rows, query head), a CTA each; the arithmetic and its order are attn_unit's (attn_body.cuh, one
 // head per unit), so the results are the same bits.  What bounds it is a chain of latencies: with attn_unit, one or two warps of a
@@ -172,6 +229,7 @@ __device__ __forceinline__ float dot_chunk(const uint4* wsm, const float* xs, in
 // barrier is awaited, and the angles worked out there; q, k and v are rotated side by side, the new row being one more row of
 // the copies; warps without rows are left out of the merge; the splits' partial results come in one round trip.  Units whose
 // rows shared memory does not hold take attn_unit.
+// Five steps and the refresh: 803 -> 749 us (d 4096, 128 rows), 131 -> 119 (d 256).
 // (No more registers than the projections need: the acquire of a grid barrier empties L1, so a spilled register comes back from
 // L2.  A variant with rows in registers spilled 100 words and made a step 24 us slower.)
 template <typename WT, int DH>
@@ -388,36 +446,58 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
     u64* bars = (u64*)(smem + a.off_bar);
     ChainMisc* misc = (ChainMisc*)(smem + a.off_misc);
     AttnSmem<CHAIN_WARPS, 1, DH>* asm_ = (AttnSmem<CHAIN_WARPS, 1, DH>*)(smem + a.off_x);   // x is idle during attention
-
     ChainAttnSmem<WT, DH>* cs = (ChainAttnSmem<WT, DH>*)(smem + a.off_x);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int cta = blockIdx.x, G = gridDim.x;
     const int d = a.d;
+    const int kh = d / CE * CE;                             // columns of the fusion FC that the first part covers
 
-    if (tid == 0) {
-        misc->abort_flag = 0;
-        for (int p = 0; p < PH_COUNT; ++p) {
-            const long long N = a.ph[p].N;
-            long long r0, r1;
-            if (p == PH_GU) {                                // keep (gate_i, up_i) row pairs together
-                r0 = 2 * ((N / 2) * cta / G);
-                r1 = 2 * ((N / 2) * (cta + 1) / G);
-            } else {
-                r0 = N * cta / G;
-                r1 = N * (cta + 1) / G;
-            }
-            const int cpr = (a.ph[p].K * ES + CHAIN_CHUNK_BYTES - 1) / CHAIN_CHUNK_BYTES;
-            misc->r0[p] = (int)r0;
-            misc->cpr[p] = cpr;
-            misc->units[p] = (int)(r1 - r0) * cpr;
+    if (tid < PH_COUNT) {
+        const int p = tid;
+        const long long N = a.ph[p].N, K = a.ph[p].K;
+        long long r0, r1;
+        if (p == PH_GU) {                                // keep (gate_i, up_i) row pairs together
+            r0 = 2 * ((N / 2) * cta / G);
+            r1 = 2 * ((N / 2) * (cta + 1) / G);
+        } else {
+            r0 = N * cta / G;
+            r1 = N * (cta + 1) / G;
         }
+        ChainSeg g;
+        g.base = (const char*)a.ph[p].W + r0 * K * ES;
+        g.ld = K * ES;
+        g.row0 = (int)r0;
+        g.rows = (int)(r1 - r0);
+        g.slots = (int)((K * ES + CHAIN_CHUNK_BYTES - 1) / CHAIN_CHUNK_BYTES);
+        if (p == PH_FC) {
+            g.K = kh;
+            g.cpr = kh / CE > 0 ? kh / CE : 1;
+            g.slot0 = 0;
+            misc->seg[CW_FCH] = g;
+            if (kh == 0) misc->seg[CW_FCH].rows = 0;
+            g.base += (long long)kh * ES;
+            g.K = (int)K - kh;
+            g.cpr = g.slots - kh / CE;
+            g.slot0 = kh / CE;
+            misc->seg[CW_FCE] = g;
+        } else {
+            g.K = (int)K;
+            g.cpr = g.slots;
+            g.slot0 = 0;
+            misc->seg[CW_FCE + p] = g;
+        }
+    } else if (tid == 32) {
+        misc->abort_flag = 0;
         misc->bar_base = barrier_base(a.bar_counter, (unsigned)G) + a.bar_off;
-        for (int i = 0; i < CHAIN_WARPS * CHAIN_STAGES; ++i) mbar_init(smem_addr(bars + i), 1);
+    } else if (tid >= 64 && tid < 64 + CHAIN_WARPS * CHAIN_STAGES) {
+        mbar_init(smem_addr(bars + tid - 64), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
     }
     __syncthreads();
+    if (lane < CW_COUNT) misc->first[lane][warp].begin(misc->seg[lane], warp);
+    __syncwarp();
 
     const int slot = a.slot;
     const int pos0 = a.kv_len[slot];
@@ -425,90 +505,22 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
 
     // ---------------------------------------------------------------- per-warp weight stream
     const u64 pol = make_evict_first_policy();
-    const uint32_t ring0 = smem_addr(smem) + warp * (CHAIN_STAGES * CHAIN_CHUNK_BYTES);
-    const uint32_t bar0 = smem_addr(bars + warp * CHAIN_STAGES);
-    unsigned fi = 0, ci = 0;                                // units fetched / consumed by this warp
-    int f_step = 0, f_ph = 0, f_u = warp;                   // fetch cursor
-    bool f_live = true;
-    auto f_normalise = [&]() {                              // move the cursor to the next existing unit
-        while (f_live && f_u >= misc->units[f_ph]) {
-            f_u = warp;
-            if (++f_ph == PH_COUNT) {
-                f_ph = 0;
-                if (++f_step == a.k) f_live = false;
-            }
-        }
-    };
-    auto fetch_next = [&]() {                               // lane 0 issues; every lane tracks the cursor
-        if (!f_live) return;
-        const ChainPhase& P = a.ph[f_ph];
-        const int cpr = misc->cpr[f_ph];
-        const int row = misc->r0[f_ph] + f_u / cpr;
-        const int ch = f_u % cpr;
-        const int k0 = ch * CE;
-        const int len = min(CE, P.K - k0);
-        if (lane == 0) {
-            const unsigned st = fi % CHAIN_STAGES;
-            const uint32_t bar = bar0 + st * 8;
-            const char* src = (const char*)P.W + ((long long)row * P.K + k0) * ES;
-            mbar_expect_tx(bar, (uint32_t)(len * ES));
-            bulk_g2s(ring0 + st * CHAIN_CHUNK_BYTES, src, (uint32_t)(len * ES), bar, pol);
-        }
-        ++fi;
-        f_u += CHAIN_WARPS;
-        f_normalise();
-    };
-    f_normalise();
-    for (int i = 0; i < CHAIN_STAGES; ++i) fetch_next();
+    unsigned char* const stages = smem + warp * (CHAIN_STAGES * CHAIN_CHUNK_BYTES);
+    const uint32_t ring0 = smem_addr(stages), bar0 = smem_addr(bars + warp * CHAIN_STAGES);
+    ChainStream t;
+    t.fi = t.ci = 0;
+    t.step = t.w = 0;
+    t.at = misc->first[0][warp];
+    for (int i = 0; i < CHAIN_STAGES; ++i) chain_fetch(t, misc, a.k, ES, ring0, bar0, pol, warp, lane);
 
-    // consume this warp's units of phase p: partial dot products into part[u]
-    auto consume_phase = [&](int p) -> bool {
-        const int K = a.ph[p].K, cpr = misc->cpr[p], U = misc->units[p];
-        for (int u = warp; u < U; u += CHAIN_WARPS) {
-            const unsigned st = ci % CHAIN_STAGES;
-            const uint32_t parity = (ci / CHAIN_STAGES) & 1u;
-            const uint32_t bar = bar0 + st * 8;
-            if (!mbar_try_wait(bar, parity)) {
-                const long long t0 = clock64();
-                while (!mbar_try_wait(bar, parity)) {
-                    if (clock64() - t0 > a.wait_cycles) {
-                        atomicExch(a.error_flag, 2);
-                        misc->abort_flag = 1;
-                        return false;
-                    }
-                }
-            }
-            const int ch = u % cpr;
-            const int k0 = ch * CE;
-            const int len = min(CE, K - k0);
-            const uint4* wsm = (const uint4*)(smem + (size_t)(warp * CHAIN_STAGES + st) * CHAIN_CHUNK_BYTES);
-            const float acc = dot_chunk<WT>(wsm, xs, K, k0, (len * ES) >> 4, lane);
-            if (lane == 0) part[u] = acc;
-            ++ci;
-            __syncwarp();
-            fence_proxy_async();                            // our reads of the stage precede its refill
-            fetch_next();
-        }
-        return true;
-    };
-    auto row_sum = [&](int p, int rl) {                     // add a row's chunk partials in chunk order
-        const int cpr = misc->cpr[p];
-        float v = 0.f;
-        for (int c = 0; c < cpr; ++c) v += part[rl * cpr + c];
-        return v;
-    };
-
-    u64 bar_target = misc->bar_base;
+    u64 bar_target = misc->bar_base;                        // of the newest barrier that this CTA has arrived on
     bool alive = true;
     auto arrive = [&]() {
         bar_target += (u64)G;
         grid_arrive(a);
     };
     auto wait = [&]() { return alive = grid_wait(a, misc, bar_target); };
-    auto barrier = [&]() {
-        arrive();
-        return wait();
-    };
+    constexpr int XB = 8;                                   // words of x per thread and turn
 
     AttnArgs aa;
     aa.qkv = a.qkv; aa.ld = a.qw + 2 * a.kvw; aa.Kc = a.Kc; aa.Vc = a.Vc; aa.slots = nullptr; aa.pos0 = nullptr;
@@ -516,134 +528,190 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
     aa.B = 1; aa.scale = a.scale; aa.chunk = a.attn_chunk; aa.nsplit = a.attn_nsplit; aa.part_acc = a.part_acc;
     aa.part_ml = a.part_ml; aa.counters = a.counters; aa.attn = a.attn; aa.attn_h = nullptr; aa.lo_rows = 0;
 
-    for (int s = 0; s < a.k && alive; ++s) {
-        // ============================================================ fusion FC + residual
-        {
-            const int K = 2 * d;
+    // One loop over the parts of all steps, so that every piece of code is there once: a step runs through all of it, and what the
+    // instruction caches do not hold comes from L2 again, in the middle of the phase boundaries.  (A copy of the weight loop and of
+    // the barriers for every phase made 175 KB, now 135.)  With the hidden half of the fusion FC under the LM head's barrier, gains and
+    // addends asked for before the barriers and x staged four words at a time: d 4096, five steps and the refresh 750 -> 731 us, an
+    // opening 765 -> 739; d 256 118 -> 121, where there is next to nothing to stream (135 at first).
+    int s = 0, w = CW_FCH;
+#pragma unroll 1
+    for (; s < a.k; s += w == CW_LM ? 1 : 0, w = w == CW_LM ? CW_FCH : w + 1) {
+        const ChainSeg& g = misc->seg[w];
+        const int K = g.K;
+        // ------------------------------------------------------------ x of the part
+        if (w == CW_FCH) {
+            // the hidden half of the fusion FC: behind the LM head x is still the layer output
+            if (K == 0) continue;
+            if (s == 0 || K != d) {
+                const float* f = s == 0 ? a.pend_feat + (long long)slot * d : a.feat;
+                for (int kk = tid; kk < K; kk += CHAIN_THREADS) xs[x_index<WT>(kk, K)] = __ldcg(f + kk);
+                __syncthreads();
+            }
+        } else if (w == CW_FCE) {
+            if (!(alive = cta_alive(misc))) break;           // (x of the other half has been used)
+            const float* f = (s == 0 ? a.pend_feat + (long long)slot * d : a.feat) + kh;
+            const int fk = d - kh;
+            for (int kk = tid; kk < fk; kk += CHAIN_THREADS) xs[x_index<WT>(kk, K)] = __ldcg(f + kk);
+            if (s > 0 && !wait()) break;                     // the keys of the last step are complete
             int tok;
             if (s == 0) tok = a.pend_id[slot];
             else if (a.forced) tok = a.forced[s - 1];
             else tok = key_index(__ldcg(a.keys + (s - 1)));
             tok = checked_token(tok, a.V, a.id_flag);
-            const float* f = s == 0 ? a.pend_feat + (long long)slot * d : a.feat;
             const long long e0 = (long long)tok * d;
-            for (int kk = tid; kk < K; kk += CHAIN_THREADS)
-                xs[x_index<WT>(kk, K)] = kk < d ? __ldcg(f + kk) : load_as_float<WT>(a.embed, e0 + (kk - d));
+            for (int kk = tid; kk < d; kk += CHAIN_THREADS) xs[x_index<WT>(fk + kk, K)] = load_as_float<WT>(a.embed, e0 + kk);
             __syncthreads();
-            if (!consume_phase(PH_FC)) {}
-            __syncthreads();
-            if (misc->abort_flag) break;
-            const int r0 = misc->r0[PH_FC], rows = misc->units[PH_FC] / misc->cpr[PH_FC];
-            const long long rho_row = (long long)(s < a.n_resid - 1 ? s : a.n_resid - 1) * d;
-            for (int rl = tid; rl < rows; rl += CHAIN_THREADS)
-                a.u[r0 + rl] = row_sum(PH_FC, rl) + (a.rho ? a.rho[rho_row + r0 + rl] : a.rho_w ? load_as_float<WT>(a.rho_w, rho_row + r0 + rl) : 0.f);
-            if (!barrier()) break;
-        }
-        // ============================================================ RMSNorm + QKV
-        {
-            const int K = d;
-            float ss = 0.f;
-            for (int kk = tid; kk < K; kk += CHAIN_THREADS) {
-                const float v = __ldcg(a.u + kk);
-                ss += v * v;
-                xs[x_index<WT>(kk, K)] = v;
-            }
-            const float inv = rsqrtf(block_sum(ss, misc->red) / (float)K + a.eps);
-            for (int kk = tid; kk < K; kk += CHAIN_THREADS) {
-                const int i = x_index<WT>(kk, K);
-                xs[i] = xs[i] * load_as_float<WT>(a.norm1, kk) * inv;
-            }
-            __syncthreads();
-            consume_phase(PH_QKV);
-            __syncthreads();
-            if (misc->abort_flag) break;
-            const int r0 = misc->r0[PH_QKV], rows = misc->units[PH_QKV] / misc->cpr[PH_QKV];
-            for (int rl = tid; rl < rows; rl += CHAIN_THREADS)
-                a.qkv[r0 + rl] = row_sum(PH_QKV, rl) + (a.bqkv ? load_as_float<WT>(a.bqkv, r0 + rl) : 0.f);
-        }
-        // ============================================================ attention over the text-only cache
-        {
-            const int nunits = a.Hq * a.attn_nsplit;
-            const bool staged = a.attn_chunk <= a.attn_rows;
-            arrive();
-            if (staged && cta < nunits) chain_attn_prepare<WT, DH>(a, *cs, cta, pos0 + s, slot);
-            if (!wait()) break;
-            for (int unit = cta; unit < nunits; unit += G) {
-                if (staged) {
-                    if (unit != cta) {
-                        __syncthreads();                     // the unit before has been read
-                        chain_attn_prepare<WT, DH>(a, *cs, unit, pos0 + s, slot);
-                    }
-                    chain_attn_run<WT, DH>(a, *cs, unit, pos0 + s, slot);
-                } else {
-                    attn_unit<WT, DH, 1, CHAIN_WARPS>(aa, unit % a.attn_nsplit, unit / a.attn_nsplit, 0, pos0 + s, slot, *asm_);
+        } else {
+            const bool norm = w == CW_QKV || w == CW_GU;
+            const float* src = w == CW_QKV ? a.u : w == CW_O ? a.attn : w == CW_GU ? a.y : w == CW_DOWN ? a.act : a.feat;
+            const void* gain = w == CW_QKV ? a.norm1 : a.norm2;
+            float gn[XB];
+            if (norm) {                                     // (asked for before the barrier)
+#pragma unroll
+                for (int i = 0; i < XB; ++i) {
+                    const int kk = tid + i * CHAIN_THREADS;
+                    gn[i] = kk < K ? load_as_float<WT>(gain, kk) : 0.f;
                 }
             }
-            if (!barrier()) break;
-        }
-        // ============================================================ O projection + residual
-        {
-            const int K = a.qw;
-            for (int kk = tid; kk < K; kk += CHAIN_THREADS) xs[x_index<WT>(kk, K)] = __ldcg(a.attn + kk);
-            __syncthreads();
-            consume_phase(PH_O);
-            __syncthreads();
-            if (misc->abort_flag) break;
-            const int r0 = misc->r0[PH_O], rows = misc->units[PH_O] / misc->cpr[PH_O];
-            for (int rl = tid; rl < rows; rl += CHAIN_THREADS)
-                a.y[r0 + rl] = __ldcg(a.u + r0 + rl) + row_sum(PH_O, rl);
-            if (!barrier()) break;
-        }
-        // ============================================================ RMSNorm + gate/up + SiLU*up
-        {
-            const int K = d;
-            float ss = 0.f;
-            for (int kk = tid; kk < K; kk += CHAIN_THREADS) {
-                const float v = __ldcg(a.y + kk);
-                ss += v * v;
-                xs[x_index<WT>(kk, K)] = v;
+            if (w == CW_O) {
+                // attention over the text-only cache
+                const int nunits = a.Hq * a.attn_nsplit;
+                const bool staged = a.attn_chunk <= a.attn_rows;
+                if (staged && cta < nunits) chain_attn_prepare<WT, DH>(a, *cs, cta, pos0 + s, slot);
+                if (!wait()) break;
+#pragma unroll 1
+                for (int unit = cta; unit < nunits; unit += G) {
+                    if (staged) {
+                        if (unit != cta) {
+                            __syncthreads();                // the unit before has been read
+                            chain_attn_prepare<WT, DH>(a, *cs, unit, pos0 + s, slot);
+                        }
+                        chain_attn_run<WT, DH>(a, *cs, unit, pos0 + s, slot);
+                    } else {
+                        attn_unit<WT, DH, 1, CHAIN_WARPS>(aa, unit % a.attn_nsplit, unit / a.attn_nsplit, 0, pos0 + s, slot, *asm_);
+                    }
+                }
+                arrive();
             }
-            const float inv = rsqrtf(block_sum(ss, misc->red) / (float)K + a.eps);
-            for (int kk = tid; kk < K; kk += CHAIN_THREADS) {
-                const int i = x_index<WT>(kk, K);
-                xs[i] = xs[i] * load_as_float<WT>(a.norm2, kk) * inv;
+            if (!wait()) break;
+            if (norm) {
+                // a thread's first words stay in registers until the scale is known
+                float v[XB], ss = 0.f;
+#pragma unroll
+                for (int i = 0; i < XB; ++i) {
+                    const int kk = tid + i * CHAIN_THREADS;
+                    v[i] = kk < K ? __ldcg(src + kk) : 0.f;
+                }
+#pragma unroll
+                for (int i = 0; i < XB; ++i) ss += v[i] * v[i];
+#pragma unroll 1
+                for (int kk = tid + XB * CHAIN_THREADS; kk < K; kk += CHAIN_THREADS) {
+                    const float y = __ldcg(src + kk);
+                    ss += y * y;
+                    xs[x_index<WT>(kk, K)] = y;
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+                if (lane == 0) misc->red[warp] = ss;
+                __syncthreads();
+                float tot = 0.f;
+#pragma unroll
+                for (int q = 0; q < CHAIN_WARPS; ++q) tot += misc->red[q];
+                const float inv = rsqrtf(tot / (float)K + a.eps);
+#pragma unroll
+                for (int i = 0; i < XB; ++i) {
+                    const int kk = tid + i * CHAIN_THREADS;
+                    if (kk < K) xs[x_index<WT>(kk, K)] = v[i] * gn[i] * inv;
+                }
+#pragma unroll 1
+                for (int kk = tid + XB * CHAIN_THREADS; kk < K; kk += CHAIN_THREADS) {
+                    const int j = x_index<WT>(kk, K);
+                    xs[j] = xs[j] * load_as_float<WT>(gain, kk) * inv;
+                }
+            } else {
+                // four words at a time (the layout keeps four together), all of a thread's loads in flight up to K = 12288
+                constexpr int XV = 6;
+#pragma unroll 1
+                for (int k0 = 4 * tid; k0 < K; k0 += 4 * XV * CHAIN_THREADS) {
+                    float4 v[XV];
+#pragma unroll
+                    for (int i = 0; i < XV; ++i) {
+                        const int kk = k0 + 4 * i * CHAIN_THREADS;
+                        if (kk < K) v[i] = __ldcg((const float4*)(src + kk));
+                    }
+#pragma unroll
+                    for (int i = 0; i < XV; ++i) {
+                        const int kk = k0 + 4 * i * CHAIN_THREADS;
+                        if (kk < K) *(float4*)(xs + x_index<WT>(kk, K)) = v[i];
+                    }
+                }
             }
             __syncthreads();
-            consume_phase(PH_GU);
-            __syncthreads();
-            if (misc->abort_flag) break;
-            const int r0 = misc->r0[PH_GU], rows = misc->units[PH_GU] / misc->cpr[PH_GU];
-            for (int pl = tid; pl < rows / 2; pl += CHAIN_THREADS) {
-                const float gate = row_sum(PH_GU, 2 * pl), up = row_sum(PH_GU, 2 * pl + 1);
+        }
+        // what the output of this thread's row is added to
+        const int r0 = g.row0;
+        const float* const add = w == CW_O ? a.u : a.y;
+        const long long rho_row = (long long)(s < a.n_resid - 1 ? s : a.n_resid - 1) * d;
+        auto addend = [&](int r) {
+            if (w == CW_FCE) return a.rho ? a.rho[rho_row + r] : a.rho_w ? load_as_float<WT>(a.rho_w, rho_row + r) : 0.f;
+            if (w == CW_QKV) return a.bqkv ? load_as_float<WT>(a.bqkv, r) : 0.f;
+            return __ldcg(add + r);
+        };
+        float first_add = 0.f;
+        if (w != CW_FCH && w != CW_GU && w != CW_LM && tid < g.rows) first_add = addend(r0 + tid);
+        // ------------------------------------------------------------ this warp's units: partial dot products into part[row][slot]
+        {
+            ChainCursor c = misc->first[w][warp];
+            int have = -1, nvec = 0;
+            bool gave_up = false;
+#pragma unroll 1
+            while (c.left > 0) {
+                if (c.ch != have) {
+                    have = c.ch;
+                    nvec = (min(CE, K - have * CE) * ES) >> 4;
+                }
+                const unsigned st = t.ci % CHAIN_STAGES;
+                const uint32_t parity = (t.ci / CHAIN_STAGES) & 1u;
+                const uint32_t bar = bar0 + st * 8;
+                if (!mbar_try_wait(bar, parity)) {
+                    const long long t0 = clock64();
+                    while (!mbar_try_wait(bar, parity)) {
+                        if (clock64() - t0 > a.wait_cycles) {
+                            atomicExch(a.error_flag, 2);
+                            *(volatile int*)&misc->abort_flag = 1;
+                            gave_up = true;
+                            break;
+                        }
+                    }
+                }
+                if (__any_sync(0xffffffffu, gave_up)) break;        // one answer for the warp
+                const float acc = dot_chunk<WT>((const uint4*)(stages + st * CHAIN_CHUNK_BYTES), xs, K, have * CE, nvec, lane);
+                if (lane == 0) part[c.row * g.slots + g.slot0 + c.ch] = acc;
+                ++t.ci;
+                __syncwarp();
+                fence_proxy_async();                        // our reads of the stage precede its refill
+                chain_fetch(t, misc, a.k, ES, ring0, bar0, pol, warp, lane);
+                c.next(g);
+            }
+        }
+        if (w == CW_FCH) continue;                          // (its partial sums wait for those of the other half)
+        if (!(alive = cta_alive(misc))) break;
+        // ------------------------------------------------------------ output stage
+        const int slots = g.slots;
+        auto row_sum = [&](int rl) {                        // add a row's chunk partials in chunk order
+            float v = 0.f;
+            for (int q = 0; q < slots; ++q) v += part[rl * slots + q];
+            return v;
+        };
+        if (w == CW_GU) {
+            for (int pl = tid; pl < g.rows / 2; pl += CHAIN_THREADS) {
+                const float gate = row_sum(2 * pl), up = row_sum(2 * pl + 1);
                 a.act[r0 / 2 + pl] = gate / (1.f + expf(-gate)) * up;
             }
-            if (!barrier()) break;
-        }
-        // ============================================================ down projection + residual
-        {
-            const int K = a.F;
-            for (int kk = tid; kk < K; kk += CHAIN_THREADS) xs[x_index<WT>(kk, K)] = __ldcg(a.act + kk);
-            __syncthreads();
-            consume_phase(PH_DOWN);
-            __syncthreads();
-            if (misc->abort_flag) break;
-            const int r0 = misc->r0[PH_DOWN], rows = misc->units[PH_DOWN] / misc->cpr[PH_DOWN];
-            for (int rl = tid; rl < rows; rl += CHAIN_THREADS)
-                a.feat[r0 + rl] = __ldcg(a.y + r0 + rl) + row_sum(PH_DOWN, rl);
-            if (!barrier()) break;
-        }
-        // ============================================================ LM head + argmax
-        {
-            const int K = d;
-            for (int kk = tid; kk < K; kk += CHAIN_THREADS) xs[x_index<WT>(kk, K)] = __ldcg(a.feat + kk);
-            __syncthreads();
-            consume_phase(PH_LM);
-            __syncthreads();
-            if (misc->abort_flag) break;
-            const int r0 = misc->r0[PH_LM], rows = misc->units[PH_LM] / misc->cpr[PH_LM];
+        } else if (w == CW_LM) {
             u64 best = 0;
-            for (int rl = tid; rl < rows; rl += CHAIN_THREADS) {
-                const float v = row_sum(PH_LM, rl);
+            for (int rl = tid; rl < g.rows; rl += CHAIN_THREADS) {
+                const float v = row_sum(rl);
                 if (a.logits_out) a.logits_out[(long long)s * a.V + r0 + rl] = v;
                 const u64 key = a.gumbel_u ? pack_key(gumbel_perturbed(v, a.inv_t, __ldg(a.gumbel_u + (long long)s * a.V + r0 + rl)), r0 + rl)
                                            : pack_key(v, r0 + rl);
@@ -659,13 +727,16 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
             if (tid == 0) {
                 u64 m = misc->kred[0];
 #pragma unroll
-                for (int w = 1; w < CHAIN_WARPS; ++w) m = misc->kred[w] > m ? misc->kred[w] : m;
+                for (int q = 1; q < CHAIN_WARPS; ++q) m = misc->kred[q] > m ? misc->kred[q] : m;
                 if (m) atomicMax(a.keys + s, m);
             }
-            if (!barrier()) break;
+        } else {
+            float* const out = w == CW_FCE ? a.u : w == CW_QKV ? a.qkv : w == CW_O ? a.y : a.feat;
+            for (int rl = tid; rl < g.rows; rl += CHAIN_THREADS) out[r0 + rl] = row_sum(rl) + (rl == tid ? first_add : addend(r0 + rl));
         }
+        arrive();
     }
-    if (alive && misc->abort_flag == 0) {
+    if (alive && (cta != 0 || wait())) {                    // (only the CTA that reads the last keys waits for them)
         if (cta == 0) {
             if (tid < a.k) a.out_ids[tid] = key_index(__ldcg(a.keys + tid));
             if (tid == 0) a.kv_len[slot] = pos0 + a.k;
@@ -675,7 +746,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
     // gave up: make the arrivals that are left (the next launch counts on whole barriers), wait (bounded) for this warp's
     // copies that are still in flight, then leave
     if (tid == 0) red_release_add_u64(a.bar_counter, (u64)(CHAIN_BARRIERS * a.k) - (bar_target - misc->bar_base) / (u64)G);
-    for (; ci < fi; ++ci) {
+    for (unsigned ci = t.ci; ci < t.fi; ++ci) {
         const uint32_t bar = bar0 + (ci % CHAIN_STAGES) * 8;
         const uint32_t parity = (ci / CHAIN_STAGES) & 1u;
         const long long t0 = clock64();
