@@ -20,7 +20,8 @@
 //
 // 34 800 pairs of the LLaVA shape (16 sequences of 2176): 3.5 ms, 1.35 PFLOP/s (of 1.4 to 1.7 for a library GEMM; the SM
 // clock drops to 1.3-1.5 GHz under the power cap); with 128 x 128 tiles, one per CTA and launch slot, and the tile turned in
-// shared memory for the output stage 7.9 ms.  17 to 256 pairs: 87 to 91 us, a serial chain of 128 k-blocks in GEMM 1.
+// shared memory for the output stage 7.9 ms.  17 to 256 pairs: 65 to 70 us (87 to 91 before the
+// MMAs were issued by an elected thread), a serial chain of 128 k-blocks in GEMM 1.
 //
 // Warp 0 (one thread, both CTAs) issues the copies, warp 1 (one thread of the leader, rank 0) the MMAs for both, warps
 // 2-5 run the output stage.  A stage's full barrier lives in the leader and counts the bytes of both CTAs; tcgen05.commit
@@ -465,9 +466,10 @@ cudaError_t pf_launch_t(PfParams& P, int clusters, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// Tile width, by the time of the busiest cluster in units of 10 ns a k-block (0.45 us at 256 weight rows, 0.33 at 128; below
-// that an MMA takes as long whatever its width).  117 / 500 pairs (d 4096 / 2560): 92 / 69 us at 256, 90 / 62 at 128; 600 and
-// 2048 pairs (d 4096 / 3584): 123 and 130 us at 256, 174 and 193 at 128.
+// Tile width, by the time of the busiest cluster in units of 10 ns a k-block (0.36 us at 256 weight rows, 0.24 at 128; the line
+// between them was drawn at 0.45 to 0.33, and both give the same choices but where the waves are as 7 to 5).  128 / 256 wide: 17 pairs
+// 65 / 87 us (d 4096), 72 / 103 (d 3584), 58 / 69 (d 2560); 512 pairs 85 / 98, 84 / 99, 60 / 74; 600 pairs 123 / 114, 113 / 101,
+// 59 / 76; 2048 pairs 260 / 226, 144 / 130, 96 / 102.
 // A tile is never split over clusters, and no call goes through the chain kernel, whose phases are split over CTAs (64 pairs:
 // 45 us there, 89 here): u and the cached rows are rounded to bf16, and parts of their long sums added in fp32 instead of
 // in the tensor core's accumulator move one element in forty to the other side of a rounding.  Two to eleven of a hundred
