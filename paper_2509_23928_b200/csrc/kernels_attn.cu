@@ -16,6 +16,8 @@ template <typename WT, int DH, int GQ>
 __global__ void __launch_bounds__(128) attn_decode_kernel(const AttnArgs a) {
     __shared__ AttnSmem<4, GQ, DH> sm;
     const int b = blockIdx.z;
+    pdl_wait();
+    pdl_trigger();
     attn_unit<WT, DH, GQ, 4>(a, blockIdx.x, blockIdx.y, b, a.pos0[b] + a.step, a.slots[b], sm);
 }
 
@@ -28,13 +30,12 @@ static cudaError_t launch_attn_g(const AttnArgs& a, cudaStream_t st) {
         if (G % cand[i] == 0) { gq = cand[i]; break; }
     dim3 grid((unsigned)a.nsplit, (unsigned)(a.Hq / gq), (unsigned)a.B);
     switch (gq) {
-        case 8: attn_decode_kernel<WT, DH, 8><<<grid, 128, 0, st>>>(a); break;
-        case 7: attn_decode_kernel<WT, DH, 7><<<grid, 128, 0, st>>>(a); break;
-        case 4: attn_decode_kernel<WT, DH, 4><<<grid, 128, 0, st>>>(a); break;
-        case 2: attn_decode_kernel<WT, DH, 2><<<grid, 128, 0, st>>>(a); break;
-        default: attn_decode_kernel<WT, DH, 1><<<grid, 128, 0, st>>>(a); break;
+        case 8: return launch_pdl(attn_decode_kernel<WT, DH, 8>, grid, dim3(128), 0, st, a);
+        case 7: return launch_pdl(attn_decode_kernel<WT, DH, 7>, grid, dim3(128), 0, st, a);
+        case 4: return launch_pdl(attn_decode_kernel<WT, DH, 4>, grid, dim3(128), 0, st, a);
+        case 2: return launch_pdl(attn_decode_kernel<WT, DH, 2>, grid, dim3(128), 0, st, a);
+        default: return launch_pdl(attn_decode_kernel<WT, DH, 1>, grid, dim3(128), 0, st, a);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_attention(int dtype, const AttnArgs& a, cudaStream_t st) {

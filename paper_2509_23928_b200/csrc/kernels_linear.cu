@@ -154,8 +154,9 @@ __global__ void __launch_bounds__(256) gemv_alu_kernel(const LinArgs a, int ppw)
         w1 = w0 + nch;
         fetch(0, c0, c1);
     };
-    if (valid) open_pair();          // the first weights are in flight while x is being staged
-
+    if (valid) open_pair();          // the first weights are in flight while the launch before ends and x is being staged
+    pdl_wait();
+    pdl_trigger();
     load_x<WT, PRO>(a, b, xs, red);
 
     u64 best = 0;
@@ -243,8 +244,7 @@ static cudaError_t launch_alu_t(const LinArgs& a, cudaStream_t st) {
     while (ppw < 8 && pairs / (8LL * ppw * 2) >= 1184) ppw *= 2;
     const long long ctas = (pairs + 8LL * ppw - 1) / (8LL * ppw);
     dim3 grid((unsigned)ctas, (unsigned)a.B);
-    gemv_alu_kernel<WT, PRO, EPI><<<grid, 256, smem, st>>>(a, ppw);
-    return cudaGetLastError();
+    return launch_pdl(gemv_alu_kernel<WT, PRO, EPI>, grid, dim3(256), smem, st, a, ppw);
 }
 
 template <typename WT>

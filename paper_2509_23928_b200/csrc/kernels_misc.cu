@@ -8,6 +8,8 @@
 __global__ void draft_setup_kernel(SlotList sl, int k, int d, int* d_slots, int* d_pos0, int* kv_len,
                                    const float* pend_feat, const int* pend_id, float* feat, bf16* feat_h,
                                    int* cur_id, u64* keys, int key_stride) {
+    pdl_wait();
+    pdl_trigger();
     const int b = blockIdx.x, slot = sl.slot[b];
     if (threadIdx.x == 0) {
         d_slots[b] = slot;
@@ -26,13 +28,14 @@ __global__ void draft_setup_kernel(SlotList sl, int k, int d, int* d_slots, int*
 cudaError_t launch_draft_setup(const SlotList& sl, int k, int d, int* d_slots, int* d_pos0,
                                int* kv_len, const float* pend_feat, const int* pend_id, float* feat,
                                bf16* feat_h, int* cur_id, u64* keys, int key_stride, cudaStream_t st) {
-    draft_setup_kernel<<<sl.n, 256, 0, st>>>(sl, k, d, d_slots, d_pos0, kv_len, pend_feat, pend_id, feat,
-                                             feat_h, cur_id, keys, key_stride);
-    return cudaGetLastError();
+    return launch_pdl(draft_setup_kernel, dim3(sl.n), dim3(256), 0, st, sl, k, d, d_slots, d_pos0, kv_len, pend_feat, pend_id, feat, feat_h,
+                      cur_id, keys, key_stride);
 }
 
 __global__ void draft_finish_kernel(int n, int k, const u64* keys, int key_stride, int32_t* out_ids) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
+    pdl_trigger();
     if (i >= n) return;
     const int b = i / k, s = i % k;
     out_ids[i] = key_index(keys[(long long)b * key_stride + s]);
@@ -40,8 +43,7 @@ __global__ void draft_finish_kernel(int n, int k, const u64* keys, int key_strid
 cudaError_t launch_draft_finish(int B, int k, const u64* keys, int key_stride, int32_t* out_ids,
                                 cudaStream_t st) {
     const int n = B * k;
-    draft_finish_kernel<<<(n + 127) / 128, 128, 0, st>>>(n, k, keys, key_stride, out_ids);
-    return cudaGetLastError();
+    return launch_pdl(draft_finish_kernel, dim3((n + 127) / 128), dim3(128), 0, st, n, k, keys, key_stride, out_ids);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -49,6 +51,8 @@ cudaError_t launch_draft_finish(int B, int k, const u64* keys, int key_stride, i
 // ------------------------------------------------------------------------------------------
 template <typename WT>
 __global__ void convert_rows_kernel(const void* src, float* dst, long long n) {
+    pdl_wait();
+    pdl_trigger();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         dst[i] = load_as_float<WT>(src, i);
@@ -56,9 +60,7 @@ __global__ void convert_rows_kernel(const void* src, float* dst, long long n) {
 cudaError_t launch_convert_rows(int dtype, const void* src, float* dst, long long n, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     const unsigned grid = (unsigned)((n + 255) / 256 > 1184 ? 1184 : (n + 255) / 256);
-    if (dtype == HIVIS_BF16) convert_rows_kernel<bf16><<<grid, 256, 0, st>>>(src, dst, n);
-    else convert_rows_kernel<float><<<grid, 256, 0, st>>>(src, dst, n);
-    return cudaGetLastError();
+    return launch_pdl(dtype == HIVIS_BF16 ? convert_rows_kernel<bf16> : convert_rows_kernel<float>, dim3(grid), dim3(256), 0, st, src, dst, n);
 }
 cudaError_t launch_bf16_to_f32(const bf16* src, float* dst, long long n, cudaStream_t st) {
     return launch_convert_rows(HIVIS_BF16, src, dst, n, st);
