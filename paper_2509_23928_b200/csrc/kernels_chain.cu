@@ -499,6 +499,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
     if (lane < CW_COUNT) misc->first[lane][warp].begin(misc->seg[lane], warp);
     __syncwarp();
 
+    pdl_trigger();                                          // (the launch after this one is set up as CTAs leave)
     const int slot = a.slot;
     const int pos0 = a.kv_len[slot];
     if (cta == 0 && tid < a.k) a.keys[tid] = 0ull;       // consumed after several grid barriers

@@ -116,6 +116,8 @@ cudaError_t launch_prefill_setup(int dtype, const SlotList& sl, const CuSeqlens&
 __global__ void prefill_setup_rows_kernel(SlotList sl, CuSeqlens cu, SlotList start, int d, const int32_t* ids,
                                           const bf16* hidden, int* kv_len, float* pend_feat, int* pend_id, int* slot_of,
                                           int* row_of, const bf16* embed, int vocab, bf16* xe, int* id_flag) {
+    pdl_wait();
+    pdl_trigger();
     const int upr = d >> 3, pairs = cu.v[sl.n];
     if ((int)blockIdx.x < pairs) {
         const int j = blockIdx.x;
@@ -150,9 +152,8 @@ __global__ void prefill_setup_rows_kernel(SlotList sl, CuSeqlens cu, SlotList st
 cudaError_t launch_prefill_setup_rows(const SlotList& sl, const CuSeqlens& cu, const SlotList& start, int d, const int32_t* ids,
                                       const bf16* hidden, int* kv_len, float* pend_feat, int* pend_id, int* slot_of,
                                       int* row_of, const bf16* embed, int vocab, bf16* xe, int* id_flag, cudaStream_t st) {
-    prefill_setup_rows_kernel<<<cu.v[sl.n] + sl.n, 512, 0, st>>>(sl, cu, start, d, ids, hidden, kv_len, pend_feat, pend_id, slot_of,
-                                                                 row_of, embed, vocab, xe, id_flag);
-    return cudaGetLastError();
+    return launch_pdl(prefill_setup_rows_kernel, dim3(cu.v[sl.n] + sl.n), dim3(512), 0, st, sl, cu, start, d, ids, hidden, kv_len, pend_feat,
+                      pend_id, slot_of, row_of, embed, vocab, xe, id_flag);
 }
 
 // K (rotated) and V of a pair to its cache row.  A thread takes four elements of a head and their partners half a head
@@ -233,6 +234,8 @@ __global__ void __launch_bounds__(256) verify_kernel(SlotList sl, int k, const v
                                                      const int32_t* draft_ids, u64* keys, int* arrivals,
                                                      int* kv_len, int32_t* out_accept, int32_t* out_next,
                                                      int32_t* out_kv_len) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ u64 kred[8];
     constexpr int VEC = 16 / (int)sizeof(LT);
     const int b = blockIdx.z;
@@ -332,14 +335,9 @@ cudaError_t launch_verify(int logits_dtype, const SlotList& sl, int k, int V, co
     while (passes < VERIFY_MAX_PASSES && rows * ((V + passes * per_pass - 1) / (passes * per_pass)) > 148 * 8) ++passes;
     const int chunk = passes * per_pass;
     dim3 grid((unsigned)((V + chunk - 1) / chunk), (unsigned)(k + 1), (unsigned)sl.n);
-    if (logits_dtype == HIVIS_BF16)
-        verify_kernel<bf16><<<grid, 256, 0, st>>>(sl, k, logits, V, passes, draft_ids, keys, arrivals, kv_len,
-                                                   out_accept, out_next, out_kv_len);
-    else
-        verify_kernel<float><<<grid, 256, 0, st>>>(sl, k, logits, V, passes, draft_ids, keys, arrivals, kv_len,
-                                                    out_accept, out_next, out_kv_len);
     *n_launches = 1;
-    return cudaGetLastError();
+    return launch_pdl(logits_dtype == HIVIS_BF16 ? verify_kernel<bf16> : verify_kernel<float>, grid, dim3(256), 0, st, sl, k, logits, V, passes,
+                      draft_ids, keys, arrivals, kv_len, out_accept, out_next, out_kv_len);
 }
 
 __global__ void set_int_kernel(int* p, int v) { *p = v; }

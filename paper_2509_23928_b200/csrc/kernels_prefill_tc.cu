@@ -325,6 +325,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1) prefi
     __syncthreads();
     pf_cluster_sync();
     pf_fence_after();
+    pdl_wait();                 // (set up while the launch before ended)
+    pdl_trigger();
 
     if (warp == 0) {
         if (pf_elect()) {
@@ -415,6 +417,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1) prefi
 
 // (cos, sin) of every pair's position, once per call: every K tile of GEMM 2 rotates with the same angles
 __global__ void prefill_rope_kernel(const int* row_of, int n_pairs, int half, const double* inv_freq, float2* rope) {
+    pdl_wait();
+    pdl_trigger();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (long long)n_pairs * half; i += (long long)gridDim.x * blockDim.x) {
         const int n = (int)(i / half), f = (int)(i % half);
         const int pos = row_of[n];
@@ -462,8 +466,7 @@ cudaError_t pf_launch_t(PfParams& P, int clusters, cudaStream_t st) {
     }
     P.n_tiles = (P.rows + BN - 1) / BN;
     const int units = P.m_tiles * P.n_tiles;
-    prefill_tc_kernel<EPI, BN><<<2u * (unsigned)(units < clusters ? units : clusters), PF_THREADS, smem, st>>>(P);
-    return cudaGetLastError();
+    return launch_pdl(prefill_tc_kernel<EPI, BN>, dim3(2u * (unsigned)(units < clusters ? units : clusters)), dim3(PF_THREADS), smem, st, P);
 }
 
 // Tile width, by the time of the busiest cluster in units of 10 ns a k-block (0.36 us at 256 weight rows, 0.24 at 128; the line
@@ -500,8 +503,7 @@ bool prefill_tc_supported(int d, int kvw) {
 cudaError_t launch_prefill_tc(const PrefillTcArgs& a, cudaStream_t st) {
     const int d = a.d;
     cudaError_t e;
-    prefill_rope_kernel<<<296, 256, 0, st>>>(a.row_of, a.n_pairs, a.dh / 2, a.inv_freq, a.rope);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_pdl(prefill_rope_kernel, dim3(296), dim3(256), 0, st, a.row_of, a.n_pairs, a.dh / 2, a.inv_freq, a.rope)) != cudaSuccess) return e;
     PfParams P;
     memset(&P, 0, sizeof(P));
     // ---- GEMM 1: u = W_fc [h ; E[id]] + rho_0

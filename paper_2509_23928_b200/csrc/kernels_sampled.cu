@@ -17,6 +17,8 @@ __host__ __device__ __forceinline__ int sv_pieces(int V) { return (V + SV_SPAN -
 template <typename LT>
 __global__ void __launch_bounds__(256) row_stats_kernel(const void* target, const float* draft, int n_target, int V,
                                                         float inv_t, float2* part) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ float redf[8];
     const int r = blockIdx.y, c0 = blockIdx.x * SV_SPAN;
     const bool is_t = r < n_target;
@@ -103,6 +105,8 @@ __global__ void __launch_bounds__(SV_THREADS) sampled_verify_kernel(SlotList sl,
                                                                     const float* u_accept, const float* u_sample, int* kv_len,
                                                                     int32_t* out_accept, int32_t* out_next,
                                                                     int32_t* out_kv_len) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ float2 s_st[2 * HIVIS_MAX_K + 1];      // rows 0..k: the target's, k+1..2k: the drafter's
     __shared__ int s_acc[HIVIS_MAX_K], s_n, s_found, s_chunk, s_clast, s_last[SV_THREADS / 32];
     __shared__ double s_sum[SV_MAX_CHUNKS], s_base, s_tot;
@@ -278,17 +282,12 @@ cudaError_t launch_verify_sampled(int logits_dtype, const SlotList& sl, int k, i
     const float inv_t = 1.0f / temperature;
     if ((V + SV_CHUNK - 1) / SV_CHUNK > SV_MAX_CHUNKS) return cudaErrorInvalidValue;
     const dim3 grid((unsigned)sv_pieces(V), (unsigned)(nt + nd));
-    if (logits_dtype == HIVIS_BF16) row_stats_kernel<bf16><<<grid, 256, 0, st>>>(target_logits, draft_logits, nt, V, inv_t, stats);
-    else row_stats_kernel<float><<<grid, 256, 0, st>>>(target_logits, draft_logits, nt, V, inv_t, stats);
-    cudaError_t e = cudaGetLastError();
+    const bool h = logits_dtype == HIVIS_BF16;
+    cudaError_t e = launch_pdl(h ? row_stats_kernel<bf16> : row_stats_kernel<float>, grid, dim3(256), 0, st, target_logits, draft_logits, nt, V,
+                               inv_t, stats);
     if (e != cudaSuccess) return e;
-    if (logits_dtype == HIVIS_BF16)
-        sampled_verify_kernel<bf16><<<B, SV_THREADS, 0, st>>>(sl, k, V, inv_t, draft_ids, draft_logits, target_logits, stats,
-                                                               u_accept, u_sample, kv_len, out_accept, out_next, out_kv_len);
-    else
-        sampled_verify_kernel<float><<<B, SV_THREADS, 0, st>>>(sl, k, V, inv_t, draft_ids, draft_logits, target_logits, stats,
-                                                                u_accept, u_sample, kv_len, out_accept, out_next, out_kv_len);
-    return cudaGetLastError();
+    return launch_pdl(h ? sampled_verify_kernel<bf16> : sampled_verify_kernel<float>, dim3(B), dim3(SV_THREADS), 0, st, sl, k, V, inv_t,
+                      draft_ids, draft_logits, target_logits, stats, u_accept, u_sample, kv_len, out_accept, out_next, out_kv_len);
 }
 
 int sampled_stats_entries(int max_batch, int max_k, int V) { return max_batch * (2 * max_k + 1) * sv_pieces(V); }

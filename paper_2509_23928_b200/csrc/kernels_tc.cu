@@ -17,6 +17,8 @@ cudaError_t tc_launch_t(const TcMaps& maps, const TcArgs& a, int grid, cudaStrea
 __global__ void __launch_bounds__(512) tc_setup_kernel(SlotList sl, int k, int d, int lo, int* d_slots, int* d_pos0, int* kv_len,
                                 const float* pend_feat, const int* pend_id, float* feat, bf16* feat_h, int* cur_id,
                                 u64* keys, int key_stride, const bf16* embed, int vocab, bf16* xe_h, int* id_flag) {
+    pdl_wait();
+    pdl_trigger();
     const int b = blockIdx.x, upr = d >> 3;
     uint4* xe = (uint4*)(xe_h + (long long)b * d);
     if (b >= sl.n) {
@@ -62,9 +64,8 @@ cudaError_t launch_tc_setup(const SlotList& sl, int k, int d, int lo, int* d_slo
                             const float* pend_feat, const int* pend_id, float* feat, bf16* feat_h, int* cur_id,
                             u64* keys, int key_stride, const bf16* embed, int vocab, bf16* xe_h, int* id_flag,
                             cudaStream_t st) {
-    tc_setup_kernel<<<sl.n <= TC_OP_ROWS ? TC_OP_ROWS : HIVIS_MAX_BATCH, 512, 0, st>>>(sl, k, d, lo, d_slots, d_pos0, kv_len, pend_feat, pend_id, feat, feat_h,
-                                                cur_id, keys, key_stride, embed, vocab, xe_h, id_flag);
-    return cudaGetLastError();
+    return launch_pdl(tc_setup_kernel, dim3(sl.n <= TC_OP_ROWS ? TC_OP_ROWS : HIVIS_MAX_BATCH), dim3(512), 0, st, sl, k, d, lo, d_slots, d_pos0, kv_len, pend_feat, pend_id, feat, feat_h,
+                      cur_id, keys, key_stride, embed, vocab, xe_h, id_flag);
 }
 
 // ------------------------------------------------------------------------------------------ host side

@@ -15,6 +15,8 @@
 // ------------------------------------------------------------------------------------------ begin / gather
 __global__ void tree_begin_kernel(int slot, int d, const int* kv_len, const float* pend_feat, const int* pend_id,
                                   float* feat, bf16* feat_h, int* cur_id, int* d_slots, TreeBufs T) {
+    pdl_wait();
+    pdl_trigger();
     if (threadIdx.x == 0) {
         *T.P = kv_len[slot];
         *T.cand_n = 0;
@@ -32,12 +34,13 @@ __global__ void tree_begin_kernel(int slot, int d, const int* kv_len, const floa
 }
 cudaError_t launch_tree_begin(int slot, int d, const int* kv_len, const float* pend_feat, const int* pend_id, float* feat,
                               bf16* feat_h, int* cur_id, int* d_slots, const TreeBufs& T, cudaStream_t st) {
-    tree_begin_kernel<<<1, 256, 0, st>>>(slot, d, kv_len, pend_feat, pend_id, feat, feat_h, cur_id, d_slots, T);
-    return cudaGetLastError();
+    return launch_pdl(tree_begin_kernel, dim3(1), dim3(256), 0, st, slot, d, kv_len, pend_feat, pend_id, feat, feat_h, cur_id, d_slots, T);
 }
 
 // row j of the level's input: the layer output of the forward that proposed node j, and node j's token
 __global__ void tree_gather_kernel(int d, const float* g_prev, TreeBufs T, float* feat, bf16* feat_h, int* cur_id) {
+    pdl_wait();
+    pdl_trigger();
     const int j = blockIdx.x;
     const float* src = g_prev + (long long)T.fr_pslot[j] * d;
     for (int i = threadIdx.x; i < d; i += blockDim.x) {
@@ -49,8 +52,7 @@ __global__ void tree_gather_kernel(int d, const float* g_prev, TreeBufs T, float
 }
 cudaError_t launch_tree_gather(int nb, int d, const float* g_prev, const TreeBufs& T, float* feat, bf16* feat_h, int* cur_id,
                                cudaStream_t st) {
-    tree_gather_kernel<<<nb, 256, 0, st>>>(d, g_prev, T, feat, feat_h, cur_id);
-    return cudaGetLastError();
+    return launch_pdl(tree_gather_kernel, dim3((unsigned)nb), dim3(256), 0, st, d, g_prev, T, feat, feat_h, cur_id);
 }
 
 // The level's rows in the form the tensor-core chain kernel reads them: the features as bf16 rows with their rounding
@@ -61,6 +63,8 @@ cudaError_t launch_tree_gather(int nb, int d, const float* g_prev, const TreeBuf
 __global__ void __launch_bounds__(512) tree_operands_tc_kernel(int nb, int d, int lo_rows, int slot, const int* kv_len,
                                         const float* pend_feat, const int* pend_id, const float* g_prev,
                                         TreeBufs T, const bf16* embed, int vocab, bf16* feat_h, bf16* xe_h, int* id_flag) {
+    pdl_wait();
+    pdl_trigger();
     const int j = blockIdx.x, upr = d >> 3;
     uint4* xe = (uint4*)(xe_h + (long long)j * d);
     if (j >= nb) {
@@ -96,9 +100,7 @@ __global__ void __launch_bounds__(512) tree_operands_tc_kernel(int nb, int d, in
 cudaError_t launch_tree_operands_tc(int nb, int rows, int d, int lo_rows, int slot, const int* kv_len, const float* pend_feat,
                                     const int* pend_id, const float* g_prev, const TreeBufs& T, const bf16* embed, int vocab,
                                     bf16* feat_h, bf16* xe_h, int* id_flag, cudaStream_t st) {
-    tree_operands_tc_kernel<<<rows, 512, 0, st>>>(nb, d, lo_rows, slot, kv_len, pend_feat, pend_id, g_prev, T, embed, vocab,
-                                                  feat_h, xe_h, id_flag);
-    return cudaGetLastError();
+    return launch_pdl(tree_operands_tc_kernel, dim3((unsigned)rows), dim3(512), 0, st, nb, d, lo_rows, slot, kv_len, pend_feat, pend_id, g_prev, T, embed, vocab, feat_h, xe_h, id_flag);
 }
 
 // ------------------------------------------------------------------------------------------ tree attention
@@ -140,6 +142,8 @@ template <typename WT, int DH>
 __global__ void __launch_bounds__(TREE_ATT_WARPS * 32) tree_attn_kernel(const float* qkv, int ld, int Hq, int Hkv, int max_len, int slot,
                                                         int level, TreeBufs T, const double* inv_freq, float scale,
                                                         void* Kc, void* Vc, float* attn, bf16* attn_h, int lo_rows) {
+    pdl_wait();
+    pdl_trigger();
     constexpr int EPL = DH / 32, NT = TREE_ATT_WARPS * 32;
     __shared__ float s_m[TREE_ATT_WARPS], s_l[TREE_ATT_WARPS], s_acc[TREE_ATT_WARPS][DH];
     __shared__ __align__(16) float s_q[DH];
@@ -269,14 +273,9 @@ cudaError_t launch_tree_attention(int dtype, int nb, const float* qkv, int ld, i
     const float scale = 1.0f / sqrtf((float)dh);
     const dim3 grid((unsigned)Hq, (unsigned)nb);
     const int nt = TREE_ATT_WARPS * 32;
-    if (dtype == HIVIS_BF16) {
-        if (dh == 128) tree_attn_kernel<bf16, 128><<<grid, nt, 0, st>>>(qkv, ld, Hq, Hkv, max_len, slot, level, T, inv_freq, scale, Kc, Vc, attn, attn_h, lo_rows);
-        else tree_attn_kernel<bf16, 64><<<grid, nt, 0, st>>>(qkv, ld, Hq, Hkv, max_len, slot, level, T, inv_freq, scale, Kc, Vc, attn, attn_h, lo_rows);
-    } else {
-        if (dh == 128) tree_attn_kernel<float, 128><<<grid, nt, 0, st>>>(qkv, ld, Hq, Hkv, max_len, slot, level, T, inv_freq, scale, Kc, Vc, attn, attn_h, lo_rows);
-        else tree_attn_kernel<float, 64><<<grid, nt, 0, st>>>(qkv, ld, Hq, Hkv, max_len, slot, level, T, inv_freq, scale, Kc, Vc, attn, attn_h, lo_rows);
-    }
-    return cudaGetLastError();
+    auto kernel = dtype == HIVIS_BF16 ? (dh == 128 ? tree_attn_kernel<bf16, 128> : tree_attn_kernel<bf16, 64>)
+                                      : (dh == 128 ? tree_attn_kernel<float, 128> : tree_attn_kernel<float, 64>);
+    return launch_pdl(kernel, grid, dim3(nt), 0, st, qkv, ld, Hq, Hkv, max_len, slot, level, T, inv_freq, scale, Kc, Vc, attn, attn_h, lo_rows);
 }
 
 // ------------------------------------------------------------------------------------------ log-softmax + top-k
@@ -387,6 +386,8 @@ __device__ __forceinline__ bool tree_arrive(int* counter, int count) {
 
 __global__ void __launch_bounds__(256) tree_topk_select_kernel(const float* logits, int V, int topk, int level, int depth,
                                                                float2* piece_stats, u64* piece_keys, TreeBufs T) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ float red[8];
     __shared__ u64 kred[8];
     __shared__ u64 s_keys[TREE_MERGE_CAP];
@@ -484,9 +485,7 @@ __global__ void __launch_bounds__(256) tree_topk_select_kernel(const float* logi
 }
 cudaError_t launch_tree_topk_select(int nb, const float* logits, int V, int topk, int level, int depth, const TreeBufs& T,
                                     cudaStream_t st) {
-    tree_topk_select_kernel<<<dim3((unsigned)tree_topk_pieces(V), (unsigned)nb), 256, 0, st>>>(logits, V, topk, level, depth,
-                                                                                              T.piece_stats, T.piece_keys, T);
-    return cudaGetLastError();
+    return launch_pdl(tree_topk_select_kernel, dim3((unsigned)tree_topk_pieces(V), (unsigned)nb), dim3(256), 0, st, logits, V, topk, level, depth, T.piece_stats, T.piece_keys, T);
 }
 
 // ------------------------------------------------------------------------------------------ final ranking
@@ -494,6 +493,8 @@ cudaError_t launch_tree_topk_select(int nb, const float* logits, int V, int topk
 // listed in creation order, parents re-numbered within the list.
 __global__ void __launch_bounds__(1024) tree_finalize_kernel(int keep, TreeBufs T, int32_t* out_tokens, int32_t* out_parents,
                                                              float* out_scores, int32_t* out_count) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ float s_score[TREE_MAX_CAND];
     __shared__ unsigned short s_pos[TREE_MAX_CAND];          // 1 + position among the kept, 0 = not kept
     __shared__ int s_sum[32];
@@ -543,13 +544,14 @@ __global__ void __launch_bounds__(1024) tree_finalize_kernel(int keep, TreeBufs 
 }
 cudaError_t launch_tree_finalize(int keep, const TreeBufs& T, int32_t* out_tokens, int32_t* out_parents, float* out_scores,
                                  int32_t* out_count, cudaStream_t st) {
-    tree_finalize_kernel<<<1, 1024, 0, st>>>(keep, T, out_tokens, out_parents, out_scores, out_count);
-    return cudaGetLastError();
+    return launch_pdl(tree_finalize_kernel, dim3(1), dim3(1024), 0, st, keep, T, out_tokens, out_parents, out_scores, out_count);
 }
 
 // ------------------------------------------------------------------------------------------ verification
 template <typename LT>
 __global__ void __launch_bounds__(256) tree_row_argmax_kernel(const void* logits, int V, u64* keys) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ u64 kred[8];
     const LT* row = (const LT*)logits + (long long)blockIdx.y * V;
     const int c0 = blockIdx.x * 2048, c1 = min(V, c0 + 2048);
@@ -581,6 +583,8 @@ template <typename WT>
 __global__ void __launch_bounds__(256) tree_walk_kernel(int slot, int depth, int Hkv, int dh, int max_len, TreeBufs T,
                                                         const u64* keys, void* Kc, void* Vc, int* kv_len, int32_t* out_accept,
                                                         int32_t* out_path, int32_t* out_next, int32_t* out_kv_len) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ int s_path[TREE_MAX_DEPTH], s_src[TREE_MAX_DEPTH], s_rows;
     __shared__ int s_tok[HIVIS_TREE_MAX_KEEP], s_par[HIVIS_TREE_MAX_KEEP], s_store[HIVIS_TREE_MAX_KEEP], s_arg[HIVIS_TREE_MAX_KEEP + 1];
     const int n = *T.kept_n, P = *T.P, lane = threadIdx.x & 31;
@@ -640,13 +644,8 @@ cudaError_t launch_tree_verify(int dtype, int logits_dtype, int slot, int depth,
     cudaError_t e = cudaMemsetAsync(T.row_keys, 0, sizeof(u64) * rows, st);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)((V + 2047) / 2048), (unsigned)rows);
-    if (logits_dtype == HIVIS_BF16) tree_row_argmax_kernel<bf16><<<grid, 256, 0, st>>>(logits, V, T.row_keys);
-    else tree_row_argmax_kernel<float><<<grid, 256, 0, st>>>(logits, V, T.row_keys);
-    e = cudaGetLastError();
+    e = launch_pdl(logits_dtype == HIVIS_BF16 ? tree_row_argmax_kernel<bf16> : tree_row_argmax_kernel<float>, grid, dim3(256), 0, st, logits, V, T.row_keys);
     if (e != cudaSuccess) return e;
-    if (dtype == HIVIS_BF16)
-        tree_walk_kernel<bf16><<<TREE_WALK_CTAS, 256, 0, st>>>(slot, depth, Hkv, dh, max_len, T, T.row_keys, Kc, Vc, kv_len, out_accept, out_path, out_next, out_kv_len);
-    else
-        tree_walk_kernel<float><<<TREE_WALK_CTAS, 256, 0, st>>>(slot, depth, Hkv, dh, max_len, T, T.row_keys, Kc, Vc, kv_len, out_accept, out_path, out_next, out_kv_len);
-    return cudaGetLastError();
+    return launch_pdl(dtype == HIVIS_BF16 ? tree_walk_kernel<bf16> : tree_walk_kernel<float>, dim3(TREE_WALK_CTAS), dim3(256), 0, st, slot, depth, Hkv, dh, max_len, T, T.row_keys, Kc, Vc, kv_len,
+                      out_accept, out_path, out_next, out_kv_len);
 }

@@ -1348,6 +1348,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_chain_kernel(const __grid_co
     __syncthreads();
     tc_fence_after();
 
+    pdl_trigger();              // (the launch after this one is set up as CTAs leave)
     // the split of the attention units (the same for every step) and this CTA's ring items per step
     const TcAttInfo ai = tc_att_info<GQ>(a, cta, G);
     if (warp == 0) {
