@@ -89,34 +89,54 @@ enum { CW_FCH = 0, CW_FCE, CW_QKV, CW_O, CW_GU, CW_DOWN, CW_LM, CW_COUNT };
 struct ChainSeg {
     const char* base;          // this CTA's first row, first column of the part
     long long ld;              // bytes from row to row
-    int row0, rows;            // rows of this CTA
+    int rows;                  // rows of this CTA
     int K;                     // columns of the part
-    int cpr;                   // chunks per row of the part
-    int slot0, slots;          // partial sums: chunk slots of a row, the first of this part
 };
+__device__ __forceinline__ int chain_phase(int w) { return w == CW_FCH ? PH_FC : w - 1; }
 
 // A warp's place in its units of a part.  A warp keeps to one chunk of the columns where the number of chunks divides the
 // number of warps, else it has a run of the units taken chunk by chunk.
-struct alignas(16) ChainCursor {
+struct ChainCursor {
     int row, ch, left, step;
-    __device__ void begin(const ChainSeg& g, int warp) {
-        if (CHAIN_WARPS % g.cpr == 0) {
-            step = CHAIN_WARPS / g.cpr;
-            ch = warp % g.cpr;
-            row = warp / g.cpr;
-            left = row < g.rows ? (g.rows - 1 - row) / step + 1 : 0;
+    __device__ void begin(int rows, int cpr, int warp) {
+        if (CHAIN_WARPS % cpr == 0) {
+            step = CHAIN_WARPS / cpr;
+            ch = warp % cpr;
+            row = warp / cpr;
+            left = row < rows ? (rows - 1 - row) / step + 1 : 0;
         } else {
-            const int U = g.rows * g.cpr, u0 = U * warp / CHAIN_WARPS;
+            const int U = rows * cpr, u0 = U * warp / CHAIN_WARPS;
             step = 1;
-            ch = g.rows > 0 ? u0 / g.rows : 0;
-            row = u0 - ch * g.rows;
+            ch = rows > 0 ? u0 / rows : 0;
+            row = u0 - ch * rows;
             left = U * (warp + 1) / CHAIN_WARPS - u0;
         }
     }
-    __device__ __forceinline__ void next(const ChainSeg& g) {
+    __device__ __forceinline__ void next(int rows) {
         --left;
         row += step;
-        if (row >= g.rows) { row = 0; ++ch; }        // (not reached by warps that keep to a chunk: none is left)
+        if (row >= rows) { row = 0; ++ch; }          // (not reached by warps that keep to a chunk: none is left)
+    }
+};
+// Every warp's place at the start of every part, worked out once per launch: lane w of the warp keeps that of part w, in 16 bits
+// a number (a CTA's units of a part have a partial sum each in shared memory, so there are fewer than 65536).  It is in registers
+// because shared memory is full: a table of it, and of the parts, took 2 KB from x, and drafters with the widest feed-forward
+// layers that had fitted did not fit any more.  A round of four steps at d 256: 116 us with the table, 112 with this; d 4096 level.
+struct ChainFirst {
+    uint32_t a, b;
+    __device__ __forceinline__ void set(const ChainCursor& c) {
+        a = (uint32_t)c.row | (uint32_t)c.ch << 16;
+        b = (uint32_t)c.left | (uint32_t)c.step << 16;
+    }
+    // (all lanes of the warp)
+    __device__ __forceinline__ ChainCursor get(int w) const {
+        const uint32_t x = __shfl_sync(0xffffffffu, a, w), y = __shfl_sync(0xffffffffu, b, w);
+        ChainCursor c;
+        c.row = (int)(x & 0xffffu);
+        c.ch = (int)(x >> 16);
+        c.left = (int)(y & 0xffffu);
+        c.step = (int)(y >> 16);
+        return c;
     }
 };
 // A warp's stream of units: how many it has asked for and used, and the next one to ask for.
@@ -129,10 +149,23 @@ struct ChainMisc {
     float red[CHAIN_WARPS];
     u64 kred[CHAIN_WARPS];
     int abort_flag;
-    ChainSeg seg[CW_COUNT];
-    ChainCursor first[CW_COUNT][CHAIN_WARPS];      // every warp's place at the start of every part
+    int row0[PH_COUNT], rows[PH_COUNT];            // this CTA's rows of every phase
     u64 bar_base;              // value of the barrier counter when the launch began
 };
+// What the plan sets aside for it, beside x: it decides how wide a feed-forward layer fits, and with it which drafters run here.
+#define CHAIN_MISC_BYTES 280
+static_assert(sizeof(ChainMisc) <= CHAIN_MISC_BYTES, "");
+// The rows of a part that are this CTA's (kh: columns of the fusion FC in its first part).
+template <typename WT>
+__device__ __forceinline__ ChainSeg chain_seg(const ChainArgs& a, const ChainMisc* misc, int w, int kh) {
+    const int p = chain_phase(w), K = a.ph[p].K;
+    ChainSeg g;
+    g.ld = (long long)K * (int)sizeof(WT);
+    g.base = (const char*)a.ph[p].W + misc->row0[p] * g.ld + (w == CW_FCE ? (long long)kh * (int)sizeof(WT) : 0ll);
+    g.rows = misc->rows[p];
+    g.K = w == CW_FCH ? kh : w == CW_FCE ? K - kh : K;
+    return g;
+}
 
 // CTA barrier; true, for all threads alike, while no wait of the CTA has run out.
 __device__ __forceinline__ bool cta_alive(const ChainMisc* misc) {
@@ -198,27 +231,28 @@ __device__ __forceinline__ float dot_chunk(const uint4* wsm, const float* xs, in
 }
 
 // Asks for the warp's next unit (lane 0 issues; every lane tracks the cursor).
-__device__ __forceinline__ void chain_fetch(ChainStream& t, const ChainMisc* misc, int k, int es, uint32_t ring0, uint32_t bar0, u64 pol,
-                                            int warp, int lane) {
+template <typename WT>
+__device__ __forceinline__ void chain_fetch(ChainStream& t, const ChainArgs& a, const ChainMisc* misc, const ChainFirst& first, int kh,
+                                            uint32_t ring0, uint32_t bar0, u64 pol, int lane) {
     while (t.at.left == 0) {
         if (++t.w == CW_COUNT) {
             t.w = 0;
             ++t.step;
         }
-        if (t.step >= k) return;
-        t.at = misc->first[t.w][warp];
+        if (t.step >= a.k) return;
+        t.at = first.get(t.w);
     }
-    if (t.step >= k) return;
-    const ChainSeg& g = misc->seg[t.w];
+    if (t.step >= a.k) return;
+    const ChainSeg g = chain_seg<WT>(a, misc, t.w, kh);
     if (lane == 0) {
         const unsigned st = t.fi % CHAIN_STAGES;
         const uint32_t bar = bar0 + st * 8;
-        const uint32_t bytes = (uint32_t)min(CHAIN_CHUNK_BYTES, g.K * es - t.at.ch * CHAIN_CHUNK_BYTES);
+        const uint32_t bytes = (uint32_t)min(CHAIN_CHUNK_BYTES, g.K * (int)sizeof(WT) - t.at.ch * CHAIN_CHUNK_BYTES);
         mbar_expect_tx(bar, bytes);
         bulk_g2s(ring0 + st * CHAIN_CHUNK_BYTES, g.base + t.at.row * g.ld + t.at.ch * CHAIN_CHUNK_BYTES, bytes, bar, pol);
     }
     ++t.fi;
-    t.at.next(g);
+    t.at.next(g.rows);
 }
 
 // ---- attention -----------------------------------------------------------------------------------
@@ -455,7 +489,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
 
     if (tid < PH_COUNT) {
         const int p = tid;
-        const long long N = a.ph[p].N, K = a.ph[p].K;
+        const long long N = a.ph[p].N;
         long long r0, r1;
         if (p == PH_GU) {                                // keep (gate_i, up_i) row pairs together
             r0 = 2 * ((N / 2) * cta / G);
@@ -464,29 +498,8 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
             r0 = N * cta / G;
             r1 = N * (cta + 1) / G;
         }
-        ChainSeg g;
-        g.base = (const char*)a.ph[p].W + r0 * K * ES;
-        g.ld = K * ES;
-        g.row0 = (int)r0;
-        g.rows = (int)(r1 - r0);
-        g.slots = (int)((K * ES + CHAIN_CHUNK_BYTES - 1) / CHAIN_CHUNK_BYTES);
-        if (p == PH_FC) {
-            g.K = kh;
-            g.cpr = kh / CE > 0 ? kh / CE : 1;
-            g.slot0 = 0;
-            misc->seg[CW_FCH] = g;
-            if (kh == 0) misc->seg[CW_FCH].rows = 0;
-            g.base += (long long)kh * ES;
-            g.K = (int)K - kh;
-            g.cpr = g.slots - kh / CE;
-            g.slot0 = kh / CE;
-            misc->seg[CW_FCE] = g;
-        } else {
-            g.K = (int)K;
-            g.cpr = g.slots;
-            g.slot0 = 0;
-            misc->seg[CW_FCE + p] = g;
-        }
+        misc->row0[p] = (int)r0;
+        misc->rows[p] = (int)(r1 - r0);
     } else if (tid == 32) {
         misc->abort_flag = 0;
         misc->bar_base = barrier_base(a.bar_counter, (unsigned)G) + a.bar_off;
@@ -496,7 +509,18 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
         fence_proxy_async();
     }
     __syncthreads();
-    if (lane < CW_COUNT) misc->first[lane][warp].begin(misc->seg[lane], warp);
+    // chunks of a row of part w: those that the hidden part of the fusion FC leaves are the other part's
+    auto chunks = [&](int w) {
+        const int all = (a.ph[chain_phase(w)].K * ES + CHAIN_CHUNK_BYTES - 1) / CHAIN_CHUNK_BYTES;
+        return w == CW_FCH ? max(kh / CE, 1) : w == CW_FCE ? all - kh / CE : all;
+    };
+    ChainFirst first;
+    {
+        const int w = min(lane, CW_COUNT - 1);
+        ChainCursor c;
+        c.begin(w == CW_FCH && kh == 0 ? 0 : misc->rows[chain_phase(w)], chunks(w), warp);
+        first.set(c);
+    }
     __syncwarp();
 
     pdl_trigger();                                          // (the launch after this one is set up as CTAs leave)
@@ -511,8 +535,8 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
     ChainStream t;
     t.fi = t.ci = 0;
     t.step = t.w = 0;
-    t.at = misc->first[0][warp];
-    for (int i = 0; i < CHAIN_STAGES; ++i) chain_fetch(t, misc, a.k, ES, ring0, bar0, pol, warp, lane);
+    t.at = first.get(0);
+    for (int i = 0; i < CHAIN_STAGES; ++i) chain_fetch<WT>(t, a, misc, first, kh, ring0, bar0, pol, lane);
 
     u64 bar_target = misc->bar_base;                        // of the newest barrier that this CTA has arrived on
     bool alive = true;
@@ -537,8 +561,8 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
     int s = 0, w = CW_FCH;
 #pragma unroll 1
     for (; s < a.k; s += w == CW_LM ? 1 : 0, w = w == CW_LM ? CW_FCH : w + 1) {
-        const ChainSeg& g = misc->seg[w];
-        const int K = g.K;
+        const int ph = chain_phase(w), rows = misc->rows[ph], r0 = misc->row0[ph];
+        const int K = w == CW_FCH ? kh : w == CW_FCE ? 2 * d - kh : a.ph[ph].K;
         // ------------------------------------------------------------ x of the part
         if (w == CW_FCH) {
             // the hidden half of the fusion FC: behind the LM head x is still the layer output
@@ -649,8 +673,8 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
             }
             __syncthreads();
         }
+        const int slots = (a.ph[ph].K * ES + CHAIN_CHUNK_BYTES - 1) / CHAIN_CHUNK_BYTES;   // partial sums of a row
         // what the output of this thread's row is added to
-        const int r0 = g.row0;
         const float* const add = w == CW_O ? a.u : a.y;
         const long long rho_row = (long long)(s < a.n_resid - 1 ? s : a.n_resid - 1) * d;
         auto addend = [&](int r) {
@@ -659,10 +683,11 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
             return __ldcg(add + r);
         };
         float first_add = 0.f;
-        if (w != CW_FCH && w != CW_GU && w != CW_LM && tid < g.rows) first_add = addend(r0 + tid);
+        if (w != CW_FCH && w != CW_GU && w != CW_LM && tid < rows) first_add = addend(r0 + tid);
         // ------------------------------------------------------------ this warp's units: partial dot products into part[row][slot]
         {
-            ChainCursor c = misc->first[w][warp];
+            ChainCursor c = first.get(w);
+            float* const part_w = part + (w == CW_FCE ? kh / CE : 0);
             int have = -1, nvec = 0;
             bool gave_up = false;
 #pragma unroll 1
@@ -687,31 +712,30 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
                 }
                 if (__any_sync(0xffffffffu, gave_up)) break;        // one answer for the warp
                 const float acc = dot_chunk<WT>((const uint4*)(stages + st * CHAIN_CHUNK_BYTES), xs, K, have * CE, nvec, lane);
-                if (lane == 0) part[c.row * g.slots + g.slot0 + c.ch] = acc;
+                if (lane == 0) part_w[c.row * slots + c.ch] = acc;
                 ++t.ci;
                 __syncwarp();
                 fence_proxy_async();                        // our reads of the stage precede its refill
-                chain_fetch(t, misc, a.k, ES, ring0, bar0, pol, warp, lane);
-                c.next(g);
+                chain_fetch<WT>(t, a, misc, first, kh, ring0, bar0, pol, lane);
+                c.next(rows);
             }
         }
         if (w == CW_FCH) continue;                          // (its partial sums wait for those of the other half)
         if (!(alive = cta_alive(misc))) break;
         // ------------------------------------------------------------ output stage
-        const int slots = g.slots;
         auto row_sum = [&](int rl) {                        // add a row's chunk partials in chunk order
             float v = 0.f;
             for (int q = 0; q < slots; ++q) v += part[rl * slots + q];
             return v;
         };
         if (w == CW_GU) {
-            for (int pl = tid; pl < g.rows / 2; pl += CHAIN_THREADS) {
+            for (int pl = tid; pl < rows / 2; pl += CHAIN_THREADS) {
                 const float gate = row_sum(2 * pl), up = row_sum(2 * pl + 1);
                 a.act[r0 / 2 + pl] = gate / (1.f + expf(-gate)) * up;
             }
         } else if (w == CW_LM) {
             u64 best = 0;
-            for (int rl = tid; rl < g.rows; rl += CHAIN_THREADS) {
+            for (int rl = tid; rl < rows; rl += CHAIN_THREADS) {
                 const float v = row_sum(rl);
                 if (a.logits_out) a.logits_out[(long long)s * a.V + r0 + rl] = v;
                 const u64 key = a.gumbel_u ? pack_key(gumbel_perturbed(v, a.inv_t, __ldg(a.gumbel_u + (long long)s * a.V + r0 + rl)), r0 + rl)
@@ -733,7 +757,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
             }
         } else {
             float* const out = w == CW_FCE ? a.u : w == CW_QKV ? a.qkv : w == CW_O ? a.y : a.feat;
-            for (int rl = tid; rl < g.rows; rl += CHAIN_THREADS) out[r0 + rl] = row_sum(rl) + (rl == tid ? first_add : addend(r0 + rl));
+            for (int rl = tid; rl < rows; rl += CHAIN_THREADS) out[r0 + rl] = row_sum(rl) + (rl == tid ? first_add : addend(r0 + rl));
         }
         arrive();
     }
@@ -780,7 +804,7 @@ static ChainPlan chain_plan(const ChainArgs& a, int es, int dh, int grid) {
     // the attention stages up to CHAIN_ATTN_ROWS rows of K and V, as many as fit beside the rest
     const size_t fixed = dh == 128 ? sizeof(ChainAttnSmem<float, 128>) : sizeof(ChainAttnSmem<float, 64>);
     const size_t row = (size_t)(2 * dh * es + 16);
-    const size_t other = (size_t)CHAIN_WARPS * CHAIN_STAGES * (CHAIN_CHUNK_BYTES + 8) + (size_t)slots * 4 + sizeof(ChainMisc) + 512;
+    const size_t other = (size_t)CHAIN_WARPS * CHAIN_STAGES * (CHAIN_CHUNK_BYTES + 8) + (size_t)slots * 4 + CHAIN_MISC_BYTES + 512;
     const size_t room = (size_t)227 * 1024 > other ? (size_t)227 * 1024 - other : 0;
     size_t want = fixed + CHAIN_ATTN_ROWS * row;
     if (want > room) want = room;
@@ -795,7 +819,7 @@ static ChainPlan chain_plan(const ChainArgs& a, int es, int dh, int grid) {
     off += CHAIN_WARPS * CHAIN_STAGES * 8;
     off = (off + 15) & ~(size_t)15;
     p.off_misc = (int)off;
-    off += sizeof(ChainMisc);
+    off += CHAIN_MISC_BYTES;
     p.smem_bytes = off;
     return p;
 }
