@@ -124,11 +124,14 @@ static char g_init_err[256] = "";
 // text for failures of calls that have no context; hivis_last_error(NULL) returns it
 void hivis_set_global_error(const char* msg) { snprintf(g_init_err, sizeof(g_init_err), "%s", msg); }
 
+// A failure is taken out of the runtime's last error as it is reported: launches made with <<<>>> read that, in later calls.
 #define CK(c, call)                                                                            \
     do {                                                                                       \
         cudaError_t e_ = (call);                                                               \
-        if (e_ != cudaSuccess)                                                                 \
+        if (e_ != cudaSuccess) {                                                               \
+            cudaGetLastError();                                                                \
             return fail(c, HIVIS_ERR_CUDA, "%s failed: %s", #call, cudaGetErrorString(e_));    \
+        }                                                                                      \
     } while (0)
 #define CKL(c, call)            \
     do {                        \
