@@ -5,7 +5,8 @@ from types import SimpleNamespace
 import pytest
 
 pytestmark = pytest.mark.gpu
-SHAPES = {"heads of 128": (20, 4, 128), "heads of 64": (12, 2, 64), "few heads": (4, 2, 64)}
+# "many heads": more units than CTAs, so a CTA stages one after the other (n up to 128; longer caches are not staged)
+SHAPES = {"heads of 128": (20, 4, 128), "heads of 64": (12, 2, 64), "few heads": (4, 2, 64), "many heads": (336, 48, 64)}
 
 
 # lengths: one row; the edges of a warp's block and of a split; units that are staged and units that are not (more than 128 rows: 1000

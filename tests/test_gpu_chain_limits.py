@@ -1,4 +1,5 @@
-"""One sequence at the widest feed-forward layer that the one-sequence chain kernel takes, against the oracle."""
+"""One sequence at the edges of the one-sequence chain kernel, against the oracle: the widest feed-forward layer that it takes, and the
+widths at which the fusion FC is cut in two."""
 from dataclasses import replace
 
 import numpy as np
@@ -37,5 +38,20 @@ def test_widest_feed_forward_layer(dtype):
         err = np.abs(logits[0].cpu().numpy() - ref[0]["logits"]).max(-1) / np.abs(ref[0]["logits"]).max(-1)
         assert err.max() <= (LOGIT_RTOL_F32 if dtype == "f32" else LOGIT_RTOL)
         dr.status()
+    finally:
+        case.close()
+
+
+@pytest.mark.parametrize("dtype,d", [("f32", 1000), ("f32", 1024), ("f32", 1280), ("f32", 2560), ("bf16", 2048), ("bf16", 2560)])
+def test_fusion_in_two_parts(dtype, d):
+    """The part of the hidden half that is used behind the LM head is whole chunks of 4 KB: none of it, all of it, some of it (fp32 1280
+    and 2560: 1024 and 2048 columns)."""
+    base = hi.workload("c1_tiny_f32_b1")
+    wl = hi.scaled(base, dims=replace(base.dims, d=d, vocab=1000, dtype=dtype), k=4)
+    case = Case(wl)
+    try:
+        res = check_draft_parity(case, rtol=LOGIT_RTOL_F32 if dtype == "f32" else LOGIT_RTOL)
+        check_kv_parity(case, res["ref"])
+        case.drafter.status()
     finally:
         case.close()
