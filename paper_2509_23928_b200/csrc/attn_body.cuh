@@ -1,5 +1,5 @@
 // Body of the split-KV decode attention, shared by the stand-alone kernel (4 warps per unit) and the
-// persistent chain kernel (8 warps per unit).  One call handles one unit = (split of the cache rows,
+// one-sequence chain kernel (16 warps per unit).  One call handles one unit = (split of the cache rows,
 // group of GQ query heads on one KV head, sequence); every thread of the CTA must make the call.
 #pragma once
 #include "hivis_internal.cuh"

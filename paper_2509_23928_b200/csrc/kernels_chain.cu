@@ -781,7 +781,10 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1) draft_chain_kernel(const Cha
 }
 
 // ------------------------------------------------------------------------------------------ host side
-#define CHAIN_ATTN_ROWS 128     // cache rows of a unit that are staged (a head's 600 rows at 32 heads, with four units each)
+// Cache rows of a unit that are staged, at most.  With 32 heads a head has four units, of a quarter of the rows in whole blocks of 32:
+// all of up to 512 rows in bf16, and at d 4096 in fp32, where x leaves room for 84, of up to 256.  Longer ones are attn_unit's: five
+// steps at d 4096 take 661 us at 128 to 512 rows, 709 from 513 on, 725 at 1024.
+#define CHAIN_ATTN_ROWS 128
 struct ChainPlan {
     int off_x, off_part, off_bar, off_misc;
     int attn_rows;             // rows of K and V that the room of x holds

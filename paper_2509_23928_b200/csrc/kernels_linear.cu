@@ -382,7 +382,7 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], unsigned a0, unsigned a1
 template <int NI, int PRO, int EPI>
 __global__ void __launch_bounds__(256) gemm_mma_kernel(const LinArgs a) {
     constexpr int MI = HIVIS_MMA_TILE_ROWS / 16;
-    // k-blocks per batch of loads, two batches in flight: 64 KB per CTA.  With two k-blocks, all used before the next were asked for,
+    // k-blocks per batch of loads: 64 KB per CTA, and two batches in flight.  With two k-blocks, all used before the next were asked for,
     // and launches that began when the one before was over, the prefix rows of 1..16 pairs (d 4096) took 81..99 us; now 66..75.
     constexpr int U = 4;
     __shared__ float red[8][NI * 8][MI * 16 + 1];

@@ -474,7 +474,7 @@ cudaError_t pf_launch_t(PfParams& P, int clusters, cudaStream_t st) {
 // 65 / 87 us (d 4096), 72 / 103 (d 3584), 58 / 69 (d 2560); 512 pairs 85 / 98, 84 / 99, 60 / 74; 600 pairs 123 / 114, 113 / 101,
 // 59 / 76; 2048 pairs 260 / 226, 144 / 130, 96 / 102.
 // A tile is never split over clusters, and no call goes through the chain kernel, whose phases are split over CTAs (64 pairs:
-// 45 us there, 89 here): u and the cached rows are rounded to bf16, and parts of their long sums added in fp32 instead of
+// 45 us there, 61 here): u and the cached rows are rounded to bf16, and parts of their long sums added in fp32 instead of
 // in the tensor core's accumulator move one element in forty to the other side of a rounding.  Two to eleven of a hundred
 // cached elements then differ, enough to exchange nodes of a draft tree and to move a token drawn by inverse CDF.
 template <int EPI>
