@@ -57,7 +57,7 @@
 #define TC_TM 128
 // Geometry by the number NG of 16-sequence column groups of the launch.
 //   NG = 1 (up to 16 sequences): 32 batch columns, [0,16) the activations rounded to bf16, [16,32) their rounding
-//          remainders (an MMA of this shape costs the same for 16 and for 32 columns).
+//          remainders.
 //   NG = 2 (17..32), NG = 4 (33..64): 16 NG columns of rounded activations, no remainders.  For 64 columns the operand
 //          tile is 8 KB beside the 16 KB of weights, so the ring has nine stages instead of eleven; its bytes of weights
 //          in flight (9 x 16 KB x 148 SMs) are still three times what the memory's latency asks for.  One pass over the
@@ -249,8 +249,8 @@ __device__ __forceinline__ void phase_stamp(const TcArgs& a, int s, int e, int c
 // One thread of a converged warp, by elect.sync: the compiler then knows that a single thread runs what follows and issues
 // tcgen05 and bulk-copy instructions back to back.  Under a test of the lane number an MMA costs 53 clocks to issue (64 with a
 // commit for every four), whatever its shape; under this one the tensor core sets the pace (128 x 32 x 16: 44 clocks with the
-// commits).  Batch 16 at d 4096, five steps and refresh: 1028 -> 977 us with 64..512 rows, 1141 -> 1087 with 704; 64 sequences
-// 1514 -> 1431.
+// commits; not measured again for 16 columns).  Batch 16 at d 4096, five steps and refresh: 1028 -> 977 us with 64..512 rows,
+// 1141 -> 1087 with 704; 64 sequences 1514 -> 1431.
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
     __syncwarp();
@@ -1352,7 +1352,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_chain_kernel(const __grid_co
     // the split of the attention units (the same for every step) and this CTA's ring items per step
     const TcAttInfo ai = tc_att_info<GQ>(a, cta, G);
     if (warp == 0) {
-        if (elect_one()) tc_producer_w<DH, GQ, NG>(P, ctl, smemA, cta, G, ai);
+        // Elected for single heads, by lane number for groups of seven.  Elected, the producers of the SMs get farther apart where only
+        // weights are streamed (the Qwen shape's LM head: first to last arrival 22 us, 13 by lane number), and keep up better
+        // with the K/V blocks of single heads.  By lane number / elected, drafts alone: Qwen shape, 8 sequences of 256 rows, seven
+        // steps 1947 / 1975 us, of 704 rows 1958 / 1996, 16 of 128, five steps 1409 / 1422, 24 ragged 1465 / 1487, 64 of 300 level;
+        // single heads at d 4096, five steps: 16 sequences of 128 rows 770 / 779, of 704 rows 1010 / 996, ragged level, 32 of 704
+        // 1280 / 1245, 64 ragged level.
+        if constexpr (GQ == 1) {
+            if (elect_one()) tc_producer_w<DH, GQ, NG>(P, ctl, smemA, cta, G, ai);
+        } else {
+            if (lane == 0) tc_producer_w<DH, GQ, NG>(P, ctl, smemA, cta, G, ai);
+        }
         __syncwarp();
     } else if (warp == 1) {
         if (elect_one()) {
